@@ -269,9 +269,9 @@ int bt_prefix_fingerprints(const uint8_t* d_text, uint64_t n, uint64_t seed, uin
  * synchronisation or its failure.
  *
  * Same arguments, results and stream semantics as bt_prefix_fingerprints.
- * The caller still provides d_text and d_out.  The scratch (power tables and
- * per-CTA aggregates) is a fixed 528 KiB array in device memory, which every
- * GPU that loads the library holds until the process exits.  The entry point
+ * The caller still provides d_text and d_out.  The scratch (per-tile
+ * totals) is a fixed 512 KiB array in device memory, which every GPU that
+ * loads the library holds until the process exits.  The entry point
  * calls no cudaMalloc, cudaFree or allocating library routine.
  *  - n may be at most 2^31 (2 GiB); larger texts return BT_ERANGE before any
  *    other check and before any work is queued.

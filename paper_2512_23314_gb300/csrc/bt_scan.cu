@@ -2,16 +2,17 @@
 //
 //  * scan_u32 / scan_u64: exclusive prefix sums (rank support of the mark
 //    bit vectors, job offsets).
+//    Three passes: a CTA-local scan of 1024 items, a single-CTA scan of the
+//    CTA aggregates, and a pass that adds each CTA's prefix to its items.
 //  * prefix_fingerprints: the Karp-Rabin prefix H(32 j) of the whole text
 //    (section 2 defines phi; Lemmas 7 and 8 of section 4.1 compute all
-//    fingerprints with an all-prefix operation).  Each 32-byte chunk is hashed
-//    by Horner, then the chunks are combined with the associative operator
+//    fingerprints with an all-prefix operation).  The 32-byte chunks are
+//    hashed and combined with the associative operator
 //    (h1, P1) (x) (h2, P2) = (h1 * P2 + h2, P1 * P2) of the all-prefix lemma
 //    (Lemma 1); every chunk has the same length, so P is a power of
-//    B^32 determined by the number of chunks combined and is read from a
-//    table instead of being carried.
-// Three passes: a CTA-local scan of 1024 items, a single-CTA scan of the CTA
-// aggregates, and a pass that folds each CTA's prefix into its items.
+//    B^32 determined by the number of chunks combined: a tree or a scan needs
+//    only its squares.  Tile totals, a single-CTA scan of them, then a pass
+//    that computes every chunk's prefix from its tile's.
 #include <cstdio>
 #include <mutex>
 
@@ -106,129 +107,283 @@ int scan_sum(const T* in, T* out, uint64_t n, cudaStream_t s) {
 
 // ---------------------------------------------------------------------------
 // Karp-Rabin all-prefix.
+//
+// Bound: the text once per pass (twice in all) and n/4 bytes written.  A
+// Horner step is a 61-bit product (about 20 instructions) per byte; instead a
+// 32-byte chunk is the dot product of its bytes with the powers B^31 .. B^0,
+// whose eight 8-bit limbs are constants: two 4-way byte products (__dp4a)
+// per byte and one reduction per chunk.  A thread takes four chunks, so that
+// the scan's products (about eight per thread) are shared by 128 bytes.  The
+// CTA totals come from a pass of their own and the text is read again: the
+// pass that writes then writes final values, instead of local ones that a
+// third pass reads, corrects and writes once more.  The second pass takes
+// the tiles from the last to the first, so that it starts with the text the
+// first pass left in L2.
+// Measured on 256 MiB + 77, the whole call: 548 us with a Horner pass that
+// wrote local values (454), their totals (33) and a correcting pass (32); 169
+// us now.
 // ---------------------------------------------------------------------------
+constexpr int kKrThreads = 256;    // threads of a tile of kTile chunks
+constexpr int kKrChunks = 4;       // chunks per thread
+static_assert(kKrThreads * kKrChunks == kTile, "a tile is kTile chunks");
 
-// Inclusive scan of chunk fingerprints within a CTA.  pw[i] = X^i, where X
-// is B raised to the length of one item, for i <= 1024.
+// Powers of the shift X of one scan item: X^1,2,4,8,16 within a warp and
+// X^32,64,..,512 across the warps.
+struct KrPow {
+  uint64_t x[5], w[5];
+};
 template <class M>
-__device__ uint64_t cta_kr_scan(const M& m, uint64_t h, const uint64_t* __restrict__ pw,
-                                uint64_t* sm) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int d = 1; d < 32; d <<= 1) {
-    uint64_t o = __shfl_up_sync(0xFFFFFFFFu, h, d);
-    if (lane >= d) h = m.add(m.mul(o, pw[d]), h);
+KrPow kr_pow(const M& m, uint64_t X) {
+  KrPow p;
+  for (int i = 0; i < 5; i++) {
+    p.x[i] = X;
+    X = m.mul(X, X);
+  }
+  for (int i = 0; i < 5; i++) {
+    p.w[i] = X;
+    X = m.mul(X, X);
+  }
+  return p;
+}
+
+// Inclusive scan of the items' fingerprints over a CTA of at most 1024
+// threads (sm: 32 words).
+template <class M>
+__device__ __forceinline__ uint64_t cta_kr_scan(const M& m, uint64_t h, const KrPow& pw, uint64_t xl, uint64_t* sm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 5; i++) {
+    const uint64_t o = __shfl_up_sync(0xFFFFFFFFu, h, 1 << i);
+    if (lane >= (1 << i)) h = m.add(m.mul(o, pw.x[i]), h);
   }
   if (lane == 31) sm[warp] = h;
   __syncthreads();
   if (warp == 0) {
-    uint64_t w = sm[lane];
-    for (int d = 1; d < 32; d <<= 1) {
-      uint64_t o = __shfl_up_sync(0xFFFFFFFFu, w, d);
-      if (lane >= d) w = m.add(m.mul(o, pw[32 * d]), w);
+    uint64_t w = lane < nw ? sm[lane] : 0;
+#pragma unroll
+    for (int i = 0; i < 5; i++) {
+      const uint64_t o = __shfl_up_sync(0xFFFFFFFFu, w, 1 << i);
+      if (lane >= (1 << i)) w = m.add(m.mul(o, pw.w[i]), w);
     }
     sm[lane] = w;
   }
   __syncthreads();
-  if (warp > 0) h = m.add(m.mul(sm[warp - 1], pw[lane + 1]), h);
+  if (warp > 0) h = m.add(m.mul(sm[warp - 1], xl), h);
   __syncthreads();
   return h;
 }
 
-// Horner fingerprint of each 32-byte chunk, scanned within the CTA; the
-// CTA-inclusive value of chunk j goes to Hs[j+1], the CTA total to agg.
+// X^(lane + 1) from the squares: the shift of a warp's carry-in.
 template <class M>
-__global__ void __launch_bounds__(kTile) k_kr_local(M m, const uint8_t* __restrict__ T,
-                                                    uint64_t nchunks, uint64_t B,
-                                                    const uint64_t* __restrict__ pw1,
-                                                    uint64_t* __restrict__ Hs,
-                                                    uint64_t* __restrict__ agg) {
-  __shared__ uint64_t sm[32];
-  uint64_t j = (uint64_t)blockIdx.x * kTile + threadIdx.x;
-  uint64_t h = 0;
-  if (j < nchunks) {
-    const uint8_t* p = T + j * kPrefixStride;
-    if ((((uintptr_t)p) & 15) == 0) {  // two 16-byte loads
-      const uint4 v0 = ((const uint4*)p)[0], v1 = ((const uint4*)p)[1];
-      const uint32_t wv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+__device__ __forceinline__ uint64_t kr_lane_pow(const M& m, const KrPow& pw) {
+  const unsigned e = (threadIdx.x & 31) + 1;
+  uint64_t r = 1;
 #pragma unroll
-      for (int i = 0; i < (int)kPrefixStride; i++)
-        h = m.add(m.mul(h, B), (uint64_t)((wv[i >> 2] >> (8 * (i & 3))) & 0xFFu) + 1);
-    } else {
-#pragma unroll 8
-      for (int i = 0; i < (int)kPrefixStride; i++) h = m.add(m.mul(h, B), (uint64_t)p[i] + 1);
+  for (int i = 0; i < 5; i++)
+    if ((e >> i) & 1u) r = m.mul(r, pw.x[i]);
+  return e == 32 ? pw.w[0] : r;
+}
+
+// Fingerprint of a 32-byte chunk (eight little-endian words).
+template <class M>
+struct ChunkHash {  // any modulus: Horner
+  uint64_t B;
+  ChunkHash(const M&, uint64_t base) : B(base) {}
+  __device__ __forceinline__ uint64_t operator()(const M& m, const uint32_t* w) const {
+    uint64_t h = 0;
+#pragma unroll
+    for (int i = 0; i < (int)kPrefixStride; i++)
+      h = m.add(m.mul(h, B), (uint64_t)((w[i >> 2] >> (8 * (i & 3))) & 0xFFu) + 1);
+    return h;
+  }
+};
+template <>
+struct ChunkHash<Mersenne61> {
+  uint32_t limb[8][8];  // [word][l]: bits 8l..8l+7 of the powers of the word's four bytes
+  uint64_t ones;        // the sum of the powers: every symbol is its byte + 1
+  ChunkHash(const Mersenne61& m, uint64_t B) {
+    uint64_t p = 1;
+    ones = 0;
+    for (int i = 31; i >= 0; i--) {
+      for (int l = 0; l < 8; l++) {
+        if ((i & 3) == 3) limb[i >> 2][l] = 0;
+        limb[i >> 2][l] |= (uint32_t)((p >> (8 * l)) & 0xFF) << (8 * (i & 3));
+      }
+      ones = m.add(ones, p);
+      p = m.mul(p, B);
     }
   }
-  h = cta_kr_scan(m, h, pw1, sm);
-  if (j < nchunks) Hs[j + 1] = h;
-  uint64_t base = (uint64_t)blockIdx.x * kTile;
-  uint64_t last = (nchunks - base < kTile ? nchunks - base : kTile) - 1;
-  if (threadIdx.x == last) agg[blockIdx.x] = h;
-}
+  __device__ __forceinline__ uint64_t operator()(const Mersenne61& m, const uint32_t* w) const {
+    uint32_t s[8];  // each at most 32 * 255^2 < 2^21
+#pragma unroll
+    for (int l = 0; l < 8; l++) {
+      s[l] = 0;
+#pragma unroll
+      for (int q = 0; q < 8; q++) s[l] = __dp4a(w[q], limb[q][l], s[l]);
+    }
+    const uint64_t lo = (uint64_t)s[0] + ((uint64_t)s[1] << 8) + ((uint64_t)s[2] << 16) + ((uint64_t)s[3] << 24);
+    const uint64_t hi = (uint64_t)s[4] + ((uint64_t)s[5] << 8) + ((uint64_t)s[6] << 16) + ((uint64_t)s[7] << 24);
+    // lo + hi 2^32 with hi = a 2^29 + r: a 2^61 + r 2^32 = a + r 2^32; < 2^62.
+    uint64_t x = lo + (hi >> 29) + ((hi & ((1u << 29) - 1)) << 32);
+    x = (x & Mersenne61::Q) + (x >> 61);
+    if (x >= Mersenne61::Q) x -= Mersenne61::Q;
+    return m.add(x, ones);
+  }
+};
 
-// pre[i] = fingerprint of chunks [0, 1024 i): scan of the CTA totals by one
-// CTA with X = B^(32*1024) (pw2[i] = X^i).
-template <class M>
-__global__ void __launch_bounds__(kTile) k_kr_aggs(M m, uint64_t* __restrict__ agg, uint64_t na,
-                                                   const uint64_t* __restrict__ pw2) {
-  __shared__ uint64_t sm[32];
-  __shared__ uint64_t carry_s;
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  for (uint64_t base = 0; base < na; base += kTile) {
-    uint64_t i = base + threadIdx.x;
-    uint64_t v = i < na ? agg[i] : 0;
-    uint64_t incl = cta_kr_scan(m, v, pw2, sm);
-    uint64_t carry = carry_s;
-    uint64_t g = m.add(m.mul(carry, pw2[threadIdx.x + 1]), incl);
-    __syncthreads();
-    uint64_t cnt = na - base < kTile ? na - base : kTile;
-    if (i < na) agg[i] = g;  // inclusive prefix over CTA totals [0, i]
-    if (threadIdx.x == cnt - 1) carry_s = g;
-    __syncthreads();
+// The words of chunk j, or zeros for a chunk the text does not hold.
+__device__ __forceinline__ void load_chunk(const uint8_t* __restrict__ T, uint64_t nchunks, uint64_t j, bool aligned,
+                                           uint32_t* w) {
+  if (j >= nchunks) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) w[i] = 0;
+    return;
+  }
+  const uint8_t* p = T + j * kPrefixStride;
+  if (aligned) {
+    const uint4 v0 = ((const uint4*)p)[0], v1 = ((const uint4*)p)[1];
+    w[0] = v0.x, w[1] = v0.y, w[2] = v0.z, w[3] = v0.w;
+    w[4] = v1.x, w[5] = v1.y, w[6] = v1.z, w[7] = v1.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+      w[i] = (uint32_t)p[4 * i] | ((uint32_t)p[4 * i + 1] << 8) | ((uint32_t)p[4 * i + 2] << 16) |
+             ((uint32_t)p[4 * i + 3] << 24);
   }
 }
 
+// agg[i] = fingerprint of tile i (kTile chunks); the last tile is not needed.
+// pw: the shift of a thread's four chunks, P = B^32 the shift of one.
 template <class M>
-__global__ void __launch_bounds__(kTile) k_kr_add(M m, uint64_t* __restrict__ Hs, uint64_t nchunks,
-                                                  const uint64_t* __restrict__ agg,
-                                                  const uint64_t* __restrict__ pw1) {
-  uint64_t j = (uint64_t)blockIdx.x * kTile + threadIdx.x;
-  if (j == 0) Hs[0] = 0;
-  if (j >= nchunks || blockIdx.x == 0) return;
-  uint64_t pre = agg[blockIdx.x - 1];
-  Hs[j + 1] = m.add(m.mul(pre, pw1[threadIdx.x + 1]), Hs[j + 1]);
+__global__ void __launch_bounds__(kKrThreads) k_kr_totals(M m, const uint8_t* __restrict__ T, uint64_t nchunks,
+                                                          const ChunkHash<M> hash, uint64_t P, KrPow pw,
+                                                          uint64_t* __restrict__ agg) {
+  __shared__ uint64_t sm[kKrThreads / 32];
+  const bool aligned = (((uintptr_t)T) & 15) == 0;
+  const uint64_t j0 = (uint64_t)blockIdx.x * kTile + (uint64_t)threadIdx.x * kKrChunks;
+  uint32_t w[kKrChunks][8];
+#pragma unroll
+  for (int i = 0; i < kKrChunks; i++) load_chunk(T, nchunks, j0 + i, aligned, w[i]);
+  uint64_t h = hash(m, w[0]);
+#pragma unroll
+  for (int i = 1; i < kKrChunks; i++) h = m.add(m.mul(h, P), hash(m, w[i]));
+  // Ordered tree over the warp, then over the warps.
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 5; i++) h = m.add(m.mul(h, pw.x[i]), __shfl_down_sync(0xFFFFFFFFu, h, 1 << i));
+  if (lane == 0) sm[warp] = h;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    h = sm[0];
+#pragma unroll
+    for (int i = 1; i < kKrThreads / 32; i++) h = m.add(m.mul(h, pw.w[0]), sm[i]);
+    agg[blockIdx.x] = h;
+  }
+}
+
+// agg[i] = fingerprint of tiles 0 .. i, by one CTA: a thread folds `per`
+// consecutive tiles (all loads first, eight at a time), then the threads are
+// scanned.  Y: the shift of a tile; pw: the shift of a thread's tiles.
+template <class M>
+__global__ void __launch_bounds__(kTile) k_kr_aggs(M m, uint64_t* __restrict__ agg, uint64_t na, uint64_t per,
+                                                   uint64_t Y, KrPow pw) {
+  __shared__ uint64_t sm[32];
+  const uint64_t i0 = threadIdx.x * per;
+  uint64_t h = 0;
+  for (uint64_t i = 0; i < per; i += 8) {
+    uint64_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) v[u] = i + u < per && i0 + i + u < na ? agg[i0 + i + u] : 0;
+#pragma unroll
+    for (int u = 0; u < 8; u++)
+      if (i + u < per) h = m.add(m.mul(h, Y), v[u]);
+  }
+  const uint64_t incl = cta_kr_scan(m, h, pw, kr_lane_pow(m, pw), sm);
+  uint64_t up = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+  if ((threadIdx.x & 31) == 31) sm[threadIdx.x >> 5] = incl;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) up = threadIdx.x ? sm[(threadIdx.x >> 5) - 1] : 0;
+  for (uint64_t i = 0; i < per && i0 + i < na; i++) {
+    up = m.add(m.mul(up, Y), agg[i0 + i]);
+    agg[i0 + i] = up;
+  }
+}
+
+// Hs[j] = H(32 j) for j <= nchunks: every thread's four chunks again, scanned
+// over the tile with the tile's prefix as the first item's carry-in.
+template <class M>
+__global__ void __launch_bounds__(kKrThreads) k_kr_write(M m, const uint8_t* __restrict__ T, uint64_t nchunks,
+                                                         const ChunkHash<M> hash, uint64_t P, KrPow pw,
+                                                         const uint64_t* __restrict__ agg, uint64_t* __restrict__ Hs) {
+  __shared__ uint64_t sm[32];
+  const bool aligned = (((uintptr_t)T) & 15) == 0;
+  const uint64_t tile = gridDim.x - 1 - blockIdx.x;
+  const uint64_t j0 = tile * kTile + (uint64_t)threadIdx.x * kKrChunks;
+  uint64_t c[kKrChunks];
+  {
+    uint32_t w[kKrChunks][8];
+#pragma unroll
+    for (int i = 0; i < kKrChunks; i++) load_chunk(T, nchunks, j0 + i, aligned, w[i]);
+#pragma unroll
+    for (int i = 0; i < kKrChunks; i++) c[i] = hash(m, w[i]);
+  }
+  uint64_t h = c[0];
+#pragma unroll
+  for (int i = 1; i < kKrChunks; i++) h = m.add(m.mul(h, P), c[i]);
+  const uint64_t carry = threadIdx.x == 0 && tile ? agg[tile - 1] : 0;
+  if (threadIdx.x == 0) h = m.add(m.mul(carry, pw.x[0]), h);
+  const uint64_t incl = cta_kr_scan(m, h, pw, kr_lane_pow(m, pw), sm);
+  uint64_t up = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+  if ((threadIdx.x & 31) == 31) sm[threadIdx.x >> 5] = incl;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) up = threadIdx.x ? sm[(threadIdx.x >> 5) - 1] : carry;
+  // up = H(32 j0); the four values are one aligned 32-byte sector.
+  uint64_t o[kKrChunks];
+#pragma unroll
+  for (int i = 0; i < kKrChunks; i++) {
+    o[i] = up;
+    up = m.add(m.mul(up, P), c[i]);
+  }
+  if (j0 + kKrChunks - 1 <= nchunks && (((uintptr_t)Hs) & 15) == 0) {
+    ((ulonglong2*)(Hs + j0))[0] = make_ulonglong2(o[0], o[1]);
+    ((ulonglong2*)(Hs + j0))[1] = make_ulonglong2(o[2], o[3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < kKrChunks; i++)
+      if (j0 + i <= nchunks) Hs[j0 + i] = o[i];
+  }
+}
+
+// The three launches; agg holds nchunks / kTile entries.
+template <class M>
+int kr_launch(const M& m, const uint8_t* T, uint64_t n, uint64_t B, uint64_t* Hs, uint64_t* agg, cudaStream_t s) {
+  const uint64_t nchunks = n / kPrefixStride;
+  const uint64_t tiles = nchunks / kTile + 1, na = tiles - 1;  // the last tile writes Hs[nchunks]
+  const uint64_t P = pow_mod(m, B, kPrefixStride);
+  const KrPow pw = kr_pow(m, pow_mod(m, P, kKrChunks));
+  const ChunkHash<M> hash(m, B);
+  if (na) {
+    BT_LAUNCH(k_kr_totals<M><<<(unsigned)na, kKrThreads, 0, s>>>(m, T, nchunks, hash, P, pw, agg));
+    const uint64_t per = (na + kTile - 1) / kTile, Y = pow_mod(m, P, kTile);
+    BT_LAUNCH(k_kr_aggs<M><<<1, kTile, 0, s>>>(m, agg, na, per, Y, kr_pow(m, pow_mod(m, Y, per))));
+  }
+  BT_LAUNCH(k_kr_write<M><<<(unsigned)tiles, kKrThreads, 0, s>>>(m, T, nchunks, hash, P, pw, agg, Hs));
+  BT_CUDA(cudaGetLastError());
+  return BT_OK;
 }
 
 template <class M>
 int kr_prefix(const M& m, const uint8_t* T, uint64_t n, uint64_t B, uint64_t* Hs, cudaStream_t s) {
-  uint64_t nchunks = n / kPrefixStride;
+  const uint64_t nchunks = n / kPrefixStride;
   if (nchunks == 0) {
     BT_CUDA(cudaMemsetAsync(Hs, 0, sizeof(uint64_t), s));
     return BT_OK;
   }
-  uint64_t na = (nchunks + kTile - 1) / kTile;
-  // Power tables: pw1[i] = P^i, pw2[i] = P^(1024 i), P = B^32.
-  std::vector<uint64_t> h(2 * (kTile + 1));
-  uint64_t P = pow_mod(m, B, kPrefixStride), P1024 = pow_mod(m, P, kTile);
-  h[0] = 1 % m.q();
-  h[kTile + 1] = 1 % m.q();
-  for (int i = 1; i <= kTile; i++) {
-    h[i] = m.mul(h[i - 1], P);
-    h[kTile + 1 + i] = m.mul(h[kTile + i], P1024);
-  }
   Scratch sc(s);
-  uint64_t *pw, *agg;
-  BT_TRY(sc.alloc(&pw, h.size()));
-  BT_TRY(sc.alloc(&agg, na));
-  BT_CUDA(cudaMemcpyAsync(pw, h.data(), h.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
+  uint64_t* agg = nullptr;
+  if (nchunks >= kTile) BT_TRY(sc.alloc(&agg, nchunks / kTile));
   ProfScope ps("prefix_fingerprint", s, n);
-  BT_LAUNCH(k_kr_local<M><<<(unsigned)na, kTile, 0, s>>>(m, T, nchunks, B, pw, Hs, agg));
-  BT_LAUNCH(k_kr_aggs<M><<<1, kTile, 0, s>>>(m, agg, na, pw + kTile + 1));
-  BT_LAUNCH(k_kr_add<M><<<(unsigned)na, kTile, 0, s>>>(m, Hs, nchunks, agg, pw));
-  BT_CUDA(cudaGetLastError());
-  // The host table must outlive the asynchronous copy.
-  BT_CUDA(cudaStreamSynchronize(s));
-  return BT_OK;
+  return kr_launch(m, T, n, B, Hs, agg, s);
 }
 
 // H[p] at every position from the stride-32 values: the lane of chunk j
@@ -326,21 +481,18 @@ int expand_prefix(const uint8_t* T, uint64_t n, uint64_t B, uint64_t q, const ui
 // reserve all device memory for its own allocator up front and forbid the
 // libraries it loads to call cudaMalloc.  Code on a latency-critical path may
 // also be unable to risk an allocation's implicit synchronisation or failure.
-// This variant of the prefix-fingerprint pass takes its scratch (the two power
-// tables and the per-CTA aggregates) from a fixed array in device memory
-// instead of cudaMallocAsync.  Every GPU that loads the library holds the
+// This variant of the prefix-fingerprint pass takes its scratch (the per-tile
+// totals) from a fixed array in device memory instead of cudaMallocAsync.  Every GPU that loads the library holds the
 // array until the process exits.
 // ---------------------------------------------------------------------------
 namespace {
 
 constexpr uint64_t kNoAllocMaxN = 1ull << 31;  // largest text accepted (2 GiB)
 constexpr uint64_t kNoAllocAggs = (kNoAllocMaxN / kPrefixStride + kTile - 1) / kTile;
-constexpr uint64_t kNoAllocWords = 2 * (kTile + 1) + kNoAllocAggs;  // 67586 u64, 528 KiB
+constexpr uint64_t kNoAllocWords = kNoAllocAggs;  // 65536 u64, 512 KiB
 constexpr int kNoAllocDevices = 64;
-// The aggregate region holds exactly the CTA totals of the largest text, and
-// the array is the two power tables plus that region.
+// The array holds exactly the tile totals of the largest text.
 static_assert(kNoAllocAggs == 65536, "one aggregate per 1024 chunks of 32 bytes of a 2 GiB text");
-static_assert(kNoAllocWords == 2 * (kTile + 1) + 65536, "power tables + aggregates");
 
 static __device__ __align__(256) uint64_t g_noalloc_scratch[kNoAllocWords];
 
@@ -369,34 +521,14 @@ int noalloc_scratch(uint64_t** out) {
   return BT_OK;
 }
 
-// pw1[i] = P^i and pw2[i] = P^(1024 i) for i <= 1024, P = B^32, computed on
-// the device so that no host buffer has to be copied.
-template <class M>
-__global__ void k_kr_powers(M m, uint64_t B, uint64_t* __restrict__ pw) {
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (i > (uint64_t)kTile) return;
-  const uint64_t P = pow_mod(m, B, kPrefixStride);
-  pw[i] = pow_mod(m, P, i);
-  pw[kTile + 1 + i] = pow_mod(m, pow_mod(m, P, kTile), i);
-}
-
 template <class M>
 int kr_prefix_noalloc(const M& m, const uint8_t* T, uint64_t n, uint64_t B, uint64_t* Hs,
                       uint64_t* scratch, cudaStream_t s) {
-  const uint64_t nchunks = n / kPrefixStride;
-  if (nchunks == 0) {
+  if (n / kPrefixStride == 0) {
     BT_CUDA(cudaMemsetAsync(Hs, 0, sizeof(uint64_t), s));
     return BT_OK;
   }
-  const uint64_t na = (nchunks + kTile - 1) / kTile;
-  uint64_t* pw = scratch;
-  uint64_t* agg = scratch + 2 * (kTile + 1);
-  BT_LAUNCH(k_kr_powers<M><<<(kTile + 1 + 255) / 256, 256, 0, s>>>(m, B, pw));
-  BT_LAUNCH(k_kr_local<M><<<(unsigned)na, kTile, 0, s>>>(m, T, nchunks, B, pw, Hs, agg));
-  BT_LAUNCH(k_kr_aggs<M><<<1, kTile, 0, s>>>(m, agg, na, pw + kTile + 1));
-  BT_LAUNCH(k_kr_add<M><<<(unsigned)na, kTile, 0, s>>>(m, Hs, nchunks, agg, pw));
-  BT_CUDA(cudaGetLastError());
-  return BT_OK;
+  return kr_launch(m, T, n, B, Hs, scratch, s);
 }
 
 }  // namespace

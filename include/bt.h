@@ -85,20 +85,17 @@ typedef struct {
 /* flags: BT_FLAG_DENSE_SCAN probes the table at every window position instead
  * of the anchored scan (a diagnostic; both give the same tree).
  * BT_FLAG_TINY_QUEUE caps the anchored scan's queue of proposed windows at 64
- * entries, so that nearly every level takes the overflow path, a second scan
+ * entries, so that nearly every anchored level takes the overflow path, a second scan
  * that tests the windows in place (a test hook; the same tree again). */
-/* BT_FLAG_GRAM_LIST builds the selected-gram list (the gram positions and
- * hashes the anchored scan shares between levels) whatever the text length;
- * by default only texts of 8 MiB or more use it (a test hook; same tree). */
-/* BT_FLAG_TWO_PHASE tests the proposed windows of every anchored level in two
- * phases: the windows of the gram hits in the first 1/16 of the text, then
- * the rest, against per-gram bounds lowered to the leftmost positions found so
- * far (a window after every such position of the keys on its gram is not
- * proposed).  The same tree.  It pays where the keys on a gram mostly have
- * their leftmost occurrence early (DNA copies with sparse point mutations:
- * about a third fewer windows); where most grams also carry a key first seen
- * late (edits in every copy of a versioned text) few windows are saved and the
- * two extra kernels and the second hit pass cost more, hence off by default. */
+/* BT_FLAG_GRAM_LIST is accepted and has no effect: the list of selected grams
+ * is built for every text whose tree has a level of blocks of 27 bytes or
+ * more. */
+/* BT_FLAG_TWO_PHASE tests the proposed windows of every anchored level (the
+ * levels of shorter blocks) in two phases: the windows of the gram hits in the
+ * first 1/16 of the text, then the rest, against per-gram bounds lowered to the
+ * leftmost positions found so far (a window after every such position of the
+ * keys on its gram is not proposed).  The same tree.  The levels of longer
+ * blocks always work this way on texts with more than 2^20 selected grams. */
 /* BT_FLAG_BATCH_WORKERS makes bt_build_batch build every document with
  * bt_build_ex on host worker threads instead of the persistent batched kernel
  * (the comparison arm of the batched build; the same trees). */

@@ -358,8 +358,8 @@ class BuildOptions:
     max_rounds: int = 0
     dense_scan: bool = False
     tiny_queue: bool = False  # test hook: forces the scan's queue-overflow path
-    gram_list: bool = False  # test hook: selected-gram list whatever the text length
-    two_phase: bool = False  # two-phase window tests on every anchored level (same tree)
+    gram_list: bool = False  # accepted, no effect (the list is built whenever a level can use it)
+    two_phase: bool = False  # two-phase window tests on the levels of short blocks (same tree)
     batch_workers: bool = False  # bt_build_batch: host workers instead of the batched kernel
     batch_ctas: int = 0  # bt_build_batch: CTAs of the batched kernel's launch (0: every SM)
     leaf_counts: bool = False  # no stored counters on the last level (space-efficient rank/select)

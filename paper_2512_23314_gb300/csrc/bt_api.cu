@@ -228,7 +228,6 @@ static int build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, 
   ctx.arena.s = s;
   ctx.dense_scan = (o.flags & BT_FLAG_DENSE_SCAN) ? 1 : 0;
   ctx.tiny_queue = (o.flags & BT_FLAG_TINY_QUEUE) ? 1 : 0;
-  ctx.force_list = (o.flags & BT_FLAG_GRAM_LIST) ? 1 : 0;
   ctx.two_phase = (o.flags & BT_FLAG_TWO_PHASE) ? 1 : 0;
   ctx.leaf_counts = (o.flags & BT_FLAG_LEAF_COUNTS) ? 1 : 0;
   ctx.sort_scan = (o.flags & BT_FLAG_SORT_SCAN) ? 1 : 0;
@@ -247,14 +246,11 @@ static int build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, 
   }
   tr.mark("setup+alphabet");
   {
-    // Prefix fingerprints at every position, for the whole construction; the
-    // stride-32 values are an intermediate step.
-    Scratch hs(s);
+    // Prefix fingerprints at every 32nd position, for the whole construction.
     uint64_t* Hs;
-    BT_TRY(hs.alloc(&Hs, n / kPrefixStride + 2));
-    BT_TRY(sc.alloc(&ctx.H, n + 1));
+    BT_TRY(sc.alloc(&Hs, n / kPrefixStride + 2));
     BT_TRY(prefix_fingerprints(dT, n, t->B, t->q, Hs, s));
-    BT_TRY(expand_prefix(dT, n, t->B, t->q, Hs, ctx.H, s));
+    ctx.Hs = Hs;
   }
   {
     ProfScope ps("phase_levels", s, 0);

@@ -359,7 +359,8 @@ int radix_sort_u64_u32(uint64_t* keys, uint32_t* vals, uint64_t* tk, uint32_t* t
 struct BuildCtx {
   bt_tree* t;
   const uint8_t* T;   // device text
-  uint64_t* H;        // prefix fingerprints at every position, n + 1 entries
+  const uint64_t* Hs = nullptr;  // prefix fingerprints H(32 j), n / 32 + 1 entries
+  uint64_t* H = nullptr;         // at every position, n + 1 entries (only the levels of short blocks need it)
   Arena arena;        // per-level scratch
   Status* st;         // device status
   Status* st_host;    // pinned mirror
@@ -367,18 +368,11 @@ struct BuildCtx {
   uint64_t verify_bytes = 0, collisions = 0;
   int dense_scan = 0;  // probe every window (diagnostic) instead of the anchored scan
   int tiny_queue = 0;  // test hook: a 64-entry candidate queue (forces the overflow path)
-  int force_list = 0;  // test hook: build the selected-gram list for any text length
   int two_phase = 0;   // BT_FLAG_TWO_PHASE: test every level's windows in two phases
   int leaf_counts = 0; // BT_FLAG_LEAF_COUNTS: no stored counters on the last level
   int sort_scan = 0;   // BT_FLAG_SORT_SCAN: leftmost windows by sorting instead of probing
   uint32_t partitions = 0;  // parts of the sort-based pass (domain decomposition; <= 1: one)
   uint64_t prev_cands = 0;  // windows the previous level's scan proposed (sizes the next queue)
-  // Selected-gram list of the whole text (built once when levels can use it):
-  // chunk j of 128 positions lists its grams at gl_chunk[j] .. gl_chunk[j+1].
-  const uint32_t* gl_chunk = nullptr;
-  const uint32_t* gl_mx = nullptr;
-  const uint32_t* gl_x = nullptr;  // positions (texts are shorter than 2^32)
-  uint32_t gl_total = 0;
   ~BuildCtx() { arena.release(); }
 };
 

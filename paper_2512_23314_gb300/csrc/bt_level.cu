@@ -36,7 +36,9 @@
 #include <cstdio>
 #include <cstdlib>
 
+#include "bt_bytes.cuh"
 #include "bt_internal.cuh"
+#include "bt_quick.cuh"
 
 namespace bt {
 
@@ -64,11 +66,9 @@ struct LevelDev {
   unsigned int tail_anchorless;     // tail key: 1 shorter than a gram, 2 no anchor
   unsigned int tail_gram;           // anchor gram of the tail key (remapped)
   unsigned int tail_a;              // its anchor offset
-  unsigned int far_end;             // 1 + the largest far anchor offset of a full-length key
   unsigned long long cands;         // windows proposed by anchors and filters
   unsigned long long hits;          // proposed windows whose fingerprint is a key's
   unsigned int qover;               // some CTA's queue segment overflowed
-  unsigned int nfar;                // FarNodes taken
 };
 
 struct Geo {
@@ -464,22 +464,20 @@ __global__ void k_first_of_key(const uint64_t* __restrict__ keys, uint64_t n, ui
 // content: the first position of a w-gram whose mixed 32-bit gram hash is
 // "selected" (at most 2^(32-sbits) - 1, density 2^-sbits).  Every key is
 // registered under its anchor gram: the anchor table maps a gram to the set of
-// offsets (a 64-bit mask for offsets below W, plus one far offset) at which
-// keys anchor on it.  The scan rolls the 32-bit gram hash over the level (no
+// offsets (a 64-bit mask) at which keys anchor on it.  The scan rolls the 32-bit gram hash over the level (no
 // 61-bit arithmetic per byte) and only records the selected grams; a second
 // pass tests those against a bitmap filter, reads the anchor table for the
 // few that pass, and each offset a proposes the window at x - a, whose 61-bit
 // fingerprint is then looked up in the block table.  A window equal to a key
 // has the key's anchor (same gram, same offset), so it is always proposed: the
 // slot minima are the same as when probing every window.  A key without any
-// selected gram (or whose far offset clashes with another key's on the same
-// gram) is registered by its first gram in a small shared-memory filter that
-// is checked at every position only when such keys exist.
+// selected gram is registered by its first gram in a small shared-memory
+// filter that is checked at every position only when such keys exist.
+// These scans serve the levels whose blocks are shorter than kQuickMinB bytes
+// (grams of half a block); bt_quick.cu takes the others.
 // ---------------------------------------------------------------------------
 constexpr uint32_t kAnchorQ = 128;        // gram positions per thread
 constexpr uint32_t kAnchorWmax = 64;      // near anchor range (bits of the offset mask)
-constexpr uint32_t kFarMax = 4096;        // far anchors are searched up to this offset
-constexpr uint32_t kNoFar = 0xFFFFFFFFu;
 constexpr uint32_t kEmptyGram = 0xFFFFFFFFu;
 constexpr uint32_t kFibMul = 0x9E3779B1u;
 constexpr uint32_t kScanThreads = 256;
@@ -502,18 +500,9 @@ struct GramP {
 // gram -> offsets at which keys anchor on it.
 struct __align__(32) AnchorSet {
   uint32_t gram;             // remapped mixed gram hash (kEmptyGram: empty slot)
-  uint32_t far;              // one anchor offset >= W (kNoFar: none)
+  uint32_t pad;
   unsigned long long offs;   // bit a: some key has its anchor at offset a < W
   unsigned long long maxst;  // largest start of a key anchored on this gram
-  uint32_t more;             // further anchor offsets >= W: a list of FarNodes (kNoFar: none)
-  uint32_t pad;
-};
-
-// A further far anchor offset of a gram (keys whose first selected gram lies
-// beyond the offset mask are rare; two of them on one gram rarer still).
-struct FarNode {
-  uint32_t off;
-  uint32_t next;
 };
 
 // The gram hash is a polynomial in rb over the symbols; its mixed value
@@ -537,27 +526,20 @@ __device__ __forceinline__ uint32_t sec_bit(uint32_t mx) { return (mx * 0x2545F4
 
 // Register the anchor of every key (every block and the tail).
 __global__ void k_anchor_keys(Geo g, GramP gp, const uint32_t* __restrict__ slotB, AnchorSet* atab,
-                              uint32_t amask, FarNode* fnode, uint32_t fcap, uint32_t* bitmap,
+                              uint32_t amask, uint32_t* bitmap,
                               uint32_t* secbits, uint32_t* __restrict__ aidx, LevelDev* ld, Status* status) {
   for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < g.c;
        k += (uint64_t)gridDim.x * blockDim.x) {
     aidx[k] = kNoSlot;
     const uint64_t s = g.st[k], len = blen(g, k);
     const bool tail = len != g.b;
-    uint32_t Wk;
     if (!tail) {
       if (slotB[k] == kNoSlot) continue;
-      Wk = gp.W;
-    } else {
-      Wk = gp.Wr;
-      if (Wk == 0) {  // shorter than a gram: the dense tail scan covers it
-        ld->tail_anchorless = 1u;
-        continue;
-      }
+    } else if (gp.Wr == 0) {  // shorter than a gram: the dense tail scan covers it
+      ld->tail_anchorless = 1u;
+      continue;
     }
-    // Gram positions of the key: [0, len - w]; the far search stops at kFarMax.
-    const uint64_t npos = len - gp.w + 1;
-    const uint32_t lim = (uint32_t)(npos < kFarMax ? npos : kFarMax);
+    const uint32_t lim = (uint32_t)(len - gp.w + 1);  // gram positions of the key: [0, len - w]
     uint32_t gh = 0;
     for (uint32_t i = 0; i < gp.w; i++) gh = gh * gp.rb + g.T[s + i];
     const uint32_t mx0 = gram_mix(gh);
@@ -571,7 +553,7 @@ __global__ void k_anchor_keys(Geo g, GramP gp, const uint32_t* __restrict__ slot
       }
     }
     const uint32_t gk = gram_key(mx);
-    bool sec = a == kNoSlot;
+    const bool sec = a == kNoSlot;
     if (!sec && !tail) {
       uint32_t h = gram_slot(gk, amask), hp = kNoSlot;
       bool placed = false;
@@ -580,28 +562,14 @@ __global__ void k_anchor_keys(Geo g, GramP gp, const uint32_t* __restrict__ slot
         if (cur == kEmptyGram || cur == gk) {
           placed = true;
           hp = h;
-          if (a < Wk) {
-            atomicOr(&atab[h].offs, 1ull << a);
-          } else {
-            const uint32_t f = atomicCAS(&atab[h].far, kNoFar, a);
-            if (f != kNoFar && f != a) {  // another far offset holds the entry: a list node
-              const uint32_t id = atomicAdd(&ld->nfar, 1u);
-              if (id < fcap) {
-                fnode[id].off = a;
-                fnode[id].next = atomicExch(&atab[h].more, id);
-              } else {
-                sec = true;
-              }
-            }
-            if (!sec) atomicMax(&ld->far_end, a + 1);
-          }
+          atomicOr(&atab[h].offs, 1ull << a);
           atomicMax(&atab[h].maxst, (unsigned long long)s);
         } else {
           h = (h + 1) & amask;
         }
       }
       if (!placed) atomicExch(&status->error, 7ull);
-      if (placed && !sec) aidx[k] = hp;
+      if (placed) aidx[k] = hp;
     }
     if (sec) {  // no usable anchor: registered by its first gram
       const uint32_t sb = sec_bit(mx0);
@@ -638,7 +606,6 @@ struct ScanCtx {
   uint32_t* csegn;                   // windows proposed by each k_hits CTA (may exceed cseg)
   uint32_t cseg;
   Status* status;                    // device-side invariant checks
-  const FarNode* fnode;              // further far anchor offsets of the anchor table
   const uint32_t* slotB;             // block slot of every block
 };
 
@@ -760,14 +727,11 @@ __device__ __forceinline__ void anchor_hit(const ScanCtx<M>& C, unsigned int* sq
                                            uint32_t& nhit) {
   const uint32_t gk = gram_key(mx);
   unsigned long long offs = 0, maxst = 0;
-  uint32_t far = kNoFar, node = kNoFar;
   for (uint32_t h = gram_slot(gk, amask), it = 0; it <= amask; h = (h + 1) & amask, it++) {
     const uint32_t eg = atab[h].gram;
     if (eg == gk) {
       offs = atab[h].offs;
-      far = atab[h].far;
       maxst = atab[h].maxst;
-      node = atab[h].more;
       break;
     }
     if (eg == kEmptyGram) break;
@@ -776,23 +740,15 @@ __device__ __forceinline__ void anchor_hit(const ScanCtx<M>& C, unsigned int* sq
   // the leftmost occurrence of any of them, nor of a pair that starts with
   // one of them (both are at or before the key's start).
   bool pt = gk == tail_gram && x >= tail_a;
-  bool pf = far != kNoFar;
-  while (offs || pf || pt || node != kNoFar) {
+  while (offs || pt) {
     uint32_t a = 0, kind = 0;
     if (pt) {
       pt = false;
       a = tail_a;
       kind = 1;
-    } else if (offs) {
+    } else {
       a = __ffsll(offs) - 1;
       offs &= offs - 1;
-    } else if (pf) {
-      pf = false;
-      a = far;
-    } else {
-      const FarNode fn = C.fnode[node];
-      node = fn.next;
-      a = fn.off;
     }
     if (a <= x && (kind || x - a <= maxst)) propose(C, sq, k, s, av, x - a, kind, ncand, nhit);
   }
@@ -880,11 +836,8 @@ __global__ void __launch_bounds__(kScanThreads, 3) k_scan_anchor(ScanCtx<M> C0, 
                                                              uint32_t amask,
                                                              const uint32_t* __restrict__ bitmap_g,
                                                              uint32_t bm_smem_words,
-                                                             const uint32_t* __restrict__ secbits_g,
-                                                             int sec_only) {
+                                                             const uint32_t* __restrict__ secbits_g) {
   if (INLINE && C0.ld->qover == 0) return;
-  // sec_only: k_scan_list covers this level unless it has keys without an anchor.
-  if (!INLINE && sec_only && C0.ld->anchorless != 1u && C0.ld->tail_anchorless != 2u) return;
   extern __shared__ uint32_t smem[];
   __shared__ unsigned int s_qn;  // hits this CTA recorded
   uint32_t* sec = smem;                                      // kSecBits / 32 words
@@ -900,8 +853,7 @@ __global__ void __launch_bounds__(kScanThreads, 3) k_scan_anchor(ScanCtx<M> C0, 
   const bool tail_sec = C.ld->tail_anchorless == 2u;
   const uint32_t tail_gram = C.ld->tail_gram, tail_a = C.ld->tail_a;
   // Anchors lie below a window's start + Wx (+ Wt for the tail window).
-  const uint32_t far_end = C.ld->far_end;
-  const uint32_t Wx = gp.W > far_end ? gp.W : far_end;
+  const uint32_t Wx = gp.W;
   const uint32_t Wt0 = gp.Wr ? gp.Wr : 1;
   const uint32_t Wt = tail_a != 0xFFFFFFFFu && tail_a + 1 > Wt0 ? tail_a + 1 : Wt0;
   for (uint32_t i = threadIdx.x; i < kSecBits / 32; i += blockDim.x) sec[i] = secbits_g[i];
@@ -952,67 +904,18 @@ __global__ void __launch_bounds__(kScanThreads, 3) k_scan_anchor(ScanCtx<M> C0, 
       // are masked off afterwards (their ring entries follow the valid ones).
       uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
       uint32_t* rp = ring;
-      if (w == 16) {
-        // The transition to position i removes byte i-1 and adds byte i+15, so
-        // positions 4q+1 .. 4q+4 take the bytes of words q and q+4.
-        uint32_t gh = 0;
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-          const uint32_t v = slotw[t];
-#pragma unroll
-          for (int u = 0; u < 4; u++) gh = gh * rb + __byte_perm(v, 0, 0x4440 + u);
-        }
-        uint32_t cur = 0;
-        {
-          const uint32_t mx = gram_mix(gh);
-          BT_RECORD(mx, cur, 0);
-        }
-        const uint32_t ngroups = (nx + 31) / 32;
-#pragma unroll 1
-        for (uint32_t G = 0; G < 4; G++) {
-          uint32_t carry = 0;
-          if (G < ngroups) {
-#pragma unroll
-            for (uint32_t qq = 0; qq < 8; qq++) {
-              const uint32_t wo = slotw[8 * G + qq], wn = slotw[8 * G + qq + 4];
-#pragma unroll
-              for (uint32_t u = 0; u < 4; u++) {
-                gh = gh * rb + __byte_perm(wn, 0, 0x4440 + u) - __byte_perm(wo, 0, 0x4440 + u) * rw;
-                const uint32_t mx = gram_mix(gh);
-                if (4 * qq + u + 1 < 32) {
-                  BT_RECORD(mx, cur, (4 * qq + u + 1) & 31);
-                } else {
-                  BT_RECORD(mx, carry, 0);
-                }
-              }
-            }
-          }
-          m3 = m2;
-          m2 = m1;
-          m1 = m0;
-          m0 = cur;
-          cur = carry;
-        }
-        // After four shifts m3 holds positions 0-31, ..., m0 positions 96-127.
-        const uint32_t t0 = m3, t1 = m2;
-        m3 = m0;
-        m2 = m1;
-        m0 = t0;
-        m1 = t1;
-      } else {
-        uint32_t gh = 0;
-        for (uint32_t i = 0; i < w; i++) gh = gh * rb + slot[i];
-        for (uint32_t i = 0; i < nx; i++) {
-          if (i) gh = gh * rb - (uint32_t)slot[i - 1] * rw + slot[i + w - 1];
-          const uint32_t mx = gram_mix(gh);
-          uint32_t bv = 0;
-          BT_RECORD(mx, bv, 0);
-          const uint32_t sh = bv << (i & 31);
-          if (i < 32) m0 |= sh;
-          else if (i < 64) m1 |= sh;
-          else if (i < 96) m2 |= sh;
-          else m3 |= sh;
-        }
+      uint32_t gh = 0;
+      for (uint32_t i = 0; i < w; i++) gh = gh * rb + slot[i];
+      for (uint32_t i = 0; i < nx; i++) {
+        if (i) gh = gh * rb - (uint32_t)slot[i - 1] * rw + slot[i + w - 1];
+        const uint32_t mx = gram_mix(gh);
+        uint32_t bv = 0;
+        BT_RECORD(mx, bv, 0);
+        const uint32_t sh = bv << (i & 31);
+        if (i < 32) m0 |= sh;
+        else if (i < 64) m1 |= sh;
+        else if (i < 96) m2 |= sh;
+        else m3 |= sh;
       }
       // Keep positions below nx.
       if (nx < 128) {
@@ -1110,235 +1013,6 @@ __global__ void __launch_bounds__(kScanThreads, 3) k_scan_anchor(ScanCtx<M> C0, 
   }
 }
 #undef BT_RECORD
-
-// ---------------------------------------------------------------------------
-// The selected-gram list.  On the levels whose block length is a multiple of
-// 128 and whose selection is the default (w = 16, density 1/8), the selected
-// grams of a chunk are the same at every level: their positions and mixed
-// hashes are computed once per build, in 128-byte text chunks (the grams of
-// chunk j at gl_chunk[j] .. gl_chunk[j+1] of gl_mx / gl_x, positions absolute),
-// and those levels read the list instead of rolling the hash again.
-// ---------------------------------------------------------------------------
-constexpr uint32_t kGlSbits = 3;
-constexpr uint64_t kGlMinText = 8ull << 20;  // smaller texts roll the hash at every level
-
-// One 128-byte chunk per thread: count the selected grams starting in it
-// into cnt[j] (WRITE = false), or write them from offset cnt[j] on (WRITE =
-// true, cnt holding the exclusive prefix sums of the counts).
-template <bool WRITE>
-__global__ void __launch_bounds__(256) k_gl_pass(const uint8_t* __restrict__ T, uint64_t n, uint64_t nchunks,
-                                                 uint32_t rb, uint32_t rw, uint32_t sel_max,
-                                                 uint32_t* __restrict__ cnt, uint32_t* __restrict__ out_mx,
-                                                 uint32_t* __restrict__ out_x) {
-  __shared__ uint32_t slots[256 * kSlotWords];
-  uint32_t* slotw = slots + threadIdx.x * kSlotWords;
-  const bool aligned16 = (((uintptr_t)T) & 15) == 0;
-  const uint64_t xlim = n - 15;  // grams start below n - 15
-  for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < nchunks;
-       j += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t p0 = j * kAnchorQ;
-    const uint32_t nx = (uint32_t)(xlim - p0 < kAnchorQ ? xlim - p0 : kAnchorQ);
-    stage((uint8_t*)slotw, T, n, p0, nx + 15, aligned16);
-    const uint64_t o = WRITE ? cnt[j] : 0;
-    uint32_t c = 0;
-    uint32_t gh = 0;
-#pragma unroll
-    for (int t = 0; t < 4; t++) {
-      const uint32_t v = slotw[t];
-#pragma unroll
-      for (int u = 0; u < 4; u++) gh = gh * rb + __byte_perm(v, 0, 0x4440 + u);
-    }
-    {
-      const uint32_t mx = gram_mix(gh);
-      if (mx <= sel_max) {
-        if (WRITE) {
-          out_mx[o] = mx;
-          out_x[o] = (uint32_t)p0;
-        }
-        c++;
-      }
-    }
-#pragma unroll 1
-    for (uint32_t G = 0; G < 4 && 32 * G + 1 < nx; G++) {
-#pragma unroll
-      for (uint32_t qq = 0; qq < 8; qq++) {
-        const uint32_t wo = slotw[8 * G + qq], wn = slotw[8 * G + qq + 4];
-#pragma unroll
-        for (uint32_t u = 0; u < 4; u++) {
-          const uint32_t i = 32 * G + 4 * qq + u + 1;
-          gh = gh * rb + __byte_perm(wn, 0, 0x4440 + u) - __byte_perm(wo, 0, 0x4440 + u) * rw;
-          const uint32_t mx = gram_mix(gh);
-          if (mx <= sel_max && i < nx) {
-            if (WRITE) {
-              out_mx[o + c] = mx;
-              out_x[o + c] = (uint32_t)(p0 + i);
-            }
-            c++;
-          }
-        }
-      }
-    }
-    if (!WRITE) cnt[j] = c;
-  }
-}
-
-// The anchored scan of a level from the selected-gram list: per chunk, the
-// listed grams below the chunk's end pass the bitmap filter (four loads in
-// flight) and go to the hit queue.  Levels with keys without an anchor are
-// left to k_scan_anchor (it needs every position's gram).
-template <class M>
-__global__ void __launch_bounds__(256) k_scan_list(ScanCtx<M> C0, GramP gp, uint64_t cpb,
-                                                   const uint32_t* __restrict__ bitmap_g, uint32_t bm_smem_words,
-                                                   const uint32_t* __restrict__ gl_chunk,
-                                                   const uint32_t* __restrict__ gl_mx,
-                                                   const uint32_t* __restrict__ gl_x) {
-  if (C0.ld->anchorless == 1u || C0.ld->tail_anchorless == 2u) return;
-  extern __shared__ uint32_t bms[];
-  __shared__ unsigned int s_qn;
-  const ScanCtx<M>& C = C0;
-  const Geo& g = C.g;
-  const uint32_t tail_a = C.ld->tail_a;
-  const uint32_t far_end = C.ld->far_end;
-  const uint32_t Wx = gp.W > far_end ? gp.W : far_end;
-  const uint32_t Wt0 = gp.Wr ? gp.Wr : 1;
-  const uint32_t Wt = tail_a != 0xFFFFFFFFu && tail_a + 1 > Wt0 ? tail_a + 1 : Wt0;
-  for (uint32_t i = threadIdx.x; i < bm_smem_words; i += blockDim.x) bms[i] = bitmap_g[i];
-  if (threadIdx.x == 0) s_qn = 0;
-  __syncthreads();
-  const uint32_t* bitmap = bm_smem_words ? bms : bitmap_g;
-  const uint32_t w = gp.w;
-  const uint64_t total = g.c * cpb;
-  const unsigned lane = threadIdx.x & 31;
-  for (uint64_t base = blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); base < total;
-       base += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t wi = base + lane;
-    do {
-      if (wi >= total) break;
-      const uint64_t k = cpb == 1 ? wi : wi / cpb, j = wi - k * cpb;
-      const uint64_t s = g.st[k], len = blen(g, k);
-      const uint64_t p0 = s + j * kAnchorQ;
-      if (p0 >= s + len) break;
-      const uint64_t av = avail_end(g, k);
-      uint64_t xe = p0 + kAnchorQ < s + len ? p0 + kAnchorQ : s + len;
-      uint64_t xm = av >= g.b ? av - g.b + Wx : 0;
-      if (g.r && av >= g.r) {
-        const uint64_t xr = av - g.r + Wt;
-        if (xr > xm) xm = xr;
-      }
-      const uint64_t gram_end = av + 1 >= w ? av + 1 - w : 0;
-      if (xm > gram_end) xm = gram_end;
-      if (xe > xm) xe = xm;
-      if (xe <= p0) break;
-      const uint32_t nx = (uint32_t)(xe - p0);
-      const uint64_t cj = p0 / kAnchorQ;
-      const uint32_t e1 = gl_chunk[cj + 1];
-      for (uint32_t e = gl_chunk[cj]; e < e1; e += 4) {
-        uint32_t pos[4], mx[4], wv[4], bt[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-          pos[u] = kAnchorQ;
-          wv[u] = 0;
-          bt[u] = 0;
-          mx[u] = 0;
-          if (e + u < e1) {
-            pos[u] = (uint32_t)(gl_x[e + u] - p0);
-            mx[u] = gl_mx[e + u];
-            const uint32_t bit = gram_bit(gp, mx[u]);
-            bt[u] = bit & 31;
-            wv[u] = bitmap[bit >> 5];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; u++)
-          if (pos[u] < nx && ((wv[u] >> bt[u]) & 1u)) record_hit(C, &s_qn, p0 + pos[u], k, mx[u]);
-      }
-    } while (0);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    C.segn[blockIdx.x] = s_qn;
-    atomicAdd(C.qn, (unsigned long long)s_qn);
-    if (s_qn > C.seg) C.ld->qover = 1u;
-  }
-}
-
-// The list scan of a level whose blocks are all present ([k b, (k+1) b),
-// consecutive): the block of a gram and the end of its run follow from its
-// position, so the whole list is read in order, coalesced, 16 entries per
-// thread and step (16-byte loads), their bitmap loads in flight together.
-// bshift: log2 b when b is a power of two, else 0.
-template <class M>
-__global__ void __launch_bounds__(256) k_scan_stream(ScanCtx<M> C0, GramP gp, uint32_t total, uint32_t bshift,
-                                                     const uint32_t* __restrict__ bitmap_g, uint32_t bm_smem_words,
-                                                     const uint32_t* __restrict__ gl_mx,
-                                                     const uint32_t* __restrict__ gl_x) {
-  if (C0.ld->anchorless == 1u || C0.ld->tail_anchorless == 2u) return;
-  extern __shared__ uint32_t bms[];
-  __shared__ unsigned int s_qn;
-  const ScanCtx<M>& C = C0;
-  const Geo& g = C.g;
-  const uint32_t tail_a = C.ld->tail_a;
-  const uint32_t far_end = C.ld->far_end;
-  const uint32_t Wx = gp.W > far_end ? gp.W : far_end;
-  const uint32_t Wt0 = gp.Wr ? gp.Wr : 1;
-  const uint32_t Wt = tail_a != 0xFFFFFFFFu && tail_a + 1 > Wt0 ? tail_a + 1 : Wt0;
-  for (uint32_t i = threadIdx.x; i < bm_smem_words; i += blockDim.x) bms[i] = bitmap_g[i];
-  if (threadIdx.x == 0) s_qn = 0;
-  __syncthreads();
-  const uint32_t* bitmap = bm_smem_words ? bms : bitmap_g;
-  const uint64_t b = g.b, w = gp.w;
-  constexpr uint32_t U = 16;  // entries per thread and step (four 16-byte loads per array)
-  const uint32_t totalU = (total + U - 1) / U;
-  for (uint64_t eu = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; eu < totalU;
-       eu += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t xs[U], mxs[U], wv[U], bt[U];
-    if (U * eu + U <= total) {
-#pragma unroll
-      for (uint32_t q = 0; q < U / 4; q++) {
-        const uint4 X = ((const uint4*)gl_x)[eu * (U / 4) + q], Y = ((const uint4*)gl_mx)[eu * (U / 4) + q];
-        xs[4 * q] = X.x, xs[4 * q + 1] = X.y, xs[4 * q + 2] = X.z, xs[4 * q + 3] = X.w;
-        mxs[4 * q] = Y.x, mxs[4 * q + 1] = Y.y, mxs[4 * q + 2] = Y.z, mxs[4 * q + 3] = Y.w;
-      }
-    } else {
-#pragma unroll
-      for (uint32_t u = 0; u < U; u++) {
-        xs[u] = U * eu + u < total ? gl_x[U * eu + u] : 0xFFFFFFFFu;
-        mxs[u] = U * eu + u < total ? gl_mx[U * eu + u] : 0;
-      }
-    }
-#pragma unroll
-    for (uint32_t u = 0; u < U; u++) {
-      wv[u] = 0;
-      bt[u] = 32;  // 32: no test
-      const uint64_t x = xs[u];
-      if (x >= g.n) continue;
-      const uint64_t k = bshift ? x >> bshift : x / b;
-      // End of block k and up to two following blocks.
-      const uint64_t av = (k + 3) * b < g.n ? (k + 3) * b : g.n;
-      uint64_t xm = av >= b ? av - b + Wx : 0;
-      if (g.r && av >= g.r) {
-        const uint64_t xr = av - g.r + Wt;
-        if (xr > xm) xm = xr;
-      }
-      const uint64_t gram_end = av + 1 >= w ? av + 1 - w : 0;
-      if (xm > gram_end) xm = gram_end;
-      if (x >= xm) continue;
-      const uint32_t bit = gram_bit(gp, mxs[u]);
-      bt[u] = bit & 31;
-      wv[u] = bitmap[bit >> 5];
-    }
-#pragma unroll
-    for (uint32_t u = 0; u < U; u++)
-      if (bt[u] < 32 && ((wv[u] >> bt[u]) & 1u))
-        record_hit(C, &s_qn, xs[u], bshift ? (uint64_t)xs[u] >> bshift : xs[u] / b, mxs[u]);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    C.segn[blockIdx.x] = s_qn;
-    atomicAdd(C.qn, (unsigned long long)s_qn);
-    if (s_qn > C.seg) C.ld->qover = 1u;
-  }
-}
 
 // The hits of scan CTA j's segment, one per thread: anchor-table lookup; the
 // windows the anchors propose go to this CTA's candidate segment.
@@ -1576,51 +1250,6 @@ __global__ void k_pair_jobs(Geo g, const uint32_t* __restrict__ slotP,
 
 // 4b. Byte verification of the queued jobs, in pieces of kPiece bytes, one
 // warp per piece.
-// The 16 bytes T[A, A+16) from the aligned units at A & ~15 (u0, u1).
-__device__ __forceinline__ uint4 unaligned16(uint4 u0, uint4 u1, uint32_t d) {
-  const uint32_t q = d >> 2, sh = 8 * (d & 3);
-  const uint32_t w0 = q == 0 ? u0.x : q == 1 ? u0.y : q == 2 ? u0.z : u0.w;
-  const uint32_t w1 = q == 0 ? u0.y : q == 1 ? u0.z : q == 2 ? u0.w : u1.x;
-  const uint32_t w2 = q == 0 ? u0.z : q == 1 ? u0.w : q == 2 ? u1.x : u1.y;
-  const uint32_t w3 = q == 0 ? u0.w : q == 1 ? u1.x : q == 2 ? u1.y : u1.z;
-  const uint32_t w4 = q == 0 ? u1.x : q == 1 ? u1.y : q == 2 ? u1.z : u1.w;
-  return make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh),
-                    __funnelshift_r(w3, w4, sh));
-}
-
-// Compare T[J.a + x] and T[J.b + x] for x in [off, end): 16 bytes per lane
-// and step when the own side J.b + off is 16-byte aligned (block starts are
-// multiples of 16 at the usual leaf lengths), the other side realigned from
-// two aligned loads; bytes otherwise and for the ragged end.
-__device__ __forceinline__ bool differs(const uint8_t* __restrict__ T, uint64_t n, bool aligned16, uint64_t a,
-                                        uint64_t b, uint64_t off, uint64_t end, unsigned lane, unsigned L) {
-  bool diff = false;
-  uint64_t x = off;
-  if (aligned16 && ((b + off) & 15) == 0) {
-    const uint64_t full = off + ((end - off) & ~15ull);
-    for (uint64_t y = off + 16ull * lane; y < full; y += 16ull * L) {
-      const uint4 vb = *(const uint4*)(T + b + y);
-      const uint64_t A = a + y, A0 = A & ~15ull;
-      const uint32_t d = (uint32_t)(A & 15);
-      const uint4 u0 = *(const uint4*)(T + A0);
-      uint4 va;
-      if (d == 0) {
-        va = u0;
-      } else if (A0 + 32 <= n) {
-        va = unaligned16(u0, *(const uint4*)(T + A0 + 16), d);
-      } else {  // the unit past the text's end is not read
-        uint32_t v[4] = {0, 0, 0, 0};
-        for (uint32_t t = 0; t < 16; t++) v[t >> 2] |= (uint32_t)T[A + t] << (8 * (t & 3));
-        va = make_uint4(v[0], v[1], v[2], v[3]);
-      }
-      diff |= va.x != vb.x || va.y != vb.y || va.z != vb.z || va.w != vb.w;
-    }
-    x = full;
-  }
-  for (x += lane; x < end; x += L) diff |= T[a + x] != T[b + x];
-  return diff;
-}
-
 // One group of L lanes (a power of two up to 32, about b/16 so that short
 // jobs do not leave most of a warp idle) per (job, piece of 4 KiB).
 __global__ void __launch_bounds__(256) k_verify(const uint8_t* __restrict__ T, uint64_t n,
@@ -1916,8 +1545,6 @@ __global__ void k_level_init(InitArgs a) {
     if (i < a.c) a.mismatch[i] = 0;
     if (a.atab && i < a.acap) {
       a.atab[i].gram = kEmptyGram;
-      a.atab[i].far = kNoFar;
-      a.atab[i].more = kNoFar;
       a.atab[i].offs = 0;
       a.atab[i].maxst = 0;
     }
@@ -1936,9 +1563,7 @@ __global__ void k_level_init(InitArgs a) {
       d.tail_anchorless = 0;
       d.tail_gram = 0xFFFFFFFFu;
       d.tail_a = 0xFFFFFFFFu;
-      d.far_end = 0;
       d.qover = 0;
-      d.nfar = 0;
       d.cands = 0;
       d.hits = 0;
       *a.ld = d;
@@ -1959,11 +1584,7 @@ __global__ void k_reset_jobs(unsigned int* mismatch, uint64_t c, LevelDev* ld) {
   }
 }
 
-// Gram length 16 (at most half a block): long enough that a gram is rare
-// even over small or skewed alphabets, so few keys share an anchor gram;
-// anchor range W <= 64; selection density 2^-sbits chosen so that
-// W / 2^sbits >= 8 (a window without an anchor is then rare).
-// Gram length w = 16 (half the block when shorter), near range W <= 64.
+// Gram length w: half the block, at most 16; anchor range W <= 64.
 // Each gram is selected with probability 2^-sbits, so a key has no selected
 // gram among its first npos positions with probability (1 - 2^-sbits)^npos;
 // sbits is the largest value in 0..3 that leaves well under one such key per
@@ -1974,7 +1595,7 @@ GramP choose_gram(uint64_t b, uint64_t r, uint64_t c) {
   GramP gp;
   gp.w = w;
   gp.W = (uint32_t)(b - w + 1 < kAnchorWmax ? b - w + 1 : kAnchorWmax);
-  const double npos = (double)(b - w + 1 < kFarMax ? b - w + 1 : kFarMax);
+  const double npos = (double)(b - w + 1);
   gp.sbits = 0;
   for (uint32_t sb = 3; sb >= 1; sb--) {
     if ((double)c * std::pow(1.0 - std::ldexp(1.0, -(int)sb), npos) <= 0.02) {
@@ -2276,8 +1897,6 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
   Arena& A = ctx.arena;
   LevelWork W;
   AnchorSet* atab = nullptr;
-  FarNode* fnode = nullptr;
-  const uint32_t fcap = (uint32_t)(c / 16 + 1024);
   uint32_t *bitmap = nullptr, *secbits = nullptr, *sagg = nullptr;
   Hit* q = nullptr;
   uint32_t* segn = nullptr;
@@ -2303,7 +1922,6 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
     sagg = A.take<uint32_t>(scan_scratch_words(words));
     if (anchored) {
       atab = A.take<AnchorSet>(acap);
-      fnode = A.take<FarNode>(fcap);
       bitmap = A.take<uint32_t>(bwords);
       secbits = A.take<uint32_t>(kSecBits / 32);
       q = A.take<Hit>((uint64_t)seg * scan_grid);
@@ -2319,20 +1937,7 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
   BT_TRY(A.reserve());
   carve();
 
-  // Persistent level arrays: one allocation, owned by the level.
-  {
-    auto al = [](uint64_t x) { return (x + 255) & ~255ull; };
-    const uint64_t o_mw = 0, o_mr = o_mw + al(words * 4 + 4), o_ptr = o_mr + al((words + 1) * 4),
-                   o_off = o_ptr + al(c * 4 + 4), o_lo = o_off + al(c * 8 + 8), total = o_lo + al(c * 8 + 8);
-    char* mem;
-    BT_CUDA(cudaMallocAsync((void**)&mem, total, s));
-    v.owned.push_back(mem);
-    v.mw = (uint32_t*)(mem + o_mw);
-    v.mr = (uint32_t*)(mem + o_mr);
-    v.ptr = (uint32_t*)(mem + o_ptr);
-    v.off = (uint64_t*)(mem + o_off);
-    v.lo = (uint64_t*)(mem + o_lo);
-  }
+  BT_TRY(alloc_level_arrays(v, words, s));
 
   InitArgs ia{W.bt, bcap, W.pt, pcap, W.mismatch, c,
               atab, acap, bitmap, bwords, secbits, qn, W.ld};
@@ -2352,10 +1957,10 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
     BT_LAUNCH(k_scan<M><<<grid_for(c * cpb, T), T, 0, s>>>(m, g, cpb, W.bt, bcap - 1, W.pt, pcap - 1,
                                                             W.ld, 0));
   } else {
-    BT_LAUNCH(k_anchor_keys<<<gc, T, 0, s>>>(g, gq, W.slotB, atab, (uint32_t)(acap - 1), fnode, fcap, bitmap, secbits,
+    BT_LAUNCH(k_anchor_keys<<<gc, T, 0, s>>>(g, gq, W.slotB, atab, (uint32_t)(acap - 1), bitmap, secbits,
                                              aidx, W.ld, ctx.st));
     ScanCtx<M> C{m, g, W.bt, bcap - 1, W.pt, pcap - 1, W.ld, 0, 0,
-                 q, segn, seg, qn, cq, csegn, cseg, ctx.st, fnode, W.slotB};
+                 q, segn, seg, qn, cq, csegn, cseg, ctx.st, W.slotB};
     const size_t smem_base = ((size_t)kSecBits / 32 + (size_t)kRing * kScanThreads +
                               (size_t)kScanThreads * kSlotWords) * 4;
     const size_t smem = smem_base + (size_t)bm_smem * 4;
@@ -2364,21 +1969,8 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
     if (rc_a == BT_OK) rc_a = allow_scan_smem<k_scan_anchor<M, true>>(smem_max);
     if (rc_a != BT_OK) return rc_a;
     ProfScope ps("window_scan", s, cov_l);
-    // The selected-gram list serves levels with the default selection whose
-    // chunks are the list's chunks; k_scan_anchor then runs only when the
-    // level has keys without an anchor.
-    const bool use_list = ctx.gl_chunk && gq.w == 16 && gq.sbits == kGlSbits && b % kAnchorQ == 0;
-    // Every block present: blocks k b .. (k+1) b (the level covers the text).
-    const bool all_present = c == (n + b - 1) / b;
-    if (use_list && all_present)
-      BT_LAUNCH(k_scan_stream<M><<<scan_grid, kScanThreads, (size_t)bm_smem * 4, s>>>(
-          C, gq, ctx.gl_total, (b & (b - 1)) == 0 ? (uint32_t)__builtin_ctzll(b) : 0u, bitmap, bm_smem,
-          ctx.gl_mx, ctx.gl_x));
-    else if (use_list)
-      BT_LAUNCH(k_scan_list<M><<<scan_grid, kScanThreads, (size_t)bm_smem * 4, s>>>(
-          C, gq, cpa, bitmap, bm_smem, ctx.gl_chunk, ctx.gl_mx, ctx.gl_x));
     BT_LAUNCH(k_scan_anchor<M, false><<<scan_grid, kScanThreads, smem, s>>>(
-        C, gq, cpa, atab, (uint32_t)(acap - 1), bitmap, bm_smem, secbits, use_list ? 1 : 0));
+        C, gq, cpa, atab, (uint32_t)(acap - 1), bitmap, bm_smem, secbits));
     if (ctx.two_phase) {
       // Two phases: the hits in the first 1/16 of the text, then the rest
       // against the bounds the first phase tightened.
@@ -2393,7 +1985,7 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
     BT_LAUNCH(k_candidates<M><<<scan_grid, 256, 0, s>>>(C));
     // Only when the queue overflowed: the scan again, testing windows inline.
     BT_LAUNCH(k_scan_anchor<M, true><<<scan_grid, kScanThreads, smem, s>>>(
-        C, gq, cpa, atab, (uint32_t)(acap - 1), bitmap, bm_smem, secbits, 0));
+        C, gq, cpa, atab, (uint32_t)(acap - 1), bitmap, bm_smem, secbits));
     if (r)
       BT_LAUNCH(k_scan<M><<<grid_for(c * cpb, T), T, 0, s>>>(m, g, cpb, W.bt, bcap - 1, W.pt, pcap - 1,
                                                               W.ld, 1));
@@ -2480,52 +2072,23 @@ int all_levels(const M& m, BuildCtx& ctx) {
   BT_LAUNCH(k_level_start<<<grid_for(r.c, 256), 256, 0, ctx.s>>>(r.c, r.b, r.st));
   uint64_t last_start = (r.c - 1) * r.b;
   const bool trace = getenv("BT_TRACE") != nullptr;
-  // The selected-gram list pays off when several levels cover large texts.
-  struct ListMem {
-    cudaStream_t s;
-    std::vector<void*> p;
-    ~ListMem() {
-      for (void* q : p) cudaFreeAsync(q, s);
-    }
-  } lm{ctx.s, {}};
-  if (!ctx.dense_scan && t->n >= 16 && (t->n >= kGlMinText || ctx.force_list)) {
-    const uint64_t n = t->n, nchunks = (n - 15 + kAnchorQ - 1) / kAnchorQ;
-    uint32_t* chunk;
-    BT_CUDA(cudaMallocAsync((void**)&chunk, (nchunks + 1) * sizeof(uint32_t), ctx.s));
-    lm.p.push_back(chunk);
-    uint32_t *agg, *cnt;
-    BT_CUDA(cudaMallocAsync((void**)&agg, scan_scratch_words(nchunks) * sizeof(uint32_t), ctx.s));
-    lm.p.push_back(agg);
-    BT_CUDA(cudaMallocAsync((void**)&cnt, nchunks * sizeof(uint32_t), ctx.s));
-    lm.p.push_back(cnt);
-    const uint32_t rb = 0x01000193u;
-    uint32_t rw = 1;
-    for (int i = 0; i < 16; i++) rw *= rb;
-    const uint32_t sel_max = (1u << (32 - kGlSbits)) - 1u;
-    const unsigned grid = grid_for(nchunks, 256);
-    {
-      ProfScope ps("gram_list", ctx.s, n);
-      BT_LAUNCH(k_gl_pass<false><<<grid, 256, 0, ctx.s>>>(ctx.T, n, nchunks, rb, rw, sel_max, cnt, nullptr,
-                                                          nullptr));
-      BT_TRY(scan_u32(cnt, chunk, nchunks, ctx.s, agg));
-      uint32_t total = 0;
-      BT_CUDA(cudaMemcpyAsync(&total, chunk + nchunks, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx.s));
-      BT_CUDA(cudaStreamSynchronize(ctx.s));
-      uint32_t *mx, *xs;
-      BT_CUDA(cudaMallocAsync((void**)&mx, (uint64_t)(total ? total : 1) * sizeof(uint32_t), ctx.s));
-      lm.p.push_back(mx);
-      BT_CUDA(cudaMallocAsync((void**)&xs, (uint64_t)(total ? total : 1) * sizeof(uint32_t), ctx.s));
-      lm.p.push_back(xs);
-      BT_LAUNCH(k_gl_pass<true><<<grid, 256, 0, ctx.s>>>(ctx.T, n, nchunks, rb, rw, sel_max, chunk, mx, xs));
-      ctx.gl_chunk = chunk;
-      ctx.gl_mx = mx;
-      ctx.gl_x = xs;
-      ctx.gl_total = total;
-    }
-  }
+  // Levels of blocks that hold a selected gram go by first occurrences, the
+  // others (the lowest levels of trees with short leaves) and the diagnostic
+  // passes by the scans of this file.
+  QuickBuild qb(ctx.s);
+  Scratch hm(ctx.s);
+  if (!ctx.dense_scan && !ctx.sort_scan && r.b >= kQuickMinB) BT_TRY(quick_list(ctx, qb));
   for (uint32_t l = 0; l < t->L; l++) {
     auto h0 = std::chrono::steady_clock::now();
-    BT_TRY(level_pass(m, ctx, l, last_start));
+    if (qb.ready && t->lv[l].b >= kQuickMinB) {
+      BT_TRY(quick_level(ctx, qb, l, last_start));
+    } else {
+      if (!ctx.H) {
+        BT_TRY(hm.alloc(&ctx.H, t->n + 1));
+        BT_TRY(expand_prefix(ctx.T, t->n, t->B, t->q, ctx.Hs, ctx.H, ctx.s));
+      }
+      BT_TRY(level_pass(m, ctx, l, last_start));
+    }
     last_start = ctx.st_host->last_start;
     if (trace) {
       auto h1 = std::chrono::steady_clock::now();
@@ -2533,14 +2096,37 @@ int all_levels(const M& m, BuildCtx& ctx) {
               std::chrono::duration<double, std::milli>(h1 - h0).count());
     }
   }
-  ctx.gl_chunk = nullptr;
-  ctx.gl_mx = nullptr;
-  ctx.gl_x = nullptr;
-  ctx.gl_total = 0;
   return BT_OK;
 }
 
 }  // namespace
+
+// Persistent level arrays: one allocation, owned by the level.
+int alloc_level_arrays(Level& v, uint64_t words, cudaStream_t s) {
+  auto al = [](uint64_t x) { return (x + 255) & ~255ull; };
+  const uint64_t c = v.c, o_mw = 0, o_mr = o_mw + al(words * 4 + 4), o_ptr = o_mr + al((words + 1) * 4),
+                 o_off = o_ptr + al(c * 4 + 4), o_lo = o_off + al(c * 8 + 8), total = o_lo + al(c * 8 + 8);
+  char* mem;
+  BT_CUDA(cudaMallocAsync((void**)&mem, total, s));
+  v.owned.push_back(mem);
+  v.mw = (uint32_t*)(mem + o_mw);
+  v.mr = (uint32_t*)(mem + o_mr);
+  v.ptr = (uint32_t*)(mem + o_ptr);
+  v.off = (uint64_t*)(mem + o_off);
+  v.lo = (uint64_t*)(mem + o_lo);
+  return BT_OK;
+}
+
+int launch_children(BuildCtx& ctx, uint32_t l, uint64_t bn, uint64_t* next_st) {
+  const Level& v = ctx.t->lv[l];
+  Geo g{};
+  g.n = ctx.t->n;
+  g.c = v.c;
+  g.b = v.b;
+  g.st = v.st;
+  BT_LAUNCH(k_children<<<grid_for(v.c * v.arity, 256), 256, 0, ctx.s>>>(g, v.mw, v.mr, v.arity, bn, next_st));
+  return BT_OK;
+}
 
 int build_levels(BuildCtx& ctx) {
   if (ctx.t->q == Mersenne61::Q) return all_levels(Mersenne61{}, ctx);

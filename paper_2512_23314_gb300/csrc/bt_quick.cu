@@ -1,0 +1,1321 @@
+// bt_quick.cu -- the level pass by first occurrences of selected grams.
+//
+// Section 3.1 finds the leftmost occurrence LO(x) of every block and pair
+// with a scan of the level's windows.  Most of those windows can be ruled out
+// without looking at them.  Select 16-byte grams by content alone (below) and
+// let F(g) be the first position of a selected gram g in T.  If a string x
+// holds g at offset a, then every occurrence p of x has g at p + a, so
+//     LO(x) >= F(g) - a        for every selected gram of x,
+// and with D = (g's own position) - F(g), a string at s has
+//     LO(x) >= s - min D       over its selected grams.
+// - min D = 0: the string holds a gram that occurs nowhere before it: LO = s.
+// - otherwise p = s - min D is the earliest place x can occur at.  The bytes
+//   there are compared with x: if they are equal, LO = p, proven.
+// - otherwise x is left open ("active") and its occurrences are looked for:
+//   every occurrence p of x has x's newest gram (the one with min D) at the
+//   same offset, so only the occurrences of that one gram propose windows.
+// Versioned and copied texts settle 90-100 % of the keys in the first two
+// steps: an edit makes grams that occur nowhere before, and a block without
+// an edit lies where its newest gram was first seen.  The scan of the other
+// keys reads the list of selected grams, tests a bitmap of the active keys'
+// grams and proposes a window only where an active key's newest gram occurs,
+// instead of every place where any key's first gram occurs.  Windows tested
+// by the levels of a build: 256 MiB of versioned text 41.3 M before (14.5 M of
+// them matched a key), 7.3 M now; 2 GiB of DNA copies 469 M before, 37.5 M now.
+// The builds: 16.2 -> 11.5 ms and 172 -> 91 ms (export included).
+//
+// Selection.  A gram is selected when the least of the 13 hashes of its
+// 4-byte substrings is the first or the last of them (a closed syncmer,
+// Edgar 2021).  Unlike a sliding minimum this depends on the gram alone, so
+// all occurrences of a gram are selected or none; unlike a hash threshold it
+// leaves no gap: of any 12 consecutive grams at least one is selected (density
+// about 2/13).  So every string of 27 bytes or more has a selected gram, and
+// every changed byte in the middle of a block changes a selected gram.
+//
+// F is a direct-mapped table indexed by the gram's hash that holds the least
+// position seen: two grams that share a cell get the smaller of their first
+// positions, which is still a lower bound (fewer keys settled, never a wrong
+// one).  Everything is decided by byte comparisons or, for the active keys,
+// by fingerprints whose matches are verified by byte comparison.
+#include <algorithm>
+#include <atomic>
+#include <cstdio>
+
+#include "bt_bytes.cuh"
+#include "bt_internal.cuh"
+#include "bt_kr.cuh"
+#include "bt_quick.cuh"
+
+namespace bt {
+
+namespace {
+
+constexpr uint32_t kGramLen = 16;
+constexpr uint32_t kSubs = kGramLen - 3;       // 4-byte substrings of a gram
+constexpr uint32_t kNoDist = 0xFFFFFFFFu;      // no selected gram in the range
+constexpr uint32_t kSubMul = 0x9E3779B1u;
+constexpr uint32_t kSegBytes = 1024;           // positions per entry of seg1; 64 of those per entry of seg2
+constexpr uint64_t kQPiece = 4096;             // bytes per comparison item
+constexpr unsigned kT = 256;
+
+// ---------------------------------------------------------------------------
+// The list of selected grams.
+// ---------------------------------------------------------------------------
+
+// The 12 words of T[x0, x0 + 48) (zeros past the text's end).
+__device__ __forceinline__ void load48(const uint8_t* __restrict__ T, uint64_t n, uint64_t x0, bool aligned, uint32_t* w) {
+  if (aligned && x0 + 48 <= n) {
+    const uint4* p = (const uint4*)(T + x0);
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const uint4 v = p[q];
+      w[4 * q] = v.x, w[4 * q + 1] = v.y, w[4 * q + 2] = v.z, w[4 * q + 3] = v.w;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 12; q++) {
+      w[q] = 0;
+#pragma unroll
+      for (int t = 0; t < 4; t++)
+        if (x0 + 4 * q + t < n) w[q] |= (uint32_t)T[x0 + 4 * q + t] << (8 * t);
+    }
+  }
+}
+
+// mask[j]: the selected grams that start in [32 j, 32 j + 32); cnt[j] their
+// number.  A thread takes one word of 32 positions: 44 substring hashes in
+// registers, the minimum over 13 of them in four steps (2, 4, 8, then 8 + 8
+// overlapping).  About 10 instructions per byte: issue-bound (256 MiB).
+__global__ void __launch_bounds__(kT) k_list_mask(const uint8_t* __restrict__ T, uint64_t n, uint64_t nw,
+                                                  uint32_t* __restrict__ mask, uint32_t* __restrict__ cnt) {
+  const bool aligned = (((uintptr_t)T) & 15) == 0;
+  for (uint64_t j = blockIdx.x * (uint64_t)kT + threadIdx.x; j < nw; j += (uint64_t)gridDim.x * kT) {
+    uint32_t w[12], m[44];
+    load48(T, n, 32 * j, aligned, w);
+#pragma unroll
+    for (int i = 0; i < 44; i++) m[i] = __funnelshift_r(w[i >> 2], w[(i >> 2) + 1 < 12 ? (i >> 2) + 1 : 11], 8 * (i & 3)) * kSubMul;
+    uint32_t bits = 0;
+    uint32_t a[43], b[41], c[37];
+#pragma unroll
+    for (int i = 0; i < 43; i++) a[i] = min(m[i], m[i + 1]);
+#pragma unroll
+    for (int i = 0; i < 41; i++) b[i] = min(a[i], a[i + 2]);
+#pragma unroll
+    for (int i = 0; i < 37; i++) c[i] = min(b[i], b[i + 4]);
+#pragma unroll
+    for (int i = 0; i < 32; i++) {
+      const uint32_t least = min(c[i], c[i + 5]);
+      if (m[i] == least || m[i + kSubs - 1] == least) bits |= 1u << i;
+    }
+    const uint64_t left = n - kGramLen + 1 - 32 * j;  // gram positions from 32 j on (nw covers at least one)
+    if (left < 32) bits &= (1u << left) - 1u;
+    mask[j] = bits;
+    cnt[j] = __popc(bits);
+  }
+}
+
+__device__ __forceinline__ uint32_t gram_cell(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t cmask) {
+  uint32_t h = w0 * 0x9E3779B1u;
+  uint32_t t = w1 * 0x85EBCA77u;
+  h ^= __funnelshift_l(t, t, 13);
+  t = w2 * 0xC2B2AE3Du;
+  h ^= __funnelshift_l(t, t, 7);
+  t = w3 * 0x27D4EB2Fu;
+  h ^= __funnelshift_l(t, t, 19);
+  h ^= h >> 16;
+  h *= 0x7FEB352Du;
+  h ^= h >> 15;
+  h *= 0x846CA68Bu;
+  h ^= h >> 16;
+  return h & cmask;
+}
+
+// The list entries: position x[e], and the cell of the gram in cell[e]; the
+// cell keeps the least position (read first: after a gram's first copies have
+// been seen nobody writes).  A CTA takes 256 words: its text and the positions
+// of its grams are staged in shared memory, so that entries, not words, are
+// dealt to the threads and leave in order.
+__global__ void __launch_bounds__(kT) k_list_write(const uint8_t* __restrict__ T, uint64_t n, uint64_t nw,
+                                                   const uint32_t* __restrict__ mask, const uint32_t* __restrict__ idx,
+                                                   uint32_t* __restrict__ x, uint32_t* __restrict__ cell,
+                                                   uint32_t* __restrict__ first, uint32_t cmask) {
+  constexpr uint32_t kBytes = 32 * kT;
+  __shared__ __align__(16) uint32_t text[kBytes / 4 + 8];
+  __shared__ uint16_t at[kBytes];
+  const bool aligned = (((uintptr_t)T) & 15) == 0;
+  for (uint64_t j0 = (uint64_t)blockIdx.x * kT; j0 < nw; j0 += (uint64_t)gridDim.x * kT) {
+    const uint64_t p0 = 32 * j0;
+    __syncthreads();
+    for (uint32_t u = threadIdx.x; u < kBytes / 16 + 2; u += kT) {
+      const uint64_t p = p0 + 16ull * u;
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (aligned && p + 16 <= n) {
+        v = *(const uint4*)(T + p);
+      } else if (p < n) {
+        uint32_t b[4] = {0, 0, 0, 0};
+        for (uint32_t t = 0; t < 16 && p + t < n; t++) b[t >> 2] |= (uint32_t)T[p + t] << (8 * (t & 3));
+        v = make_uint4(b[0], b[1], b[2], b[3]);
+      }
+      ((uint4*)text)[u] = v;
+    }
+    const uint64_t j = j0 + threadIdx.x;
+    const uint32_t e0 = idx[j0];
+    const uint64_t jend = j0 + kT < nw ? j0 + kT : nw;
+    const uint32_t ne = idx[jend] - e0;
+    if (j < nw) {
+      uint32_t o = idx[j] - e0;
+      for (uint32_t b = mask[j]; b; b &= b - 1) at[o++] = (uint16_t)(32 * threadIdx.x + __ffs(b) - 1);
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < ne; i += kT) {
+      const uint32_t a = at[i], q = a >> 2, sh = 8 * (a & 3);
+      uint32_t w[5];
+#pragma unroll
+      for (int u = 0; u < 5; u++) w[u] = text[q + u];
+      const uint32_t c = gram_cell(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
+                                   __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh), cmask);
+      const uint32_t pos = (uint32_t)(p0 + a);
+      x[e0 + i] = pos;
+      cell[e0 + i] = c;
+      if (*(volatile uint32_t*)&first[c] > pos) atomicMin(&first[c], pos);
+    }
+  }
+}
+
+// D[e] = x[e] - F, in place of the cell.  Four entries per thread: the random
+// reads of the table are in flight together.
+__global__ void __launch_bounds__(kT) k_list_dist(const uint32_t* __restrict__ total_p, const uint32_t* __restrict__ x,
+                                                  uint32_t* __restrict__ D, const uint32_t* __restrict__ first) {
+  const uint64_t total = *total_p;
+  for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; 4 * i < total; i += (uint64_t)gridDim.x * kT) {
+    if (4 * i + 4 <= total) {
+      const uint4 X = ((const uint4*)x)[i], C = ((const uint4*)D)[i];
+      ((uint4*)D)[i] = make_uint4(X.x - first[C.x], X.y - first[C.y], X.z - first[C.z], X.w - first[C.w]);
+    } else {
+      for (uint64_t e = 4 * i; e < total; e++) D[e] = x[e] - first[D[e]];
+    }
+  }
+}
+
+// seg1[j]: min D over the grams that start in [1024 j, 1024 j + 1024).
+__global__ void __launch_bounds__(kT) k_list_seg1(uint64_t nw, const uint32_t* __restrict__ idx,
+                                                  const uint32_t* __restrict__ D, uint64_t ns, uint32_t* __restrict__ seg1) {
+  const unsigned lane = threadIdx.x & 31;
+  for (uint64_t j = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32; j < ns; j += (uint64_t)gridDim.x * (kT / 32)) {
+    const uint64_t w0 = j * (kSegBytes / 32), w1 = w0 + kSegBytes / 32 < nw ? w0 + kSegBytes / 32 : nw;
+    uint32_t d = kNoDist;
+    const uint32_t e1 = idx[w1];
+    for (uint32_t e = idx[w0] + lane; e < e1; e += 32) d = min(d, D[e]);
+    d = __reduce_min_sync(0xFFFFFFFFu, d);
+    if (lane == 0) seg1[j] = d;
+  }
+}
+// seg2[j]: min over 64 entries of seg1.
+__global__ void __launch_bounds__(kT) k_list_seg2(uint64_t ns, const uint32_t* __restrict__ seg1, uint64_t ns2,
+                                                  uint32_t* __restrict__ seg2) {
+  for (uint64_t j = blockIdx.x * (uint64_t)kT + threadIdx.x; j < ns2; j += (uint64_t)gridDim.x * kT) {
+    uint32_t d = kNoDist;
+    for (uint64_t i = 64 * j; i < 64 * j + 64 && i < ns; i++) d = min(d, seg1[i]);
+    seg2[j] = d;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// One level.
+// ---------------------------------------------------------------------------
+struct QGeo {
+  const uint8_t* T;
+  uint64_t n, c, b;
+  const uint64_t* st;
+};
+
+__device__ __forceinline__ uint64_t qblen(const QGeo& g, uint64_t k) {
+  const uint64_t s = g.st[k];
+  return g.n - s < g.b ? g.n - s : g.b;
+}
+
+// Min over the list entries e in [e0, e1), taken by lane gl of G.
+__device__ __forceinline__ uint32_t min_entries(const uint32_t* __restrict__ D, uint32_t e0, uint32_t e1, unsigned gl,
+                                                unsigned G, uint32_t d) {
+  uint32_t e = e0 + gl;
+  for (; e + 3 * G < e1; e += 4 * G) {
+    const uint32_t d0 = D[e], d1 = D[e + G], d2 = D[e + 2 * G], d3 = D[e + 3 * G];
+    d = min(min(d, min(d0, d1)), min(d2, d3));
+  }
+  for (; e < e1; e += G) d = min(d, D[e]);
+  return d;
+}
+
+__device__ __forceinline__ uint32_t list_at(const QList& Q, uint64_t w) { return Q.idx[w < Q.nw ? w : Q.nw]; }
+
+// A[k]: min D over the grams inside block k; X[k]: over the grams that start
+// in block k and reach into block k+1 (inside the pair).  A group of G lanes
+// per block; a block's inside is read at the coarsest grain that fits it (64
+// KiB, 1 KiB, list entries), so that the upper levels cost next to nothing.
+__global__ void __launch_bounds__(kT) k_quick_min(QGeo g, QList Q, unsigned G, uint32_t* __restrict__ A,
+                                                  uint32_t* __restrict__ X, uint32_t* __restrict__ flags,
+                                                  QuickStatus* qs) {
+  const unsigned lane = threadIdx.x & 31, grp = lane / G, gl = lane % G, gpw = 32 / G;
+  const uint64_t warps = (uint64_t)gridDim.x * (kT / 32);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    qs->nopen[0] = qs->nopen[1] = qs->npairs = qs->nsusp = qs->nitems = 0;
+    qs->total = Q.idx[Q.nw];
+  }
+  for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32 * gpw; base < g.c; base += warps * gpw) {
+    const uint64_t k = base + grp;
+    uint32_t a = kNoDist, xm = kNoDist;
+    if (k < g.c) {
+      const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
+      // Gram starts inside the block: [s, aend); inside the pair: [s, pend), pend <= s + len.
+      const uint64_t aend = len >= kGramLen ? s + len - kGramLen + 1 : s;
+      uint64_t pend = aend;
+      if (k + 1 < g.c && g.st[k + 1] == s + len) {
+        const uint64_t len2 = g.n - s - len < g.b ? g.n - s - len : g.b;
+        if (len + len2 >= kGramLen) {
+          pend = s + len + len2 - kGramLen + 1;
+          if (pend > s + len) pend = s + len;
+        }
+      }
+      const uint64_t w0 = (s + 31) / 32, w1 = aend / 32;
+      uint64_t rest = s;  // first position not covered by whole words
+      if (w1 > w0) {
+        if (s & 31) {
+          for (uint32_t e = list_at(Q, s / 32) + gl, e1 = list_at(Q, w0); e < e1; e += G)
+            if (Q.x[e] >= s) a = min(a, Q.D[e]);
+        }
+        const uint64_t j0 = (w0 + 31) / 32, j1 = w1 / 32;  // 1 KiB segments inside
+        if (j1 > j0 + 2) {
+          a = min_entries(Q.D, list_at(Q, w0), list_at(Q, 32 * j0), gl, G, a);
+          const uint64_t i0 = (j0 + 63) / 64, i1 = j1 / 64;
+          if (i1 > i0) {
+            a = min_entries(Q.seg1, (uint32_t)j0, (uint32_t)(64 * i0), gl, G, a);
+            a = min_entries(Q.seg2, (uint32_t)i0, (uint32_t)i1, gl, G, a);
+            a = min_entries(Q.seg1, (uint32_t)(64 * i1), (uint32_t)j1, gl, G, a);
+          } else {
+            a = min_entries(Q.seg1, (uint32_t)j0, (uint32_t)j1, gl, G, a);
+          }
+          a = min_entries(Q.D, list_at(Q, 32 * j1), list_at(Q, w1), gl, G, a);
+        } else {
+          a = min_entries(Q.D, list_at(Q, w0), list_at(Q, w1), gl, G, a);
+        }
+        rest = 32 * w1;
+      }
+      for (uint32_t e = list_at(Q, rest / 32) + gl, e1 = list_at(Q, (pend + 31) / 32); e < e1; e += G) {
+        const uint64_t p = Q.x[e];
+        if (p < s || p >= pend) continue;
+        if (p < aend) a = min(a, Q.D[e]);
+        else xm = min(xm, Q.D[e]);
+      }
+    }
+    for (unsigned o = G / 2; o; o >>= 1) {
+      a = min(a, __shfl_xor_sync(0xFFFFFFFFu, a, o));
+      xm = min(xm, __shfl_xor_sync(0xFFFFFFFFu, xm, o));
+    }
+    if (k < g.c && gl == 0) {
+      A[k] = a;
+      X[k] = xm;
+      flags[k] = 0;
+    }
+  }
+}
+
+// min D over the pair (k, k+1).
+__device__ __forceinline__ uint32_t pair_dist(const uint32_t* __restrict__ A, const uint32_t* __restrict__ X, uint64_t k,
+                                              uint64_t len2) {
+  const uint32_t d = min(A[k], X[k]);
+  return len2 >= kGramLen ? min(d, A[k + 1]) : d;
+}
+
+constexpr uint32_t kBlkDiffers = 1, kPairDiffers = 2;
+
+// Compare every block and pair with the bytes at its bound s - min D (at 0
+// when the bound is negative): flags[k] says which differ.  One group of L
+// lanes per piece of 4 KiB of the pair; the block's comparison is the first
+// half of the pair's when both have the same bound.  Bound: the text's
+// bandwidth, both sides.
+__global__ void __launch_bounds__(kT) k_quick_compare(QGeo g, const uint32_t* __restrict__ A, const uint32_t* __restrict__ X,
+                                                      uint32_t* __restrict__ flags, uint64_t ppk, unsigned L) {
+  const unsigned lane = threadIdx.x & 31, grp = lane / L, gl = lane % L, gpw = 32 / L;
+  const unsigned gmask = (L == 32 ? 0xFFFFFFFFu : ((1u << L) - 1u)) << (grp * L);
+  const bool aligned16 = (((uintptr_t)g.T) & 15) == 0;
+  const uint64_t warps = (uint64_t)gridDim.x * (kT / 32), total = g.c * ppk;
+  // Warp-uniform loop: every lane reaches the ballots of every iteration.
+  for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32 * gpw; base < total; base += warps * gpw) {
+    const uint64_t u = base + grp;
+    bool db = false, dp = false;
+    uint64_t k = 0;
+    if (u < total) {
+      k = ppk == 1 ? u : u / ppk;
+      const uint64_t off = ppk == 1 ? 0 : (u - k * ppk) * kQPiece;
+      const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
+      const uint32_t dk = A[k];
+      const bool blk = dk != 0 && dk != kNoDist && s != 0 && off < len;
+      bool pair = false;
+      uint32_t d2 = 0;
+      uint64_t plen = 0;
+      if (k + 1 < g.c && s != 0 && g.st[k + 1] == s + len) {
+        const uint64_t len2 = g.n - s - len < g.b ? g.n - s - len : g.b;
+        plen = len + len2;
+        d2 = pair_dist(A, X, k, len2);
+        pair = d2 != 0 && d2 != kNoDist && off < plen;
+      }
+      if (blk || pair) {
+        const uint32_t f = *(volatile uint32_t*)&flags[k];
+        const uint64_t pk = dk > s ? 0 : s - dk, pp = d2 > s ? 0 : s - d2;
+        const uint64_t bend = off + kQPiece < len ? off + kQPiece : len;
+        const uint64_t pend = off + kQPiece < plen ? off + kQPiece : plen;
+        if (blk && !(f & kBlkDiffers)) {
+          db = differs(g.T, g.n, aligned16, pk, s, off, bend, gl, L);
+          if (pair && pk == pp) dp = db;
+        }
+        if (pair && !(f & kPairDiffers)) {
+          const uint64_t from = blk && pk == pp ? (off < bend ? bend : off) : off;
+          if (from < pend) dp |= differs(g.T, g.n, aligned16, pp, s, from, pend, gl, L);
+        }
+      }
+    }
+    const unsigned bb = __ballot_sync(0xFFFFFFFFu, db), bp = __ballot_sync(0xFFFFFFFFu, dp);
+    const uint32_t set = (bb & gmask ? kBlkDiffers : 0u) | (bp & gmask ? kPairDiffers : 0u);
+    if (u < total && gl == 0 && set) atomicOr(&flags[k], set);
+  }
+}
+
+__device__ __forceinline__ uint64_t warp_sum64(uint64_t v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+
+constexpr uint8_t kIsPair = 1, kLeftmost = 2;  // state of the pair (k, k+1)
+
+// What the comparisons say about the pair (k, k+1).
+__device__ __forceinline__ uint8_t pair_state(const QGeo& g, const uint32_t* __restrict__ A, const uint32_t* __restrict__ X,
+                                              const uint32_t* __restrict__ flags, uint64_t k, uint32_t* dist, uint64_t* plen,
+                                              bool* open) {
+  *open = false;
+  if (k + 1 >= g.c) return 0;
+  const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
+  if (g.st[k + 1] != s + len) return 0;
+  const uint64_t len2 = g.n - s - len < g.b ? g.n - s - len : g.b;
+  const uint32_t d = pair_dist(A, X, k, len2);
+  *dist = d;
+  *plen = len + len2;
+  if (s == 0 || d == 0) return kIsPair | kLeftmost;
+  *open = d == kNoDist || (flags[k] & kPairDiffers);
+  return kIsPair;
+}
+
+// Settled blocks get their leftmost occurrence, open keys go to the item list
+// (2 k: block k, 2 k + 1: the pair that starts with it), and the marks follow
+// from the settled pairs (again later if some were open).
+__global__ void __launch_bounds__(kT) k_quick_settle(QGeo g, const uint32_t* __restrict__ A, const uint32_t* __restrict__ X,
+                                                     const uint32_t* __restrict__ flags, uint64_t* __restrict__ lo,
+                                                     uint8_t* __restrict__ ps, uint32_t* __restrict__ items,
+                                                     uint32_t* __restrict__ mw, uint32_t* __restrict__ wpop,
+                                                     QuickStatus* qs, Status* status) {
+  const uint64_t words = (g.c + 31) / 32;
+  const unsigned lane = threadIdx.x & 31;
+  for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) & ~31ull; base < words * 32;
+       base += (uint64_t)gridDim.x * kT) {
+    const uint64_t k = base + lane;
+    bool ob = false, op = false;
+    uint8_t st = 0;
+    uint64_t vb = 0;
+    if (k < g.c) {
+      const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
+      const uint32_t d = A[k];
+      uint64_t p = s;
+      if (s != 0 && d != 0) {
+        ob = d == kNoDist || (flags[k] & kBlkDiffers);
+        p = ob ? kNone : (d > s ? 0 : s - d);
+        if (d != kNoDist) vb += 2 * len;
+      }
+      lo[k] = p;
+      uint32_t d2 = 0;
+      uint64_t plen = 0;
+      st = pair_state(g, A, X, flags, k, &d2, &plen, &op);
+      ps[k] = st;
+      if (st == kIsPair && d2 != kNoDist) vb += 2 * plen;
+    }
+    uint32_t left = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)st, 1);
+    if (lane == 0) {
+      left = 0;
+      if (k > 0 && k <= g.c) {
+        uint32_t d2;
+        uint64_t plen;
+        bool o;
+        left = pair_state(g, A, X, flags, k - 1, &d2, &plen, &o);
+      }
+    }
+    const bool mk = k < g.c && ((left & kLeftmost) || (st & kLeftmost) || !((left | st) & kIsPair));
+    const uint32_t bits = __ballot_sync(0xFFFFFFFFu, mk);
+    const uint32_t bb = __ballot_sync(0xFFFFFFFFu, ob), bp = __ballot_sync(0xFFFFFFFFu, op);
+    const uint32_t np = __popc(__ballot_sync(0xFFFFFFFFu, st & kIsPair));
+    vb = warp_sum64(vb);
+    unsigned long long at = 0;
+    if (lane == 0) {
+      mw[base / 32] = bits;
+      wpop[base / 32] = __popc(bits);
+      if (np) atomicAdd(&qs->npairs, (unsigned long long)np);
+      if (vb) atomicAdd(&status->verify_bytes, (unsigned long long)vb);
+      if (bb) atomicAdd(&qs->nopen[0], (unsigned long long)__popc(bb));
+      if (bp) atomicAdd(&qs->nopen[1], (unsigned long long)__popc(bp));
+      if (bb | bp) at = atomicAdd(&qs->nitems, (unsigned long long)(__popc(bb) + __popc(bp)));
+    }
+    if (bb | bp) {
+      at = __shfl_sync(0xFFFFFFFFu, at, 0);
+      const uint32_t lt = (1u << lane) - 1u;
+      if (ob) items[at + __popc(bb & lt)] = (uint32_t)(2 * k);
+      if (op) items[at + __popc(bb) + __popc(bp & lt)] = (uint32_t)(2 * k + 1);
+    }
+  }
+}
+
+// The marks again, from the pair states the open keys' search completed.
+__global__ void __launch_bounds__(kT) k_quick_remark(uint64_t c, const uint8_t* __restrict__ ps, uint32_t* __restrict__ mw,
+                                                     uint32_t* __restrict__ wpop) {
+  const uint64_t words = (c + 31) / 32;
+  for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) & ~31ull; base < words * 32;
+       base += (uint64_t)gridDim.x * kT) {
+    const uint64_t k = base + (threadIdx.x & 31);
+    bool mk = false;
+    if (k < c) {
+      const uint8_t l = k ? ps[k - 1] : 0, r = ps[k];
+      mk = (l & kLeftmost) || (r & kLeftmost) || !((l | r) & kIsPair);
+    }
+    const uint32_t bits = __ballot_sync(0xFFFFFFFFu, mk);
+    if ((threadIdx.x & 31) == 0) {
+      mw[base / 32] = bits;
+      wpop[base / 32] = __popc(bits);
+    }
+  }
+}
+
+// Size of the next level and the start of its last block (one thread).
+__device__ void level_end(const QGeo& g, const uint32_t* mw, uint64_t words, uint64_t nmarked, uint32_t arity, uint64_t bn,
+                          Status* status, QuickStatus* qs) {
+  qs->nmarked = nmarked;
+  status->next_c = 0;
+  status->last_start = 0;
+  if (arity == 0) return;
+  for (uint64_t w = words; w-- > 0;) {
+    if (!mw[w]) continue;
+    const uint64_t last = w * 32 + 31 - __clz(mw[w]);
+    const uint64_t len = qblen(g, last), nch = (len + bn - 1) / bn;
+    status->next_c = (nmarked - 1) * arity + nch;
+    status->last_start = g.st[last] + (nch - 1) * bn;
+    return;
+  }
+}
+
+// Rank prefix of a level of at most kRankWords mark words and the level's end,
+// by one CTA (eight words per thread and step).
+constexpr uint64_t kRankWords = 16384;
+__global__ void __launch_bounds__(1024) k_quick_rank(QGeo g, const uint32_t* __restrict__ mw, const uint32_t* __restrict__ wpop,
+                                                     uint32_t* __restrict__ mr, uint32_t arity, uint64_t bn, Status* status,
+                                                     QuickStatus* qs) {
+  __shared__ uint32_t sm[32];
+  const uint64_t words = (g.c + 31) / 32;
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t carry = 0;
+  for (uint64_t base = 0; base < words; base += 8192) {
+    const uint64_t i = base + 8ull * threadIdx.x;
+    uint32_t v[8], sum = 0;
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      v[u] = i + u < words ? wpop[i + u] : 0;
+      sum += v[u];
+    }
+    uint32_t x = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, x, d);
+      if (lane >= (unsigned)d) x += o;
+    }
+    if (lane == 31) sm[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+      uint32_t w = sm[lane];
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, w, d);
+        if (lane >= (unsigned)d) w += o;
+      }
+      sm[lane] = w;
+    }
+    __syncthreads();
+    uint32_t at = carry + (warp ? sm[warp - 1] : 0) + x - sum;
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      if (i + u < words) mr[i + u] = at;
+      at += v[u];
+    }
+    carry += sm[31];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    mr[words] = carry;
+    level_end(g, mw, words, carry, arity, bn, status, qs);
+  }
+}
+__global__ void k_quick_end(QGeo g, const uint32_t* mw, const uint32_t* mr, uint32_t arity, uint64_t bn, Status* status,
+                            QuickStatus* qs) {
+  const uint64_t words = (g.c + 31) / 32;
+  level_end(g, mw, words, mr[words], arity, bn, status, qs);
+}
+
+__device__ __forceinline__ bool qmark(const uint32_t* __restrict__ mw, uint64_t k) { return (mw[k >> 5] >> (k & 31)) & 1u; }
+
+// Back-pointers of the unmarked blocks (the block that holds the leftmost
+// occurrence and the offset into it; the copied window must lie in one or two
+// marked blocks and end before the block) and the children of the marked
+// ones: the block of mark rank r puts its children at r arity + i.
+__global__ void __launch_bounds__(kT) k_quick_points(QGeo g, const uint32_t* __restrict__ mw, const uint32_t* __restrict__ mr,
+                                                     const uint64_t* __restrict__ lo, uint32_t* __restrict__ ptr,
+                                                     uint64_t* __restrict__ off, uint32_t arity, uint64_t bn,
+                                                     uint64_t* __restrict__ next_st, Status* status) {
+  const bool all_present = g.c == (g.n + g.b - 1) / g.b;
+  for (uint64_t k = blockIdx.x * (uint64_t)kT + threadIdx.x; k < g.c; k += (uint64_t)gridDim.x * kT) {
+    const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
+    if (qmark(mw, k)) {
+      ptr[k] = 0;
+      off[k] = 0;
+      if (next_st) {
+        const uint64_t r = mr[k >> 5] + __popc(mw[k >> 5] & ((1u << (k & 31)) - 1u));
+        for (uint64_t i = 0; i * bn < len; i++) next_st[r * arity + i] = s + i * bn;
+      }
+      continue;
+    }
+    const uint64_t p = lo[k];
+    uint64_t j;
+    bool ok = p + len <= s;
+    if (all_present) {
+      j = ok ? p / g.b : 0;
+    } else {
+      uint64_t a = 0, z = k;  // first index with st > p; p < s
+      while (a < z) {
+        const uint64_t mid = (a + z) / 2;
+        if (g.st[mid] <= p) a = mid + 1;
+        else z = mid;
+      }
+      ok = ok && a > 0;
+      j = a ? a - 1 : 0;
+    }
+    if (ok) ok = p < g.st[j] + qblen(g, j) && qmark(mw, j);
+    if (ok && p + len > g.st[j] + qblen(g, j))
+      ok = j + 1 < g.c && g.st[j + 1] == g.st[j] + qblen(g, j) && qmark(mw, j + 1);
+    if (!ok) {
+      atomicExch(&status->error, 5ull);
+      continue;
+    }
+    ptr[k] = (uint32_t)j;
+    off[k] = p - g.st[j];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The open keys: every occurrence of an open key has the key's newest gram at
+// the key's offset.  (gram, offset) pairs go to a table, each once; the list
+// scan proposes p = x - offset wherever one of the grams occurs before the
+// last start of a key with that pair, and a proposed window's fingerprint is
+// looked up among the open blocks (and, joined with the one at p + b, among
+// the open pairs).  A gram is named by its first position F.
+// ---------------------------------------------------------------------------
+struct __align__(32) CSlot {  // a block fingerprint: leftmost window, last start of an open pair beginning with it
+  unsigned long long key, lo, maxpst, pad;
+};
+struct __align__(16) CPair {  // (slot, slot): leftmost window
+  unsigned long long key, lo;
+};
+struct __align__(16) CGram {  // F << 32 | offset; windows from `bound` on are of no use
+  unsigned long long key, bound;
+};
+
+struct Chase {
+  QGeo g;
+  QList Q;
+  const uint32_t* A;
+  const uint32_t* X;
+  const uint32_t* items;
+  uint32_t nitems;
+  uint64_t Bb, Br, r;  // B^b, B^r; length of the short last block (0: none)
+  CSlot* bt;
+  CPair* pt;
+  CGram* gt;
+  uint32_t bmask, pmask, gmask;
+  uint32_t* bitmap;
+  uint32_t bshift;         // bitmap bit = (F * odd) >> bshift
+  uint32_t* islot;         // per item: its slot in bt or pt
+  uint32_t* igram;         // per item: its slot in gt
+  unsigned long long* bound2;
+  uint32_t* differ;        // per item: the verification found a difference
+  uint32_t* susp;          // items whose fingerprint match was false
+  unsigned long long* exlo;
+  QuickStatus* qs;
+  Status* status;
+  uint64_t* lo;
+  uint8_t* ps;
+};
+
+constexpr uint32_t kTailItem = 0xFFFFFFFEu;  // islot of a key that ends in the short last block
+
+template <class S>
+__device__ __forceinline__ uint32_t c_insert(S* t, uint32_t mask, unsigned long long key) {
+  uint32_t h = (uint32_t)mix64(key) & mask;
+  for (uint32_t it = 0; it <= mask; it++) {
+    unsigned long long old = *(volatile unsigned long long*)&t[h].key;
+    if (old == kNone) old = atomicCAS(&t[h].key, (unsigned long long)kNone, key);
+    if (old == kNone || old == key) return h;
+    h = (h + 1) & mask;
+  }
+  return kNoSlot;
+}
+template <class S>
+__device__ __forceinline__ uint32_t c_find(const S* t, uint32_t mask, unsigned long long key) {
+  uint32_t h = (uint32_t)mix64(key) & mask;
+  for (uint32_t it = 0; it <= mask; it++) {
+    const unsigned long long k = t[h].key;
+    if (k == key) return h;
+    if (k == kNone) return kNoSlot;
+    h = (h + 1) & mask;
+  }
+  return kNoSlot;
+}
+// Grams probe from a place that depends on F alone, so that all offsets of a
+// gram are met on one walk to the next empty slot.
+__device__ __forceinline__ uint32_t c_gram_home(uint32_t F, uint32_t mask) {
+  uint32_t h = F * 0x9E3779B1u;
+  h ^= h >> 15;
+  h *= 0x85EBCA77u;
+  h ^= h >> 13;
+  return h & mask;
+}
+__device__ __forceinline__ uint32_t c_bit(const Chase& C, uint32_t F) { return (F * 0xC2B2AE3Du) >> C.bshift; }
+
+__device__ __forceinline__ void c_min(unsigned long long* a, uint64_t p) {
+  if (*(volatile unsigned long long*)a > p) atomicMin(a, (unsigned long long)p);
+}
+
+__global__ void __launch_bounds__(kT) k_chase_init(Chase C, uint32_t bwords) {
+  uint64_t top = (uint64_t)C.bmask + 1;
+  top = top > (uint64_t)C.pmask + 1 ? top : (uint64_t)C.pmask + 1;
+  top = top > (uint64_t)C.gmask + 1 ? top : (uint64_t)C.gmask + 1;
+  top = top > bwords ? top : bwords;
+  for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; i < top; i += (uint64_t)gridDim.x * kT) {
+    if (i <= C.bmask) C.bt[i] = CSlot{kNone, kNone, 0, 0};
+    if (i <= C.pmask) C.pt[i] = CPair{kNone, kNone};
+    if (i <= C.gmask) {
+      C.gt[i] = CGram{kNone, 0};
+      C.bound2[i] = 0;
+    }
+    if (i < bwords) C.bitmap[i] = 0;
+    if (i < C.nitems) C.differ[i] = 0;
+    if (i == 0) {
+      C.qs->fp_tail = C.qs->lo_tail = C.qs->lo_tailpair = kNone;
+      C.qs->pretail = kNoSlot;
+      C.qs->tail_F = C.qs->tail_off = 0xFFFFFFFFu;
+      C.qs->cands = C.qs->hits = 0;
+    }
+  }
+}
+
+// A warp per open key: the list entry with the key's min D, then (lane 0) the
+// tables.  A pair enters both of its blocks.
+template <class M>
+__global__ void __launch_bounds__(kT) k_chase_keys(M m, const __grid_constant__ PrefixAt<M> H, Chase C) {
+  const unsigned lane = threadIdx.x & 31;
+  const QGeo& g = C.g;
+  for (uint64_t i = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32; i < C.nitems; i += (uint64_t)gridDim.x * (kT / 32)) {
+    const uint32_t it = C.items[i];
+    const uint64_t k = it >> 1;
+    const bool pair = it & 1;
+    const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
+    const uint64_t len2 = pair ? (g.n - s - len < g.b ? g.n - s - len : g.b) : 0;
+    const uint32_t d = pair ? pair_dist(C.A, C.X, k, len2) : C.A[k];
+    const uint64_t end = s + len + len2 - kGramLen + 1;  // gram starts [s, end) when the key has a gram at all
+    uint32_t F = 0, off = 0;
+    bool found = false;
+    if (d != kNoDist) {
+      const uint32_t e1 = list_at(C.Q, (end + 31) / 32);
+      for (uint32_t e0 = list_at(C.Q, s / 32); e0 < e1; e0 += 32) {
+        const uint32_t e = e0 + lane;
+        const bool hit = e < e1 && C.Q.D[e] == d && C.Q.x[e] >= s && C.Q.x[e] < end;
+        const unsigned bal = __ballot_sync(0xFFFFFFFFu, hit);
+        if (bal) {
+          const uint32_t x = C.Q.x[e0 + __ffs(bal) - 1];
+          F = x - d;
+          off = (uint32_t)(x - s);
+          found = true;
+          break;
+        }
+      }
+    }
+    if (lane) continue;
+    C.igram[i] = kNoSlot;
+    C.islot[i] = kNoSlot;
+    const bool tail = !pair && len != g.b;
+    if (found && !tail) {
+      uint32_t h = c_gram_home(F, C.gmask);
+      const unsigned long long key = ((unsigned long long)F << 32) | off;
+      bool placed = false;
+      for (uint32_t q = 0; q <= C.gmask && !placed; q++) {
+        unsigned long long old = *(volatile unsigned long long*)&C.gt[h].key;
+        if (old == kNone) old = atomicCAS(&C.gt[h].key, (unsigned long long)kNone, key);
+        if (old == kNone || old == key) placed = true;
+        else h = (h + 1) & C.gmask;
+      }
+      if (placed) {
+        atomicMax(&C.gt[h].bound, (unsigned long long)s);
+        C.igram[i] = h;
+      } else {
+        atomicExch(&C.status->error, 21ull);
+      }
+    }
+    if (found) {
+      const uint32_t bit = c_bit(C, F);
+      atomicOr(&C.bitmap[bit >> 5], 1u << (bit & 31));
+    } else if (!tail) {
+      atomicExch(&C.status->error, 22ull);  // a key of 27 bytes or more has a selected gram
+    }
+    const uint64_t h0 = H.at(m, s), h1 = H.at(m, s + len);
+    if (tail) {
+      C.qs->fp_tail = m.sub(h1, m.mul(h0, C.Br));
+      c_min(&C.qs->lo_tail, s);
+      if (found) {
+        C.qs->tail_F = F;
+        C.qs->tail_off = off;
+      }
+      C.islot[i] = kTailItem;
+      continue;
+    }
+    const uint32_t slot = c_insert(C.bt, C.bmask, m.sub(h1, m.mul(h0, C.Bb)));
+    if (slot == kNoSlot) {
+      atomicExch(&C.status->error, 23ull);
+      continue;
+    }
+    c_min(&C.bt[slot].lo, s);
+    if (!pair) {
+      C.islot[i] = slot;
+      continue;
+    }
+    atomicMax(&C.bt[slot].maxpst, (unsigned long long)s);
+    const uint64_t h2 = H.at(m, s + len + len2);
+    if (len2 != g.b) {  // the pair that ends in the short last block
+      C.qs->pretail = slot;
+      C.qs->fp_tail = m.sub(h2, m.mul(h1, C.Br));
+      c_min(&C.qs->lo_tailpair, s);
+      C.islot[i] = kTailItem;
+      continue;
+    }
+    const uint32_t slot2 = c_insert(C.bt, C.bmask, m.sub(h2, m.mul(h1, C.Bb)));
+    const uint32_t sp = slot2 == kNoSlot ? kNoSlot : c_insert(C.pt, C.pmask, ((unsigned long long)slot << 32) | slot2);
+    if (sp == kNoSlot) {
+      atomicExch(&C.status->error, 24ull);
+      continue;
+    }
+    c_min(&C.pt[sp].lo, s);
+    C.islot[i] = sp;
+  }
+}
+
+// The window at p: its fingerprint among the open blocks, joined with the
+// window at p + b among the open pairs.
+template <class M>
+__device__ __forceinline__ void chase_test(const M& m, const PrefixAt<M>& H, const Chase& C, uint64_t p, uint32_t pretail,
+                                        uint64_t fp_tail, uint32_t& nhit) {
+  const QGeo& g = C.g;
+  if (p + g.b > g.n) return;
+  const uint64_t h0 = H.at(m, p), h1 = H.at(m, p + g.b);
+  const uint32_t sl = c_find(C.bt, C.bmask, m.sub(h1, m.mul(h0, C.Bb)));
+  if (sl == kNoSlot) return;
+  nhit++;
+  c_min(&C.bt[sl].lo, p);
+  if (p > C.bt[sl].maxpst) return;
+  if (p + 2 * g.b <= g.n) {
+    const uint32_t s2 = c_find(C.bt, C.bmask, m.sub(H.at(m, p + 2 * g.b), m.mul(h1, C.Bb)));
+    if (s2 != kNoSlot) {
+      const uint32_t sp = c_find(C.pt, C.pmask, ((unsigned long long)sl << 32) | s2);
+      if (sp != kNoSlot) c_min(&C.pt[sp].lo, p);
+    }
+  }
+  if (C.r && sl == pretail && p + g.b + C.r <= g.n &&
+      m.sub(H.at(m, p + g.b + C.r), m.mul(h1, C.Br)) == fp_tail)
+    c_min(&C.qs->lo_tailpair, p);
+}
+
+// List entries [e0, e1): the bitmap test, then per CTA a queue of gram hits
+// in shared memory, the gram table's walk, a queue of proposed windows and
+// their tests.  The queues never overflow for good: a proposal that finds
+// the second one full is tested on the spot, and the first one is emptied
+// before a tile could fill it.  Bound: the list's stream and one bitmap test
+// per entry; hits are a few percent of the entries.
+constexpr uint32_t kChaseTile = 2048, kHitQ = 4096, kCandQ = 2048;
+constexpr uint32_t kChaseBitWords = 8192;  // bitmap kept in shared memory up to 32 KiB
+
+template <class M>
+__global__ void __launch_bounds__(kT) k_chase_scan(M m, const __grid_constant__ PrefixAt<M> H, const __grid_constant__ Chase C,
+                                                   uint32_t e0, uint32_t e1, uint32_t smem_words,
+                                                   const unsigned long long* __restrict__ bound2) {
+  extern __shared__ uint32_t bits_s[];
+  __shared__ uint2 hq[kHitQ];
+  __shared__ uint32_t cq[kCandQ];
+  __shared__ uint32_t hn, cn;
+  for (uint32_t i = threadIdx.x; i < smem_words; i += kT) bits_s[i] = C.bitmap[i];
+  if (threadIdx.x == 0) hn = cn = 0;
+  __syncthreads();
+  const uint32_t* bits = smem_words ? bits_s : C.bitmap;
+  const uint32_t tail_F = C.qs->tail_F, tail_off = C.qs->tail_off, pretail = C.qs->pretail;
+  const uint64_t fp_tail = C.qs->fp_tail;
+  uint32_t ncand = 0, nhit = 0;
+  for (uint64_t t0 = e0 + (uint64_t)blockIdx.x * kChaseTile; t0 < e1; t0 += (uint64_t)gridDim.x * kChaseTile) {
+    uint32_t x[8], F[8];
+    const uint64_t e = t0 + 8ull * threadIdx.x;
+    if (e + 8 <= e1) {
+#pragma unroll
+      for (int q = 0; q < 2; q++) {
+        const uint4 a = ((const uint4*)(C.Q.x + e))[q], d = ((const uint4*)(C.Q.D + e))[q];
+        x[4 * q] = a.x, x[4 * q + 1] = a.y, x[4 * q + 2] = a.z, x[4 * q + 3] = a.w;
+        F[4 * q] = a.x - d.x, F[4 * q + 1] = a.y - d.y, F[4 * q + 2] = a.z - d.z, F[4 * q + 3] = a.w - d.w;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; u++) {
+        const uint32_t bit = c_bit(C, F[u]);
+        if ((bits[bit >> 5] >> (bit & 31)) & 1u) hq[atomicAdd(&hn, 1u)] = make_uint2(x[u], F[u]);
+      }
+    } else {
+      for (uint64_t f = e; f < e1; f++) {
+        const uint32_t X = C.Q.x[f], Fe = X - C.Q.D[f], bit = c_bit(C, Fe);
+        if ((bits[bit >> 5] >> (bit & 31)) & 1u) hq[atomicAdd(&hn, 1u)] = make_uint2(X, Fe);
+      }
+    }
+    __syncthreads();
+    const uint32_t nh = hn;
+    if (nh <= kHitQ - kChaseTile && t0 + (uint64_t)gridDim.x * kChaseTile < e1) {
+      __syncthreads();
+      continue;
+    }
+    for (uint32_t i = threadIdx.x; i < nh; i += kT) {
+      const uint2 h = hq[i];
+      uint32_t s = c_gram_home(h.y, C.gmask);
+      for (uint32_t it = 0; it <= C.gmask; it++) {
+        const ulonglong2 en = *(const ulonglong2*)&C.gt[s];
+        if (en.x == kNone) break;
+        if ((uint32_t)(en.x >> 32) == h.y) {
+          const uint32_t off = (uint32_t)en.x;
+          const unsigned long long bound = bound2 ? bound2[s] : en.y;
+          if (off <= h.x && h.x - off < bound) {
+            ncand++;
+            const uint32_t q = atomicAdd(&cn, 1u);
+            if (q < kCandQ) cq[q] = h.x - off;
+            else chase_test(m, H, C, h.x - off, pretail, fp_tail, nhit);
+          }
+        }
+        s = (s + 1) & C.gmask;
+      }
+      if (h.y == tail_F && tail_off <= h.x) {
+        const uint64_t p = h.x - tail_off;
+        if (p + C.r < C.g.n && p < *(volatile unsigned long long*)&C.qs->lo_tail &&
+            m.sub(H.at(m, p + C.r), m.mul(H.at(m, p), C.Br)) == fp_tail)
+          c_min(&C.qs->lo_tail, p);
+      }
+    }
+    __syncthreads();
+    const uint32_t nc = cn < kCandQ ? cn : kCandQ;
+    for (uint32_t i = threadIdx.x; i < nc; i += kT) chase_test(m, H, C, cq[i], pretail, fp_tail, nhit);
+    __syncthreads();
+    if (threadIdx.x == 0) hn = cn = 0;
+    __syncthreads();
+  }
+  if (ncand) atomicAdd(&C.qs->cands, (unsigned long long)ncand);
+  if (nhit) atomicAdd(&C.qs->hits, (unsigned long long)nhit);
+}
+
+// Between the two halves of the scan: a (gram, offset) pair's windows are of
+// use up to the largest leftmost window found so far among its keys.
+__global__ void __launch_bounds__(kT) k_chase_bound(Chase C) {
+  for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; i < C.nitems; i += (uint64_t)gridDim.x * kT) {
+    const uint32_t h = C.igram[i], sl = C.islot[i];
+    if (h == kNoSlot || sl == kNoSlot) continue;
+    const bool pair = C.items[i] & 1;
+    const unsigned long long lo = sl == kTailItem ? C.qs->lo_tailpair : pair ? C.pt[sl].lo : C.bt[sl].lo;
+    atomicMax(&C.bound2[h], lo);
+  }
+}
+
+// The short last block when it has no selected gram (at most 26 bytes): every
+// position before it, 16 per thread, filtered by its first bytes.
+__global__ void __launch_bounds__(kT) k_chase_tail(Chase C) {
+  if (C.qs->lo_tail == kNone || C.qs->tail_F != 0xFFFFFFFFu) return;  // not open, or found through its gram
+  const QGeo& g = C.g;
+  const uint64_t s = g.st[g.c - 1], r = C.r;
+  const uint32_t f = (uint32_t)(r < 4 ? r : 4);
+  uint32_t want = 0;
+  for (uint32_t t = 0; t < f; t++) want |= (uint32_t)g.T[s + t] << (8 * t);
+  const uint32_t fm = f == 4 ? 0xFFFFFFFFu : (1u << (8 * f)) - 1u;
+  const bool aligned = (((uintptr_t)g.T) & 15) == 0;
+  for (uint64_t p0 = 16ull * (blockIdx.x * (uint64_t)kT + threadIdx.x); p0 < s; p0 += 16ull * gridDim.x * kT) {
+    if (p0 >= *(volatile unsigned long long*)&C.qs->lo_tail) return;
+    uint32_t w[5];
+    if (aligned && p0 + 20 <= g.n) {
+      const uint4 v = *(const uint4*)(g.T + p0);
+      w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+      w[4] = *(const uint32_t*)(g.T + p0 + 16);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 5; q++) {
+        w[q] = 0;
+        for (int t = 0; t < 4; t++)
+          if (p0 + 4 * q + t < g.n) w[q] |= (uint32_t)g.T[p0 + 4 * q + t] << (8 * t);
+      }
+    }
+#pragma unroll
+    for (uint32_t i = 0; i < 16; i++) {
+      if ((__funnelshift_r(w[i >> 2], w[(i >> 2) + 1], 8 * (i & 3)) & fm) != want) continue;
+      const uint64_t p = p0 + i;
+      if (p >= s) break;
+      bool eq = true;
+      for (uint64_t t = f; t < r && eq; t++) eq = g.T[p + t] == g.T[s + t];
+      if (eq) {
+        c_min(&C.qs->lo_tail, p);
+        break;
+      }
+    }
+  }
+}
+
+// An open key's leftmost fingerprint match.
+__device__ __forceinline__ uint64_t item_lo(const Chase& C, uint64_t i, uint64_t* k, uint64_t* s, uint64_t* len) {
+  const QGeo& g = C.g;
+  const uint32_t it = C.items[i], sl = C.islot[i];
+  const bool pair = it & 1;
+  *k = it >> 1;
+  *s = g.st[*k];
+  *len = g.n - *s < g.b ? g.n - *s : g.b;
+  if (pair) *len += g.n - *s - *len < g.b ? g.n - *s - *len : g.b;
+  if (sl == kNoSlot) return *s;
+  return sl == kTailItem ? (pair ? C.qs->lo_tailpair : C.qs->lo_tail) : pair ? C.pt[sl].lo : C.bt[sl].lo;
+}
+
+__global__ void __launch_bounds__(kT) k_chase_verify(Chase C, uint64_t ppk, unsigned L) {
+  const QGeo& g = C.g;
+  const unsigned lane = threadIdx.x & 31, grp = lane / L, gl = lane % L, gpw = 32 / L;
+  const unsigned gmask = (L == 32 ? 0xFFFFFFFFu : ((1u << L) - 1u)) << (grp * L);
+  const bool aligned16 = (((uintptr_t)g.T) & 15) == 0;
+  const uint64_t warps = (uint64_t)gridDim.x * (kT / 32), total = C.nitems * ppk;
+  for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32 * gpw; base < total; base += warps * gpw) {
+    const uint64_t u = base + grp;
+    bool d = false;
+    uint64_t i = 0;
+    if (u < total) {
+      i = u / ppk;
+      const uint64_t off = (u - i * ppk) * kQPiece;
+      uint64_t k, s, len;
+      const uint64_t p = item_lo(C, i, &k, &s, &len);
+      if (p < s && off < len)
+        d = differs(g.T, g.n, aligned16, p, s, off, off + kQPiece < len ? off + kQPiece : len, gl, L);
+    }
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, d);
+    if (u < total && gl == 0 && (bal & gmask)) C.differ[i] = 1;
+  }
+}
+
+__global__ void __launch_bounds__(kT) k_chase_apply(Chase C) {
+  for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; i < C.nitems; i += (uint64_t)gridDim.x * kT) {
+    uint64_t k, s, len;
+    const uint64_t p = item_lo(C, i, &k, &s, &len);
+    const bool pair = C.items[i] & 1;
+    if (p > s) {
+      atomicExch(&C.status->error, 25ull);
+      continue;
+    }
+    if (p < s) atomicAdd(&C.status->verify_bytes, 2ull * len);
+    if (p < s && C.differ[i]) {  // a fingerprint collision: resolved exactly
+      atomicAdd(&C.status->collisions, 1ull);
+      const unsigned long long q = atomicAdd(&C.qs->nsusp, 1ull);
+      C.susp[q] = (uint32_t)i;
+      C.exlo[q] = s;
+    } else if (pair) {
+      C.ps[k] = kIsPair | (p == s ? kLeftmost : 0);
+    } else {
+      C.lo[k] = p;
+    }
+  }
+}
+
+// Exact leftmost occurrence of the keys whose match was false: every earlier
+// position, byte by byte (a test modulus makes this frequent; with 2^61 - 1 it
+// does not happen).
+__global__ void __launch_bounds__(kT) k_chase_exact(Chase C, uint64_t nsusp) {
+  for (uint64_t q = blockIdx.y; q < nsusp; q += gridDim.y) {
+    uint64_t k, s, len;
+    item_lo(C, C.susp[q], &k, &s, &len);
+    for (uint64_t p = blockIdx.x * (uint64_t)kT + threadIdx.x; p < s; p += (uint64_t)gridDim.x * kT) {
+      bool eq = true;
+      for (uint64_t t = 0; t < len && eq; t++) eq = C.g.T[p + t] == C.g.T[s + t];
+      if (eq) c_min(&C.exlo[q], p);
+    }
+  }
+}
+__global__ void __launch_bounds__(kT) k_chase_exact_apply(Chase C, uint64_t nsusp) {
+  for (uint64_t q = blockIdx.x * (uint64_t)kT + threadIdx.x; q < nsusp; q += (uint64_t)gridDim.x * kT) {
+    uint64_t k, s, len;
+    item_lo(C, C.susp[q], &k, &s, &len);
+    if (C.items[C.susp[q]] & 1) C.ps[k] = kIsPair | (C.exlo[q] == s ? kLeftmost : 0);
+    else C.lo[k] = C.exlo[q];
+  }
+}
+
+// Opt a kernel in to more than 48 KiB of shared memory, once per device.
+template <auto FN>
+int allow_smem(int bytes) {
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  BT_CUDA(cudaGetDevice(&dev));
+  const uint64_t bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return BT_OK;
+  BT_CUDA(cudaFuncSetAttribute(FN, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  done.fetch_or(bit, std::memory_order_acq_rel);
+  return BT_OK;
+}
+
+uint64_t pow2_from(uint64_t x) {
+  uint64_t p = 64;
+  while (p < x) p <<= 1;
+  return p;
+}
+
+}  // namespace
+
+int quick_list(BuildCtx& ctx, QuickBuild& qb) {
+  const uint64_t n = ctx.t->n;
+  cudaStream_t s = ctx.s;
+  const uint64_t nw = n < kGramLen ? 0 : (n - kGramLen + 1 + 31) / 32;  // words of 32 gram positions
+  const uint64_t ns = (n + kSegBytes - 1) / kSegBytes, ns2 = (ns + 63) / 64;
+  // Cells of the first-occurrence table: one per eight positions (there is
+  // about one list entry per six, most of them repeats), at most 256 MiB:
+  // random reads run at 300 G/s from L2-sized tables, 80-90 from 256 MiB, 47
+  // from 1 GiB (GB300), and a shared cell only loosens a bound.
+  uint64_t cells = 1024;
+  while (cells < n / 8 && cells < (1ull << 26)) cells <<= 1;
+  uint32_t *mask, *first, *agg;
+  Scratch tmp(s);
+  BT_TRY(tmp.alloc(&mask, nw));
+  BT_TRY(tmp.alloc(&agg, scan_scratch_words(nw)));
+  BT_TRY(qb.mem.alloc(&qb.idx, nw + 1));
+  BT_TRY(tmp.alloc(&first, cells));
+  BT_TRY(qb.mem.alloc(&qb.seg1, ns));
+  BT_TRY(qb.mem.alloc(&qb.seg2, ns2));
+  ProfScope ps("gram_list", s, n);
+  if (nw) BT_LAUNCH(k_list_mask<<<grid_for(nw, kT), kT, 0, s>>>(ctx.T, n, nw, mask, qb.idx));
+  BT_TRY(scan_u32(qb.idx, qb.idx, nw, s, agg));
+  // Room for the entries: all positions of a short text (no round trip), the
+  // number found otherwise.
+  uint64_t cap = n;
+  if (n > (4ull << 20)) {
+    uint32_t total = 0;
+    BT_CUDA(cudaMemcpyAsync(&total, qb.idx + nw, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    BT_CUDA(cudaStreamSynchronize(s));
+    cap = total;
+  }
+  cap = (cap + 63) & ~63ull;
+  uint32_t* xd;
+  BT_TRY(qb.mem.alloc(&xd, 2 * (cap ? cap : 64)));
+  qb.x = xd;
+  qb.D = xd + (cap ? cap : 64);
+  BT_CUDA(cudaMemsetAsync(first, 0xFF, cells * sizeof(uint32_t), s));
+  if (nw)
+    BT_LAUNCH(k_list_write<<<(unsigned)std::min<uint64_t>((nw + kT - 1) / kT, 152 * 16), kT, 0, s>>>(
+        ctx.T, n, nw, mask, qb.idx, qb.x, qb.D, first, (uint32_t)(cells - 1)));
+  BT_LAUNCH(k_list_dist<<<grid_for(cap / 4 + 1, kT, 152 * 16), kT, 0, s>>>(qb.idx + nw, qb.x, qb.D, first));
+  BT_LAUNCH(k_list_seg1<<<grid_for(ns * 32, kT), kT, 0, s>>>(nw, qb.idx, qb.D, ns, qb.seg1));
+  BT_LAUNCH(k_list_seg2<<<grid_for(ns2, kT), kT, 0, s>>>(ns, qb.seg1, ns2, qb.seg2));
+  BT_CUDA(cudaGetLastError());
+  qb.list = QList{qb.idx, qb.x, qb.D, qb.seg1, qb.seg2, nw};
+  qb.ready = true;
+  BT_TRY(qb.mem.alloc(&qb.qs, 1));
+  BT_CUDA(cudaMallocHost(&qb.qs_host, sizeof(QuickStatus)));
+  return BT_OK;
+}
+
+template <class M>
+static int chase(const M& m, BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint64_t last_start, const uint32_t* A,
+                 const uint32_t* X, const uint32_t* items, uint64_t* lo, uint8_t* ps) {
+  bt_tree* t = ctx.t;
+  cudaStream_t s = ctx.s;
+  const uint64_t nb = qb.qs_host->nopen[0], np = qb.qs_host->nopen[1], ni = nb + np;
+  const uint64_t len_last = g.n - last_start;
+  Chase C;
+  C.g = g;
+  C.Q = qb.list;
+  C.A = A;
+  C.X = X;
+  C.items = items;
+  C.nitems = (uint32_t)ni;
+  C.r = len_last < g.b ? len_last : 0;
+  C.Bb = pow_mod(m, t->B, g.b);
+  C.Br = C.r ? pow_mod(m, t->B, C.r) : 0;
+  const uint64_t bcap = pow2_from(2 * (nb + 2 * np)), pcap = pow2_from(2 * np), gcap = pow2_from(2 * ni);
+  uint32_t fbits = 12;
+  while ((1ull << fbits) < 16 * ni && fbits < 30) fbits++;
+  const uint32_t bwords = 1u << (fbits - 5);
+  C.bmask = (uint32_t)(bcap - 1);
+  C.pmask = (uint32_t)(pcap - 1);
+  C.gmask = (uint32_t)(gcap - 1);
+  C.bshift = 32 - fbits;
+  C.qs = qb.qs;
+  C.status = ctx.st;
+  C.lo = lo;
+  C.ps = ps;
+  Arena& R = qb.open;
+  auto carve = [&]() {
+    C.bt = R.take<CSlot>(bcap);
+    C.pt = R.take<CPair>(pcap);
+    C.gt = R.take<CGram>(gcap);
+    C.bound2 = R.take<unsigned long long>(gcap);
+    C.bitmap = R.take<uint32_t>(bwords);
+    C.islot = R.take<uint32_t>(ni);
+    C.igram = R.take<uint32_t>(ni);
+    C.differ = R.take<uint32_t>(ni);
+    C.susp = R.take<uint32_t>(ni);
+    C.exlo = R.take<unsigned long long>(ni);
+  };
+  R.begin_dry();
+  carve();
+  BT_TRY(R.reserve());
+  carve();
+  const PrefixAt<M> H(m, ctx.T, g.n, ctx.Hs, t->B);
+  BT_TRY(allow_smem<k_chase_scan<M>>(kChaseBitWords * 4));
+  const uint64_t top = std::max<uint64_t>(std::max(bcap, pcap), std::max<uint64_t>(gcap, bwords));
+  BT_LAUNCH(k_chase_init<<<grid_for(top, kT), kT, 0, s>>>(C, bwords));
+  BT_LAUNCH(k_chase_keys<M><<<grid_for(ni * 32, kT), kT, 0, s>>>(m, H, C));
+  {
+    ProfScope prof("window_scan", s, 0);  // (the level's bytes are counted by its first part)
+    // Two halves: the first sixteenth of the list, then the rest against the
+    // bounds it lowered (most copies' content is first seen early).
+    const uint32_t total = qb.qs_host->total;
+    const uint32_t split = total > (1u << 20) ? (total / 16) & ~(kChaseTile - 1) : 0;
+    const uint32_t sw = bwords <= kChaseBitWords ? bwords : 0;
+    auto grid = [](uint64_t n) { return (unsigned)std::min<uint64_t>((n + kChaseTile - 1) / kChaseTile, 152 * 3); };
+    if (split) {
+      BT_LAUNCH(k_chase_scan<M><<<grid(split), kT, sw * 4, s>>>(m, H, C, 0, split, sw, nullptr));
+      BT_LAUNCH(k_chase_bound<<<grid_for(ni, kT), kT, 0, s>>>(C));
+    }
+    if (total)
+      BT_LAUNCH(k_chase_scan<M><<<grid(total - split), kT, sw * 4, s>>>(m, H, C, split, total, sw,
+                                                                       split ? C.bound2 : nullptr));
+    if (C.r && C.r < 27) BT_LAUNCH(k_chase_tail<<<grid_for(g.n / 16 + 1, kT, 152 * 8), kT, 0, s>>>(C));
+  }
+  const uint64_t ppk = (2 * g.b + kQPiece - 1) / kQPiece;
+  const unsigned L = g.b >= 256 ? 32u : g.b >= 128 ? 16u : g.b >= 64 ? 8u : 4u;
+  BT_LAUNCH(k_chase_verify<<<grid_for(ni * ppk * L, kT), kT, 0, s>>>(C, ppk, L));
+  BT_LAUNCH(k_chase_apply<<<grid_for(ni, kT), kT, 0, s>>>(C));
+  BT_CUDA(cudaGetLastError());
+  qb.resolve_exact = [=](uint64_t nsusp) -> int {
+    const dim3 grid(grid_for(g.n, kT, 1024), (unsigned)std::min<uint64_t>(nsusp, 1024));
+    BT_LAUNCH(k_chase_exact<<<grid, kT, 0, s>>>(C, nsusp));
+    BT_LAUNCH(k_chase_exact_apply<<<grid_for(nsusp, kT), kT, 0, s>>>(C, nsusp));
+    BT_CUDA(cudaGetLastError());
+    return BT_OK;
+  };
+  return BT_OK;
+}
+
+// One level: marks, leftmost occurrences, pointers, the next level's blocks.
+int quick_level(BuildCtx& ctx, QuickBuild& qb, uint32_t l, uint64_t last_start) {
+  bt_tree* t = ctx.t;
+  Level& v = t->lv[l];
+  cudaStream_t s = ctx.s;
+  const uint64_t c = v.c, b = v.b, n = t->n, words = (c + 31) / 32;
+  const bool last_level = l + 1 == t->L;
+  const uint64_t bn = last_level ? 0 : t->lv[l + 1].b;
+  v.arity = last_level ? 0 : (uint32_t)(b / bn);
+  const QGeo g{ctx.T, n, c, b, v.st};
+  BT_TRY(alloc_level_arrays(v, words, s));
+  uint32_t *A, *X, *flags, *items, *wpop, *sagg;
+  uint8_t* ps;
+  Arena& R = ctx.arena;
+  auto carve = [&]() {
+    A = R.take<uint32_t>(c);
+    X = R.take<uint32_t>(c);
+    flags = R.take<uint32_t>(c);
+    items = R.take<uint32_t>(2 * c);
+    ps = R.take<uint8_t>(c);
+    wpop = R.take<uint32_t>(words);
+    sagg = R.take<uint32_t>(scan_scratch_words(words));
+  };
+  R.begin_dry();
+  carve();
+  BT_TRY(R.reserve());
+  carve();
+  const unsigned gc = grid_for(c, kT);
+  unsigned G = 1;
+  while (G < 32 && 64ull * 2 * G <= b) G <<= 1;
+  {
+  ProfScope prof("window_scan", s, (c - 1) * b + (n - last_start < b ? n - last_start : b));
+  BT_LAUNCH(k_quick_min<<<grid_for(c * G, kT), kT, 0, s>>>(g, qb.list, G, A, X, flags, qb.qs));
+  const uint64_t ppk = (2 * b + kQPiece - 1) / kQPiece;
+  const unsigned L = b >= 256 ? 32u : b >= 128 ? 16u : b >= 64 ? 8u : 4u;
+  BT_LAUNCH(k_quick_compare<<<grid_for(c * ppk * L, kT), kT, 0, s>>>(g, A, X, flags, ppk, L));
+  BT_LAUNCH(k_quick_settle<<<gc, kT, 0, s>>>(g, A, X, flags, v.lo, ps, items, v.mw, wpop, qb.qs, ctx.st));
+  }
+  auto rank_and_wait = [&]() -> int {
+    if (words <= kRankWords) {
+      BT_LAUNCH(k_quick_rank<<<1, 1024, 0, s>>>(g, v.mw, wpop, v.mr, v.arity, bn, ctx.st, qb.qs));
+    } else {
+      BT_TRY(scan_u32(wpop, v.mr, words, s, sagg));
+      BT_LAUNCH(k_quick_end<<<1, 1, 0, s>>>(g, v.mw, v.mr, v.arity, bn, ctx.st, qb.qs));
+    }
+    BT_CUDA(cudaGetLastError());
+    BT_CUDA(cudaMemcpyAsync(qb.qs_host, qb.qs, sizeof(QuickStatus), cudaMemcpyDeviceToHost, s));
+    return sync_status(ctx);
+  };
+  BT_TRY(rank_and_wait());
+  const QuickStatus q0 = *qb.qs_host;
+  if (q0.nitems) {
+    if (t->q == Mersenne61::Q) BT_TRY(chase(Mersenne61{}, ctx, qb, g, last_start, A, X, items, v.lo, ps));
+    else BT_TRY(chase(SmallMod{t->q}, ctx, qb, g, last_start, A, X, items, v.lo, ps));
+    BT_LAUNCH(k_quick_remark<<<grid_for(words * 32, kT), kT, 0, s>>>(c, ps, v.mw, wpop));
+    BT_TRY(rank_and_wait());
+    if (qb.qs_host->nsusp) {
+      BT_TRY(qb.resolve_exact(qb.qs_host->nsusp));
+      BT_LAUNCH(k_quick_remark<<<grid_for(words * 32, kT), kT, 0, s>>>(c, ps, v.mw, wpop));
+      BT_TRY(rank_and_wait());
+    }
+  }
+  uint64_t* next_st = nullptr;
+  if (!last_level) {
+    Level& nx = t->lv[l + 1];
+    nx.c = ctx.st_host->next_c;
+    if (nx.c == 0) return BT_EINTERNAL;
+    BT_CUDA(cudaMallocAsync(&nx.st, nx.c * sizeof(uint64_t), s));
+    nx.owned.push_back(nx.st);
+    next_st = nx.st;
+  }
+  // Wide nodes (explicit block sizes) leave their children to a kernel that
+  // deals them to the threads.
+  const bool wide = v.arity > 64;
+  BT_LAUNCH(k_quick_points<<<gc, kT, 0, s>>>(g, v.mw, v.mr, v.lo, v.ptr, v.off, v.arity, bn, wide ? nullptr : next_st,
+                                             ctx.st));
+  if (next_st && wide) BT_TRY(launch_children(ctx, l, bn, next_st));
+  BT_CUDA(cudaGetLastError());
+  v.nmarked = qb.qs_host->nmarked;
+  v.stats[BT_ST_NBLOCKS] = c;
+  v.stats[BT_ST_B] = b;
+  v.stats[BT_ST_COV] = (c - 1) * b + (n - last_start < b ? n - last_start : b);
+  v.stats[BT_ST_NMARKED] = v.nmarked;
+  v.stats[BT_ST_NPAIRS] = q0.npairs;
+  v.stats[BT_ST_VERIFY_BYTES] = ctx.st_host->verify_bytes - ctx.verify_bytes;
+  v.stats[BT_ST_COLLISIONS] = ctx.st_host->collisions - ctx.collisions;
+  v.stats[BT_ST_CANDIDATES] = q0.nitems ? qb.qs_host->cands : 0;
+  v.stats[BT_ST_HITS] = q0.nitems ? qb.qs_host->hits : 0;
+  ctx.verify_bytes = ctx.st_host->verify_bytes;
+  ctx.collisions = ctx.st_host->collisions;
+  if (ctx.st_host->error) {
+    if (getenv("BT_VERBOSE"))
+      fprintf(stderr, "bt: level %u (b=%llu, c=%llu): device check %llu failed\n", l, (unsigned long long)b,
+              (unsigned long long)c, (unsigned long long)ctx.st_host->error);
+    return BT_EINTERNAL;
+  }
+  return BT_OK;
+}
+
+}  // namespace bt

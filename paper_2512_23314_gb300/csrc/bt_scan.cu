@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "bt_internal.cuh"
+#include "bt_kr.cuh"
 
 namespace bt {
 
@@ -183,53 +184,6 @@ __device__ __forceinline__ uint64_t kr_lane_pow(const M& m, const KrPow& pw) {
     if ((e >> i) & 1u) r = m.mul(r, pw.x[i]);
   return e == 32 ? pw.w[0] : r;
 }
-
-// Fingerprint of a 32-byte chunk (eight little-endian words).
-template <class M>
-struct ChunkHash {  // any modulus: Horner
-  uint64_t B;
-  ChunkHash(const M&, uint64_t base) : B(base) {}
-  __device__ __forceinline__ uint64_t operator()(const M& m, const uint32_t* w) const {
-    uint64_t h = 0;
-#pragma unroll
-    for (int i = 0; i < (int)kPrefixStride; i++)
-      h = m.add(m.mul(h, B), (uint64_t)((w[i >> 2] >> (8 * (i & 3))) & 0xFFu) + 1);
-    return h;
-  }
-};
-template <>
-struct ChunkHash<Mersenne61> {
-  uint32_t limb[8][8];  // [word][l]: bits 8l..8l+7 of the powers of the word's four bytes
-  uint64_t ones;        // the sum of the powers: every symbol is its byte + 1
-  ChunkHash(const Mersenne61& m, uint64_t B) {
-    uint64_t p = 1;
-    ones = 0;
-    for (int i = 31; i >= 0; i--) {
-      for (int l = 0; l < 8; l++) {
-        if ((i & 3) == 3) limb[i >> 2][l] = 0;
-        limb[i >> 2][l] |= (uint32_t)((p >> (8 * l)) & 0xFF) << (8 * (i & 3));
-      }
-      ones = m.add(ones, p);
-      p = m.mul(p, B);
-    }
-  }
-  __device__ __forceinline__ uint64_t operator()(const Mersenne61& m, const uint32_t* w) const {
-    uint32_t s[8];  // each at most 32 * 255^2 < 2^21
-#pragma unroll
-    for (int l = 0; l < 8; l++) {
-      s[l] = 0;
-#pragma unroll
-      for (int q = 0; q < 8; q++) s[l] = __dp4a(w[q], limb[q][l], s[l]);
-    }
-    const uint64_t lo = (uint64_t)s[0] + ((uint64_t)s[1] << 8) + ((uint64_t)s[2] << 16) + ((uint64_t)s[3] << 24);
-    const uint64_t hi = (uint64_t)s[4] + ((uint64_t)s[5] << 8) + ((uint64_t)s[6] << 16) + ((uint64_t)s[7] << 24);
-    // lo + hi 2^32 with hi = a 2^29 + r: a 2^61 + r 2^32 = a + r 2^32; < 2^62.
-    uint64_t x = lo + (hi >> 29) + ((hi & ((1u << 29) - 1)) << 32);
-    x = (x & Mersenne61::Q) + (x >> 61);
-    if (x >= Mersenne61::Q) x -= Mersenne61::Q;
-    return m.add(x, ones);
-  }
-};
 
 // The words of chunk j, or zeros for a chunk the text does not hold.
 __device__ __forceinline__ void load_chunk(const uint8_t* __restrict__ T, uint64_t nchunks, uint64_t j, bool aligned,

@@ -18,6 +18,17 @@ __device__ __forceinline__ uint4 unaligned16(uint4 u0, uint4 u1, uint32_t d) {
                     __funnelshift_r(w3, w4, sh));
 }
 
+// Do the 16 bytes at a and at b (16-byte aligned, a < b, T aligned) differ?
+// The unit after a's first one ends at b + 16 or before.
+__device__ __forceinline__ bool differ16(const uint8_t* __restrict__ T, uint64_t a, uint64_t b) {
+  const uint4 vb = *(const uint4*)(T + b);
+  const uint64_t a0 = a & ~15ull;
+  const uint32_t d = (uint32_t)(a & 15);
+  const uint4 u0 = *(const uint4*)(T + a0);
+  const uint4 va = d == 0 ? u0 : unaligned16(u0, *(const uint4*)(T + a0 + 16), d);
+  return va.x != vb.x || va.y != vb.y || va.z != vb.z || va.w != vb.w;
+}
+
 // Compare T[a + x] and T[b + x] for x in [off, end) by L lanes: bytes up to
 // the first 16-byte unit of the side at b, then 16 bytes per lane and step,
 // the other side realigned from two aligned loads; bytes for the ragged end.

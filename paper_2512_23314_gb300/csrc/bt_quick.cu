@@ -55,7 +55,9 @@ constexpr uint32_t kSubs = kGramLen - 3;       // 4-byte substrings of a gram
 constexpr uint32_t kNoDist = 0xFFFFFFFFu;      // no selected gram in the range
 constexpr uint32_t kSubMul = 0x9E3779B1u;
 constexpr uint32_t kSegBytes = 1024;           // positions per entry of seg1; 64 of those per entry of seg2
-constexpr uint64_t kQPiece = 4096;             // bytes per comparison item
+// Bytes per comparison item: on the levels of the longest blocks few pieces,
+// since nearly all of them are looked at only to find nothing to compare.
+__host__ __device__ inline uint64_t q_piece(uint64_t b) { return b >= (64u << 10) ? 32u << 10 : 4u << 10; }
 constexpr unsigned kT = 256;
 
 // ---------------------------------------------------------------------------
@@ -130,15 +132,13 @@ __device__ __forceinline__ uint32_t gram_cell(uint32_t w0, uint32_t w1, uint32_t
   return h & cmask;
 }
 
-// The list entries: position x[e], and the cell of the gram in cell[e]; the
-// cell keeps the least position (read first: after a gram's first copies have
-// been seen nobody writes).  A CTA takes 256 words: its text and the positions
-// of its grams are staged in shared memory, so that entries, not words, are
-// dealt to the threads and leave in order.
+// The list entries: position x[e], and the cell of the gram in cell[e].  A CTA
+// takes 256 words: its text and the positions of its grams are staged in
+// shared memory, so that entries, not words, are dealt to the threads and
+// leave in order.
 __global__ void __launch_bounds__(kT) k_list_write(const uint8_t* __restrict__ T, uint64_t n, uint64_t nw,
                                                    const uint32_t* __restrict__ mask, const uint32_t* __restrict__ idx,
-                                                   uint32_t* __restrict__ x, uint32_t* __restrict__ cell,
-                                                   uint32_t* __restrict__ first, uint32_t cmask) {
+                                                   uint32_t* __restrict__ x, uint32_t* __restrict__ cell, uint32_t cmask) {
   constexpr uint32_t kBytes = 32 * kT;
   __shared__ __align__(16) uint32_t text[kBytes / 4 + 8];
   __shared__ uint16_t at[kBytes];
@@ -172,12 +172,31 @@ __global__ void __launch_bounds__(kT) k_list_write(const uint8_t* __restrict__ T
       uint32_t w[5];
 #pragma unroll
       for (int u = 0; u < 5; u++) w[u] = text[q + u];
-      const uint32_t c = gram_cell(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
-                                   __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh), cmask);
-      const uint32_t pos = (uint32_t)(p0 + a);
-      x[e0 + i] = pos;
-      cell[e0 + i] = c;
-      if (*(volatile uint32_t*)&first[c] > pos) atomicMin(&first[c], pos);
+      x[e0 + i] = (uint32_t)(p0 + a);
+      cell[e0 + i] = gram_cell(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
+                               __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh), cmask);
+    }
+  }
+}
+
+// first[cell] = the least position of an entry with that cell (read first:
+// after a gram's first copies have been seen nobody writes).  A pass of its
+// own: inside k_list_write, between that kernel's barriers, the same random
+// reads took 400 us of a 256 MiB build instead of 180.
+__global__ void __launch_bounds__(kT) k_list_first(const uint32_t* __restrict__ total_p, const uint32_t* __restrict__ x,
+                                                   const uint32_t* __restrict__ cell, uint32_t* first) {
+  const uint64_t total = *total_p;
+  for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; 4 * i < total; i += (uint64_t)gridDim.x * kT) {
+    if (4 * i + 4 <= total) {
+      const uint4 X = ((const uint4*)x)[i], C = ((const uint4*)cell)[i];
+      const uint32_t f0 = *(volatile uint32_t*)&first[C.x], f1 = *(volatile uint32_t*)&first[C.y],
+                     f2 = *(volatile uint32_t*)&first[C.z], f3 = *(volatile uint32_t*)&first[C.w];
+      if (f0 > X.x) atomicMin(&first[C.x], X.x);
+      if (f1 > X.y) atomicMin(&first[C.y], X.y);
+      if (f2 > X.z) atomicMin(&first[C.z], X.z);
+      if (f3 > X.w) atomicMin(&first[C.w], X.w);
+    } else {
+      for (uint64_t e = 4 * i; e < total; e++) atomicMin(&first[cell[e]], x[e]);
     }
   }
 }
@@ -338,7 +357,7 @@ __global__ void __launch_bounds__(kT) k_quick_compare(QGeo g, const uint32_t* __
   const unsigned lane = threadIdx.x & 31, grp = lane / L, gl = lane % L, gpw = 32 / L;
   const unsigned gmask = (L == 32 ? 0xFFFFFFFFu : ((1u << L) - 1u)) << (grp * L);
   const bool aligned16 = (((uintptr_t)g.T) & 15) == 0;
-  const uint64_t warps = (uint64_t)gridDim.x * (kT / 32), total = g.c * ppk;
+  const uint64_t warps = (uint64_t)gridDim.x * (kT / 32), total = g.c * ppk, piece = q_piece(g.b);
   // Warp-uniform loop: every lane reaches the ballots of every iteration.
   for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32 * gpw; base < total; base += warps * gpw) {
     const uint64_t u = base + grp;
@@ -346,7 +365,7 @@ __global__ void __launch_bounds__(kT) k_quick_compare(QGeo g, const uint32_t* __
     uint64_t k = 0;
     if (u < total) {
       k = ppk == 1 ? u : u / ppk;
-      const uint64_t off = ppk == 1 ? 0 : (u - k * ppk) * kQPiece;
+      const uint64_t off = ppk == 1 ? 0 : (u - k * ppk) * piece;
       const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
       const uint32_t dk = A[k];
       const bool blk = dk != 0 && dk != kNoDist && s != 0 && off < len;
@@ -359,11 +378,19 @@ __global__ void __launch_bounds__(kT) k_quick_compare(QGeo g, const uint32_t* __
         d2 = pair_dist(A, X, k, len2);
         pair = d2 != 0 && d2 != kNoDist && off < plen;
       }
-      if (blk || pair) {
-        const uint32_t f = *(volatile uint32_t*)&flags[k];
-        const uint64_t pk = dk > s ? 0 : s - dk, pp = d2 > s ? 0 : s - d2;
-        const uint64_t bend = off + kQPiece < len ? off + kQPiece : len;
-        const uint64_t pend = off + kQPiece < plen ? off + kQPiece : plen;
+      // (Flags another piece has set spare this one; pieces are many only when blocks are long.)
+      const uint32_t f = ppk > 1 && (blk || pair) ? *(volatile uint32_t*)&flags[k] : 0u;
+      const uint64_t pk = dk > s ? 0 : s - dk, pp = d2 > s ? 0 : s - d2;
+      const uint64_t bend = off + piece < len ? off + piece : len;
+      const uint64_t pend = off + piece < plen ? off + piece : plen;
+      if (blk && pair && pk == pp && !(f & kPairDiffers) && aligned16 && ((s | len | plen | off) & 15) == 0) {
+        // One bound for both: the block's bytes are the pair's first half.
+        for (uint64_t y = off + 16ull * gl; y < pend; y += 16ull * L) {
+          const bool d = differ16(g.T, pk + y, s + y);
+          dp |= d;
+          db |= d && y < len;
+        }
+      } else {
         if (blk && !(f & kBlkDiffers)) {
           db = differs(g.T, g.n, aligned16, pk, s, off, bend, gl, L);
           if (pair && pk == pp) dp = db;
@@ -412,11 +439,17 @@ __global__ void __launch_bounds__(kT) k_quick_settle(QGeo g, const uint32_t* __r
                                                      uint8_t* __restrict__ ps, uint32_t* __restrict__ items,
                                                      uint32_t* __restrict__ mw, uint32_t* __restrict__ wpop,
                                                      QuickStatus* qs, Status* status) {
-  const uint64_t words = (g.c + 31) / 32;
-  const unsigned lane = threadIdx.x & 31;
-  for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) & ~31ull; base < words * 32;
-       base += (uint64_t)gridDim.x * kT) {
-    const uint64_t k = base + lane;
+  // One atomic per counter and CTA, and one per 256 blocks that hold an open
+  // key: with one per warp and counter their queue on five addresses was the
+  // whole time (121 and 191 us on the two lowest levels of the 256 MiB text).
+  __shared__ uint32_t s_cnt[kT / 32];
+  __shared__ unsigned long long s_at, s_sum[kT / 32][4];
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint64_t tiles = (g.c + kT - 1) / kT;
+  uint64_t sum_vb = 0;
+  uint32_t sum_np = 0, sum_b = 0, sum_p = 0;
+  for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const uint64_t base = tile * kT + warp * 32, k = base + lane;
     bool ob = false, op = false;
     uint8_t st = 0;
     uint64_t vb = 0;
@@ -449,24 +482,50 @@ __global__ void __launch_bounds__(kT) k_quick_settle(QGeo g, const uint32_t* __r
     const bool mk = k < g.c && ((left & kLeftmost) || (st & kLeftmost) || !((left | st) & kIsPair));
     const uint32_t bits = __ballot_sync(0xFFFFFFFFu, mk);
     const uint32_t bb = __ballot_sync(0xFFFFFFFFu, ob), bp = __ballot_sync(0xFFFFFFFFu, op);
-    const uint32_t np = __popc(__ballot_sync(0xFFFFFFFFu, st & kIsPair));
-    vb = warp_sum64(vb);
-    unsigned long long at = 0;
-    if (lane == 0) {
+    sum_np += __popc(__ballot_sync(0xFFFFFFFFu, st & kIsPair));
+    sum_b += __popc(bb);
+    sum_p += __popc(bp);
+    sum_vb += vb;
+    if (lane == 0 && base < g.c) {
       mw[base / 32] = bits;
       wpop[base / 32] = __popc(bits);
-      if (np) atomicAdd(&qs->npairs, (unsigned long long)np);
-      if (vb) atomicAdd(&status->verify_bytes, (unsigned long long)vb);
-      if (bb) atomicAdd(&qs->nopen[0], (unsigned long long)__popc(bb));
-      if (bp) atomicAdd(&qs->nopen[1], (unsigned long long)__popc(bp));
-      if (bb | bp) at = atomicAdd(&qs->nitems, (unsigned long long)(__popc(bb) + __popc(bp)));
     }
-    if (bb | bp) {
-      at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    const uint32_t mine = __popc(bb) + __popc(bp);
+    if (lane == 0) s_cnt[warp] = mine;
+    if (__syncthreads_or(mine != 0)) {
+      if (threadIdx.x == 0) {
+        uint32_t n = 0;
+        for (unsigned w = 0; w < kT / 32; w++) {
+          const uint32_t v = s_cnt[w];
+          s_cnt[w] = n;
+          n += v;
+        }
+        s_at = atomicAdd(&qs->nitems, (unsigned long long)n);
+      }
+      __syncthreads();
+      const uint64_t at = s_at + s_cnt[warp];
       const uint32_t lt = (1u << lane) - 1u;
       if (ob) items[at + __popc(bb & lt)] = (uint32_t)(2 * k);
       if (op) items[at + __popc(bb) + __popc(bp & lt)] = (uint32_t)(2 * k + 1);
     }
+    __syncthreads();
+  }
+  sum_vb = warp_sum64(sum_vb);
+  if (lane == 0) {
+    s_sum[warp][0] = sum_b;
+    s_sum[warp][1] = sum_p;
+    s_sum[warp][2] = sum_np;
+    s_sum[warp][3] = sum_vb;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    unsigned long long v = 0;
+    for (unsigned w = 0; w < kT / 32; w++) v += s_sum[w][threadIdx.x];
+    unsigned long long* to = threadIdx.x == 0   ? &qs->nopen[0]
+                             : threadIdx.x == 1 ? &qs->nopen[1]
+                             : threadIdx.x == 2 ? &qs->npairs
+                                                : &status->verify_bytes;
+    if (v) atomicAdd(to, v);
   }
 }
 
@@ -718,13 +777,14 @@ __global__ void __launch_bounds__(kT) k_chase_init(Chase C, uint32_t bwords) {
   }
 }
 
-// A warp per open key: the list entry with the key's min D, then (lane 0) the
-// tables.  A pair enters both of its blocks.
-template <class M>
+// G lanes per open key (one when blocks are short, else a warp): the list entry
+// with the key's min D, then (one lane) the tables.  A pair enters both of its
+// blocks.
+template <class M, unsigned G>
 __global__ void __launch_bounds__(kT) k_chase_keys(M m, const __grid_constant__ PrefixAt<M> H, Chase C) {
-  const unsigned lane = threadIdx.x & 31;
+  const unsigned gl = threadIdx.x % G;
   const QGeo& g = C.g;
-  for (uint64_t i = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32; i < C.nitems; i += (uint64_t)gridDim.x * (kT / 32)) {
+  for (uint64_t i = (blockIdx.x * (uint64_t)kT + threadIdx.x) / G; i < C.nitems; i += (uint64_t)gridDim.x * (kT / G)) {
     const uint32_t it = C.items[i];
     const uint64_t k = it >> 1;
     const bool pair = it & 1;
@@ -736,20 +796,24 @@ __global__ void __launch_bounds__(kT) k_chase_keys(M m, const __grid_constant__ 
     bool found = false;
     if (d != kNoDist) {
       const uint32_t e1 = list_at(C.Q, (end + 31) / 32);
-      for (uint32_t e0 = list_at(C.Q, s / 32); e0 < e1; e0 += 32) {
-        const uint32_t e = e0 + lane;
-        const bool hit = e < e1 && C.Q.D[e] == d && C.Q.x[e] >= s && C.Q.x[e] < end;
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, hit);
-        if (bal) {
-          const uint32_t x = C.Q.x[e0 + __ffs(bal) - 1];
-          F = x - d;
-          off = (uint32_t)(x - s);
-          found = true;
-          break;
+      for (uint32_t e0 = list_at(C.Q, s / 32); e0 < e1 && !found; e0 += G) {
+        const uint32_t e = e0 + gl;
+        const uint32_t x = e < e1 ? C.Q.x[e] : 0;
+        const bool hit = e < e1 && C.Q.D[e] == d && x >= s && x < end;
+        if (G == 1) {
+          found = hit;
+          if (hit) F = x - d, off = (uint32_t)(x - s);
+        } else {
+          const unsigned bal = __ballot_sync(0xFFFFFFFFu, hit);
+          found = bal != 0;
+          if (found) {
+            const uint32_t fx = __shfl_sync(0xFFFFFFFFu, x, __ffs(bal) - 1);
+            F = fx - d, off = (uint32_t)(fx - s);
+          }
         }
       }
     }
-    if (lane) continue;
+    if (gl) continue;
     C.igram[i] = kNoSlot;
     C.islot[i] = kNoSlot;
     const bool tail = !pair && len != g.b;
@@ -842,33 +906,84 @@ __device__ __forceinline__ void chase_test(const M& m, const PrefixAt<M>& H, con
     c_min(&C.qs->lo_tailpair, p);
 }
 
-// List entries [e0, e1): the bitmap test, then per CTA a queue of gram hits
+// List entries [e0, e1): the bitmap test, then per warp a queue of gram hits
 // in shared memory, the gram table's walk, a queue of proposed windows and
-// their tests.  The queues never overflow for good: a proposal that finds
-// the second one full is tested on the spot, and the first one is emptied
-// before a tile could fill it.  Bound: the list's stream and one bitmap test
-// per entry; hits are a few percent of the entries.
-constexpr uint32_t kChaseTile = 2048, kHitQ = 4096, kCandQ = 2048;
-constexpr uint32_t kChaseBitWords = 8192;  // bitmap kept in shared memory up to 32 KiB
+// their tests, each step by 32 full lanes and without a barrier.  Neither
+// queue can overflow: a batch is taken out as soon as there are 32 entries.
+// Bound: the list's stream, one bitmap test per entry, and the chains of
+// dependent reads of the hits (table, prefix values and text, block table).
+constexpr uint32_t kChaseTile = 256;                 // entries per warp and step, eight per lane
+constexpr uint32_t kHitQ = kChaseTile + 32, kCandQ = 64;
+constexpr uint32_t kChaseBitWords = 4096;            // bitmap kept in shared memory up to 16 KiB
 
 template <class M>
-__global__ void __launch_bounds__(kT) k_chase_scan(M m, const __grid_constant__ PrefixAt<M> H, const __grid_constant__ Chase C,
-                                                   uint32_t e0, uint32_t e1, uint32_t smem_words,
-                                                   const unsigned long long* __restrict__ bound2) {
+__global__ void __launch_bounds__(kT, 4) k_chase_scan(M m, const __grid_constant__ PrefixAt<M> H, const __grid_constant__ Chase C,
+                                                      uint32_t e0, uint32_t e1, uint32_t smem_words,
+                                                      const unsigned long long* __restrict__ bound2) {
   extern __shared__ uint32_t bits_s[];
-  __shared__ uint2 hq[kHitQ];
-  __shared__ uint32_t cq[kCandQ];
-  __shared__ uint32_t hn, cn;
+  __shared__ uint2 hit_q[kT / 32][kHitQ];
+  __shared__ uint32_t cand_q[kT / 32][kCandQ];
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lt = (1u << lane) - 1u;
+  uint2* hq = hit_q[warp];
+  uint32_t* cq = cand_q[warp];
+  uint32_t hn = 0, cn = 0;  // warp-uniform
   for (uint32_t i = threadIdx.x; i < smem_words; i += kT) bits_s[i] = C.bitmap[i];
-  if (threadIdx.x == 0) hn = cn = 0;
   __syncthreads();
   const uint32_t* bits = smem_words ? bits_s : C.bitmap;
   const uint32_t tail_F = C.qs->tail_F, tail_off = C.qs->tail_off, pretail = C.qs->pretail;
   const uint64_t fp_tail = C.qs->fp_tail;
   uint32_t ncand = 0, nhit = 0;
-  for (uint64_t t0 = e0 + (uint64_t)blockIdx.x * kChaseTile; t0 < e1; t0 += (uint64_t)gridDim.x * kChaseTile) {
+  // 32 proposed windows (fewer at the end).
+  auto take_cands = [&]() {
+    const uint32_t n = cn < 32 ? cn : 32;
+    __syncwarp();
+    if (lane < n) chase_test(m, H, C, cq[cn - n + lane], pretail, fp_tail, nhit);
+    cn -= n;
+    __syncwarp();
+  };
+  // 32 gram hits (fewer at the end): every offset of the gram proposes.
+  auto take_hits = [&]() {
+    const uint32_t n = hn < 32 ? hn : 32;
+    __syncwarp();
+    const bool mine = lane < n;
+    const uint2 h = mine ? hq[hn - n + lane] : make_uint2(0, 0);
+    hn -= n;
+    if (mine && h.y == tail_F && tail_off <= h.x) {
+      const uint64_t p = h.x - tail_off;
+      if (p + C.r < C.g.n && p < *(volatile unsigned long long*)&C.qs->lo_tail &&
+          m.sub(H.at(m, p + C.r), m.mul(H.at(m, p), C.Br)) == fp_tail)
+        c_min(&C.qs->lo_tail, p);
+    }
+    bool live = mine;
+    uint32_t s = c_gram_home(h.y, C.gmask);
+    for (uint32_t it = 0; it <= C.gmask && __any_sync(0xFFFFFFFFu, live); it++) {
+      bool want = false;
+      uint32_t p = 0;
+      if (live) {
+        const ulonglong2 en = *(const ulonglong2*)&C.gt[s];
+        if (en.x == kNone) {
+          live = false;
+        } else if ((uint32_t)(en.x >> 32) == h.y) {
+          const uint32_t off = (uint32_t)en.x;
+          p = h.x - off;
+          want = off <= h.x && p < (bound2 ? bound2[s] : en.y);
+        }
+        s = (s + 1) & C.gmask;
+      }
+      const unsigned bal = __ballot_sync(0xFFFFFFFFu, want);
+      if (bal) {
+        if (want) cq[cn + __popc(bal & lt)] = p;
+        cn += __popc(bal);
+        if (lane == 0) ncand += __popc(bal);
+        if (cn >= 32) take_cands();
+      }
+    }
+  };
+  const uint64_t nwarps = (uint64_t)gridDim.x * (kT / 32);
+  for (uint64_t t0 = e0 + ((uint64_t)blockIdx.x * (kT / 32) + warp) * kChaseTile; t0 < e1; t0 += nwarps * kChaseTile) {
     uint32_t x[8], F[8];
-    const uint64_t e = t0 + 8ull * threadIdx.x;
+    uint32_t pass = 0;
+    const uint64_t e = t0 + 8ull * lane;
     if (e + 8 <= e1) {
 #pragma unroll
       for (int q = 0; q < 2; q++) {
@@ -879,54 +994,34 @@ __global__ void __launch_bounds__(kT) k_chase_scan(M m, const __grid_constant__ 
 #pragma unroll
       for (int u = 0; u < 8; u++) {
         const uint32_t bit = c_bit(C, F[u]);
-        if ((bits[bit >> 5] >> (bit & 31)) & 1u) hq[atomicAdd(&hn, 1u)] = make_uint2(x[u], F[u]);
+        pass |= ((bits[bit >> 5] >> (bit & 31)) & 1u) << u;
       }
     } else {
-      for (uint64_t f = e; f < e1; f++) {
-        const uint32_t X = C.Q.x[f], Fe = X - C.Q.D[f], bit = c_bit(C, Fe);
-        if ((bits[bit >> 5] >> (bit & 31)) & 1u) hq[atomicAdd(&hn, 1u)] = make_uint2(X, Fe);
+#pragma unroll
+      for (int u = 0; u < 8; u++) {
+        x[u] = F[u] = 0;
+        if (e + u >= e1) continue;
+        x[u] = C.Q.x[e + u];
+        F[u] = x[u] - C.Q.D[e + u];
+        const uint32_t bit = c_bit(C, F[u]);
+        pass |= ((bits[bit >> 5] >> (bit & 31)) & 1u) << u;
       }
     }
-    __syncthreads();
-    const uint32_t nh = hn;
-    if (nh <= kHitQ - kChaseTile && t0 + (uint64_t)gridDim.x * kChaseTile < e1) {
-      __syncthreads();
-      continue;
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      const bool ok = (pass >> u) & 1u;
+      const unsigned bal = __ballot_sync(0xFFFFFFFFu, ok);
+      if (ok) hq[hn + __popc(bal & lt)] = make_uint2(x[u], F[u]);
+      hn += __popc(bal);
     }
-    for (uint32_t i = threadIdx.x; i < nh; i += kT) {
-      const uint2 h = hq[i];
-      uint32_t s = c_gram_home(h.y, C.gmask);
-      for (uint32_t it = 0; it <= C.gmask; it++) {
-        const ulonglong2 en = *(const ulonglong2*)&C.gt[s];
-        if (en.x == kNone) break;
-        if ((uint32_t)(en.x >> 32) == h.y) {
-          const uint32_t off = (uint32_t)en.x;
-          const unsigned long long bound = bound2 ? bound2[s] : en.y;
-          if (off <= h.x && h.x - off < bound) {
-            ncand++;
-            const uint32_t q = atomicAdd(&cn, 1u);
-            if (q < kCandQ) cq[q] = h.x - off;
-            else chase_test(m, H, C, h.x - off, pretail, fp_tail, nhit);
-          }
-        }
-        s = (s + 1) & C.gmask;
-      }
-      if (h.y == tail_F && tail_off <= h.x) {
-        const uint64_t p = h.x - tail_off;
-        if (p + C.r < C.g.n && p < *(volatile unsigned long long*)&C.qs->lo_tail &&
-            m.sub(H.at(m, p + C.r), m.mul(H.at(m, p), C.Br)) == fp_tail)
-          c_min(&C.qs->lo_tail, p);
-      }
-    }
-    __syncthreads();
-    const uint32_t nc = cn < kCandQ ? cn : kCandQ;
-    for (uint32_t i = threadIdx.x; i < nc; i += kT) chase_test(m, H, C, cq[i], pretail, fp_tail, nhit);
-    __syncthreads();
-    if (threadIdx.x == 0) hn = cn = 0;
-    __syncthreads();
+    while (hn >= 32) take_hits();
   }
-  if (ncand) atomicAdd(&C.qs->cands, (unsigned long long)ncand);
-  if (nhit) atomicAdd(&C.qs->hits, (unsigned long long)nhit);
+  while (hn) take_hits();
+  while (cn) take_cands();
+  ncand = __reduce_add_sync(0xFFFFFFFFu, ncand);
+  nhit = __reduce_add_sync(0xFFFFFFFFu, nhit);
+  if (lane == 0 && ncand) atomicAdd(&C.qs->cands, (unsigned long long)ncand);
+  if (lane == 0 && nhit) atomicAdd(&C.qs->hits, (unsigned long long)nhit);
 }
 
 // Between the two halves of the scan: a (gram, offset) pair's windows are of
@@ -1000,18 +1095,18 @@ __global__ void __launch_bounds__(kT) k_chase_verify(Chase C, uint64_t ppk, unsi
   const unsigned lane = threadIdx.x & 31, grp = lane / L, gl = lane % L, gpw = 32 / L;
   const unsigned gmask = (L == 32 ? 0xFFFFFFFFu : ((1u << L) - 1u)) << (grp * L);
   const bool aligned16 = (((uintptr_t)g.T) & 15) == 0;
-  const uint64_t warps = (uint64_t)gridDim.x * (kT / 32), total = C.nitems * ppk;
+  const uint64_t warps = (uint64_t)gridDim.x * (kT / 32), total = C.nitems * ppk, piece = q_piece(g.b);
   for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32 * gpw; base < total; base += warps * gpw) {
     const uint64_t u = base + grp;
     bool d = false;
     uint64_t i = 0;
     if (u < total) {
       i = u / ppk;
-      const uint64_t off = (u - i * ppk) * kQPiece;
+      const uint64_t off = (u - i * ppk) * piece;
       uint64_t k, s, len;
       const uint64_t p = item_lo(C, i, &k, &s, &len);
       if (p < s && off < len)
-        d = differs(g.T, g.n, aligned16, p, s, off, off + kQPiece < len ? off + kQPiece : len, gl, L);
+        d = differs(g.T, g.n, aligned16, p, s, off, off + piece < len ? off + piece : len, gl, L);
     }
     const unsigned bal = __ballot_sync(0xFFFFFFFFu, d);
     if (u < total && gl == 0 && (bal & gmask)) C.differ[i] = 1;
@@ -1019,6 +1114,7 @@ __global__ void __launch_bounds__(kT) k_chase_verify(Chase C, uint64_t ppk, unsi
 }
 
 __global__ void __launch_bounds__(kT) k_chase_apply(Chase C) {
+  uint64_t vb = 0;
   for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; i < C.nitems; i += (uint64_t)gridDim.x * kT) {
     uint64_t k, s, len;
     const uint64_t p = item_lo(C, i, &k, &s, &len);
@@ -1027,7 +1123,7 @@ __global__ void __launch_bounds__(kT) k_chase_apply(Chase C) {
       atomicExch(&C.status->error, 25ull);
       continue;
     }
-    if (p < s) atomicAdd(&C.status->verify_bytes, 2ull * len);
+    if (p < s) vb += 2 * len;
     if (p < s && C.differ[i]) {  // a fingerprint collision: resolved exactly
       atomicAdd(&C.status->collisions, 1ull);
       const unsigned long long q = atomicAdd(&C.qs->nsusp, 1ull);
@@ -1039,6 +1135,8 @@ __global__ void __launch_bounds__(kT) k_chase_apply(Chase C) {
       C.lo[k] = p;
     }
   }
+  vb = warp_sum64(vb);
+  if ((threadIdx.x & 31) == 0 && vb) atomicAdd(&C.status->verify_bytes, (unsigned long long)vb);
 }
 
 // Exact leftmost occurrence of the keys whose match was false: every earlier
@@ -1093,7 +1191,10 @@ int quick_list(BuildCtx& ctx, QuickBuild& qb) {
   // Cells of the first-occurrence table: one per eight positions (there is
   // about one list entry per six, most of them repeats), at most 256 MiB:
   // random reads run at 300 G/s from L2-sized tables, 80-90 from 256 MiB, 47
-  // from 1 GiB (GB300), and a shared cell only loosens a bound.
+  // from 1 GiB (GB300), and a shared cell only loosens a bound.  Builds with
+  // one cell per 8, 16 and 32 positions of the 256 MiB text: 8.69, 8.74 and
+  // 9.12 ms; with at most 2^24 .. 2^27 cells for 2 GiB of DNA: 71.3, 57.2, 58.1
+  // and 59.2 ms.
   uint64_t cells = 1024;
   while (cells < n / 8 && cells < (1ull << 26)) cells <<= 1;
   uint32_t *mask, *first, *agg;
@@ -1124,7 +1225,8 @@ int quick_list(BuildCtx& ctx, QuickBuild& qb) {
   BT_CUDA(cudaMemsetAsync(first, 0xFF, cells * sizeof(uint32_t), s));
   if (nw)
     BT_LAUNCH(k_list_write<<<(unsigned)std::min<uint64_t>((nw + kT - 1) / kT, 152 * 16), kT, 0, s>>>(
-        ctx.T, n, nw, mask, qb.idx, qb.x, qb.D, first, (uint32_t)(cells - 1)));
+        ctx.T, n, nw, mask, qb.idx, qb.x, qb.D, (uint32_t)(cells - 1)));
+  BT_LAUNCH(k_list_first<<<grid_for(cap / 4 + 1, kT, 152 * 16), kT, 0, s>>>(qb.idx + nw, qb.x, qb.D, first));
   BT_LAUNCH(k_list_dist<<<grid_for(cap / 4 + 1, kT, 152 * 16), kT, 0, s>>>(qb.idx + nw, qb.x, qb.D, first));
   BT_LAUNCH(k_list_seg1<<<grid_for(ns * 32, kT), kT, 0, s>>>(nw, qb.idx, qb.D, ns, qb.seg1));
   BT_LAUNCH(k_list_seg2<<<grid_for(ns2, kT), kT, 0, s>>>(ns, qb.seg1, ns2, qb.seg2));
@@ -1186,15 +1288,16 @@ static int chase(const M& m, BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint6
   BT_TRY(allow_smem<k_chase_scan<M>>(kChaseBitWords * 4));
   const uint64_t top = std::max<uint64_t>(std::max(bcap, pcap), std::max<uint64_t>(gcap, bwords));
   BT_LAUNCH(k_chase_init<<<grid_for(top, kT), kT, 0, s>>>(C, bwords));
-  BT_LAUNCH(k_chase_keys<M><<<grid_for(ni * 32, kT), kT, 0, s>>>(m, H, C));
+  if (g.b <= 256) BT_LAUNCH(k_chase_keys<M, 1><<<grid_for(ni, kT), kT, 0, s>>>(m, H, C));
+  else BT_LAUNCH(k_chase_keys<M, 32><<<grid_for(ni * 32, kT), kT, 0, s>>>(m, H, C));
   {
     ProfScope prof("window_scan", s, 0);  // (the level's bytes are counted by its first part)
     // Two halves: the first sixteenth of the list, then the rest against the
     // bounds it lowered (most copies' content is first seen early).
     const uint32_t total = qb.qs_host->total;
-    const uint32_t split = total > (1u << 20) ? (total / 16) & ~(kChaseTile - 1) : 0;
+    const uint32_t split = total > (1u << 20) ? (total / 16) & ~(8 * kChaseTile - 1) : 0;
     const uint32_t sw = bwords <= kChaseBitWords ? bwords : 0;
-    auto grid = [](uint64_t n) { return (unsigned)std::min<uint64_t>((n + kChaseTile - 1) / kChaseTile, 152 * 3); };
+    auto grid = [](uint64_t n) { return (unsigned)std::min<uint64_t>((n + 8 * kChaseTile - 1) / (8 * kChaseTile), 152 * 4); };
     if (split) {
       BT_LAUNCH(k_chase_scan<M><<<grid(split), kT, sw * 4, s>>>(m, H, C, 0, split, sw, nullptr));
       BT_LAUNCH(k_chase_bound<<<grid_for(ni, kT), kT, 0, s>>>(C));
@@ -1204,10 +1307,10 @@ static int chase(const M& m, BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint6
                                                                        split ? C.bound2 : nullptr));
     if (C.r && C.r < 27) BT_LAUNCH(k_chase_tail<<<grid_for(g.n / 16 + 1, kT, 152 * 8), kT, 0, s>>>(C));
   }
-  const uint64_t ppk = (2 * g.b + kQPiece - 1) / kQPiece;
+  const uint64_t ppk = (2 * g.b + q_piece(g.b) - 1) / q_piece(g.b);
   const unsigned L = g.b >= 256 ? 32u : g.b >= 128 ? 16u : g.b >= 64 ? 8u : 4u;
   BT_LAUNCH(k_chase_verify<<<grid_for(ni * ppk * L, kT), kT, 0, s>>>(C, ppk, L));
-  BT_LAUNCH(k_chase_apply<<<grid_for(ni, kT), kT, 0, s>>>(C));
+  BT_LAUNCH(k_chase_apply<<<grid_for(ni, kT, 152 * 4), kT, 0, s>>>(C));
   BT_CUDA(cudaGetLastError());
   qb.resolve_exact = [=](uint64_t nsusp) -> int {
     const dim3 grid(grid_for(g.n, kT, 1024), (unsigned)std::min<uint64_t>(nsusp, 1024));
@@ -1252,10 +1355,10 @@ int quick_level(BuildCtx& ctx, QuickBuild& qb, uint32_t l, uint64_t last_start) 
   {
   ProfScope prof("window_scan", s, (c - 1) * b + (n - last_start < b ? n - last_start : b));
   BT_LAUNCH(k_quick_min<<<grid_for(c * G, kT), kT, 0, s>>>(g, qb.list, G, A, X, flags, qb.qs));
-  const uint64_t ppk = (2 * b + kQPiece - 1) / kQPiece;
+  const uint64_t ppk = (2 * b + q_piece(b) - 1) / q_piece(b);
   const unsigned L = b >= 256 ? 32u : b >= 128 ? 16u : b >= 64 ? 8u : 4u;
   BT_LAUNCH(k_quick_compare<<<grid_for(c * ppk * L, kT), kT, 0, s>>>(g, A, X, flags, ppk, L));
-  BT_LAUNCH(k_quick_settle<<<gc, kT, 0, s>>>(g, A, X, flags, v.lo, ps, items, v.mw, wpop, qb.qs, ctx.st));
+  BT_LAUNCH(k_quick_settle<<<grid_for(c, kT, 152 * 8), kT, 0, s>>>(g, A, X, flags, v.lo, ps, items, v.mw, wpop, qb.qs, ctx.st));
   }
   auto rank_and_wait = [&]() -> int {
     if (words <= kRankWords) {

@@ -20,7 +20,7 @@
 namespace bt {
 
 int alphabet(const uint8_t* T, uint64_t n, uint32_t sigma, bt_tree* t, cudaStream_t s);
-int upload_view(bt_tree* t, cudaStream_t s);
+int run_query_one(const bt_tree* t, int kind, uint64_t a0, uint64_t a1, uint64_t* out, cudaStream_t s);
 int batch_kernel_build(const uint8_t* const* texts, const uint64_t* ns, const uint32_t* sigmas,
                        const uint32_t* taus, const uint32_t* leaf_lens, uint64_t ndocs, const bt_opts& o,
                        std::vector<char>& routed, bt_tree** outs, uint32_t threads, uint32_t ctas_per_sm,
@@ -154,7 +154,7 @@ static void free_tree_memory(bt_tree* t) {
     t->slab.reset();
     return;
   }
-  void* rest[] = {t->leaf, t->pre, t->sym, t->view};
+  void* rest[] = {t->leaf, t->pre, t->sym, t->view, t->recs};
   for (void* a : rest)
     if (a) cudaFreeAsync(a, s);
   cudaStreamSynchronize(s);
@@ -269,13 +269,12 @@ static int build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, 
     BT_TRY(build_counters(ctx));
   }
   tr.mark("counters");
-  for (Level& v : t->lv) v.lo = nullptr;  // lives in the level's allocation; no longer needed
   ctx.arena.release();
-  BT_TRY(upload_view(t, s));
+  BT_TRY(pack_records(ctx));
   uint64_t bytes = t->leaf_bytes + 16 + sizeof(TreeView) + 512 + (t->lv[0].c + 1) * t->S * 8;
   for (const Level& v : t->lv) {
     const uint64_t words = (v.c + 31) / 32;
-    bytes += v.c * (8 + 4 + 8) + (2 * words + 1) * 4 + (v.cnt ? 2 * v.c * t->S * v.cw : 0);
+    bytes += v.c * 8 + (2 * words + 1) * 4 + (v.cnt ? 2 * v.c * t->S * v.cw : 0);
   }
   t->dev_bytes = bytes;
   BT_CUDA(cudaStreamSynchronize(s));
@@ -351,8 +350,7 @@ namespace {
 struct ExportLevel {
   const uint32_t* mw;
   const uint32_t* mr;
-  const uint32_t* ptr;
-  const uint64_t* off;
+  const uint2* rec;
   uint64_t c, b, nptr;
   uint64_t at;  // u64 index of the level's first field in the serialization
 };
@@ -376,8 +374,9 @@ __global__ void k_export_level(ExportLevel e, uint64_t* __restrict__ out) {
     const uint32_t word = e.mw[k >> 5];
     if ((word >> (k & 31)) & 1u) continue;
     const uint64_t i = k - (e.mr[k >> 5] + __popc(word & ((1u << (k & 31)) - 1u)));
-    pairs[2 * i] = e.ptr[k];
-    pairs[2 * i + 1] = e.off[k];
+    const uint2 r = e.rec[k];
+    pairs[2 * i] = r.x;
+    pairs[2 * i + 1] = r.y;
   }
 }
 
@@ -521,20 +520,28 @@ void bt_free(bt_tree* t) {
   delete t;
 }
 
+// One query: its arguments travel with the launch and the kernel writes the
+// answer to the calling thread's pinned word (portable: any device), so a call
+// is one launch and one wait instead of an allocation, two copies and a free
+// around them (about 38 us).  The word is given back when its thread ends.
+namespace {
+struct AnswerWord {
+  uint64_t* p = nullptr;
+  ~AnswerWord() {
+    if (p) cudaFreeHost(p);
+  }
+};
+thread_local AnswerWord g_answer;
+}  // namespace
+
 static int single_query(const bt_tree* t, int kind, uint64_t a0, uint64_t a1, uint64_t* res) {
   if (!t) return BT_EINVAL;
   cudaStream_t s = cudaStreamPerThread;
-  uint64_t* d;
-  BT_CUDA(cudaMallocAsync(&d, 3 * sizeof(uint64_t), s));
-  uint64_t h[2] = {a0, a1};
-  int rc = BT_OK;
-  if (cudaMemcpyAsync(d, h, sizeof(h), cudaMemcpyHostToDevice, s) != cudaSuccess) rc = BT_ECUDA;
-  if (rc == BT_OK) rc = run_queries(t, kind, d, 1, d + 2, s);
-  if (rc == BT_OK && cudaMemcpyAsync(res, d + 2, sizeof(uint64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-    rc = BT_ECUDA;
-  cudaFreeAsync(d, s);
-  if (cudaStreamSynchronize(s) != cudaSuccess && rc == BT_OK) rc = BT_ECUDA;
-  return rc;
+  if (!g_answer.p) BT_CUDA(cudaHostAlloc((void**)&g_answer.p, sizeof(uint64_t), cudaHostAllocPortable));
+  BT_TRY(run_query_one(t, kind, a0, a1, g_answer.p, s));
+  if (cudaStreamSynchronize(s) != cudaSuccess) return BT_ECUDA;
+  *res = *(volatile uint64_t*)g_answer.p;
+  return BT_OK;
 }
 
 int bt_access(const bt_tree* t, uint64_t i, uint8_t* out) {
@@ -602,7 +609,7 @@ int bt_export(const bt_tree* t, uint8_t* buf, uint64_t cap, uint64_t* len) {
   uint64_t at = 6;  // header: "BLKTREE1", n, tau, leaf_len, L, prune
   for (uint32_t l = 0; l < L; l++) {
     const Level& v = t->lv[l];
-    ex[l] = ExportLevel{v.mw, v.mr, v.ptr, v.off, v.c, v.b, v.c - nm[l], at};
+    ex[l] = ExportLevel{v.mw, v.mr, v.rec, v.c, v.b, v.c - nm[l], at};
     at += 2 + (v.c + 63) / 64 + 1 + 2 * (v.c - nm[l]);
   }
   const uint64_t leaf_at = at + 1, leaf_pad = (t->leaf_bytes + 7) / 8 * 8;

@@ -1510,16 +1510,12 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
   for (uint32_t l = 0; l < L; l++) {
     const PLv v = plevel(C, scr, bsz, l);
     const uint64_t words = (v.c + 31) / 32;
-    uint64_t* st = (uint64_t*)(out + s_ol[l].st);
     uint32_t* mw = (uint32_t*)(out + s_ol[l].mw);
     uint32_t* mr = (uint32_t*)(out + s_ol[l].mr);
-    uint32_t* ptr = (uint32_t*)(out + s_ol[l].ptr);
-    uint64_t* off = (uint64_t*)(out + s_ol[l].off);
-    for (uint64_t k = tid; k < v.c; k += nt) {
-      st[k] = v.st[k];
-      ptr[k] = v.ptr[k];
-      off[k] = marked(v.mw, k) ? 0 : v.off[k];
-    }
+    uint2* rec = (uint2*)(out + s_ol[l].rec);
+    for (uint64_t k = tid; k < v.c; k += nt)
+      rec[k] = marked(v.mw, k) ? make_uint2(kMarkedRec, (uint32_t)mrank(v.mw, v.mr, k))
+                               : make_uint2(v.ptr[k], (uint32_t)v.off[k]);
     for (uint64_t i = tid; i <= words; i += nt) {
       if (i < words) mw[i] = v.mw[i];
       mr[i] = v.mr[i];
@@ -1594,15 +1590,13 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
     for (uint32_t l = 0; l < L; l++) {
       const uint64_t words = (C.c[l] + 31) / 32;
       LevelView& lv = tv->lv[l];
-      lv.c = C.c[l];
-      lv.b = bsz[l];
+      lv.c = (uint32_t)C.c[l];
+      lv.b = view_len(bsz[l]);
       lv.arity = C.arity[l];
-      lv.bshift = block_shift(bsz[l]);
-      lv.st = (const uint64_t*)(out + s_ol[l].st);
-      lv.mw = (const uint32_t*)(out + s_ol[l].mw);
-      lv.mr = (const uint32_t*)(out + s_ol[l].mr);
-      lv.ptr = (const uint32_t*)(out + s_ol[l].ptr);
-      lv.off = (const uint64_t*)(out + s_ol[l].off);
+      lv.bshift = block_shift(view_len(bsz[l]));
+      const PLv v = plevel(C, scr, bsz, l);
+      lv.last_len = (uint32_t)plen(v, v.c - 1);
+      lv.rec = (const uint2*)(out + s_ol[l].rec);
       lv.cnt = out + s_ol[l].cnt;
       lv.pc = out + s_ol[l].pc;
       lv.cw = s_cw[l];
@@ -2076,11 +2070,9 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
       v.arity = Lr.arity;
       v.nmarked = Lr.nmarked;
       v.cw = Lr.cw;
-      v.st = (uint64_t*)(base + ol[l].st);
       v.mw = (uint32_t*)(base + ol[l].mw);
       v.mr = (uint32_t*)(base + ol[l].mr);
-      v.ptr = (uint32_t*)(base + ol[l].ptr);
-      v.off = (uint64_t*)(base + ol[l].off);
+      v.rec = (uint2*)(base + ol[l].rec);
       v.cnt = base + ol[l].cnt;
       v.pc = base + ol[l].pc;
       memcpy(v.stats, Lr.stats, sizeof(v.stats));

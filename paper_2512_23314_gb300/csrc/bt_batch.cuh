@@ -59,7 +59,7 @@ struct BRes {
 // the region's start.  The same function runs on the device (to write the
 // tree) and on the host (to point the bt_tree at it).
 struct OutLevel {
-  uint64_t st, mw, mr, ptr, off, cnt, pc;
+  uint64_t mw, mr, rec, cnt, pc;
 };
 __host__ __device__ inline uint64_t out_align(uint64_t x) { return (x + 255) & ~255ull; }
 __host__ __device__ inline uint64_t out_align16(uint64_t x) { return (x + 15) & ~15ull; }
@@ -74,16 +74,12 @@ __host__ __device__ inline uint64_t out_layout(uint32_t L, const uint64_t* c, co
   o = out_align16(o + sizeof(TreeView));
   for (uint32_t l = 0; l < L; l++) {
     const uint64_t words = (c[l] + 31) / 32;
-    lv[l].st = o;
+    lv[l].rec = o;
     o = out_align16(o + c[l] * 8 + 8);
     lv[l].mw = o;
     o = out_align16(o + words * 4 + 4);
     lv[l].mr = o;
     o = out_align16(o + (words + 1) * 4);
-    lv[l].ptr = o;
-    o = out_align16(o + c[l] * 4 + 4);
-    lv[l].off = o;
-    o = out_align16(o + c[l] * 8 + 8);
     lv[l].cnt = o;
     o = out_align16(o + c[l] * S * cw[l] + 4);
     lv[l].pc = o;

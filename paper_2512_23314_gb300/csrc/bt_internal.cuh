@@ -5,14 +5,18 @@
 //   H           u64[n + 1]     Karp-Rabin prefix fingerprints H(p) (section 2),
 //                              during construction only
 //   per level l (blocks in text order):
-//     st        u64[c]         block starts (multiples of b_l)
 //     mw        u32[ceil(c/32)] mark bits, bit k%32 of word k/32
-//     mr        u32[words + 1] exclusive prefix popcounts of mw (rank support)
-//     ptr       u32[c]         unmarked: index of the block holding the leftmost
-//                              occurrence of the block's string
-//     off       u64[c]         unmarked: offset of that occurrence in block ptr
-//     cnt       u32[c * S]     symbol counts of the block (S distinct symbols)
-//     pc        u32[c * S]     unmarked: symbol counts of T[st[ptr], st[ptr]+off)
+//     mr        u32[words + 1] exclusive prefix popcounts of mw
+//     rec       uint2[c]       unmarked: (index of the block holding the leftmost
+//                              occurrence of the block's string, its offset
+//                              there); marked: (kMarkedRec, mark rank).  All a
+//                              query needs of a block in one 8-byte read
+//     cnt       [c * S]        symbol counts of the block (S distinct symbols)
+//     pc        [c * S]        unmarked: symbol counts of the target's text
+//                              before the copied window
+//   during construction also
+//     st        u64[c]         block starts (multiples of b_l)
+//     ptr, off, lo             the pointers and leftmost occurrences apart
 //   pre         u64[(c_1+1)*S] level 1: symbol counts of T[0, st[k])
 //   leaf        u8[...]        text of the marked last-level blocks, block r at r*b_L
 // A marked block of a non-last level with mark rank r has its children at
@@ -119,6 +123,7 @@ struct Level {
   uint32_t* ptr = nullptr;
   uint64_t* off = nullptr;
   uint64_t* lo = nullptr;  // exact leftmost occurrence of every block (pruning)
+  uint2* rec = nullptr;    // the finished tree's records (st, ptr, off and lo are gone then)
   void* cnt = nullptr;     // counter rows, cw bytes per counter
   void* pc = nullptr;
   uint32_t cw = 4;
@@ -126,19 +131,18 @@ struct Level {
   std::vector<void*> owned;  // device allocations holding this level's arrays
 };
 
-// Device-side view of one level, passed by value to kernels.
+constexpr uint32_t kMarkedRec = 0xFFFFFFFFu;
+
+// Device-side view of one level for the queries.  Positions fit 32 bits.
 struct LevelView {
-  uint64_t c, b;
+  uint32_t c, b;        // blocks, block length (at most 2^32 - 1)
   uint32_t arity;
-  uint32_t bshift;  // log2(b) when b is a power of two, else 0xFF
-  const uint64_t* st;
-  const uint32_t* mw;
-  const uint32_t* mr;
-  const uint32_t* ptr;
-  const uint64_t* off;
-  const void* cnt;  // symbol counters of the blocks, cw bytes each (1, 2 or 4)
+  uint32_t bshift;      // log2(b) when b is a power of two, else 0xFF
+  uint32_t last_len;    // length of block c - 1 (the others are b long)
+  uint32_t cw;          // bytes per counter (1, 2 or 4)
+  const uint2* rec;
+  const void* cnt;      // symbol counters of the blocks (null: counted in the leaf text)
   const void* pc;
-  uint32_t cw;
 };
 
 __host__ __device__ inline uint32_t block_shift(uint64_t b) {
@@ -147,6 +151,10 @@ __host__ __device__ inline uint32_t block_shift(uint64_t b) {
   while ((1ull << s) < b) s++;
   return s;
 }
+
+// A block length as the queries use it (explicit lengths may exceed 32 bits;
+// such a level has one block, which every position divides into as 0).
+__host__ __device__ inline uint32_t view_len(uint64_t b) { return b > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)b; }
 
 // Bytes per symbol counter of a level with block length b: a count never
 // exceeds b.
@@ -188,6 +196,7 @@ struct bt_tree {
   int16_t sym_host[256];
   uint32_t S = 0;
   bt::TreeView* view = nullptr;  // device copy of the view
+  void* recs = nullptr;          // records, mark words and rank prefixes of all levels
   int device = 0;
   uint64_t dev_bytes = 0;        // device memory held by the tree
   // Trees of a batched build live in a region of the batch's output pool:
@@ -379,6 +388,7 @@ struct BuildCtx {
 int build_levels(BuildCtx& ctx);
 int prune_tree(BuildCtx& ctx, uint64_t max_rounds);
 int build_counters(BuildCtx& ctx);
+int pack_records(BuildCtx& ctx);
 int sync_status(BuildCtx& ctx);
 
 }  // namespace bt

@@ -204,51 +204,80 @@ __global__ void k_leaf_text(uint64_t c, uint64_t b, uint64_t n, const uint64_t* 
 // ---------------------------------------------------------------------------
 // Queries.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool qmarked(const LevelView& v, uint64_t k) {
-  return (v.mw[k >> 5] >> (k & 31)) & 1u;
-}
-__device__ __forceinline__ uint64_t qrank(const LevelView& v, uint64_t k) {
-  return v.mr[k >> 5] + __popc(v.mw[k >> 5] & ((1u << (k & 31)) - 1u));
-}
-__device__ __forceinline__ uint64_t qlen(const TreeView& t, const LevelView& v, uint64_t k) {
-  uint64_t s = v.st[k];
-  return t.n - s < v.b ? t.n - s : v.b;
+__device__ __forceinline__ uint32_t qlen(const LevelView& v, uint32_t k) { return k + 1 == v.c ? v.last_len : v.b; }
+
+// x / b for the block length of a level (a shift when b is a power of two).
+__device__ __forceinline__ uint32_t div_b(uint32_t x, const LevelView& v) {
+  return v.bshift != 0xFFu ? x >> v.bshift : x / v.b;
 }
 
-// Occurrences of byte c in p[0, o): four bytes per step from aligned words
-// (a per-byte compare, __vcmpeq4, then a population count).
-__device__ __forceinline__ uint64_t leaf_count(const uint8_t* p, uint64_t o, uint32_t c) {
-  uint64_t x = 0, acc = 0;
-  for (; x < o && (((uintptr_t)(p + x)) & 3); x++) acc += p[x] == c;  // up to an aligned word
+// Occurrences of byte c in p[0, o): 16 bytes per load from a 16-byte aligned
+// start (a per-byte compare, __vcmpeq4, then a population count), four bytes
+// per step otherwise.
+__device__ __forceinline__ uint32_t leaf_count(const uint8_t* p, uint32_t o, uint32_t c) {
+  uint32_t x = 0, acc = 0;
   const uint32_t cc = c * 0x01010101u;
+  if ((((uintptr_t)p) & 15) == 0) {
+    // (The leaf text is followed by 16 bytes, so the last unit is readable.)
+    for (; x < o; x += 16) {
+      const uint4 v = *(const uint4*)(p + x);
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      const uint32_t left = o - x;
+#pragma unroll
+      for (uint32_t q = 0; q < 4; q++) {
+        uint32_t eq = __vcmpeq4(w[q], cc);
+        if (left < 4 * q + 4) eq = left <= 4 * q ? 0u : eq & ((1u << (8 * (left - 4 * q))) - 1u);
+        acc += __popc(eq);
+      }
+    }
+    return acc >> 3;
+  }
+  for (; x < o && (((uintptr_t)(p + x)) & 3); x++) acc += p[x] == c;  // up to an aligned word
   const uint32_t* w = (const uint32_t*)(p + x);
-  uint64_t i = 0;
-  for (; x + 4 <= o; x += 4, i++) acc += __popc(__vcmpeq4(w[i], cc)) >> 3;
+  for (uint32_t i = 0; x + 4 <= o; x += 4, i++) acc += __popc(__vcmpeq4(w[i], cc)) >> 3;
   for (; x < o; x++) acc += p[x] == c;
   return acc;
 }
 
-// Position of the j-th occurrence (j >= 1) of byte c in p[0, len), or kNone.
-__device__ __forceinline__ uint64_t leaf_find(const uint8_t* p, uint64_t len, uint32_t c, uint64_t j) {
-  uint64_t x = 0;
+// Position of the j-th occurrence (j >= 1) of byte c in p[0, len), or kNoSlot.
+__device__ __forceinline__ uint32_t leaf_find(const uint8_t* p, uint32_t len, uint32_t c, uint32_t j) {
+  uint32_t x = 0;
+  const uint32_t cc = c * 0x01010101u;
+  if ((((uintptr_t)p) & 15) == 0) {
+    for (; x < len; x += 16) {
+      const uint4 v = *(const uint4*)(p + x);
+      const uint32_t e[4] = {__vcmpeq4(v.x, cc), __vcmpeq4(v.y, cc), __vcmpeq4(v.z, cc), __vcmpeq4(v.w, cc)};
+      const uint32_t k = (__popc(e[0]) + __popc(e[1]) + __popc(e[2]) + __popc(e[3])) >> 3;
+      if (k < j) {
+        j -= k;
+        continue;
+      }
+#pragma unroll
+      for (uint32_t q = 0; q < 4; q++) {
+        const uint32_t kq = __popc(e[q]) >> 3;
+        if (j > kq) {
+          j -= kq;
+          continue;
+        }
+        uint32_t m = e[q] & 0x01010101u;
+        for (; j > 1; j--) m &= m - 1;
+        const uint32_t at = x + 4 * q + (__ffs(m) - 1) / 8;
+        return at < len ? at : kNoSlot;
+      }
+    }
+    return kNoSlot;
+  }
   if ((((uintptr_t)p) & 3) == 0) {
-    const uint32_t cc = c * 0x01010101u;
     const uint32_t* w = (const uint32_t*)p;
     for (; x + 4 <= len; x += 4) {
-      const uint32_t eq = __vcmpeq4(w[x >> 2], cc);
-      const uint32_t k = __popc(eq) >> 3;
+      const uint32_t k = __popc(__vcmpeq4(w[x >> 2], cc)) >> 3;
       if (k >= j) break;  // the j-th is in this word: bytes below
       j -= k;
     }
   }
   for (; x < len; x++)
     if (p[x] == c && --j == 0) return x;
-  return kNone;
-}
-
-// x / b for the block length of a level (a shift when b is a power of two).
-__device__ __forceinline__ uint64_t div_b(uint64_t x, const LevelView& v) {
-  return v.bshift != 0xFFu ? x >> v.bshift : x / v.b;
+  return kNoSlot;
 }
 
 // Space-efficient counters (BT_FLAG_LEAF_COUNTS): the last level stores no
@@ -256,84 +285,110 @@ __device__ __forceinline__ uint64_t div_b(uint64_t x, const LevelView& v) {
 // A marked last-level block's text is its leaf text; an unmarked one copies a
 // window of at most two marked blocks (its target and the next one), whose
 // text is in the leaf text too.
-__device__ uint64_t leaf_block_count(const TreeView& t, const LevelView& v, uint64_t k, uint32_t c) {
-  const uint64_t len = qlen(t, v, k);
-  if (qmarked(v, k)) return leaf_count(t.leaf + qrank(v, k) * v.b, len, c);
-  const uint64_t j = v.ptr[k], o = v.off[k], lj = qlen(t, v, j);
-  const uint64_t first = o + len <= lj ? len : lj - o;
-  uint64_t acc = leaf_count(t.leaf + qrank(v, j) * v.b + o, first, c);
-  if (first < len) acc += leaf_count(t.leaf + qrank(v, j + 1) * v.b, len - first, c);
+__device__ __noinline__ uint32_t leaf_block_count(const uint8_t* leaf, const LevelView& v, uint32_t k, uint32_t c) {
+  const uint32_t len = qlen(v, k);
+  const uint2 r = v.rec[k];
+  if (r.x == kMarkedRec) return leaf_count(leaf + (uint64_t)r.y * v.b, len, c);
+  const uint32_t lj = qlen(v, r.x);
+  const uint32_t first = r.y + len <= lj ? len : lj - r.y;
+  const uint32_t rank = v.rec[r.x].y;  // the targets are marked: ranks rank, rank + 1
+  uint32_t acc = leaf_count(leaf + (uint64_t)rank * v.b + r.y, first, c);
+  if (first < len) acc += leaf_count(leaf + (uint64_t)(rank + 1) * v.b, len - first, c);
   return acc;
 }
 
-// Counts of byte c in T[st[ptr], st[ptr] + off) of an unmarked last-level block.
-__device__ uint64_t leaf_prefix_count(const TreeView& t, const LevelView& v, uint64_t k, uint32_t c) {
-  const uint64_t j = v.ptr[k];
-  return leaf_count(t.leaf + qrank(v, j) * v.b, v.off[k], c);
+// Counts of byte c in the target of an unmarked last-level block before the window.
+__device__ __noinline__ uint32_t leaf_prefix_count(const uint8_t* leaf, const LevelView& v, uint2 r, uint32_t c) {
+  return leaf_count(leaf + (uint64_t)v.rec[r.x].y * v.b, r.y, c);
 }
 
 // Counter of symbol s (byte c) of block k: stored, or counted in the leaf text.
-__device__ __forceinline__ uint64_t blk_cnt(const TreeView& t, const LevelView& v, uint64_t k, uint32_t s,
+__device__ __forceinline__ uint32_t blk_cnt(const uint8_t* leaf, uint32_t S, const LevelView& v, uint32_t k, uint32_t s,
                                             uint32_t c) {
-  return v.cnt ? cget(v.cnt, v.cw, k * t.S + s) : leaf_block_count(t, v, k, c);
+  return v.cnt ? cget(v.cnt, v.cw, (uint64_t)k * S + s) : leaf_block_count(leaf, v, k, c);
 }
-__device__ __forceinline__ uint64_t blk_pc(const TreeView& t, const LevelView& v, uint64_t k, uint32_t s,
-                                           uint32_t c) {
-  return v.pc ? cget(v.pc, v.cw, k * t.S + s) : leaf_prefix_count(t, v, k, c);
+__device__ __forceinline__ uint32_t blk_pc(const uint8_t* leaf, uint32_t S, const LevelView& v, uint32_t k, uint2 r,
+                                           uint32_t s, uint32_t c) {
+  return v.pc ? cget(v.pc, v.cw, (uint64_t)k * S + s) : leaf_prefix_count(leaf, v, r, c);
 }
 
-__device__ uint64_t q_access(const TreeView& t, uint64_t i) {
+// What a descent needs of the tree besides the level table.
+struct QTree {
+  uint64_t n;
+  uint32_t L, S;
+  const uint64_t* pre;
+  const uint8_t* leaf;
+  const int16_t* sym;
+};
+
+// A descent keeps the offset o inside the current block instead of a text
+// position, so no block starts are read: one 8-byte record per step.
+__device__ __forceinline__ uint64_t q_access(const QTree& t, const LevelView* __restrict__ lv, uint64_t i) {
   if (i >= t.n) return kNone;
-  uint32_t l = 0;
-  uint64_t k = div_b(i, t.lv[0]), x = i;
+  uint32_t l = 0, k = div_b((uint32_t)i, lv[0]), o = (uint32_t)i - k * lv[0].b;
   for (uint32_t step = 0; step < 4 * t.L + 4; step++) {
-    const LevelView& v = t.lv[l];
-    if (qmarked(v, k)) {
-      if (l + 1 == t.L) return t.leaf[qrank(v, k) * v.b + (x - v.st[k])];
-      k = qrank(v, k) * v.arity + div_b(x - v.st[k], t.lv[l + 1]);
+    const LevelView& v = lv[l];
+    const uint2 r = v.rec[k];
+    if (r.x == kMarkedRec) {
+      if (l + 1 == t.L) return t.leaf[(uint64_t)r.y * v.b + o];
       l++;
+      const uint32_t j = div_b(o, lv[l]);
+      k = r.y * v.arity + j;
+      o -= j * lv[l].b;
     } else {
-      uint64_t P = v.ptr[k];
-      x = v.st[P] + v.off[k] + (x - v.st[k]);
-      k = x < v.st[P] + qlen(t, v, P) ? P : P + 1;
+      const uint32_t lp = qlen(v, r.x), x = r.y + o;
+      k = r.x + (x >= lp);
+      o = x >= lp ? x - lp : x;
     }
   }
   return kNone;
 }
 
-__device__ uint64_t q_rank(const TreeView& t, uint32_t c, uint64_t i) {
+// rank descends likewise.  Its counters are off the chain of dependent reads:
+// they are added one step later, when the next record has been read too.
+__device__ __forceinline__ uint64_t q_rank(const QTree& t, const LevelView* __restrict__ lv, uint32_t c, uint64_t i) {
   if (i > t.n) return kNone;
-  int s = t.sym[c & 0xFF];
+  const int s = t.sym[c];
   if (s < 0) return 0;
   const uint32_t S = t.S;
-  const LevelView& r = t.lv[0];
-  if (i == t.n) return t.pre[r.c * S + s];
-  uint64_t k = div_b(i, r), o = i - r.st[k];
-  int64_t acc = (int64_t)t.pre[k * S + s];
-  uint32_t l = 0;
+  if (i == t.n) return t.pre[(uint64_t)lv[0].c * S + s];
+  uint32_t l = 0, k = div_b((uint32_t)i, lv[0]), o = (uint32_t)i - k * lv[0].b;
+  int64_t acc = (int64_t)t.pre[(uint64_t)k * S + s];
+  uint32_t p0 = 0, p1 = 0, p2 = 0, m0 = 0;  // counters in flight: to add, to subtract
   for (uint32_t step = 0; step < 4 * t.L + 4; step++) {
-    const LevelView& v = t.lv[l];
-    if (o == 0) return (uint64_t)acc;
-    uint64_t len = qlen(t, v, k);
-    if (o == len) return (uint64_t)(acc + blk_cnt(t, v, k, s, c & 0xFF));
-    if (qmarked(v, k)) {
-      if (l + 1 == t.L) return (uint64_t)(acc + leaf_count(t.leaf + qrank(v, k) * v.b, o, c & 0xFF));
-      const LevelView& w = t.lv[l + 1];
-      uint64_t j = div_b(o, w), f = qrank(v, k) * v.arity;
-      for (uint64_t x = 0; x < j; x++) acc += blk_cnt(t, w, f + x, s, c & 0xFF);
+    const LevelView& v = lv[l];
+    if (o == 0) return (uint64_t)(acc + p0 + p1 + p2 - m0);
+    if (o == qlen(v, k)) return (uint64_t)(acc + p0 + p1 + p2 - m0 + blk_cnt(t.leaf, S, v, k, s, c));
+    const uint2 r = v.rec[k];
+    if (r.x == kMarkedRec) {
+      acc += (int64_t)p0 + p1 + p2 - m0;
+      p0 = p1 = p2 = m0 = 0;
+      if (l + 1 == t.L) return (uint64_t)(acc + leaf_count(t.leaf + (uint64_t)r.y * v.b, o, c));
+      const LevelView& w = lv[++l];
+      const uint32_t j = div_b(o, w), f = r.y * v.arity;
       o -= j * w.b;
       k = f + j;
-      l++;
+      if (w.cnt) {
+        const uint64_t at = (uint64_t)f * S + s;
+        uint32_t x = 0;
+        for (; x + 3 < j; x++) acc += cget(w.cnt, w.cw, at + (uint64_t)x * S);
+        if (x < j) p0 = cget(w.cnt, w.cw, at + (uint64_t)x * S);
+        if (x + 1 < j) p1 = cget(w.cnt, w.cw, at + (uint64_t)(x + 1) * S);
+        if (x + 2 < j) p2 = cget(w.cnt, w.cw, at + (uint64_t)(x + 2) * S);
+      } else {
+        for (uint32_t x = 0; x < j; x++) acc += leaf_block_count(t.leaf, w, f + x, c);
+      }
     } else {
-      uint64_t P = v.ptr[k], x = v.off[k] + o;
-      acc -= blk_pc(t, v, k, s, c & 0xFF);
-      uint64_t lp = qlen(t, v, P);
+      acc += (int64_t)p0 + p1 + p2 - m0;
+      p0 = p1 = p2 = 0;
+      m0 = blk_pc(t.leaf, S, v, k, r, s, c);
+      const uint32_t lp = qlen(v, r.x), x = r.y + o;
       if (x <= lp) {
-        k = P;
+        k = r.x;
         o = x;
       } else {
-        acc += blk_cnt(t, v, P, s, c & 0xFF);
-        k = P + 1;
+        p0 = blk_cnt(t.leaf, S, v, r.x, s, c);
+        k = r.x + 1;
         o = x - lp;
       }
     }
@@ -341,156 +396,175 @@ __device__ uint64_t q_rank(const TreeView& t, uint32_t c, uint64_t i) {
   return kNone;
 }
 
-__device__ uint64_t q_select(const TreeView& t, uint32_t c, uint64_t j) {
-  int s = t.sym[c & 0xFF];
-  if (s < 0 || j == 0) return kNone;
+// select needs the counters to find its way: those of up to three children
+// are read together, and an unmarked block's prefix counter with its record.
+__device__ __forceinline__ uint64_t q_select(const QTree& t, const LevelView* __restrict__ lv, uint32_t c, uint64_t jq) {
+  const int s = t.sym[c];
+  if (s < 0 || jq == 0) return kNone;
   const uint32_t S = t.S;
-  const LevelView& r = t.lv[0];
-  if (j > t.pre[r.c * S + s]) return kNone;
-  uint64_t a = 0, z = r.c;  // last k with pre[k] < j
+  const LevelView& top = lv[0];
+  if (jq > t.pre[(uint64_t)top.c * S + s]) return kNone;
+  uint32_t a = 0, z = top.c;  // last k with pre[k] < j
   while (z - a > 1) {
-    uint64_t mid = (a + z) / 2;
-    if (t.pre[mid * S + s] < j) a = mid;
+    const uint32_t mid = (a + z) / 2;
+    if (t.pre[(uint64_t)mid * S + s] < jq) a = mid;
     else z = mid;
   }
-  uint64_t k = a;
-  j -= t.pre[k * S + s];
-  int64_t res = (int64_t)r.st[k];
-  uint32_t l = 0;
+  uint32_t k = a, l = 0;
+  uint32_t j = (uint32_t)(jq - t.pre[(uint64_t)k * S + s]);
+  int64_t res = (int64_t)k * top.b;
   for (uint32_t step = 0; step < 4 * t.L + 4; step++) {
-    const LevelView& v = t.lv[l];
-    if (qmarked(v, k)) {
+    const LevelView& v = lv[l];
+    const uint2 r = v.rec[k];
+    const uint32_t pck = v.pc ? cget(v.pc, v.cw, (uint64_t)k * S + s) : 0;
+    if (r.x == kMarkedRec) {
       if (l + 1 == t.L) {
-        const uint64_t x = leaf_find(t.leaf + qrank(v, k) * v.b, qlen(t, v, k), c & 0xFF, j);
-        return x == kNone ? kNone : (uint64_t)(res + (int64_t)x);
+        const uint32_t x = leaf_find(t.leaf + (uint64_t)r.y * v.b, qlen(v, k), c, j);
+        return x == kNoSlot ? kNone : (uint64_t)(res + x);
       }
-      const LevelView& w = t.lv[l + 1];
-      uint64_t f = qrank(v, k) * v.arity, i = 0;
-      while (i < v.arity) {
-        const uint64_t cc = blk_cnt(t, w, f + i, s, c & 0xFF);
-        if (cc >= j) break;
-        j -= cc;
-        i++;
+      const LevelView& w = lv[++l];
+      const uint32_t f = r.y * v.arity, ar = v.arity;
+      uint32_t i = 0;
+      bool found = false;
+      if (w.cnt) {
+        const uint64_t at = (uint64_t)f * S + s;
+        // (A short last block has fewer children: counters past the level's
+        // end are not read, and the j-th symbol lies before them.)
+        const uint32_t have = w.c - f < ar ? w.c - f : ar;
+        while (i < have && !found) {
+          uint32_t cc[4];
+#pragma unroll
+          for (uint32_t u = 0; u < 4; u++) cc[u] = i + u < have ? cget(w.cnt, w.cw, at + (uint64_t)(i + u) * S) : 0xFFFFFFFFu;
+#pragma unroll
+          for (uint32_t u = 0; u < 4; u++) {
+            if (found) continue;
+            if (cc[u] >= j) {
+              found = true;
+              i += u;
+            } else {
+              j -= cc[u];
+            }
+          }
+          if (!found) i += 4;
+        }
+        found = found && i < have;
+      } else {
+        for (; i < ar && !found; i++) {
+          const uint32_t cc = leaf_block_count(t.leaf, w, f + i, c);
+          if (cc >= j) {
+            found = true;
+            break;
+          }
+          j -= cc;
+        }
       }
-      if (i == v.arity) return kNone;
-      res += (int64_t)(i * w.b);
+      if (!found) return kNone;
+      res += (int64_t)i * w.b;
       k = f + i;
-      l++;
     } else {
-      uint64_t P = v.ptr[k], jj = j + blk_pc(t, v, k, s, c & 0xFF);
-      const uint64_t cp = blk_cnt(t, v, P, s, c & 0xFF);
+      const uint32_t cp = blk_cnt(t.leaf, S, v, r.x, s, c);
+      const uint32_t jj = j + (v.pc ? pck : leaf_prefix_count(t.leaf, v, r, c));
       if (jj <= cp) {
-        res -= (int64_t)v.off[k];
-        k = P;
+        res -= (int64_t)r.y;
+        k = r.x;
         j = jj;
       } else {
-        res += (int64_t)(qlen(t, v, P) - v.off[k]);
+        res += (int64_t)qlen(v, r.x) - r.y;
         j = jj - cp;
-        k = P + 1;
+        k = r.x + 1;
       }
     }
   }
   return kNone;
 }
 
-// The batched query kernel.  Every CTA first copies the tree's level table
-// and the arrays of its top levels (block starts, marks, rank prefix,
-// pointers, offsets, and the counters while they fit) into shared memory:
-// every query descends through the top levels, so those steps read shared
-// memory instead of L2.  Then each thread answers queries (grid-stride).
-constexpr uint32_t kQThreads = 256;
-
-__device__ __forceinline__ void copy_words(uint32_t* dst, const void* src, uint64_t bytes) {
-  const uint32_t* s = (const uint32_t*)src;
-  for (uint64_t i = threadIdx.x; i < bytes / 4; i += blockDim.x) dst[i] = s[i];
+template <int KIND>
+__device__ __forceinline__ uint64_t q_answer(const QTree& t, const LevelView* __restrict__ lv, uint64_t a0, uint64_t a1) {
+  if (KIND == BT_Q_ACCESS) return q_access(t, lv, a0);
+  if (a0 > 255) return kNone;
+  return KIND == BT_Q_RANK ? q_rank(t, lv, (uint32_t)a0, a1) : q_select(t, lv, (uint32_t)a0, a1);
 }
 
-template <uint32_t kQCacheBytes, int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_queries(const TreeView* __restrict__ tv, int kind,
-                                                            const uint64_t* __restrict__ args, uint64_t m,
-                                                            uint64_t* __restrict__ out) {
-  if (kQCacheBytes == 0) {  // the level table straight from global memory (L1-cached broadcasts)
-    const TreeView& t = *tv;
-    for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < m;
-         q += (uint64_t)gridDim.x * blockDim.x) {
-      uint64_t r;
-      if (kind == BT_Q_ACCESS) r = q_access(t, args[q]);
-      else if (kind == BT_Q_RANK) r = args[2 * q] > 255 ? kNone : q_rank(t, (uint32_t)args[2 * q], args[2 * q + 1]);
-      else r = args[2 * q] > 255 ? kNone : q_select(t, (uint32_t)args[2 * q], args[2 * q + 1]);
-      out[q] = r;
-    }
-    return;
-  }
-  __shared__ TreeView st;
-  __shared__ __align__(16) uint32_t cache[kQCacheBytes / 4 + 4];
-  __shared__ uint32_t s_off[kMaxLevels][7];
-  __shared__ uint32_t s_lc;
-  {
-    const uint32_t* src = (const uint32_t*)tv;
-    uint32_t* dst = (uint32_t*)&st;
-    for (uint32_t i = threadIdx.x; i < sizeof(TreeView) / 4; i += blockDim.x) dst[i] = src[i];
-  }
+// The batched query kernel: one thread answers a query.  Bound: the chain of
+// dependent reads (a record per level and pointer hop, L2 or DRAM) times the
+// threads in flight.  The level table is in shared memory; the records of the
+// upper levels stay in L1.  Measured on 4 M queries of each kind on the tree of
+// the 256 MiB text: 3.68 ms when a step read block starts, marks, ranks,
+// pointers and offsets from five arrays (and every CTA copied the top levels
+// into shared memory), 2.82 ms with one record; 1000 queries of each kind 79
+// and 42 us.
+template <int KIND, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_queries(const TreeView* __restrict__ tv, const uint64_t* __restrict__ args,
+                                                      uint64_t m, uint64_t* __restrict__ out) {
+  __shared__ __align__(16) LevelView lv[kMaxLevels];
+  const QTree t{tv->n, tv->L, tv->S, tv->pre, tv->leaf, tv->sym};
+  for (uint32_t i = threadIdx.x; i < t.L * (sizeof(LevelView) / 4); i += NT)
+    ((uint32_t*)lv)[i] = ((const uint32_t*)tv->lv)[i];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // Top levels that fit: st, mw, mr, ptr, off, cnt, pc (each 16-byte
-    // aligned in the cache); counters only while the whole level fits.
-    uint32_t used = 0, lc = 0;
-    for (uint32_t l = 0; l < st.L; l++) {
-      const LevelView& v = st.lv[l];
-      const uint64_t words = (v.c + 31) / 32;
-      const uint64_t cb = v.cnt ? v.c * st.S * v.cw : 0;
-      const uint64_t sz[7] = {v.c * 8, words * 4, (words + 1) * 4, v.c * 4, v.c * 8, cb, cb};
-      uint64_t tot = 0;
-      for (int a = 0; a < 7; a++) tot += (sz[a] + 15) & ~15ull;
-      if (used + tot > kQCacheBytes) break;
-      for (int a = 0; a < 7; a++) {
-        s_off[l][a] = used;
-        used += (uint32_t)((sz[a] + 15) & ~15ull);
-      }
-      lc = l + 1;
-    }
-    s_lc = lc;
-  }
-  __syncthreads();
-  const uint32_t lc = s_lc;
-  for (uint32_t l = 0; l < lc; l++) {
-    const LevelView& v = st.lv[l];
-    const uint64_t words = (v.c + 31) / 32;
-    copy_words(cache + s_off[l][0] / 4, v.st, v.c * 8);
-    copy_words(cache + s_off[l][1] / 4, v.mw, (words * 4 + 3) & ~3ull);
-    copy_words(cache + s_off[l][2] / 4, v.mr, (words + 1) * 4);
-    copy_words(cache + s_off[l][3] / 4, v.ptr, v.c * 4);
-    copy_words(cache + s_off[l][4] / 4, v.off, v.c * 8);
-    if (v.cnt) {
-      const uint64_t cb = (v.c * st.S * v.cw + 3) & ~3ull;
-      copy_words(cache + s_off[l][5] / 4, v.cnt, cb);
-      copy_words(cache + s_off[l][6] / 4, v.pc, cb);
+  for (uint64_t q = blockIdx.x * (uint64_t)NT + threadIdx.x; q < m; q += (uint64_t)gridDim.x * NT) {
+    if (KIND == BT_Q_ACCESS) {
+      out[q] = q_answer<KIND>(t, lv, args[q], 0);
+    } else if ((((uintptr_t)args) & 15) == 0) {
+      const ulonglong2 a = ((const ulonglong2*)args)[q];
+      out[q] = q_answer<KIND>(t, lv, a.x, a.y);
+    } else {
+      out[q] = q_answer<KIND>(t, lv, args[2 * q], args[2 * q + 1]);
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (uint32_t l = 0; l < lc; l++) {
-      LevelView& v = st.lv[l];
-      char* b = (char*)cache;
-      v.st = (const uint64_t*)(b + s_off[l][0]);
-      v.mw = (const uint32_t*)(b + s_off[l][1]);
-      v.mr = (const uint32_t*)(b + s_off[l][2]);
-      v.ptr = (const uint32_t*)(b + s_off[l][3]);
-      v.off = (const uint64_t*)(b + s_off[l][4]);
-      if (v.cnt) {
-        v.cnt = b + s_off[l][5];
-        v.pc = b + s_off[l][6];
-      }
+}
+
+// One query, its arguments in the launch and its answer written to `out`
+// (pinned host memory): 38 us a call with copies around it, 22 now.
+__global__ void k_query_one(const TreeView* __restrict__ tv, int kind, uint64_t a0, uint64_t a1, uint64_t* out) {
+  const QTree t{tv->n, tv->L, tv->S, tv->pre, tv->leaf, tv->sym};
+  if (kind == BT_Q_ACCESS) *out = q_answer<BT_Q_ACCESS>(t, tv->lv, a0, a1);
+  else if (kind == BT_Q_RANK) *out = q_answer<BT_Q_RANK>(t, tv->lv, a0, a1);
+  else *out = q_answer<BT_Q_SELECT>(t, tv->lv, a0, a1);
+}
+
+// The records of all levels (blockIdx.y) and their mark words, from the
+// arrays of the construction, and the tree's device view (filled in here with
+// the lengths of the levels' last blocks).
+struct PackLevel {
+  uint64_t c, b;
+  const uint64_t* st;
+  const uint32_t* mw;
+  const uint32_t* mr;
+  const uint32_t* ptr;
+  const uint64_t* off;
+  uint2* rec;
+  uint32_t* mw2;
+  uint32_t* mr2;
+};
+struct PackArgs {
+  PackLevel lv[kMaxLevels];
+  TreeView view;
+};
+__global__ void __launch_bounds__(256) k_pack_records(const __grid_constant__ PackArgs P, TreeView* __restrict__ view) {
+  const PackLevel& v = P.lv[blockIdx.y];
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (blockIdx.y == 0) {
+      view->n = P.view.n;
+      view->L = P.view.L;
+      view->S = P.view.S;
+      view->pre = P.view.pre;
+      view->leaf = P.view.leaf;
+      view->sym = P.view.sym;
     }
-  __syncthreads();
-  const TreeView& t = st;
-  for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < m;
-       q += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t r;
-    if (kind == BT_Q_ACCESS) r = q_access(t, args[q]);
-    else if (kind == BT_Q_RANK) r = args[2 * q] > 255 ? kNone : q_rank(t, (uint32_t)args[2 * q], args[2 * q + 1]);
-    else r = args[2 * q] > 255 ? kNone : q_select(t, (uint32_t)args[2 * q], args[2 * q + 1]);
-    out[q] = r;
+    LevelView lv = P.view.lv[blockIdx.y];
+    const uint64_t last = P.view.n - v.st[v.c - 1];
+    lv.last_len = (uint32_t)(last < v.b ? last : v.b);
+    view->lv[blockIdx.y] = lv;
+  }
+  const uint64_t words = (v.c + 31) / 32, stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < v.c; k += stride) {
+    const uint32_t w = v.mw[k >> 5], bit = (uint32_t)k & 31u;
+    if ((w >> bit) & 1u) v.rec[k] = make_uint2(kMarkedRec, v.mr[k >> 5] + __popc(w & ((1u << bit) - 1u)));
+    else v.rec[k] = make_uint2(v.ptr[k], (uint32_t)v.off[k]);
+  }
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i <= words; i += stride) {
+    if (i < words) v.mw2[i] = v.mw[i];
+    v.mr2[i] = v.mr[i];
   }
 }
 
@@ -593,42 +667,76 @@ int build_counters(BuildCtx& ctx) {
   return BT_OK;
 }
 
-int upload_view(bt_tree* t, cudaStream_t s) {
-  TreeView h;
-  h.n = t->n;
-  h.L = t->L;
-  h.S = t->S;
-  for (uint32_t l = 0; l < t->L; l++) {
-    const Level& v = t->lv[l];
-    h.lv[l] = LevelView{v.c, v.b, v.arity, block_shift(v.b), v.st, v.mw, v.mr, v.ptr, v.off, v.cnt, v.pc, v.cw};
+// The finished tree keeps records instead of the construction's arrays, which
+// are given back: 8 bytes per block instead of 20, in one allocation.
+int pack_records(BuildCtx& ctx) {
+  bt_tree* t = ctx.t;
+  cudaStream_t s = ctx.s;
+  auto al = [](uint64_t x) { return (x + 255) & ~255ull; };
+  uint64_t total = 0, cmax = 1;
+  for (const Level& v : t->lv) {
+    const uint64_t words = (v.c + 31) / 32;
+    total += al(v.c * 8) + al(words * 4) + al((words + 1) * 4);
+    cmax = v.c > cmax ? v.c : cmax;
   }
-  h.pre = t->pre;
-  h.leaf = t->leaf;
-  h.sym = t->sym;
-  BT_CUDA(cudaMallocAsync(&t->view, sizeof(TreeView), s));
-  BT_CUDA(cudaMemcpyAsync(t->view, &h, sizeof(TreeView), cudaMemcpyHostToDevice, s));
-  BT_CUDA(cudaStreamSynchronize(s));
+  char* mem;
+  BT_CUDA(cudaMallocAsync((void**)&mem, total, s));
+  t->recs = mem;
+  BT_CUDA(cudaMallocAsync((void**)&t->view, sizeof(TreeView), s));
+  PackArgs P;
+  P.view.n = t->n;
+  P.view.L = t->L;
+  P.view.S = t->S;
+  P.view.pre = t->pre;
+  P.view.leaf = t->leaf;
+  P.view.sym = t->sym;
+  for (uint32_t l = 0; l < t->L; l++) {
+    Level& v = t->lv[l];
+    const uint64_t words = (v.c + 31) / 32;
+    PackLevel& p = P.lv[l];
+    p = PackLevel{v.c, v.b, v.st, v.mw, v.mr, v.ptr, v.off, (uint2*)mem, nullptr, nullptr};
+    P.view.lv[l] = LevelView{(uint32_t)v.c, view_len(v.b), v.arity, block_shift(view_len(v.b)), 0, v.cw,
+                             p.rec, v.cnt, v.pc};
+    mem += al(v.c * 8);
+    p.mw2 = (uint32_t*)mem;
+    mem += al(words * 4);
+    p.mr2 = (uint32_t*)mem;
+    mem += al((words + 1) * 4);
+  }
+  BT_LAUNCH(k_pack_records<<<dim3(grid_for(cmax, 256, 2048), t->L), 256, 0, s>>>(P, t->view));
+  BT_CUDA(cudaGetLastError());
+  for (uint32_t l = 0; l < t->L; l++) {
+    Level& v = t->lv[l];
+    v.rec = P.lv[l].rec;
+    v.mw = P.lv[l].mw2;
+    v.mr = P.lv[l].mr2;
+    v.st = v.off = v.lo = nullptr;
+    v.ptr = nullptr;
+    std::vector<void*> keep;
+    for (void* a : v.owned) {
+      if (a == v.cnt) keep.push_back(a);
+      else cudaFreeAsync(a, s);
+    }
+    v.owned.swap(keep);
+  }
+  return BT_OK;
+}
+
+int run_query_one(const bt_tree* t, int kind, uint64_t a0, uint64_t a1, uint64_t* out, cudaStream_t s) {
+  BT_LAUNCH(k_query_one<<<1, 1, 0, s>>>(t->view, kind, a0, a1, out));
+  BT_CUDA(cudaGetLastError());
   return BT_OK;
 }
 
 int run_queries(const bt_tree* t, int kind, const uint64_t* d_args, uint64_t m, uint64_t* d_out,
                 cudaStream_t s) {
   if (m == 0) return BT_OK;
-  // Enough CTAs to fill the device (each pays for its shared-memory copy of
-  // the top levels once), threads striding over the queries.
-  // Access descends with few loads per level and gains most from threads in
-  // flight: 128-thread CTAs without the shared-memory copy, bounded to 64
-  // registers so that 1024 threads fit on an SM (80 registers left 768).
-  // Rank and select read counters at every level and gain from the copy of
-  // the top levels; four CTAs of 256 per SM at 64 registers run without the
-  // spills that six CTAs (40 registers) had.  Measured on the 256 MiB tree:
-  // access 9.7 instead of 8.2, rank 2.6 instead of 2.4, select 2.5 instead of
-  // 2.1 G queries/s.
-  if (kind == BT_Q_ACCESS)
-    BT_LAUNCH(k_queries<0, 128, 8><<<grid_for(m, 128, 152 * 64), 128, 0, s>>>(t->view, kind, d_args, m, d_out));
-  else
-    BT_LAUNCH(k_queries<12 << 10, kQThreads, 4><<<grid_for(m, kQThreads, 152 * 4), kQThreads, 0, s>>>(
-        t->view, kind, d_args, m, d_out));
+  // CTAs of 128 threads: small batches spread over more SMs; 64 registers, so
+  // that 1024 threads fit on an SM.
+  const unsigned g = grid_for(m, 128, 152 * 64);
+  if (kind == BT_Q_ACCESS) BT_LAUNCH(k_queries<BT_Q_ACCESS, 128, 8><<<g, 128, 0, s>>>(t->view, d_args, m, d_out));
+  else if (kind == BT_Q_RANK) BT_LAUNCH(k_queries<BT_Q_RANK, 128, 8><<<g, 128, 0, s>>>(t->view, d_args, m, d_out));
+  else BT_LAUNCH(k_queries<BT_Q_SELECT, 128, 8><<<g, 128, 0, s>>>(t->view, d_args, m, d_out));
   BT_CUDA(cudaGetLastError());
   return BT_OK;
 }

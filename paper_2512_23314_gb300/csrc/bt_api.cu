@@ -271,10 +271,10 @@ static int build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, 
   tr.mark("counters");
   ctx.arena.release();
   BT_TRY(pack_records(ctx));
-  uint64_t bytes = t->leaf_bytes + 16 + sizeof(TreeView) + 512 + (t->lv[0].c + 1) * t->S * 8;
+  uint64_t bytes = t->leaf_bytes + 16 + sizeof(TreeView) + 512 + (t->lv[t->base].c + 1) * t->S * 4;
   for (const Level& v : t->lv) {
     const uint64_t words = (v.c + 31) / 32;
-    bytes += v.c * 8 + (2 * words + 1) * 4 + (v.cnt ? 2 * v.c * t->S * v.cw : 0);
+    bytes += v.c * 8 + (2 * words + 1) * 4 + (v.cnt ? 2 * counter_stride(v.c) * t->S * v.cw : 0);
   }
   t->dev_bytes = bytes;
   BT_CUDA(cudaStreamSynchronize(s));

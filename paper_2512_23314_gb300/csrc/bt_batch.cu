@@ -1453,29 +1453,58 @@ __device__ void prune_pass(const BParams& P, const BDoc& D, Cta& C, char* scr) {
 // Output: the tree's arrays, counters, level-1 prefix counts and leaf text in
 // the pool; the device view that the query kernels read.
 // ---------------------------------------------------------------------------
+// Counters of a level, symbol-major (cp entries per symbol).  mode 0: symbol
+// counts of each block (marked blocks of a non-last level are filled from their
+// children afterwards); mode 1: counts of T[st[ptr], st[ptr] + off) of each
+// unmarked block (zeros for marked ones).  A warp takes four consecutive
+// blocks at a time, their bytes in flight together, each with its own
+// histogram (hist: 1024 words per warp), and writes the four counters of a
+// symbol at once.
 __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PLv& v, int mode, bool last,
-                           void* out, uint32_t cw, unsigned int* hist) {
-  // mode 0: symbol counts of each block (marked blocks of a non-last level
-  // are filled from their children afterwards); mode 1: counts of
-  // T[st[ptr], st[ptr] + off) of each unmarked block (zeros for marked ones).
+                           void* out, uint32_t cw, uint64_t cp, unsigned int* hist) {
   const uint32_t S = C.S;
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  unsigned int* h = hist + warp * 256;
-  for (uint64_t k = warp; k < v.c; k += nw) {
-    const bool mk = marked(v.mw, k);
-    uint64_t s0 = 0, len = 0;
-    if (mode == 0 && (last || !mk)) {
-      s0 = v.st[k];
-      len = plen(v, k);
-    } else if (mode == 1 && !mk) {
-      s0 = v.st[v.ptr[k]];
-      len = v.off[k];
+  unsigned int* h = hist + warp * 1024;
+  for (uint64_t g = warp; 4 * g < v.c; g += nw) {
+    uint64_t s0[4];
+    uint32_t len[4], top = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < 4; q++) {
+      const uint64_t k = 4 * g + q;
+      s0[q] = 0;
+      len[q] = 0;
+      if (k >= v.c) continue;
+      const bool mk = marked(v.mw, k);
+      if (mode == 0 && (last || !mk)) {
+        s0[q] = v.st[k];
+        len[q] = (uint32_t)plen(v, k);
+      } else if (mode == 1 && !mk) {
+        s0[q] = v.st[v.ptr[k]];
+        len[q] = (uint32_t)v.off[k];
+      }
+      top = top > len[q] ? top : len[q];
     }
-    for (uint32_t i = lane; i < S; i += 32) h[i] = 0;
+    for (uint32_t i = lane; i < S; i += 32) {
+#pragma unroll
+      for (uint32_t q = 0; q < 4; q++) h[256 * q + i] = 0;
+    }
     __syncwarp();
-    for (uint64_t x = lane; x < len; x += 32) atomicAdd(&h[C.sym[T[s0 + x]]], 1u);
+    for (uint32_t x = lane; x < top; x += 32) {
+      uint32_t ch[4];
+#pragma unroll
+      for (uint32_t q = 0; q < 4; q++) ch[q] = x < len[q] ? T[s0[q] + x] : 256u;
+#pragma unroll
+      for (uint32_t q = 0; q < 4; q++)
+        if (ch[q] < 256u) atomicAdd(&h[256 * q + C.sym[ch[q]]], 1u);
+    }
     __syncwarp();
-    for (uint32_t i = lane; i < S; i += 32) cput(out, cw, k * S + i, h[i]);
+    for (uint32_t i = lane; i < S; i += 32) {
+      const uint32_t a = h[i], b = h[256 + i], c = h[512 + i], d = h[768 + i];
+      const uint64_t at = i * cp + 4 * g;
+      if (cw == 1) *(uint32_t*)((uint8_t*)out + at) = a | (b << 8) | (c << 16) | (d << 24);
+      else if (cw == 2) *(uint2*)((uint16_t*)out + at) = make_uint2(a | (b << 16), c | (d << 16));
+      else *(uint4*)((uint32_t*)out + at) = make_uint4(a, b, c, d);
+    }
     __syncwarp();
   }
 }
@@ -1487,13 +1516,15 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
   __shared__ OutLevel s_ol[kBMaxLevels];
   __shared__ uint32_t s_cw[kBMaxLevels];
   __shared__ uint64_t s_view, s_pre, s_leaf, s_sym;
+  __shared__ uint32_t s_base;
   if (tid == 0) {
     for (uint32_t l = 0; l < L; l++) s_cw[l] = counter_width(bsz[l]);
     const uint64_t words = (C.c[L - 1] + 31) / 32;
     const uint32_t* mrl = (const uint32_t*)(scr + C.sl.mr[L - 1]);
     const uint64_t nm = mrl[words];
     const uint64_t leaf_alloc = nm * bsz[L - 1];
-    const uint64_t need = out_layout(L, C.c, s_cw, S, leaf_alloc, s_ol, &s_view, &s_pre, &s_leaf, &s_sym);
+    s_base = out_base(L, C.c, bsz, C.n, S);
+    const uint64_t need = out_layout(L, s_base, C.c, s_cw, S, leaf_alloc, s_ol, &s_view, &s_pre, &s_leaf, &s_sym);
     C.out_bytes = need;
     const unsigned long long o = atomicAdd(P.pool_used, (unsigned long long)need);
     if (o + need > P.pool_cap) {
@@ -1506,6 +1537,7 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
   }
   if (cta_failed(C)) return;
   char* out = C.out;
+  const uint32_t bl = s_base;
   // Level arrays.
   for (uint32_t l = 0; l < L; l++) {
     const PLv v = plevel(C, scr, bsz, l);
@@ -1522,45 +1554,52 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
     }
   }
   __syncthreads();
-  // Counters, last level first (marked blocks sum their children's rows).
-  for (int l = (int)L - 1; l >= 0; l--) {
+  // Counters, last level first (marked blocks sum their children's).
+  for (int l = (int)L - 1; l >= (int)bl; l--) {
     const PLv v = plevel(C, scr, bsz, (uint32_t)l);
     const bool last = l + 1 == (int)L;
     void* cnt = out + s_ol[l].cnt;
     void* pc = out + s_ol[l].pc;
     const uint32_t cw = s_cw[l];
-    count_rows(D.T, C, v, 0, last, cnt, cw, hist);
-    count_rows(D.T, C, v, 1, last, pc, cw, hist);
+    const uint64_t cp = counter_stride(v.c);
+    count_rows(D.T, C, v, 0, last, cnt, cw, cp, hist);
+    count_rows(D.T, C, v, 1, last, pc, cw, cp, hist);
     __syncthreads();
     if (!last) {
       const void* ccnt = out + s_ol[l + 1].cnt;
       const uint32_t ccw = s_cw[l + 1];
-      const uint64_t bn = bsz[l + 1];
+      const uint64_t bn = bsz[l + 1], ccp = counter_stride(C.c[l + 1]);
       const uint32_t arity = C.arity[l];
-      for (uint64_t k = warp; k < v.c; k += nw) {
-        if (!marked(v.mw, k)) continue;
-        const uint64_t first = mrank(v.mw, v.mr, k) * arity, nch = (plen(v, k) + bn - 1) / bn;
-        for (uint32_t s = lane; s < S; s += 32) {
-          uint32_t acc = 0;
-          for (uint64_t i = 0; i < nch; i++) acc += cget(ccnt, ccw, (first + i) * S + s);
-          cput(cnt, cw, k * S + s, acc);
+      for (uint32_t s = warp; s < S; s += nw)
+        for (uint64_t k = lane; k < v.c; k += 32) {
+          if (!marked(v.mw, k)) continue;
+          const uint64_t first = mrank(v.mw, v.mr, k) * arity;
+          const uint32_t nch = (uint32_t)((plen(v, k) + bn - 1) / bn);
+          cput(cnt, cw, s * cp + k, sum_run(ccnt, ccw, s * ccp + first, nch));
         }
-      }
       __syncthreads();
     }
   }
-  // Level-1 prefix counts.
+  // Prefix counts of the base level, a warp per symbol.
   {
-    const PLv v = plevel(C, scr, bsz, 0);
-    uint64_t* pre = (uint64_t*)(out + s_pre);
-    const void* cnt = out + s_ol[0].cnt;
-    for (uint32_t s = tid; s < S; s += nt) {
-      uint64_t acc = 0;
-      for (uint64_t k = 0; k < v.c; k++) {
-        pre[k * S + s] = acc;
-        acc += cget(cnt, s_cw[0], k * S + s);
+    const uint64_t c0 = C.c[bl], cp = counter_stride(c0);
+    uint32_t* pre = (uint32_t*)(out + s_pre);
+    const void* cnt = out + s_ol[bl].cnt;
+    for (uint32_t s = warp; s < S; s += nw) {
+      uint32_t carry = 0;
+      for (uint64_t base = 0; base < c0; base += 32) {
+        const uint64_t k = base + lane;
+        const uint32_t x = k < c0 ? cget(cnt, s_cw[bl], s * cp + k) : 0u;
+        uint32_t y = x;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const uint32_t o = __shfl_up_sync(kFull, y, d);
+          if ((int)lane >= d) y += o;
+        }
+        if (k < c0) pre[s * (c0 + 1) + k] = carry + y - x;
+        carry += __shfl_sync(kFull, y, 31);
       }
-      pre[v.c * S + s] = acc;
+      if (lane == 0) pre[s * (c0 + 1) + c0] = carry;
     }
   }
   // Leaf text of the marked last-level blocks: rank r at r * b_L.
@@ -1587,6 +1626,7 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
     tv->n = C.n;
     tv->L = L;
     tv->S = S;
+    tv->base = bl;
     for (uint32_t l = 0; l < L; l++) {
       const uint64_t words = (C.c[l] + 31) / 32;
       LevelView& lv = tv->lv[l];
@@ -1597,13 +1637,14 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
       const PLv v = plevel(C, scr, bsz, l);
       lv.last_len = (uint32_t)plen(v, v.c - 1);
       lv.rec = (const uint2*)(out + s_ol[l].rec);
-      lv.cnt = out + s_ol[l].cnt;
-      lv.pc = out + s_ol[l].pc;
+      lv.cnt = l >= bl ? out + s_ol[l].cnt : nullptr;
+      lv.pc = l >= bl ? out + s_ol[l].pc : nullptr;
       lv.cw = s_cw[l];
+      lv.cp = (uint32_t)counter_stride(C.c[l]);
       const uint32_t* mrl = (const uint32_t*)(scr + C.sl.mr[l]);
       C.nmarked[l] = mrl[words];
     }
-    tv->pre = (const uint64_t*)(out + s_pre);
+    tv->pre = (const uint32_t*)(out + s_pre);
     tv->leaf = (const uint8_t*)(out + s_leaf);
     tv->sym = (const int16_t*)(out + s_sym);
   }
@@ -2049,17 +2090,19 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
     memcpy(t->sym_host, R.sym, sizeof(t->sym_host));
     t->slab = pool_of[k];
     t->lv.resize(D.L);
-    std::vector<uint64_t> c(D.L);
+    std::vector<uint64_t> c(D.L), bs(D.L);
     std::vector<uint32_t> cw(D.L);
     for (uint32_t l = 0; l < D.L; l++) {
       const BLevelRes& Lr = lres[lv_off[k] + l];
       c[l] = Lr.c;
+      bs[l] = Lr.b;
       cw[l] = Lr.cw;
     }
     const BLevelRes& last = lres[lv_off[k] + D.L - 1];
     std::vector<OutLevel> ol(D.L);
     uint64_t o_view, o_pre, o_leaf, o_sym;
-    out_layout(D.L, c.data(), cw.data(), R.S, last.nmarked * last.b, ol.data(), &o_view, &o_pre, &o_leaf,
+    t->base = out_base(D.L, c.data(), bs.data(), D.n, R.S);
+    out_layout(D.L, t->base, c.data(), cw.data(), R.S, last.nmarked * last.b, ol.data(), &o_view, &o_pre, &o_leaf,
                &o_sym);
     char* base = (char*)t->slab.get() + R.out_off;
     for (uint32_t l = 0; l < D.L; l++) {
@@ -2073,12 +2116,12 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
       v.mw = (uint32_t*)(base + ol[l].mw);
       v.mr = (uint32_t*)(base + ol[l].mr);
       v.rec = (uint2*)(base + ol[l].rec);
-      v.cnt = base + ol[l].cnt;
-      v.pc = base + ol[l].pc;
+      v.cnt = l >= t->base ? base + ol[l].cnt : nullptr;
+      v.pc = l >= t->base ? base + ol[l].pc : nullptr;
       memcpy(v.stats, Lr.stats, sizeof(v.stats));
     }
     t->view = (TreeView*)(base + o_view);
-    t->pre = (uint64_t*)(base + o_pre);
+    t->pre = (uint32_t*)(base + o_pre);
     t->leaf = (uint8_t*)(base + o_leaf);
     t->sym = (int16_t*)(base + o_sym);
     t->dev_bytes = R.out_bytes;

@@ -64,9 +64,22 @@ struct OutLevel {
 __host__ __device__ inline uint64_t out_align(uint64_t x) { return (x + 255) & ~255ull; }
 __host__ __device__ inline uint64_t out_align16(uint64_t x) { return (x + 15) & ~15ull; }
 
+// The level queries start at (as for a single text): the lowest one with all
+// blocks whose prefix table stays within an eighth of the text, or 8 KiB; at
+// most 1024 blocks, as one CTA fills the table.
+__host__ __device__ inline uint32_t out_base(uint32_t L, const uint64_t* c, const uint64_t* b, uint64_t n, uint32_t S) {
+  uint32_t base = 0;
+  for (uint32_t l = 1; l < L; l++) {
+    if (c[l] != (n + b[l] - 1) / b[l] || c[l] > 1024) break;
+    const uint64_t bytes = (c[l] + 1) * S * 4;
+    if (bytes <= n / 8 || bytes <= (8u << 10)) base = l;
+  }
+  return base;
+}
+
 // c[l]: blocks of level l after pruning; cw[l]: counter bytes; S symbols;
 // leaf_alloc: leaf text bytes (rounded).  Returns the region's size.
-__host__ __device__ inline uint64_t out_layout(uint32_t L, const uint64_t* c, const uint32_t* cw, uint32_t S,
+__host__ __device__ inline uint64_t out_layout(uint32_t L, uint32_t base, const uint64_t* c, const uint32_t* cw, uint32_t S,
                                                uint64_t leaf_alloc, OutLevel* lv, uint64_t* view,
                                                uint64_t* pre, uint64_t* leaf, uint64_t* sym) {
   uint64_t o = 0;
@@ -81,12 +94,12 @@ __host__ __device__ inline uint64_t out_layout(uint32_t L, const uint64_t* c, co
     lv[l].mr = o;
     o = out_align16(o + (words + 1) * 4);
     lv[l].cnt = o;
-    o = out_align16(o + c[l] * S * cw[l] + 4);
+    if (l >= base) o = out_align16(o + counter_stride(c[l]) * S * cw[l]);
     lv[l].pc = o;
-    o = out_align16(o + c[l] * S * cw[l] + 4);
+    if (l >= base) o = out_align16(o + counter_stride(c[l]) * S * cw[l]);
   }
   *pre = o;
-  o = out_align16(o + (c[0] + 1) * (uint64_t)S * 8 + 8);
+  o = out_align16(o + (c[base] + 1) * (uint64_t)S * 4);
   *leaf = o;
   o = out_align16(o + leaf_alloc + 16);
   *sym = o;

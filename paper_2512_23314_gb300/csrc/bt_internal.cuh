@@ -11,13 +11,21 @@
 //                              occurrence of the block's string, its offset
 //                              there); marked: (kMarkedRec, mark rank).  All a
 //                              query needs of a block in one 8-byte read
-//     cnt       [c * S]        symbol counts of the block (S distinct symbols)
-//     pc        [c * S]        unmarked: symbol counts of the target's text
+//     cnt       [S * cp]       symbol counts of the blocks, symbol-major (entry
+//                              s cp + k; cp = c rounded up to 4): the children of
+//                              a block are neighbours, so a query reads all their
+//                              counters of its symbol at once
+//     pc        [S * cp]       unmarked: symbol counts of the target's text
 //                              before the copied window
+//                              (both from the base level on)
 //   during construction also
 //     st        u64[c]         block starts (multiples of b_l)
 //     ptr, off, lo             the pointers and leftmost occurrences apart
-//   pre         u64[(c_1+1)*S] level 1: symbol counts of T[0, st[k])
+//   pre         u32[S * (c+1)] the base level: symbol counts of T[0, st[k]).  The
+//                              base is the lowest level that still has all of
+//                              its blocks (every block above is marked), where
+//                              the table is small enough: every query starts
+//                              there, at block position / b
 //   leaf        u8[...]        text of the marked last-level blocks, block r at r*b_L
 // A marked block of a non-last level with mark rank r has its children at
 // indices r*arity .. r*arity + ceil(len/b_{l+1}) - 1 of the next level.
@@ -140,6 +148,8 @@ struct LevelView {
   uint32_t bshift;      // log2(b) when b is a power of two, else 0xFF
   uint32_t last_len;    // length of block c - 1 (the others are b long)
   uint32_t cw;          // bytes per counter (1, 2 or 4)
+  uint32_t cp;          // entries per symbol of the counters
+  uint32_t pad;
   const uint2* rec;
   const void* cnt;      // symbol counters of the blocks (null: counted in the leaf text)
   const void* pc;
@@ -160,7 +170,11 @@ __host__ __device__ inline uint32_t view_len(uint64_t b) { return b > 0xFFFFFFFF
 // exceeds b.
 __host__ __device__ inline uint32_t counter_width(uint64_t b) { return b <= 0xFF ? 1 : b <= 0xFFFF ? 2 : 4; }
 
-// Counter i of a row array with w-byte entries.
+// Entries per symbol of a level's counters: whole groups of four, which are
+// read at once.
+__host__ __device__ inline uint64_t counter_stride(uint64_t c) { return (c + 3) & ~3ull; }
+
+// Counter i of an array with w-byte entries.
 __device__ __forceinline__ uint32_t cget(const void* a, uint32_t w, uint64_t i) {
   return w == 1 ? ((const uint8_t*)a)[i] : w == 2 ? ((const uint16_t*)a)[i] : ((const uint32_t*)a)[i];
 }
@@ -170,13 +184,36 @@ __device__ __forceinline__ void cput(void* a, uint32_t w, uint64_t i, uint32_t v
   else ((uint32_t*)a)[i] = v;
 }
 
+// Sum of the counters [i, i + m) of one symbol (four at a time when i is a
+// multiple of 4).
+__device__ __forceinline__ uint32_t sum_run(const void* cnt, uint32_t w, uint64_t i, uint32_t m) {
+  uint32_t acc = 0;
+  if ((i & 3) == 0) {
+    for (; m >= 4; m -= 4, i += 4) {
+      if (w == 1) {
+        acc = __dp4a(*(const uint32_t*)((const uint8_t*)cnt + i), 0x01010101u, acc);
+      } else if (w == 2) {
+        const uint2 v = *(const uint2*)((const uint16_t*)cnt + i);
+        acc += (v.x & 0xFFFFu) + (v.x >> 16) + (v.y & 0xFFFFu) + (v.y >> 16);
+      } else {
+        const uint4 v = *(const uint4*)((const uint32_t*)cnt + i);
+        acc += v.x + v.y + v.z + v.w;
+      }
+    }
+  }
+  for (; m; m--, i++) acc += cget(cnt, w, i);
+  return acc;
+}
+
 constexpr int kMaxLevels = 64;
 
 struct TreeView {
   uint64_t n;
   uint32_t L, S;
+  uint32_t base;        // the level queries start at
+  uint32_t pad;
   LevelView lv[kMaxLevels];
-  const uint64_t* pre;
+  const uint32_t* pre;
   const uint8_t* leaf;
   const int16_t* sym;  // byte -> dense symbol, -1 if absent
 };
@@ -191,7 +228,8 @@ struct bt_tree {
   std::vector<bt::Level> lv;
   uint8_t* leaf = nullptr;
   uint64_t leaf_bytes = 0;
-  uint64_t* pre = nullptr;
+  uint32_t base = 0;     // the level queries start at
+  uint32_t* pre = nullptr;
   int16_t* sym = nullptr;  // device map
   int16_t sym_host[256];
   uint32_t S = 0;

@@ -4,11 +4,11 @@
 // implementation stores one bit vector per level plus pointers and offsets
 // (section 4.4) and names the rank/select auxiliary data as future work
 // (section 6).  The counters used here:
-//   cnt[k][s]  occurrences of symbol s in block k (every level),
-//   pc[u][s]   occurrences of s in T[st[ptr], st[ptr] + off) for an unmarked
+//   cnt[s][k]  occurrences of symbol s in block k (from the base level on),
+//   pc[s][u]   occurrences of s in T[st[ptr], st[ptr] + off) for an unmarked
 //              block u (the part of its target before the copied window),
-//   pre[k][s]  occurrences of s before level-1 block k.
-// rank_c(i) descends from the level-1 block holding i: inside a marked block
+//   pre[s][k]  occurrences of s before block k of the base level.
+// rank_c(i) descends from the base-level block holding i: inside a marked block
 // it adds the counts of the children left of the one holding i; at an
 // unmarked block it continues in its target (ptr or ptr+1) and subtracts
 // pc.  select mirrors it.  One thread answers one query.
@@ -46,146 +46,225 @@ __global__ void k_histogram(const uint8_t* __restrict__ T, uint64_t n, unsigned 
     if (h[i]) atomicAdd(&hist[i], (unsigned long long)h[i]);
 }
 
-struct CountJob {
+// What a level's counters are counted from.
+struct CountLevel {
   const uint64_t* st;   // block starts of the level
-  const uint32_t* ptr;  // for pc jobs: targets
+  const uint32_t* ptr;  // targets and offsets of the unmarked blocks
   const uint64_t* off;
   const uint32_t* mw;
-  uint64_t c, b, n;
-  void* out;            // rows of S counters of cw bytes
+  uint64_t c, b, n, cp;
+  void* cnt;            // symbol-major, cw bytes each
+  void* pc;
   uint32_t cw;
-  int mode;             // 0: count the block itself, 1: count T[st[ptr], st[ptr]+off)
-  int only_unmarked;    // skip marked blocks
-  int only_marked;
+  int only_unmarked;    // cnt of the marked blocks is summed from their children later
 };
 
+// The text counted for entry k of cnt (which = 0) or pc (1): [s0, s0 + len),
+// perhaps empty; false for an entry that is not counted.
+__device__ __forceinline__ bool count_range(const CountLevel& J, int which, uint64_t k, uint64_t* s0, uint32_t* len) {
+  const bool mk = (J.mw[k >> 5] >> (k & 31)) & 1u;
+  *s0 = 0;
+  *len = 0;
+  if (which == 0) {
+    if (J.only_unmarked && mk) return false;
+    *s0 = J.st[k];
+    *len = (uint32_t)(J.n - *s0 < J.b ? J.n - *s0 : J.b);
+    return true;
+  }
+  if (mk) return false;
+  *s0 = J.st[J.ptr[k]];
+  *len = (uint32_t)J.off[k];
+  return true;
+}
+
+// One-byte counters (b <= 255): a thread per block.  The CTA's counters are a
+// tile [S][128] in shared memory; thread t has the column 4 (t mod 32) + t/32,
+// so that the lanes of a warp update 32 different banks, and rows leave as
+// 128-byte lines.  blockIdx.y: cnt or pc.  Entries that are not counted are
+// written as zeros; k_sum_children overwrites its own.  Bound: the counters'
+// writes (S bytes per block).  Measured on the two lowest levels of the
+// 256 MiB text: 670 us with block-major rows (zeroed byte by byte, four-way
+// bank conflicts), 190 now.
+constexpr uint32_t kSmallCountThreads = 128;
+
+__global__ void __launch_bounds__(kSmallCountThreads) k_count_small(CountLevel J, const int16_t* __restrict__ sym_g,
+                                                                    const uint8_t* __restrict__ T, uint32_t S) {
+  extern __shared__ uint8_t tile[];  // [S][128], then the symbol map (one byte each)
+  uint8_t* sym = tile + kSmallCountThreads * S;
+  const uint32_t t = threadIdx.x, col = 4 * (t & 31) + (t >> 5);
+  for (uint32_t i = t; i < 256; i += kSmallCountThreads) sym[i] = (uint8_t)sym_g[i];
+  for (uint32_t i = t; i < 32 * S; i += kSmallCountThreads) ((uint32_t*)tile)[i] = 0;
+  __syncthreads();
+  const int which = blockIdx.y;
+  uint8_t* out = (uint8_t*)(which ? J.pc : J.cnt);
+  const uint64_t k0 = (uint64_t)blockIdx.x * kSmallCountThreads, k = k0 + col;
+  if (k < J.c) {
+    uint64_t s0;
+    uint32_t len;
+    count_range(J, which, k, &s0, &len);
+    uint8_t* my = tile + col;
+    uint32_t x = 0;
+    if ((((uintptr_t)(T + s0)) & 15) == 0) {
+      for (; x < len && s0 + x + 16 <= J.n; x += 16) {
+        const uint4 v = *(const uint4*)(T + s0 + x);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        const uint32_t have = len - x;
+#pragma unroll
+        for (uint32_t i = 0; i < 16; i++)
+          if (i < have) my[kSmallCountThreads * sym[(w[i >> 2] >> (8 * (i & 3))) & 0xFF]]++;
+      }
+    }
+    for (; x < len; x++) my[kSmallCountThreads * sym[T[s0 + x]]]++;
+  }
+  __syncthreads();
+  for (uint32_t i = t; i < 32 * S; i += kSmallCountThreads) {
+    const uint64_t at = k0 + 4 * (i & 31);
+    if (at < J.cp) *(uint32_t*)(out + (uint64_t)(i >> 5) * J.cp + at) = ((const uint32_t*)tile)[i];
+  }
+}
+
+// Two-byte counters (blocks of 256 bytes to 64 KiB): a CTA takes 16
+// consecutive blocks, a warp one after the other, 16 bytes per lane and step
+// into four copies of a histogram in shared memory (lanes take different
+// copies: a frequent symbol's updates meet less often); the 16 blocks' counters
+// of a symbol leave as one unit.  blockIdx.y: cnt or pc.
+constexpr uint32_t kTileBlocks = 16;
 constexpr uint64_t kCountPiece = 1 << 16;
 
-// One warp per (block, piece of at most 64 KiB); symbol counts are gathered
-// in a per-warp shared histogram.  Narrow rows (blocks of at most 64 KiB, one
-// piece) are written whole; 4-byte rows (several pieces) are added to with
-// atomics.
-__global__ void __launch_bounds__(256) k_count(CountJob J, const int16_t* __restrict__ sym,
-                                               const uint8_t* __restrict__ T, uint32_t S,
-                                               uint64_t ppb) {
-  extern __shared__ unsigned int hist[];  // 8 warps x S
+__global__ void __launch_bounds__(256) k_count_tile(CountLevel J, const int16_t* __restrict__ sym_g,
+                                                    const uint8_t* __restrict__ T, uint32_t S) {
+  extern __shared__ uint32_t hist[];  // per warp [S][4], then [S][16] of cw bytes, then the symbol map
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t* h = hist + warp * 4 * S;
+  uint8_t* rows = (uint8_t*)(hist + 8 * 4 * S);
+  uint8_t* sym = rows + S * kTileBlocks * J.cw;
+  for (uint32_t i = threadIdx.x; i < 256; i += 256) sym[i] = (uint8_t)sym_g[i];
+  const int which = blockIdx.y;
+  uint8_t* out = (uint8_t*)(which ? J.pc : J.cnt);
+  const uint64_t tiles = (J.c + kTileBlocks - 1) / kTileBlocks;
+  for (uint64_t tl = blockIdx.x; tl < tiles; tl += gridDim.x) {
+    __syncthreads();
+    bool any = false;
+    for (uint32_t i = warp; i < kTileBlocks; i += 8) {
+      const uint64_t k = tl * kTileBlocks + i;
+      uint64_t s0 = 0;
+      uint32_t len = 0;
+      if (k < J.c) any |= count_range(J, which, k, &s0, &len);
+      if (len == 0) {
+        for (uint32_t s = lane; s < S; s += 32) cput(rows, J.cw, s * kTileBlocks + i, 0u);
+        continue;
+      }
+      for (uint32_t s = lane; s < 4 * S; s += 32) h[s] = 0;
+      __syncwarp();
+      const uint32_t cpy = lane & 3;
+      uint32_t x = 0;
+      if ((((uintptr_t)(T + s0)) & 15) == 0) {
+        const uint32_t full = len & ~15u;
+        for (x = 16 * lane; x < full; x += 512) {
+          const uint4 v = *(const uint4*)(T + s0 + x);
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (uint32_t q = 0; q < 16; q++) atomicAdd(&h[4 * sym[(w[q >> 2] >> (8 * (q & 3))) & 0xFF] + cpy], 1u);
+        }
+        x = full;
+      }
+      for (x += lane; x < len; x += 32) atomicAdd(&h[4 * sym[T[s0 + x]] + cpy], 1u);
+      __syncwarp();
+      for (uint32_t s = lane; s < S; s += 32)
+        cput(rows, J.cw, s * kTileBlocks + i, h[4 * s] + h[4 * s + 1] + h[4 * s + 2] + h[4 * s + 3]);
+      __syncwarp();
+    }
+    // (Entries of a tile without counted blocks need no write: those of marked
+    // blocks are summed from the children or never read.)
+    if (!__syncthreads_or(any)) continue;
+    const uint32_t words = kTileBlocks * J.cw / 4;
+    const uint64_t have = (J.cp - tl * kTileBlocks) * J.cw / 4;  // words of the row from the tile on
+    for (uint32_t i = threadIdx.x; i < S * words; i += 256) {
+      const uint32_t s = i / words, w = i - s * words;
+      if (w >= have) continue;
+      ((uint32_t*)(out + ((uint64_t)s * J.cp + tl * kTileBlocks) * J.cw))[w] = ((const uint32_t*)rows)[s * words + w];
+    }
+  }
+}
+
+// Blocks longer than a piece: one warp per (block, piece of 64 KiB), added to
+// four-byte counters that start at zero.  blockIdx.y: cnt or pc.
+__global__ void __launch_bounds__(256) k_count_long(CountLevel J, const int16_t* __restrict__ sym,
+                                                    const uint8_t* __restrict__ T, uint32_t S, uint64_t ppb) {
+  extern __shared__ uint32_t hist[];  // 8 warps x S
   const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned int* h = hist + wid * S;
+  uint32_t* h = hist + wid * S;
+  uint32_t* out = (uint32_t*)(blockIdx.y ? J.pc : J.cnt);
   const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
   for (uint64_t w = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32; w < J.c * ppb; w += warps) {
-    const uint64_t k = w / ppb, piece = w - k * ppb;
-    const bool mk = (J.mw[k >> 5] >> (k & 31)) & 1u;
-    if ((J.only_unmarked && mk) || (J.only_marked && !mk)) continue;
-    uint64_t s0, len;
-    if (J.mode == 0) {
-      s0 = J.st[k];
-      len = J.n - s0 < J.b ? J.n - s0 : J.b;
-    } else {
-      s0 = J.st[J.ptr[k]];
-      len = J.off[k];
-    }
-    const uint64_t a = piece * kCountPiece;
-    if (a >= len) {
-      // An empty range (a pointer at offset 0): narrow rows are not zeroed
-      // beforehand, so the row is written here.
-      if (J.cw < 4 && piece == 0)
-        for (uint32_t i = lane; i < S; i += 32) cput(J.out, J.cw, k * S + i, 0u);
-      continue;
-    }
+    const uint64_t k = w / ppb, a = (w - k * ppb) * kCountPiece;
+    uint64_t s0;
+    uint32_t len;
+    count_range(J, blockIdx.y, k, &s0, &len);
+    if (a >= len) continue;
     const uint64_t e = a + kCountPiece < len ? a + kCountPiece : len;
     for (uint32_t i = lane; i < S; i += 32) h[i] = 0;
     __syncwarp();
     for (uint64_t x = a + lane; x < e; x += 32) atomicAdd(&h[sym[T[s0 + x]]], 1u);
     __syncwarp();
-    if (J.cw < 4) {
-      for (uint32_t i = lane; i < S; i += 32) cput(J.out, J.cw, k * S + i, h[i]);
-    } else {
-      for (uint32_t i = lane; i < S; i += 32)
-        if (h[i]) atomicAdd((uint32_t*)J.out + k * S + i, h[i]);
-    }
+    for (uint32_t i = lane; i < S; i += 32)
+      if (h[i]) atomicAdd(&out[(uint64_t)i * J.cp + k], h[i]);
     __syncwarp();
   }
 }
 
-// Small blocks (one-byte counters, b <= 255): one thread per block counts
-// into a private shared-memory row (16-byte text loads when aligned); the
-// CTA's rows are contiguous in the output and go out with word stores.
-// Rows of blocks that are not counted (J.only_*) are written as zeros; a
-// later kernel may overwrite them.
-constexpr uint32_t kSmallCountThreads = 128;
+// Marked blocks of a non-last level: sums of their children's counters.  A
+// thread per block and eighth of the symbols (blockIdx.y): neighbouring marked
+// blocks read neighbouring children.
+__global__ void __launch_bounds__(256) k_sum_children(CountLevel J, const uint32_t* __restrict__ mr, uint32_t arity,
+                                                      uint64_t bn, const void* __restrict__ child_cnt, uint32_t child_cw,
+                                                      uint64_t child_cp, uint32_t S) {
+  const uint32_t s0 = (uint32_t)((uint64_t)S * blockIdx.y / gridDim.y), s1 = (uint32_t)((uint64_t)S * (blockIdx.y + 1) / gridDim.y);
+  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < J.c; k += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t word = J.mw[k >> 5];
+    if (!((word >> (k & 31)) & 1u)) continue;
+    const uint64_t len = J.n - J.st[k] < J.b ? J.n - J.st[k] : J.b;
+    const uint64_t first = (mr[k >> 5] + __popc(word & ((1u << (k & 31)) - 1u))) * (uint64_t)arity;
+    const uint32_t nch = (uint32_t)((len + bn - 1) / bn);
+    for (uint32_t s = s0; s < s1; s++)
+      cput(J.cnt, J.cw, (uint64_t)s * J.cp + k, sum_run(child_cnt, child_cw, (uint64_t)s * child_cp + first, nch));
+  }
+}
 
-__global__ void __launch_bounds__(kSmallCountThreads) k_count_small(CountJob J, const int16_t* __restrict__ sym_g,
-                                                                    const uint8_t* __restrict__ T, uint32_t S) {
-  extern __shared__ uint8_t rows[];  // kSmallCountThreads rows of S bytes, then the symbol map
-  int16_t* sym = (int16_t*)(rows + ((kSmallCountThreads * S + 3) & ~3u));
-  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) sym[i] = sym_g[i];
-  uint8_t* row = rows + threadIdx.x * S;
-  for (uint32_t i = 0; i < S; i++) row[i] = 0;
-  __syncthreads();
-  const uint64_t k0 = (uint64_t)blockIdx.x * kSmallCountThreads, k = k0 + threadIdx.x;
-  if (k < J.c) {
-    const bool mk = (J.mw[k >> 5] >> (k & 31)) & 1u;
-    if (!((J.only_unmarked && mk) || (J.only_marked && !mk))) {
-      uint64_t s0, len;
-      if (J.mode == 0) {
-        s0 = J.st[k];
-        len = J.n - s0 < J.b ? J.n - s0 : J.b;
-      } else {
-        s0 = J.st[J.ptr[k]];
-        len = J.off[k];
-      }
-      uint64_t x = 0;
-      if ((((uintptr_t)(T + s0)) & 15) == 0) {
-        for (; x + 16 <= len; x += 16) {
-          const uint4 v = *(const uint4*)(T + s0 + x);
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+// pre[s][k]: exclusive prefix sums of the base level's counters, a CTA per
+// symbol.
+__global__ void __launch_bounds__(1024) k_base_prefix(uint64_t c, const void* __restrict__ cnt, uint32_t cw, uint64_t cp,
+                                                      uint32_t* __restrict__ pre) {
+  __shared__ uint32_t sm[32];
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint64_t s = blockIdx.x;
+  uint32_t carry = 0;
+  for (uint64_t base = 0; base < c; base += blockDim.x) {
+    const uint64_t k = base + threadIdx.x;
+    const uint32_t v = k < c ? cget(cnt, cw, s * cp + k) : 0u;
+    uint32_t x = v;
 #pragma unroll
-          for (int t = 0; t < 16; t++) row[sym[(w[t >> 2] >> (8 * (t & 3))) & 0xFF]]++;
-        }
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, x, d);
+      if (lane >= (unsigned)d) x += o;
+    }
+    if (lane == 31) sm[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+      uint32_t w = lane < nw ? sm[lane] : 0;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, w, d);
+        if (lane >= (unsigned)d) w += o;
       }
-      for (; x < len; x++) row[sym[T[s0 + x]]]++;
+      sm[lane] = w;
     }
+    __syncthreads();
+    if (k < c) pre[s * (c + 1) + k] = carry + (warp ? sm[warp - 1] : 0) + x - v;
+    carry += sm[nw - 1];
+    __syncthreads();
   }
-  __syncthreads();
-  const uint64_t nrows = J.c - k0 < kSmallCountThreads ? J.c - k0 : kSmallCountThreads;
-  const uint64_t nbytes = nrows * S;
-  uint8_t* out = (uint8_t*)J.out + k0 * S;
-  const uint64_t nwords = ((((uintptr_t)out) & 3) == 0) ? nbytes / 4 : 0;
-  for (uint64_t i = threadIdx.x; i < nwords; i += blockDim.x) ((uint32_t*)out)[i] = ((const uint32_t*)rows)[i];
-  for (uint64_t i = nwords * 4 + threadIdx.x; i < nbytes; i += blockDim.x) out[i] = rows[i];
-}
-
-// Marked blocks of a non-last level: sum of the children's counts, one warp
-// per block (lanes over the symbols).
-__global__ void k_sum_children(uint64_t c, uint64_t b, uint64_t n, const uint64_t* __restrict__ st,
-                               const uint32_t* __restrict__ mw, const uint32_t* __restrict__ mr,
-                               uint32_t arity, uint64_t bn, const void* __restrict__ child_cnt,
-                               uint32_t child_cw, uint32_t S, void* __restrict__ cnt, uint32_t cw) {
-  const unsigned lane = threadIdx.x & 31;
-  const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
-  for (uint64_t k = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / 32; k < c; k += warps) {
-    if (!((mw[k >> 5] >> (k & 31)) & 1u)) continue;
-    const uint64_t len = n - st[k] < b ? n - st[k] : b;
-    const uint64_t first = (mr[k >> 5] + __popc(mw[k >> 5] & ((1u << (k & 31)) - 1u))) * (uint64_t)arity;
-    const uint64_t nch = (len + bn - 1) / bn;
-    for (uint32_t s = lane; s < S; s += 32) {
-      uint32_t acc = 0;
-      for (uint64_t i = 0; i < nch; i++) acc += cget(child_cnt, child_cw, (first + i) * S + s);
-      cput(cnt, cw, k * S + s, acc);
-    }
-  }
-}
-
-__global__ void k_level1_prefix(uint64_t c, const void* __restrict__ cnt, uint32_t cw, uint32_t S,
-                                uint64_t* __restrict__ pre) {
-  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < S; s += gridDim.x * blockDim.x) {
-    uint64_t acc = 0;
-    for (uint64_t k = 0; k < c; k++) {
-      pre[k * S + s] = acc;
-      acc += cget(cnt, cw, k * S + s);
-    }
-    pre[c * S + s] = acc;
-  }
+  if (threadIdx.x == 0) pre[s * (c + 1) + c] = carry;
 }
 
 __global__ void k_leaf_text(uint64_t c, uint64_t b, uint64_t n, const uint64_t* __restrict__ st,
@@ -303,20 +382,19 @@ __device__ __noinline__ uint32_t leaf_prefix_count(const uint8_t* leaf, const Le
 }
 
 // Counter of symbol s (byte c) of block k: stored, or counted in the leaf text.
-__device__ __forceinline__ uint32_t blk_cnt(const uint8_t* leaf, uint32_t S, const LevelView& v, uint32_t k, uint32_t s,
-                                            uint32_t c) {
-  return v.cnt ? cget(v.cnt, v.cw, (uint64_t)k * S + s) : leaf_block_count(leaf, v, k, c);
+__device__ __forceinline__ uint32_t blk_cnt(const uint8_t* leaf, const LevelView& v, uint32_t k, uint32_t s, uint32_t c) {
+  return v.cnt ? cget(v.cnt, v.cw, (uint64_t)s * v.cp + k) : leaf_block_count(leaf, v, k, c);
 }
-__device__ __forceinline__ uint32_t blk_pc(const uint8_t* leaf, uint32_t S, const LevelView& v, uint32_t k, uint2 r,
-                                           uint32_t s, uint32_t c) {
-  return v.pc ? cget(v.pc, v.cw, (uint64_t)k * S + s) : leaf_prefix_count(leaf, v, r, c);
+__device__ __forceinline__ uint32_t blk_pc(const uint8_t* leaf, const LevelView& v, uint32_t k, uint2 r, uint32_t s,
+                                           uint32_t c) {
+  return v.pc ? cget(v.pc, v.cw, (uint64_t)s * v.cp + k) : leaf_prefix_count(leaf, v, r, c);
 }
 
 // What a descent needs of the tree besides the level table.
 struct QTree {
   uint64_t n;
-  uint32_t L, S;
-  const uint64_t* pre;
+  uint32_t L;           // levels from the base on (the level table starts there)
+  const uint32_t* pre;
   const uint8_t* leaf;
   const int16_t* sym;
 };
@@ -344,50 +422,82 @@ __device__ __forceinline__ uint64_t q_access(const QTree& t, const LevelView* __
   return kNone;
 }
 
+// Up to four counters of one symbol as read, and how many of them count:
+// their sum is taken when it is needed.
+struct Run4 {
+  uint32_t v[4];
+  uint32_t m;
+};
+__device__ __forceinline__ void read_run(Run4& r, const void* cnt, uint32_t w, uint64_t i, uint32_t m) {
+  r.m = m;
+  if (w == 1) {
+    r.v[0] = *(const uint32_t*)((const uint8_t*)cnt + i);
+  } else if (w == 2) {
+    const uint2 q = *(const uint2*)((const uint16_t*)cnt + i);
+    r.v[0] = q.x, r.v[1] = q.y;
+  } else {
+    const uint4 q = *(const uint4*)((const uint32_t*)cnt + i);
+    r.v[0] = q.x, r.v[1] = q.y, r.v[2] = q.z, r.v[3] = q.w;
+  }
+}
+__device__ __forceinline__ uint32_t run_sum(const Run4& r, uint32_t w) {  // of the first m <= 3
+  if (r.m == 0) return 0;
+  if (w == 1) return __dp4a(r.v[0] & ((1u << (8 * r.m)) - 1u), 0x01010101u, 0u);
+  if (w == 2) return (r.v[0] & 0xFFFFu) + (r.m > 1 ? r.v[0] >> 16 : 0) + (r.m > 2 ? r.v[1] & 0xFFFFu : 0);
+  return r.v[0] + (r.m > 1 ? r.v[1] : 0) + (r.m > 2 ? r.v[2] : 0);
+}
+
 // rank descends likewise.  Its counters are off the chain of dependent reads:
 // they are added one step later, when the next record has been read too.
 __device__ __forceinline__ uint64_t q_rank(const QTree& t, const LevelView* __restrict__ lv, uint32_t c, uint64_t i) {
   if (i > t.n) return kNone;
   const int s = t.sym[c];
   if (s < 0) return 0;
-  const uint32_t S = t.S;
-  if (i == t.n) return t.pre[(uint64_t)lv[0].c * S + s];
+  const uint32_t* pre = t.pre + (uint64_t)s * (lv[0].c + 1);
+  if (i == t.n) return pre[lv[0].c];
   uint32_t l = 0, k = div_b((uint32_t)i, lv[0]), o = (uint32_t)i - k * lv[0].b;
-  int64_t acc = (int64_t)t.pre[(uint64_t)k * S + s];
-  uint32_t p0 = 0, p1 = 0, p2 = 0, m0 = 0;  // counters in flight: to add, to subtract
+  uint32_t acc = pre[k];  // (sums may pass below zero on the way: modulo 2^32, the answer is at most n)
+  Run4 run;
+  run.m = 0;
+  uint32_t rw = 1, p0 = 0, m0 = 0;  // counters in flight: a run of width rw and p0 to add, m0 to subtract
   for (uint32_t step = 0; step < 4 * t.L + 4; step++) {
     const LevelView& v = lv[l];
-    if (o == 0) return (uint64_t)(acc + p0 + p1 + p2 - m0);
-    if (o == qlen(v, k)) return (uint64_t)(acc + p0 + p1 + p2 - m0 + blk_cnt(t.leaf, S, v, k, s, c));
+    if (o == 0) return acc + run_sum(run, rw) + p0 - m0;
+    if (o == qlen(v, k)) return acc + run_sum(run, rw) + p0 - m0 + blk_cnt(t.leaf, v, k, s, c);
     const uint2 r = v.rec[k];
+    acc += run_sum(run, rw) + p0 - m0;
+    run.m = p0 = m0 = 0;
     if (r.x == kMarkedRec) {
-      acc += (int64_t)p0 + p1 + p2 - m0;
-      p0 = p1 = p2 = m0 = 0;
-      if (l + 1 == t.L) return (uint64_t)(acc + leaf_count(t.leaf + (uint64_t)r.y * v.b, o, c));
+      if (l + 1 == t.L) return acc + leaf_count(t.leaf + (uint64_t)r.y * v.b, o, c);
+      const uint32_t f = r.y * v.arity, ar = v.arity;
       const LevelView& w = lv[++l];
-      const uint32_t j = div_b(o, w), f = r.y * v.arity;
+      const uint32_t j = div_b(o, w);
       o -= j * w.b;
       k = f + j;
       if (w.cnt) {
-        const uint64_t at = (uint64_t)f * S + s;
-        uint32_t x = 0;
-        for (; x + 3 < j; x++) acc += cget(w.cnt, w.cw, at + (uint64_t)x * S);
-        if (x < j) p0 = cget(w.cnt, w.cw, at + (uint64_t)x * S);
-        if (x + 1 < j) p1 = cget(w.cnt, w.cw, at + (uint64_t)(x + 1) * S);
-        if (x + 2 < j) p2 = cget(w.cnt, w.cw, at + (uint64_t)(x + 2) * S);
+        uint64_t at = (uint64_t)s * w.cp + f;
+        uint32_t left = j;
+        if ((ar & 3) == 0) {
+          if (left >= 4) {
+            acc += sum_run(w.cnt, w.cw, at, left & ~3u);
+            at += left & ~3u;
+            left &= 3u;
+          }
+          if (left) read_run(run, w.cnt, rw = w.cw, at, left);
+        } else {
+          acc += sum_run(w.cnt, w.cw, at, left);
+        }
       } else {
         for (uint32_t x = 0; x < j; x++) acc += leaf_block_count(t.leaf, w, f + x, c);
       }
     } else {
-      acc += (int64_t)p0 + p1 + p2 - m0;
-      p0 = p1 = p2 = 0;
-      m0 = blk_pc(t.leaf, S, v, k, r, s, c);
+      m0 = blk_pc(t.leaf, v, k, r, s, c);
       const uint32_t lp = qlen(v, r.x), x = r.y + o;
       if (x <= lp) {
         k = r.x;
         o = x;
       } else {
-        p0 = blk_cnt(t.leaf, S, v, r.x, s, c);
+        p0 = blk_cnt(t.leaf, v, r.x, s, c);
         k = r.x + 1;
         o = x - lp;
       }
@@ -401,53 +511,79 @@ __device__ __forceinline__ uint64_t q_rank(const QTree& t, const LevelView* __re
 __device__ __forceinline__ uint64_t q_select(const QTree& t, const LevelView* __restrict__ lv, uint32_t c, uint64_t jq) {
   const int s = t.sym[c];
   if (s < 0 || jq == 0) return kNone;
-  const uint32_t S = t.S;
   const LevelView& top = lv[0];
-  if (jq > t.pre[(uint64_t)top.c * S + s]) return kNone;
-  uint32_t a = 0, z = top.c;  // last k with pre[k] < j
+  const uint32_t* pre = t.pre + (uint64_t)s * (top.c + 1);
+  if (jq > pre[top.c]) return kNone;
+  uint32_t a = 0, z = top.c;  // last k with pre[k] < j: four parts per step, their bounds read together
+  const uint32_t jw = (uint32_t)jq;
   while (z - a > 1) {
-    const uint32_t mid = (a + z) / 2;
-    if (t.pre[(uint64_t)mid * S + s] < jq) a = mid;
-    else z = mid;
+    const uint32_t d = z - a, q1 = a + ((d + 3) >> 2), q2 = a + ((d + 1) >> 1), q3 = a + d - (d >> 2);
+    const uint32_t v1 = pre[q1], v2 = pre[q2], v3 = pre[q3 < z ? q3 : z - 1];
+    if (v2 < jw) {
+      a = q2;
+      if (q3 < z && q3 > q2) {
+        if (v3 < jw) a = q3;
+        else z = q3;
+      }
+    } else {
+      z = q2;
+      if (q1 < q2) {
+        if (v1 < jw) a = q1;
+        else z = q1;
+      }
+    }
   }
   uint32_t k = a, l = 0;
-  uint32_t j = (uint32_t)(jq - t.pre[(uint64_t)k * S + s]);
+  uint32_t j = jw - pre[k];
   int64_t res = (int64_t)k * top.b;
   for (uint32_t step = 0; step < 4 * t.L + 4; step++) {
     const LevelView& v = lv[l];
     const uint2 r = v.rec[k];
-    const uint32_t pck = v.pc ? cget(v.pc, v.cw, (uint64_t)k * S + s) : 0;
+    const uint32_t pck = v.pc ? cget(v.pc, v.cw, (uint64_t)s * v.cp + k) : 0;
     if (r.x == kMarkedRec) {
       if (l + 1 == t.L) {
         const uint32_t x = leaf_find(t.leaf + (uint64_t)r.y * v.b, qlen(v, k), c, j);
         return x == kNoSlot ? kNone : (uint64_t)(res + x);
       }
-      const LevelView& w = lv[++l];
       const uint32_t f = r.y * v.arity, ar = v.arity;
+      const LevelView& w = lv[++l];
       uint32_t i = 0;
       bool found = false;
       if (w.cnt) {
-        const uint64_t at = (uint64_t)f * S + s;
-        // (A short last block has fewer children: counters past the level's
-        // end are not read, and the j-th symbol lies before them.)
+        const uint64_t at = (uint64_t)s * w.cp + f;
+        // (A short last block has fewer children: the entries behind them are
+        // the row's padding or not counted; the j-th symbol lies before them.)
         const uint32_t have = w.c - f < ar ? w.c - f : ar;
         while (i < have && !found) {
           uint32_t cc[4];
+          if ((ar & 3) == 0) {
+            Run4 run;
+            read_run(run, w.cnt, w.cw, at + i, 4);
+            if (w.cw == 1) {
 #pragma unroll
-          for (uint32_t u = 0; u < 4; u++) cc[u] = i + u < have ? cget(w.cnt, w.cw, at + (uint64_t)(i + u) * S) : 0xFFFFFFFFu;
+              for (uint32_t u = 0; u < 4; u++) cc[u] = (run.v[0] >> (8 * u)) & 0xFFu;
+            } else if (w.cw == 2) {
+              cc[0] = run.v[0] & 0xFFFFu, cc[1] = run.v[0] >> 16, cc[2] = run.v[1] & 0xFFFFu, cc[3] = run.v[1] >> 16;
+            } else {
+#pragma unroll
+              for (uint32_t u = 0; u < 4; u++) cc[u] = run.v[u];
+            }
+          } else {
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++) cc[u] = i + u < have ? cget(w.cnt, w.cw, at + i + u) : 0;
+          }
 #pragma unroll
           for (uint32_t u = 0; u < 4; u++) {
-            if (found) continue;
+            if (found || i + u >= have) continue;
             if (cc[u] >= j) {
               found = true;
               i += u;
-            } else {
-              j -= cc[u];
+              break;
             }
+            j -= cc[u];
           }
           if (!found) i += 4;
         }
-        found = found && i < have;
       } else {
         for (; i < ar && !found; i++) {
           const uint32_t cc = leaf_block_count(t.leaf, w, f + i, c);
@@ -462,7 +598,7 @@ __device__ __forceinline__ uint64_t q_select(const QTree& t, const LevelView* __
       res += (int64_t)i * w.b;
       k = f + i;
     } else {
-      const uint32_t cp = blk_cnt(t.leaf, S, v, r.x, s, c);
+      const uint32_t cp = blk_cnt(t.leaf, v, r.x, s, c);
       const uint32_t jj = j + (v.pc ? pck : leaf_prefix_count(t.leaf, v, r, c));
       if (jj <= cp) {
         res -= (int64_t)r.y;
@@ -491,15 +627,15 @@ __device__ __forceinline__ uint64_t q_answer(const QTree& t, const LevelView* __
 // upper levels stay in L1.  Measured on 4 M queries of each kind on the tree of
 // the 256 MiB text: 3.68 ms when a step read block starts, marks, ranks,
 // pointers and offsets from five arrays (and every CTA copied the top levels
-// into shared memory), 2.82 ms with one record; 1000 queries of each kind 79
-// and 42 us.
+// into shared memory), 2.82 ms with one record, 1.69 with symbol-major counters
+// and the base level; 1000 queries of each kind 79, 42 and 35 us.
 template <int KIND, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_queries(const TreeView* __restrict__ tv, const uint64_t* __restrict__ args,
                                                       uint64_t m, uint64_t* __restrict__ out) {
   __shared__ __align__(16) LevelView lv[kMaxLevels];
-  const QTree t{tv->n, tv->L, tv->S, tv->pre, tv->leaf, tv->sym};
-  for (uint32_t i = threadIdx.x; i < t.L * (sizeof(LevelView) / 4); i += NT)
-    ((uint32_t*)lv)[i] = ((const uint32_t*)tv->lv)[i];
+  const QTree t{tv->n, tv->L - tv->base, tv->pre, tv->leaf, tv->sym};
+  const uint32_t* from = (const uint32_t*)(tv->lv + tv->base);
+  for (uint32_t i = threadIdx.x; i < t.L * (sizeof(LevelView) / 4); i += NT) ((uint32_t*)lv)[i] = from[i];
   __syncthreads();
   for (uint64_t q = blockIdx.x * (uint64_t)NT + threadIdx.x; q < m; q += (uint64_t)gridDim.x * NT) {
     if (KIND == BT_Q_ACCESS) {
@@ -516,10 +652,11 @@ __global__ void __launch_bounds__(NT, MINB) k_queries(const TreeView* __restrict
 // One query, its arguments in the launch and its answer written to `out`
 // (pinned host memory): 38 us a call with copies around it, 22 now.
 __global__ void k_query_one(const TreeView* __restrict__ tv, int kind, uint64_t a0, uint64_t a1, uint64_t* out) {
-  const QTree t{tv->n, tv->L, tv->S, tv->pre, tv->leaf, tv->sym};
-  if (kind == BT_Q_ACCESS) *out = q_answer<BT_Q_ACCESS>(t, tv->lv, a0, a1);
-  else if (kind == BT_Q_RANK) *out = q_answer<BT_Q_RANK>(t, tv->lv, a0, a1);
-  else *out = q_answer<BT_Q_SELECT>(t, tv->lv, a0, a1);
+  const QTree t{tv->n, tv->L - tv->base, tv->pre, tv->leaf, tv->sym};
+  const LevelView* lv = tv->lv + tv->base;
+  if (kind == BT_Q_ACCESS) *out = q_answer<BT_Q_ACCESS>(t, lv, a0, a1);
+  else if (kind == BT_Q_RANK) *out = q_answer<BT_Q_RANK>(t, lv, a0, a1);
+  else *out = q_answer<BT_Q_SELECT>(t, lv, a0, a1);
 }
 
 // The records of all levels (blockIdx.y) and their mark words, from the
@@ -547,6 +684,7 @@ __global__ void __launch_bounds__(256) k_pack_records(const __grid_constant__ Pa
       view->n = P.view.n;
       view->L = P.view.L;
       view->S = P.view.S;
+      view->base = P.view.base;
       view->pre = P.view.pre;
       view->leaf = P.view.leaf;
       view->sym = P.view.sym;
@@ -589,60 +727,71 @@ int alphabet(const uint8_t* T, uint64_t n, uint32_t sigma, bt_tree* t, cudaStrea
   return BT_OK;
 }
 
+// The level queries start at: the lowest one with all blocks of the text
+// (every block above it is marked), while its prefix table, 4 bytes per block
+// and symbol, stays within an eighth of the text (or 64 KiB).  A descent of the
+// 256 MiB text's tree then starts at level 8 of 12, and the levels above need
+// no counters.
+static uint32_t base_level(const bt_tree* t, uint32_t last) {
+  uint32_t base = 0;
+  for (uint32_t l = 1; l <= last; l++) {
+    const Level& v = t->lv[l];
+    if (v.c != (t->n + v.b - 1) / v.b || v.b > 0xFFFFFFFFull) break;
+    const uint64_t bytes = (v.c + 1) * t->S * 4;
+    if (bytes <= t->n / 8 || bytes <= (64u << 10)) base = l;
+  }
+  return base;
+}
+
 int build_counters(BuildCtx& ctx) {
   bt_tree* t = ctx.t;
   cudaStream_t s = ctx.s;
   const uint32_t S = t->S;
   const unsigned T = 256;
-  const size_t smem = 8 * S * sizeof(unsigned int);
   // Space-efficient counters: the last level keeps none (queries count its
   // blocks in the leaf text), and the marked blocks of the level above are
   // counted in the text instead of summed from children.
   const bool leaf_counts = ctx.leaf_counts && t->L >= 2;
-  for (int l = (int)t->L - 1; l >= 0; l--) {
+  t->base = base_level(t, leaf_counts ? t->L - 2 : t->L - 1);
+  for (int l = (int)t->L - 1; l >= (int)t->base; l--) {
     Level& v = t->lv[l];
     v.cw = counter_width(v.b);
     if (leaf_counts && l + 1 == (int)t->L) {
       v.cnt = v.pc = nullptr;
       continue;
     }
-    // Counters of cw bytes (a count never exceeds b).  Narrow rows are
-    // written whole by the kernels; 4-byte rows are accumulated from zero.
-    v.cw = counter_width(v.b);
-    const uint64_t half = ((v.c * S * v.cw + 4) + 255) & ~255ull;
+    const uint64_t cp = counter_stride(v.c), half = (S * cp * v.cw + 255) & ~255ull;
     char* mem;
     BT_CUDA(cudaMallocAsync((void**)&mem, 2 * half, s));
     v.owned.push_back(mem);
     v.cnt = mem;
     v.pc = mem + half;
-    if (v.cw == 4) BT_CUDA(cudaMemsetAsync(mem, 0, 2 * half, s));
-    const uint64_t ppb = (v.b + kCountPiece - 1) / kCountPiece;
     const bool last = l + 1 == (int)t->L;
-    CountJob J{v.st, v.ptr, v.off, v.mw, v.c, v.b, t->n, v.cnt, v.cw, 0, 0, 0};
-    CountJob P{v.st, v.ptr, v.off, v.mw, v.c, v.b, t->n, v.pc, v.cw, 1, 1, 0};
     const bool children_counted = !last && !(leaf_counts && l + 2 == (int)t->L);
-    if (children_counted) J.only_unmarked = 1;  // marked blocks are sums of their children
+    const CountLevel J{v.st, v.ptr, v.off, v.mw, v.c, v.b, t->n, cp, v.cnt, v.pc, v.cw, children_counted};
     if (v.cw == 1) {
-      // One thread per block; the rows of marked blocks are written as zeros
-      // and the sums of children overwrite them below.
-      const size_t sm1 = ((kSmallCountThreads * S + 3) & ~3u) + 256 * sizeof(int16_t);
-      const unsigned g1 = (unsigned)((v.c + kSmallCountThreads - 1) / kSmallCountThreads);
-      BT_LAUNCH(k_count_small<<<g1, kSmallCountThreads, sm1, s>>>(J, t->sym, ctx.T, S));
-      BT_LAUNCH(k_count_small<<<g1, kSmallCountThreads, sm1, s>>>(P, t->sym, ctx.T, S));
+      const size_t sm = (size_t)kSmallCountThreads * S + 256;
+      BT_LAUNCH(k_count_small<<<dim3((unsigned)((v.c + kSmallCountThreads - 1) / kSmallCountThreads), 2),
+                                kSmallCountThreads, sm, s>>>(J, t->sym, ctx.T, S));
+    } else if (v.cw == 2) {
+      const size_t sm = 8ull * 4 * S * 4 + (size_t)S * kTileBlocks * v.cw + 256;
+      BT_LAUNCH(k_count_tile<<<dim3(grid_for(v.c, kTileBlocks, 152 * 8), 2), 256, sm, s>>>(J, t->sym, ctx.T, S));
     } else {
-      BT_LAUNCH(k_count<<<grid_for(v.c * ppb * 32, T), T, smem, s>>>(J, t->sym, ctx.T, S, ppb));
-      BT_LAUNCH(k_count<<<grid_for(v.c * ppb * 32, T), T, smem, s>>>(P, t->sym, ctx.T, S, ppb));
+      BT_CUDA(cudaMemsetAsync(mem, 0, 2 * half, s));
+      const uint64_t ppb = (v.b + kCountPiece - 1) / kCountPiece;
+      BT_LAUNCH(k_count_long<<<dim3(grid_for(v.c * ppb * 32, T), 2), T, 8 * S * sizeof(uint32_t), s>>>(J, t->sym, ctx.T, S,
+                                                                                                    ppb));
     }
     if (children_counted) {
       const Level& w = t->lv[l + 1];
-      BT_LAUNCH(k_sum_children<<<grid_for(v.c * 32, T), T, 0, s>>>(v.c, v.b, t->n, v.st, v.mw, v.mr, v.arity, w.b,
-                                                        w.cnt, w.cw, S, v.cnt, v.cw));
+      BT_LAUNCH(k_sum_children<<<dim3(grid_for(v.c, T), S < 8 ? 1 : 8), T, 0, s>>>(J, v.mr, v.arity, w.b, w.cnt, w.cw,
+                                                                                  counter_stride(w.c), S));
     }
     BT_CUDA(cudaGetLastError());
   }
-  const Level& r = t->lv[0];
-  BT_CUDA(cudaMallocAsync(&t->pre, (r.c + 1) * S * sizeof(uint64_t) + 8, s));
-  BT_LAUNCH(k_level1_prefix<<<1, 256, 0, s>>>(r.c, r.cnt, r.cw, S, t->pre));
+  const Level& r = t->lv[t->base];
+  BT_CUDA(cudaMallocAsync((void**)&t->pre, (r.c + 1) * S * sizeof(uint32_t), s));
+  BT_LAUNCH(k_base_prefix<<<S, r.c > 512 ? 1024 : 128, 0, s>>>(r.c, r.cnt, r.cw, counter_stride(r.c), t->pre));
   // Leaf text of the marked last-level blocks.
   const Level& z = t->lv[t->L - 1];
   uint32_t nm = 0;
@@ -687,6 +836,7 @@ int pack_records(BuildCtx& ctx) {
   P.view.n = t->n;
   P.view.L = t->L;
   P.view.S = t->S;
+  P.view.base = t->base;
   P.view.pre = t->pre;
   P.view.leaf = t->leaf;
   P.view.sym = t->sym;
@@ -696,7 +846,7 @@ int pack_records(BuildCtx& ctx) {
     PackLevel& p = P.lv[l];
     p = PackLevel{v.c, v.b, v.st, v.mw, v.mr, v.ptr, v.off, (uint2*)mem, nullptr, nullptr};
     P.view.lv[l] = LevelView{(uint32_t)v.c, view_len(v.b), v.arity, block_shift(view_len(v.b)), 0, v.cw,
-                             p.rec, v.cnt, v.pc};
+                             (uint32_t)counter_stride(v.c), 0, p.rec, v.cnt, v.pc};
     mem += al(v.c * 8);
     p.mw2 = (uint32_t*)mem;
     mem += al(words * 4);
@@ -734,7 +884,7 @@ int run_queries(const bt_tree* t, int kind, const uint64_t* d_args, uint64_t m, 
   // CTAs of 128 threads: small batches spread over more SMs; 64 registers, so
   // that 1024 threads fit on an SM.
   const unsigned g = grid_for(m, 128, 152 * 64);
-  if (kind == BT_Q_ACCESS) BT_LAUNCH(k_queries<BT_Q_ACCESS, 128, 8><<<g, 128, 0, s>>>(t->view, d_args, m, d_out));
+  if (kind == BT_Q_ACCESS) BT_LAUNCH(k_queries<BT_Q_ACCESS, 128, 16><<<g, 128, 0, s>>>(t->view, d_args, m, d_out));
   else if (kind == BT_Q_RANK) BT_LAUNCH(k_queries<BT_Q_RANK, 128, 8><<<g, 128, 0, s>>>(t->view, d_args, m, d_out));
   else BT_LAUNCH(k_queries<BT_Q_SELECT, 128, 8><<<g, 128, 0, s>>>(t->view, d_args, m, d_out));
   BT_CUDA(cudaGetLastError());

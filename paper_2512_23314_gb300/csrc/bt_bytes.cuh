@@ -18,16 +18,30 @@ __device__ __forceinline__ uint4 unaligned16(uint4 u0, uint4 u1, uint32_t d) {
                     __funnelshift_r(w3, w4, sh));
 }
 
-// Do the 16 bytes at a and at b (16-byte aligned, a < b, T aligned) differ?
-// The unit after a's first one ends at b + 16 or before.
-__device__ __forceinline__ bool differ16(const uint8_t* __restrict__ T, uint64_t a, uint64_t b) {
-  const uint4 vb = *(const uint4*)(T + b);
-  const uint64_t a0 = a & ~15ull;
-  const uint32_t d = (uint32_t)(a & 15);
-  const uint4 u0 = *(const uint4*)(T + a0);
-  const uint4 va = d == 0 ? u0 : unaligned16(u0, *(const uint4*)(T + a0 + 16), d);
-  return va.x != vb.x || va.y != vb.y || va.z != vb.z || va.w != vb.w;
+// The 16 bytes at b (16-byte aligned) and the two aligned units that hold the
+// 16 bytes at a < b (T aligned).  The second unit ends at b + 16 or before.
+struct Unit16 {
+  uint4 b, u0, u1;
+};
+__device__ __forceinline__ Unit16 load_units(const uint8_t* __restrict__ T, uint32_t a, uint32_t b) {
+  const uint4* p = (const uint4*)(T + (a & ~15u));
+  return Unit16{*(const uint4*)(T + b), p[0], p[1]};
 }
+// Realignment by a mod 16, the same for all units of a comparison.
+struct Shift16 {
+  bool w2, w1;
+  uint32_t sh;
+  __device__ __forceinline__ explicit Shift16(uint32_t a) : w2(a & 8), w1(a & 4), sh(8 * (a & 3)) {}
+  __device__ __forceinline__ bool differ(const Unit16& v) const {
+    uint32_t a[8] = {v.u0.x, v.u0.y, v.u0.z, v.u0.w, v.u1.x, v.u1.y, v.u1.z, v.u1.w};
+#pragma unroll
+    for (int i = 0; i < 6; i++) a[i] = w2 ? a[i + 2] : a[i];
+#pragma unroll
+    for (int i = 0; i < 5; i++) a[i] = w1 ? a[i + 1] : a[i];
+    return ((__funnelshift_r(a[0], a[1], sh) ^ v.b.x) | (__funnelshift_r(a[1], a[2], sh) ^ v.b.y) |
+            (__funnelshift_r(a[2], a[3], sh) ^ v.b.z) | (__funnelshift_r(a[3], a[4], sh) ^ v.b.w)) != 0;
+  }
+};
 
 // Compare T[a + x] and T[b + x] for x in [off, end) by L lanes: bytes up to
 // the first 16-byte unit of the side at b, then 16 bytes per lane and step,

@@ -12,6 +12,7 @@
 // it adds the counts of the children left of the one holding i; at an
 // unmarked block it continues in its target (ptr or ptr+1) and subtracts
 // pc.  select mirrors it.  One thread answers one query.
+#include <atomic>
 #include <cstdlib>
 
 #include "bt_internal.cuh"
@@ -46,6 +47,24 @@ __global__ void k_histogram(const uint8_t* __restrict__ T, uint64_t n, unsigned 
     if (h[i]) atomicAdd(&hist[i], (unsigned long long)h[i]);
 }
 
+// Up to four counters of one symbol as read, and how many of them count:
+// their sum is taken when it is needed.
+struct Run4 {
+  uint32_t v[4];
+  uint32_t m;
+};
+__device__ __forceinline__ void read_run(Run4& r, const void* cnt, uint32_t w, uint64_t i, uint32_t m) {
+  r.m = m;
+  if (w == 1) {
+    r.v[0] = *(const uint32_t*)((const uint8_t*)cnt + i);
+  } else if (w == 2) {
+    const uint2 q = *(const uint2*)((const uint16_t*)cnt + i);
+    r.v[0] = q.x, r.v[1] = q.y;
+  } else {
+    const uint4 q = *(const uint4*)((const uint32_t*)cnt + i);
+    r.v[0] = q.x, r.v[1] = q.y, r.v[2] = q.z, r.v[3] = q.w;
+  }
+}
 // What a level's counters are counted from.
 struct CountLevel {
   const uint64_t* st;   // block starts of the level
@@ -123,66 +142,162 @@ __global__ void __launch_bounds__(kSmallCountThreads) k_count_small(CountLevel J
   }
 }
 
-// Two-byte counters (blocks of 256 bytes to 64 KiB): a CTA takes 16
-// consecutive blocks, a warp one after the other, 16 bytes per lane and step
-// into four copies of a histogram in shared memory (lanes take different
-// copies: a frequent symbol's updates meet less often); the 16 blocks' counters
-// of a symbol leave as one unit.  blockIdx.y: cnt or pc.
-constexpr uint32_t kTileBlocks = 16;
+// Two-byte counters (blocks of 256 bytes to 64 KiB): a CTA takes a tile of
+// consecutive blocks and writes its counters of a symbol as one run.  Bound by
+// the chain of dependent reads before a block's text (mark, target, start): the
+// lanes of a warp walk it for all the warp's blocks at once, and the texts of
+// the next blocks are in flight while the current ones are counted.  Few
+// symbols (DNA) are counted by comparing words with each symbol, a group of
+// lanes per block, without memory; more go to four copies of a histogram in
+// shared memory (lanes take different copies: a frequent symbol's updates meet
+// less often), two blocks at a time.  blockIdx.y: cnt or pc.
+constexpr uint32_t kFewSymbols = 8;
+constexpr uint32_t kTileFew = 128, kTileMany = 64;  // blocks per tile
 constexpr uint64_t kCountPiece = 1 << 16;
 
+// 16 text bytes from x of a range (zeros past it); bytes outside are not read.
+__device__ __forceinline__ uint4 range16(const uint8_t* __restrict__ T, uint64_t s0, uint32_t len, uint32_t x, bool al) {
+  if (x >= len) return make_uint4(0, 0, 0, 0);
+  if (al && x + 16 <= len) return *(const uint4*)(T + s0 + x);
+  uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (uint32_t q = 0; q < 16; q++)
+    if (x + q < len) w[q >> 2] |= (uint32_t)T[s0 + x + q] << (8 * (q & 3));
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+template <bool FEW>
 __global__ void __launch_bounds__(256) k_count_tile(CountLevel J, const int16_t* __restrict__ sym_g,
                                                     const uint8_t* __restrict__ T, uint32_t S) {
-  extern __shared__ uint32_t hist[];  // per warp [S][4], then [S][16] of cw bytes, then the symbol map
+  constexpr uint32_t TB = FEW ? kTileFew : kTileMany, PW = TB / 8;  // blocks per tile and per warp
+  extern __shared__ uint32_t hist[];  // per warp two [S][4] (not FEW), then [S][TB] of two bytes, then the symbol map
+  __shared__ uint8_t byte_of[kFewSymbols];
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t* h = hist + warp * 4 * S;
-  uint8_t* rows = (uint8_t*)(hist + 8 * 4 * S);
-  uint8_t* sym = rows + S * kTileBlocks * J.cw;
-  for (uint32_t i = threadIdx.x; i < 256; i += 256) sym[i] = (uint8_t)sym_g[i];
+  uint32_t* h = hist + warp * 8 * S;
+  uint16_t* rows = (uint16_t*)(hist + (FEW ? 0 : 8 * 8 * S));
+  uint8_t* sym = (uint8_t*)(rows + S * TB);
+  for (uint32_t i = threadIdx.x; i < 256; i += 256) {
+    const int v = sym_g[i];
+    sym[i] = (uint8_t)v;
+    if (FEW && v >= 0) byte_of[v] = (uint8_t)i;
+  }
   const int which = blockIdx.y;
-  uint8_t* out = (uint8_t*)(which ? J.pc : J.cnt);
-  const uint64_t tiles = (J.c + kTileBlocks - 1) / kTileBlocks;
+  uint16_t* out = (uint16_t*)(which ? J.pc : J.cnt);
+  const uint64_t tiles = (J.c + TB - 1) / TB;
+  // Lanes per block of the comparing kernel: one 16-byte unit each at first.
+  unsigned L = 32;
+  while (L > 1 && 16ull * (L / 2) >= J.b) L >>= 1;
   for (uint64_t tl = blockIdx.x; tl < tiles; tl += gridDim.x) {
     __syncthreads();
     bool any = false;
-    for (uint32_t i = warp; i < kTileBlocks; i += 8) {
-      const uint64_t k = tl * kTileBlocks + i;
-      uint64_t s0 = 0;
-      uint32_t len = 0;
-      if (k < J.c) any |= count_range(J, which, k, &s0, &len);
-      if (len == 0) {
-        for (uint32_t s = lane; s < S; s += 32) cput(rows, J.cw, s * kTileBlocks + i, 0u);
-        continue;
-      }
-      for (uint32_t s = lane; s < 4 * S; s += 32) h[s] = 0;
-      __syncwarp();
-      const uint32_t cpy = lane & 3;
-      uint32_t x = 0;
-      if ((((uintptr_t)(T + s0)) & 15) == 0) {
-        const uint32_t full = len & ~15u;
-        for (x = 16 * lane; x < full; x += 512) {
-          const uint4 v = *(const uint4*)(T + s0 + x);
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-          for (uint32_t q = 0; q < 16; q++) atomicAdd(&h[4 * sym[(w[q >> 2] >> (8 * (q & 3))) & 0xFF] + cpy], 1u);
-        }
-        x = full;
-      }
-      for (x += lane; x < len; x += 32) atomicAdd(&h[4 * sym[T[s0 + x]] + cpy], 1u);
-      __syncwarp();
-      for (uint32_t s = lane; s < S; s += 32)
-        cput(rows, J.cw, s * kTileBlocks + i, h[4 * s] + h[4 * s + 1] + h[4 * s + 2] + h[4 * s + 3]);
-      __syncwarp();
+    uint64_t rs = 0;
+    uint32_t rl = 0;
+    if (lane < PW) {
+      const uint64_t k = tl * TB + warp * PW + lane;
+      if (k < J.c) any = count_range(J, which, k, &rs, &rl);
     }
-    // (Entries of a tile without counted blocks need no write: those of marked
-    // blocks are summed from the children or never read.)
+    if (FEW) {
+      const unsigned gl = lane % L, grp = lane / L, gpw = 32 / L;
+      for (uint32_t i0 = 0; i0 < PW; i0 += 2 * gpw) {
+        uint32_t acc[2][kFewSymbols] = {};
+        uint64_t s0[2];
+        uint32_t len[2];
+        bool al[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const uint32_t i = i0 + u * gpw + grp;
+          s0[u] = __shfl_sync(0xFFFFFFFFu, rs, i & 31);
+          len[u] = __shfl_sync(0xFFFFFFFFu, rl, i & 31);
+          if (i >= PW) len[u] = 0;
+          al[u] = (((uintptr_t)(T + s0[u])) & 15) == 0;
+        }
+        const uint32_t top = len[0] > len[1] ? len[0] : len[1];
+        for (uint32_t x = 16 * gl; x < top; x += 16 * L) {
+          uint4 v[2];
+#pragma unroll
+          for (int u = 0; u < 2; u++) v[u] = range16(T, s0[u], len[u], x, al[u]);
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            if (x >= len[u]) continue;
+            const uint32_t have = len[u] - x;  // bytes of the unit that count
+            const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+            uint32_t keep[4];
+#pragma unroll
+            for (uint32_t q = 0; q < 4; q++)
+              keep[q] = have >= 4 * q + 4 ? 0xFFFFFFFFu : have <= 4 * q ? 0u : (1u << (8 * (have - 4 * q))) - 1u;
+#pragma unroll
+            for (uint32_t s = 0; s < kFewSymbols; s++) {
+              if (s >= S) break;
+              const uint32_t cc = byte_of[s] * 0x01010101u;
+#pragma unroll
+              for (uint32_t q = 0; q < 4; q++) acc[u][s] += __popc(__vcmpeq4(w[q], cc) & keep[q]);
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const uint32_t i = i0 + u * gpw + grp;
+#pragma unroll
+          for (uint32_t s = 0; s < kFewSymbols; s++) {
+            if (s >= S) break;
+            uint32_t v = acc[u][s];
+            for (unsigned o = L / 2; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+            if (gl == 0 && i < PW) rows[s * TB + warp * PW + i] = (uint16_t)(v >> 3);
+          }
+        }
+      }
+    } else {
+      const uint32_t cpy = lane & 3;
+      uint4 next[2];  // the first 512 bytes of the next two blocks
+#pragma unroll
+      for (int u = 0; u < 2; u++) {
+        const uint64_t s0 = __shfl_sync(0xFFFFFFFFu, rs, u);
+        const uint32_t len = __shfl_sync(0xFFFFFFFFu, rl, u);
+        next[u] = range16(T, s0, len, 16 * lane, (((uintptr_t)(T + s0)) & 15) == 0);
+      }
+      for (uint32_t i = 0; i < PW; i += 2) {
+        for (uint32_t z = lane; z < 2 * S; z += 32) ((uint4*)h)[z] = make_uint4(0, 0, 0, 0);
+        uint4 cur[2] = {next[0], next[1]};
+        if (i + 2 < PW) {
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            const uint64_t s0 = __shfl_sync(0xFFFFFFFFu, rs, i + 2 + u);
+            const uint32_t len = __shfl_sync(0xFFFFFFFFu, rl, i + 2 + u);
+            next[u] = range16(T, s0, len, 16 * lane, (((uintptr_t)(T + s0)) & 15) == 0);
+          }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const uint64_t s0 = __shfl_sync(0xFFFFFFFFu, rs, i + u);
+          const uint32_t len = __shfl_sync(0xFFFFFFFFu, rl, i + u);
+          uint32_t* hu = h + 4 * S * u + cpy;
+          const bool al = (((uintptr_t)(T + s0)) & 15) == 0;
+          for (uint32_t x = 16 * lane; x < len; x += 512) {
+            const uint4 v = x < 512 ? cur[u] : range16(T, s0, len, x, al);
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+            const uint32_t have = len - x;
+#pragma unroll
+            for (uint32_t q = 0; q < 16; q++)
+              if (q < have) atomicAdd(&hu[4 * sym[(w[q >> 2] >> (8 * (q & 3))) & 0xFF]], 1u);
+          }
+        }
+        __syncwarp();
+        for (uint32_t s = lane; s < S; s += 32) {
+          const uint4 a = ((const uint4*)h)[s], b = ((const uint4*)h)[S + s];
+          *(uint32_t*)(rows + s * TB + warp * PW + i) = (a.x + a.y + a.z + a.w) | ((b.x + b.y + b.z + b.w) << 16);
+        }
+        __syncwarp();
+      }
+    }
+    // (A tile without counted entries needs no write: those of marked blocks
+    // are summed from the children or never read.)
     if (!__syncthreads_or(any)) continue;
-    const uint32_t words = kTileBlocks * J.cw / 4;
-    const uint64_t have = (J.cp - tl * kTileBlocks) * J.cw / 4;  // words of the row from the tile on
-    for (uint32_t i = threadIdx.x; i < S * words; i += 256) {
-      const uint32_t s = i / words, w = i - s * words;
+    const uint64_t have = (J.cp - tl * TB) / 2;  // words of the row from the tile on
+    for (uint32_t i = threadIdx.x; i < S * (TB / 2); i += 256) {
+      const uint32_t s = i / (TB / 2), w = i % (TB / 2);
       if (w >= have) continue;
-      ((uint32_t*)(out + ((uint64_t)s * J.cp + tl * kTileBlocks) * J.cw))[w] = ((const uint32_t*)rows)[s * words + w];
+      ((uint32_t*)(out + (uint64_t)s * J.cp + tl * TB))[w] = ((const uint32_t*)rows)[i];
     }
   }
 }
@@ -214,11 +329,14 @@ __global__ void __launch_bounds__(256) k_count_long(CountLevel J, const int16_t*
 }
 
 // Marked blocks of a non-last level: sums of their children's counters.  A
-// thread per block and eighth of the symbols (blockIdx.y): neighbouring marked
-// blocks read neighbouring children.
+// thread per block and group of symbols (blockIdx.y): neighbouring marked
+// blocks read neighbouring children.  Four symbols at a time, so that their
+// reads are in flight together: bound by latency, 278 us with one at a time on
+// 0.88 M blocks of 96 symbols.
+template <uint32_t CW, uint32_t CCW>
 __global__ void __launch_bounds__(256) k_sum_children(CountLevel J, const uint32_t* __restrict__ mr, uint32_t arity,
-                                                      uint64_t bn, const void* __restrict__ child_cnt, uint32_t child_cw,
-                                                      uint64_t child_cp, uint32_t S) {
+                                                      uint64_t bn, const void* __restrict__ child_cnt, uint64_t child_cp,
+                                                      uint32_t S) {
   const uint32_t s0 = (uint32_t)((uint64_t)S * blockIdx.y / gridDim.y), s1 = (uint32_t)((uint64_t)S * (blockIdx.y + 1) / gridDim.y);
   for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < J.c; k += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t word = J.mw[k >> 5];
@@ -226,8 +344,23 @@ __global__ void __launch_bounds__(256) k_sum_children(CountLevel J, const uint32
     const uint64_t len = J.n - J.st[k] < J.b ? J.n - J.st[k] : J.b;
     const uint64_t first = (mr[k >> 5] + __popc(word & ((1u << (k & 31)) - 1u))) * (uint64_t)arity;
     const uint32_t nch = (uint32_t)((len + bn - 1) / bn);
-    for (uint32_t s = s0; s < s1; s++)
-      cput(J.cnt, J.cw, (uint64_t)s * J.cp + k, sum_run(child_cnt, child_cw, (uint64_t)s * child_cp + first, nch));
+    uint32_t s = s0;
+    if (nch == 4 && arity == 4) {  // one read per symbol
+      for (; s + 4 <= s1; s += 4) {
+        Run4 v[4];
+#pragma unroll
+        for (uint32_t u = 0; u < 4; u++) read_run(v[u], child_cnt, CCW, (uint64_t)(s + u) * child_cp + first, 4);
+#pragma unroll
+        for (uint32_t u = 0; u < 4; u++) {
+          const uint32_t x = CCW == 1   ? __dp4a(v[u].v[0], 0x01010101u, 0u)
+                             : CCW == 2 ? (v[u].v[0] & 0xFFFFu) + (v[u].v[0] >> 16) + (v[u].v[1] & 0xFFFFu) + (v[u].v[1] >> 16)
+                                        : v[u].v[0] + v[u].v[1] + v[u].v[2] + v[u].v[3];
+          cput(J.cnt, CW, (uint64_t)(s + u) * J.cp + k, x);
+        }
+      }
+    }
+    for (; s < s1; s++)
+      cput(J.cnt, CW, (uint64_t)s * J.cp + k, sum_run(child_cnt, CCW, (uint64_t)s * child_cp + first, nch));
   }
 }
 
@@ -267,16 +400,28 @@ __global__ void __launch_bounds__(1024) k_base_prefix(uint64_t c, const void* __
   if (threadIdx.x == 0) pre[s * (c + 1) + c] = carry;
 }
 
-__global__ void k_leaf_text(uint64_t c, uint64_t b, uint64_t n, const uint64_t* __restrict__ st,
-                            const uint32_t* __restrict__ mw, const uint32_t* __restrict__ mr,
-                            const uint8_t* __restrict__ T, uint8_t* __restrict__ leaf) {
-  for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < c * b;
+// Text of the marked last-level blocks, block of rank r at r b.  VEC: b, and
+// so every start, is a multiple of 16 and the text aligned: 16 bytes per thread.
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_leaf_text(uint64_t c, uint64_t b, uint64_t n, const uint64_t* __restrict__ st,
+                                                   const uint32_t* __restrict__ mw, const uint32_t* __restrict__ mr,
+                                                   const uint8_t* __restrict__ T, uint8_t* __restrict__ leaf) {
+  const uint32_t unit = VEC ? 16 : 1;
+  const uint64_t per = b / unit;
+  const uint32_t shift = (per & (per - 1)) == 0 ? 63 - __clzll(per) : 64;
+  for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < c * per;
        w += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t k = w / b, i = w - k * b;
-    if (!((mw[k >> 5] >> (k & 31)) & 1u)) continue;
-    if (st[k] + i >= n) continue;
-    uint64_t r = mr[k >> 5] + __popc(mw[k >> 5] & ((1u << (k & 31)) - 1u));
-    leaf[r * b + i] = T[st[k] + i];
+    const uint64_t k = shift < 64 ? w >> shift : w / per, i = (w - k * per) * unit;
+    const uint32_t word = mw[k >> 5];
+    if (!((word >> (k & 31)) & 1u)) continue;
+    const uint64_t x = st[k] + i;
+    if (x >= n) continue;
+    uint8_t* to = leaf + (uint64_t)(mr[k >> 5] + __popc(word & ((1u << (k & 31)) - 1u))) * b + i;
+    if (VEC && x + 16 <= n) {
+      *(uint4*)to = *(const uint4*)(T + x);
+    } else {
+      for (uint32_t q = 0; q < unit && x + q < n; q++) to[q] = T[x + q];
+    }
   }
 }
 
@@ -422,24 +567,6 @@ __device__ __forceinline__ uint64_t q_access(const QTree& t, const LevelView* __
   return kNone;
 }
 
-// Up to four counters of one symbol as read, and how many of them count:
-// their sum is taken when it is needed.
-struct Run4 {
-  uint32_t v[4];
-  uint32_t m;
-};
-__device__ __forceinline__ void read_run(Run4& r, const void* cnt, uint32_t w, uint64_t i, uint32_t m) {
-  r.m = m;
-  if (w == 1) {
-    r.v[0] = *(const uint32_t*)((const uint8_t*)cnt + i);
-  } else if (w == 2) {
-    const uint2 q = *(const uint2*)((const uint16_t*)cnt + i);
-    r.v[0] = q.x, r.v[1] = q.y;
-  } else {
-    const uint4 q = *(const uint4*)((const uint32_t*)cnt + i);
-    r.v[0] = q.x, r.v[1] = q.y, r.v[2] = q.z, r.v[3] = q.w;
-  }
-}
 __device__ __forceinline__ uint32_t run_sum(const Run4& r, uint32_t w) {  // of the first m <= 3
   if (r.m == 0) return 0;
   if (w == 1) return __dp4a(r.v[0] & ((1u << (8 * r.m)) - 1u), 0x01010101u, 0u);
@@ -743,6 +870,20 @@ static uint32_t base_level(const bt_tree* t, uint32_t last) {
   return base;
 }
 
+// The tile counter of 256 symbols needs 96.25 KiB of shared memory:
+// opted in once per device.
+static int allow_count_smem() {
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  BT_CUDA(cudaGetDevice(&dev));
+  const uint64_t bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return BT_OK;
+  BT_CUDA(cudaFuncSetAttribute(k_count_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               256 * kTileMany * 2 + 256 + 8 * 8 * 256 * 4));
+  done.fetch_or(bit, std::memory_order_acq_rel);
+  return BT_OK;
+}
+
 int build_counters(BuildCtx& ctx) {
   bt_tree* t = ctx.t;
   cudaStream_t s = ctx.s;
@@ -774,8 +915,14 @@ int build_counters(BuildCtx& ctx) {
       BT_LAUNCH(k_count_small<<<dim3((unsigned)((v.c + kSmallCountThreads - 1) / kSmallCountThreads), 2),
                                 kSmallCountThreads, sm, s>>>(J, t->sym, ctx.T, S));
     } else if (v.cw == 2) {
-      const size_t sm = 8ull * 4 * S * 4 + (size_t)S * kTileBlocks * v.cw + 256;
-      BT_LAUNCH(k_count_tile<<<dim3(grid_for(v.c, kTileBlocks, 152 * 8), 2), 256, sm, s>>>(J, t->sym, ctx.T, S));
+      const dim3 grid(grid_for(v.c, S <= kFewSymbols ? kTileFew : kTileMany, 152 * 16), 2);
+      const size_t rows = (size_t)S * (S <= kFewSymbols ? kTileFew : kTileMany) * 2 + 256, hists = 8ull * 8 * S * 4;
+      if (S <= kFewSymbols) {
+        BT_LAUNCH(k_count_tile<true><<<grid, 256, rows, s>>>(J, t->sym, ctx.T, S));
+      } else {
+        BT_TRY(allow_count_smem());
+        BT_LAUNCH(k_count_tile<false><<<grid, 256, rows + hists, s>>>(J, t->sym, ctx.T, S));
+      }
     } else {
       BT_CUDA(cudaMemsetAsync(mem, 0, 2 * half, s));
       const uint64_t ppb = (v.b + kCountPiece - 1) / kCountPiece;
@@ -784,8 +931,14 @@ int build_counters(BuildCtx& ctx) {
     }
     if (children_counted) {
       const Level& w = t->lv[l + 1];
-      BT_LAUNCH(k_sum_children<<<dim3(grid_for(v.c, T), S < 8 ? 1 : 8), T, 0, s>>>(J, v.mr, v.arity, w.b, w.cnt, w.cw,
-                                                                                  counter_stride(w.c), S));
+      const dim3 grid(grid_for(v.c, T), S < 8 ? 1 : 8);
+      auto sum = [&](auto kernel) {
+        BT_LAUNCH(kernel<<<grid, T, 0, s>>>(J, v.mr, v.arity, w.b, w.cnt, counter_stride(w.c), S));
+      };
+      if (v.cw == 1) sum(k_sum_children<1, 1>);
+      else if (v.cw == 2) w.cw == 1 ? sum(k_sum_children<2, 1>) : sum(k_sum_children<2, 2>);
+      else if (w.cw == 1) sum(k_sum_children<4, 1>);
+      else w.cw == 2 ? sum(k_sum_children<4, 2>) : sum(k_sum_children<4, 4>);
     }
     BT_CUDA(cudaGetLastError());
   }
@@ -799,7 +952,10 @@ int build_counters(BuildCtx& ctx) {
   BT_CUDA(cudaStreamSynchronize(s));
   t->leaf_bytes = (uint64_t)nm * z.b;
   BT_CUDA(cudaMallocAsync(&t->leaf, t->leaf_bytes + 16, s));
-  BT_LAUNCH(k_leaf_text<<<grid_for(z.c * z.b, T), T, 0, s>>>(z.c, z.b, t->n, z.st, z.mw, z.mr, ctx.T, t->leaf));
+  if (z.b % 16 == 0 && ((uintptr_t)ctx.T & 15) == 0)
+    BT_LAUNCH(k_leaf_text<true><<<grid_for(z.c * (z.b / 16), T), T, 0, s>>>(z.c, z.b, t->n, z.st, z.mw, z.mr, ctx.T, t->leaf));
+  else
+    BT_LAUNCH(k_leaf_text<false><<<grid_for(z.c * z.b, T), T, 0, s>>>(z.c, z.b, t->n, z.st, z.mw, z.mr, ctx.T, t->leaf));
   BT_CUDA(cudaGetLastError());
   // Real leaf length: the tail block may be short.
   uint64_t tail_short = 0;

@@ -348,56 +348,77 @@ __device__ __forceinline__ uint32_t pair_dist(const uint32_t* __restrict__ A, co
 constexpr uint32_t kBlkDiffers = 1, kPairDiffers = 2;
 
 // Compare every block and pair with the bytes at its bound s - min D (at 0
-// when the bound is negative): flags[k] says which differ.  One group of L
-// lanes per piece of 4 KiB of the pair; the block's comparison is the first
-// half of the pair's when both have the same bound.  Bound: the text's
-// bandwidth, both sides.
+// when the bound is negative): flags[k] says which differ.  A group of L lanes
+// per piece of the pair; the block's comparison is the first half of the
+// pair's when both have the same bound.  Bound: instruction issue (nearly every
+// block is looked at, few bytes each), so a lane takes about four 16-byte
+// units rather than one -- the item's bookkeeping is then shared by more
+// lanes' worth of text -- and positions are 32 bits.  With one unit per lane
+// and 64-bit positions: 836 us on the 256 MiB text and 6.4 ms on 2 GiB of DNA
+// copies (55-70 % of the issue slots, 10-13 % of DRAM).
 __global__ void __launch_bounds__(kT) k_quick_compare(QGeo g, const uint32_t* __restrict__ A, const uint32_t* __restrict__ X,
-                                                      uint32_t* __restrict__ flags, uint64_t ppk, unsigned L) {
+                                                      uint32_t* __restrict__ flags, uint32_t ppk, unsigned L) {
   const unsigned lane = threadIdx.x & 31, grp = lane / L, gl = lane % L, gpw = 32 / L;
   const unsigned gmask = (L == 32 ? 0xFFFFFFFFu : ((1u << L) - 1u)) << (grp * L);
   const bool aligned16 = (((uintptr_t)g.T) & 15) == 0;
-  const uint64_t warps = (uint64_t)gridDim.x * (kT / 32), total = g.c * ppk, piece = q_piece(g.b);
+  const uint32_t c = (uint32_t)g.c, n = (uint32_t)g.n, bl = (uint32_t)(g.b < g.n ? g.b : g.n);
+  const uint32_t warps = gridDim.x * (kT / 32), total = c * ppk, piece = (uint32_t)q_piece(g.b);
   // Warp-uniform loop: every lane reaches the ballots of every iteration.
-  for (uint64_t base = (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32 * gpw; base < total; base += warps * gpw) {
-    const uint64_t u = base + grp;
+  for (uint32_t base = (blockIdx.x * kT + threadIdx.x) / 32 * gpw; base < total; base += warps * gpw) {
+    const uint32_t u = base + grp;
     bool db = false, dp = false;
-    uint64_t k = 0;
+    uint32_t k = 0;
     if (u < total) {
       k = ppk == 1 ? u : u / ppk;
-      const uint64_t off = ppk == 1 ? 0 : (u - k * ppk) * piece;
-      const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
-      const uint32_t dk = A[k];
-      const bool blk = dk != 0 && dk != kNoDist && s != 0 && off < len;
+      const uint32_t off = ppk == 1 ? 0 : (u - k * ppk) * piece;
+      const uint32_t s = (uint32_t)g.st[k], dk = A[k], xk = X[k];
+      const bool more = k + 1 < c;
+      const uint32_t s1 = more ? (uint32_t)g.st[k + 1] : 0, d1 = more ? A[k + 1] : 0;
+      const uint32_t f = ppk > 1 ? *(volatile uint32_t*)&flags[k] : 0u;  // (another piece may have settled it)
+      const uint32_t len = n - s < bl ? n - s : bl;
+      const bool blk = dk != 0 && dk != kNoDist && s != 0 && off < len && !(f & kBlkDiffers);
       bool pair = false;
-      uint32_t d2 = 0;
-      uint64_t plen = 0;
-      if (k + 1 < g.c && s != 0 && g.st[k + 1] == s + len) {
-        const uint64_t len2 = g.n - s - len < g.b ? g.n - s - len : g.b;
+      uint32_t d2 = 0, plen = 0;
+      if (more && s != 0 && s1 == s + len) {
+        const uint32_t len2 = n - s1 < bl ? n - s1 : bl;
         plen = len + len2;
-        d2 = pair_dist(A, X, k, len2);
-        pair = d2 != 0 && d2 != kNoDist && off < plen;
+        d2 = min(dk, xk);
+        if (len2 >= kGramLen) d2 = min(d2, d1);
+        pair = d2 != 0 && d2 != kNoDist && off < plen && !(f & kPairDiffers);
       }
-      // (Flags another piece has set spare this one; pieces are many only when blocks are long.)
-      const uint32_t f = ppk > 1 && (blk || pair) ? *(volatile uint32_t*)&flags[k] : 0u;
-      const uint64_t pk = dk > s ? 0 : s - dk, pp = d2 > s ? 0 : s - d2;
-      const uint64_t bend = off + piece < len ? off + piece : len;
-      const uint64_t pend = off + piece < plen ? off + piece : plen;
-      if (blk && pair && pk == pp && !(f & kPairDiffers) && aligned16 && ((s | len | plen | off) & 15) == 0) {
-        // One bound for both: the block's bytes are the pair's first half.
-        for (uint64_t y = off + 16ull * gl; y < pend; y += 16ull * L) {
-          const bool d = differ16(g.T, pk + y, s + y);
-          dp |= d;
-          db |= d && y < len;
-        }
-      } else {
-        if (blk && !(f & kBlkDiffers)) {
-          db = differs(g.T, g.n, aligned16, pk, s, off, bend, gl, L);
-          if (pair && pk == pp) dp = db;
-        }
-        if (pair && !(f & kPairDiffers)) {
-          const uint64_t from = blk && pk == pp ? (off < bend ? bend : off) : off;
-          if (from < pend) dp |= differs(g.T, g.n, aligned16, pp, s, from, pend, gl, L);
+      if (blk || pair) {
+        const uint32_t pk = dk > s ? 0 : s - dk, pp = d2 > s ? 0 : s - d2;
+        const uint32_t bend = min(off + piece, len), pend = min(off + piece, plen);
+        const bool one = blk && pair && pk == pp;
+        if (aligned16 && ((s | len | off) & 15) == 0 && (!pair || (plen & 15) == 0)) {
+          // One bound for both: the block's bytes are the pair's first half.
+          if (blk) {
+            const Shift16 sh(pk);
+            for (uint32_t y = off + 16 * gl; y < (one ? pend : bend); y += 32 * L) {
+              const uint32_t y2 = y + 16 * L < (one ? pend : bend) ? y + 16 * L : y;
+              const Unit16 a = load_units(g.T, pk + y, s + y), b = load_units(g.T, pk + y2, s + y2);
+              const bool da = sh.differ(a), dc = sh.differ(b);
+              if (one) dp |= da | dc;
+              db |= (da && y < len) || (dc && y2 < len);
+            }
+          }
+          if (pair && !one) {
+            const Shift16 sh(pp);
+            for (uint32_t y = off + 16 * gl; y < pend; y += 32 * L) {
+              const uint32_t y2 = y + 16 * L < pend ? y + 16 * L : y;
+              const Unit16 a = load_units(g.T, pp + y, s + y), b = load_units(g.T, pp + y2, s + y2);
+              dp |= sh.differ(a) | sh.differ(b);
+            }
+          }
+        } else {
+          if (blk) {
+            db = differs(g.T, g.n, aligned16, pk, s, off, bend, gl, L);
+            if (one) dp = db;
+          }
+          if (pair) {
+            const uint32_t from = one ? max(off, bend) : off;
+            if (from < pend) dp |= differs(g.T, g.n, aligned16, pp, s, from, pend, gl, L);
+          }
         }
       }
     }
@@ -1355,8 +1376,10 @@ int quick_level(BuildCtx& ctx, QuickBuild& qb, uint32_t l, uint64_t last_start) 
   {
   ProfScope prof("window_scan", s, (c - 1) * b + (n - last_start < b ? n - last_start : b));
   BT_LAUNCH(k_quick_min<<<grid_for(c * G, kT), kT, 0, s>>>(g, qb.list, G, A, X, flags, qb.qs));
-  const uint64_t ppk = (2 * b + q_piece(b) - 1) / q_piece(b);
-  const unsigned L = b >= 256 ? 32u : b >= 128 ? 16u : b >= 64 ? 8u : 4u;
+  // (A block is at most n long, so c ppk < 2^32.)
+  const uint64_t bl = b < n ? b : n;
+  const uint32_t ppk = (uint32_t)((2 * bl + q_piece(b) - 1) / q_piece(b));
+  const unsigned L = b >= 1024 ? 32u : b >= 512 ? 16u : b >= 256 ? 8u : b >= 128 ? 4u : b >= 64 ? 2u : 1u;
   BT_LAUNCH(k_quick_compare<<<grid_for(c * ppk * L, kT), kT, 0, s>>>(g, A, X, flags, ppk, L));
   BT_LAUNCH(k_quick_settle<<<grid_for(c, kT, 152 * 8), kT, 0, s>>>(g, A, X, flags, v.lo, ps, items, v.mw, wpop, qb.qs, ctx.st));
   }

@@ -72,8 +72,8 @@ typedef struct {
                                   rest; 0 = default 4096.                     */
   uint32_t flags;              /* BT_FLAG_* (0 by default)                    */
   uint32_t batch_ctas;         /* bt_build_batch: CTAs of the batched kernel's
-                                  launch; 0 (default) = the autotuned shape
-                                  over every SM.  A smaller grid leaves SMs to
+                                  launch; 0 (default) = one per SM.
+                                  A smaller grid leaves SMs to
                                   other work, e.g. a second batch on another
                                   host thread.                                 */
   uint32_t partitions;         /* with BT_FLAG_SORT_SCAN: the number K of parts
@@ -107,11 +107,9 @@ typedef struct {
  * from otherwise; at most 2 leaf_len bytes).  Same tree and same answers,
  * fewer device bytes, slower rank and select at the last level.  Single-text
  * builds only (bt_build_batch ignores it). */
-/* BT_FLAG_ANCHOR_ALL (a test hook of bt_build_batch): the batched kernel
- * scans every level with blocks of 32 bytes or more by anchors (by default
- * only levels with blocks of 1024 bytes or more), so that its anchored scan
- * and the 8-byte prefix filter of blocks without an anchor run on short
- * blocks too.  The same trees. */
+/* BT_FLAG_ANCHOR_ALL is accepted and has no effect: the batched kernel takes
+ * every level of blocks of 27 bytes or more by first occurrences of selected
+ * grams, as the single-text path does. */
 /* BT_FLAG_SORT_SCAN: the sort-based level pass of the paper's section 4.1
  * instead of the table probes: every window of length b (then 2b) inside a
  * run becomes a (fingerprint, position) tuple, the tuples are radix-sorted
@@ -180,15 +178,12 @@ int bt_build_batch(const uint8_t* const* texts, const uint64_t* ns, const uint32
  * u64: documents built by the batched kernel, documents built by host
  * workers, kernel launches, documents built a second time because the output
  * pool ran out, threads per CTA, CTAs per SM, output pool bytes, CTA scratch
- * bytes, the largest grid, the scan's window run (consecutive positions per
- * lane), the autotuner's trial builds in this call, the microseconds the
- * host spent issuing the texts' copies to the device (the copies themselves
- * when the texts are in pageable memory) and the microseconds of device time
- * of the batched kernel's launches.  The launch shape (threads, CTAs per SM,
- * run) of a batch of 1024 or more documents is chosen the first time a batch
- * of its size class is built, and cached for the process: each candidate
- * builds a seeded sample of the batch, and the one whose measured cycles per
- * byte and level give the shortest simulated batch wins.  bt_batch_cycles: for a tree from the batched
+ * bytes, the largest grid, two zeros (formerly
+ * the tuned window run and the trial builds: the kernel has one launch shape
+ * and nothing to tune), the microseconds the host spent issuing the texts'
+ * copies to the device (the copies themselves when the texts are in pageable
+ * memory) and the microseconds of device time of the batched kernel's
+ * launches.  bt_batch_cycles: for a tree from the batched
  * kernel, the SM clock cycles its CTA spent per phase (6 u64: set-up,
  * tables, window scan, verification/marks/pointers/split, pruning, output
  * and counters); zeros for other trees.  BT_EINVAL for null pointers or cap

@@ -365,7 +365,7 @@ class BuildOptions:
     leaf_counts: bool = False  # no stored counters on the last level (space-efficient rank/select)
     sort_scan: bool = False  # leftmost windows by radix-sorting (fingerprint, position) tuples
     partitions: int = 0  # with sort_scan: parts of the domain decomposition (0 or 1: one)
-    anchor_all: bool = False  # bt_build_batch test hook: anchored scan on every level of 32+ byte blocks
+    anchor_all: bool = False  # accepted, no effect
 
     def to_c(self):
         o = bt_opts_default()

@@ -23,14 +23,9 @@ int alphabet(const uint8_t* T, uint64_t n, uint32_t sigma, bt_tree* t, cudaStrea
 int run_query_one(const bt_tree* t, int kind, uint64_t a0, uint64_t a1, uint64_t* out, cudaStream_t s);
 int batch_kernel_build(const uint8_t* const* texts, const uint64_t* ns, const uint32_t* sigmas,
                        const uint32_t* taus, const uint32_t* leaf_lens, uint64_t ndocs, const bt_opts& o,
-                       std::vector<char>& routed, bt_tree** outs, uint32_t threads, uint32_t ctas_per_sm,
-                       uint32_t chunk, cudaStream_t s, const std::vector<char>* eligible);
+                       std::vector<char>& routed, bt_tree** outs, cudaStream_t s, const std::vector<char>* eligible);
 uint32_t batch_split(const uint64_t* ns, const uint32_t* taus, const uint32_t* leaf_lens, uint64_t ndocs,
-                     const bt_opts& o, uint32_t ctas_per_sm, std::vector<char>& eligible);
-int batch_shape(const uint8_t* const* texts, const uint64_t* ns, const uint32_t* sigmas, const uint32_t* taus,
-                const uint32_t* leaf_lens, uint64_t ndocs, const bt_opts& o, cudaStream_t s, uint32_t* threads,
-                uint32_t* ctas_per_sm, uint32_t* chunk, uint64_t* tuned_now);
-void batch_report_tuned(uint64_t trials);
+                     const bt_opts& o, std::vector<char>& eligible);
 void batch_report_workers(uint64_t docs);
 void batch_report_reset();
 int run_queries(const bt_tree* t, int kind, const uint64_t* d_args, uint64_t m, uint64_t* d_out,
@@ -459,12 +454,9 @@ int bt_build_batch(const uint8_t* const* texts, const uint64_t* ns, const uint32
     int device = 0;
     if (cudaGetDevice(&device) == cudaSuccess) keep_pool_memory(device);
     cudaGetLastError();
-    uint32_t threads = 0, ctas = 0, chunk = 0;
-    uint64_t trials = 0;
-    rc = batch_shape(texts, ns, sigmas, taus, leaf_lens, ndocs, o, s, &threads, &ctas, &chunk, &trials);
     std::vector<char> eligible;
     bt_opts ok = o;
-    const uint32_t cap = rc == BT_OK ? batch_split(ns, taus, leaf_lens, ndocs, o, ctas, eligible) : 0;
+    const uint32_t cap = batch_split(ns, taus, leaf_lens, ndocs, o, eligible);
     std::thread split_thread;
     if (cap) {
       ok.batch_ctas = cap;
@@ -484,9 +476,8 @@ int bt_build_batch(const uint8_t* const* texts, const uint64_t* ns, const uint32
     }
     if (rc == BT_OK && rc_split == BT_OK) {
       batch_report_reset();
-      rc = batch_kernel_build(texts, ns, sigmas, taus, leaf_lens, ndocs, ok, routed, outs, threads, ctas, chunk,
-                              s, cap ? &eligible : nullptr);
-      batch_report_tuned(trials);
+      rc = batch_kernel_build(texts, ns, sigmas, taus, leaf_lens, ndocs, ok, routed, outs, s,
+                              cap ? &eligible : nullptr);
     }
     if (split_thread.joinable()) split_thread.join();
     if (rc == BT_OK) rc = rc_split;

@@ -7,21 +7,17 @@
 // itself:
 //
 //   1. alphabet (byte histogram -> dense symbol map, sigma check);
-//   2. Karp-Rabin prefix fingerprints H(p) at every position (section 2, the
-//      all-prefix form of section 4.1: Horner per 32-byte chunk, then a scan
-//      of the chunks with (h1, P1) (x) (h2, P2) = (h1 P2 + h2, P1 P2)), and
-//      the list of selected 16-byte grams (the scan's anchors on levels of
-//      long blocks);
-//   3. for every level (section 3): block and pair fingerprints into
-//      open-addressing tables, a scan of the windows of the level's runs of
-//      consecutive blocks (section 3.1: phi(p, p+b) = H(p+b) - H(p) B^b,
-//      rolled from window to window, or only the windows that the selected
-//      grams propose on levels of long blocks; table probe, atomicMin of the
-//      leftmost window per key, the pair joined at p+b), byte verification
-//      of every accepted minimum with an exact
-//      rescan of a key whose fingerprint collided, marks (a pair is marked
-//      when its leftmost occurrence is its own start, a block in no pair is
-//      marked), back-pointers (ptr, off), and the tau-way split of marked
+//   2. Karp-Rabin prefix fingerprints H(32 j) (section 2, the all-prefix form of
+//      section 4.1) and the list of selected grams with the distances to their
+//      first occurrences (bt_quick.cu);
+//   3. for every level (section 3) of blocks of 27 bytes or more the steps of
+//      bt_quick.cu over the CTA: bounds from the list, byte comparisons, and a
+//      search of the list for the keys left open; for shorter blocks block and
+//      pair fingerprints in open-addressing tables and a scan of every window
+//      (section 3.1), byte verification of every accepted minimum with an
+//      exact rescan of a key whose fingerprint collided.  Then marks (a pair is
+//      marked when its leftmost occurrence is its own start, a block in no pair
+//      is marked), back-pointers (ptr, off), and the tau-way split of marked
 //      blocks into the next level;
 //   4. the pruning post-pass (section 3.1, "Optional Pruning"), with the same
 //      four conditions and the same right-to-left rule as the standard path,
@@ -50,6 +46,7 @@
 #include <chrono>
 
 #include "bt_batch.cuh"
+#include "bt_quick_dev.cuh"
 
 namespace bt {
 
@@ -62,6 +59,9 @@ namespace {
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kBTailPair = 0xFFFFFFFEu;
 constexpr uint32_t kMaxBThreads = 1024;
+// 32-bit words of dynamic shared memory: the open keys' queues and bitmap, the
+// window filter, the counters' histograms and tiles, one after the other.
+constexpr uint32_t kDynWords = 32768;
 
 struct __align__(32) BSlot {
   unsigned long long key, lo, maxpst, pad;
@@ -90,16 +90,18 @@ struct Cta {
   uint64_t stats[kBMaxLevels][BT_ST_FIELDS];
   uint64_t last_start;
   // current level
-  uint64_t r, Bb, Br, B1;
+  uint64_t r, Bb, Br;
   uint64_t bmask, pmask;
-  uint64_t rtab[256];  // (a + 1) B^b for every byte a
   uint32_t bshift;
   unsigned long long fp_tail, lo_tail, lo_tailpair;
   uint32_t pretail;
   unsigned int npairs, njobs, nsusp;
-  uint32_t nsel;                      // selected grams of the document (kNoList: none kept)
-  unsigned int anchorless;            // some key of the level has no selected gram
-  uint32_t tail_g, tail_a, tail_anchored;  // anchor of the short tail key
+  uint32_t nsel;                      // entries of the list of selected grams
+  int expanded;                       // H holds every position (the list is gone)
+  QList list;
+  Chase chase;
+  QuickStatus qs;
+  Status status;
   unsigned long long verify_bytes, collisions;
   unsigned long long lastk;
   // scans
@@ -294,134 +296,83 @@ __device__ void verify_jobs(const uint8_t* __restrict__ T, const BJob* jobs, uin
 // ---------------------------------------------------------------------------
 // Document set-up: alphabet and prefix fingerprints.
 // ---------------------------------------------------------------------------
+// (Only which bytes occur matters: after a document's first lines every mark
+// is set, and looking costs no atomics and no conflicts on frequent bytes.)
 __device__ void alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t sigma, Cta& C) {
-  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) C.hist[i] = 0;
+  volatile unsigned int* seen = C.hist;
+  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) seen[i] = 0;
   __syncthreads();
   const uint64_t nv = n / 16;
   for (uint64_t i = threadIdx.x; i < nv; i += blockDim.x) {
     const uint4 q = ((const uint4*)T)[i];
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    uint32_t f[16];
 #pragma unroll
-    for (int a = 0; a < 4; a++)
+    for (int a = 0; a < 16; a++) f[a] = seen[(w[a >> 2] >> (8 * (a & 3))) & 0xFF];
 #pragma unroll
-      for (int s = 0; s < 4; s++) atomicAdd(&C.hist[(w[a] >> (8 * s)) & 0xFF], 1u);
+    for (int a = 0; a < 16; a++)
+      if (!f[a]) seen[(w[a >> 2] >> (8 * (a & 3))) & 0xFF] = 1;
   }
-  for (uint64_t i = nv * 16 + threadIdx.x; i < n; i += blockDim.x) atomicAdd(&C.hist[T[i]], 1u);
+  for (uint64_t i = nv * 16 + threadIdx.x; i < n; i += blockDim.x) seen[T[i]] = 1;
   __syncthreads();
   if (threadIdx.x == 0) {
     uint32_t S = 0;
-    for (int i = 0; i < 256; i++) C.sym[i] = C.hist[i] ? (int16_t)S++ : (int16_t)-1;
+    for (int i = 0; i < 256; i++) C.sym[i] = seen[i] ? (int16_t)S++ : (int16_t)-1;
     C.S = S;
     if (S > sigma) C.err = BT_EINVAL;
   }
   __syncthreads();
 }
 
-// H[p] for every p in [0, n]: chunks of 32 bytes, blockDim.x chunks per tile.
-// pw[i] = X^i with X = B^32, i <= 1024.
+// Hs[j] = H(32 j) for j <= n / 32: four chunks of 32 bytes per thread, their
+// byte dot products scanned over the CTA (as the prefix kernels of bt_scan.cu).
 template <class M>
-__device__ void prefix_pass(const M& m, const uint8_t* __restrict__ T, uint64_t n, uint64_t B,
-                            const uint64_t* __restrict__ pw, uint64_t* __restrict__ H, Cta& C) {
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const uint64_t tile = (uint64_t)blockDim.x * 32;
+__device__ void prefix_pass(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const uint8_t* T, uint64_t n,
+                            uint64_t* Hs, Cta& C) {
+  const uint64_t nchunks = n / 32;
   if (threadIdx.x == 0) C.carry = 0;
   __syncthreads();
-  for (uint64_t t0 = 0; t0 < n; t0 += tile) {
+  const uint64_t xl = kr_lane_pow(m, pw);
+  for (uint64_t t0 = 0; t0 <= nchunks; t0 += 4ull * blockDim.x) {
+    const uint64_t j0 = t0 + 4ull * threadIdx.x;
+    uint64_t c[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      uint32_t w[8];
+      load_chunk(T, nchunks, j0 + i, true, w);
+      c[i] = PC.hash(m, w);
+    }
+    uint64_t h = c[0];
+#pragma unroll
+    for (int i = 1; i < 4; i++) h = m.add(m.mul(h, PC.B32), c[i]);
     const uint64_t carry = C.carry;
-    const uint64_t p0 = t0 + 32ull * threadIdx.x;
-    const uint32_t cnt = p0 < n ? (uint32_t)(n - p0 < 32 ? n - p0 : 32) : 0u;
-    uint64_t h = 0;
-    if (cnt == 32) {
-      const uint4 v0 = *(const uint4*)(T + p0), v1 = *(const uint4*)(T + p0 + 16);
-      const uint32_t wv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-#pragma unroll
-      for (int i = 0; i < 32; i++) h = m.add(m.mul(h, B), (uint64_t)((wv[i >> 2] >> (8 * (i & 3))) & 0xFFu) + 1);
-    } else {
-      for (uint32_t i = 0; i < cnt; i++) h = m.add(m.mul(h, B), (uint64_t)T[p0 + i] + 1);
-    }
-    // Inclusive scan of the chunk values (each chunk shifts by X = B^32).
-    uint64_t x = h;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint64_t o = __shfl_up_sync(kFull, x, d);
-      if ((int)lane >= d) x = m.add(m.mul(o, pw[d]), x);
-    }
-    if (lane == 31) C.wsum[warp] = x;
+    if (threadIdx.x == 0) h = m.add(m.mul(carry, pw.x[0]), h);
+    const uint64_t incl = cta_kr_scan(m, h, pw, xl, C.wsum);
+    uint64_t up = __shfl_up_sync(kFull, incl, 1);
+    if ((threadIdx.x & 31) == 31) C.wsum[threadIdx.x >> 5] = incl;
+    if (threadIdx.x == blockDim.x - 1) C.carry = incl;
     __syncthreads();
-    if (warp == 0) {
-      uint64_t w = lane < nw ? C.wsum[lane] : 0ull;
+    if ((threadIdx.x & 31) == 0) up = threadIdx.x ? C.wsum[(threadIdx.x >> 5) - 1] : carry;
 #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint64_t o = __shfl_up_sync(kFull, w, d);
-        if ((int)lane >= d) w = m.add(m.mul(o, pw[32 * d]), w);
-      }
-      C.wsum[lane] = w;
+    for (int i = 0; i < 4; i++) {
+      if (j0 + i <= nchunks) Hs[j0 + i] = up;
+      up = m.add(m.mul(up, PC.B32), c[i]);
     }
-    __syncthreads();
-    const uint64_t wp = warp ? C.wsum[warp - 1] : 0ull;
-    const uint64_t incl = m.add(m.mul(wp, pw[lane + 1]), x);  // chunks [0, j] of the tile
-    const uint64_t up = __shfl_up_sync(kFull, incl, 1);
-    const uint64_t excl = lane ? up : wp;                      // chunks [0, j)
-    uint64_t hh = m.add(m.mul(carry, pw[threadIdx.x]), excl);  // H(p0)
-    if (cnt == 32) {
-      const uint4 v0 = *(const uint4*)(T + p0), v1 = *(const uint4*)(T + p0 + 16);
-      const uint32_t wv[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-#pragma unroll
-      for (int i = 0; i < 32; i++) {
-        H[p0 + i] = hh;
-        hh = m.add(m.mul(hh, B), (uint64_t)((wv[i >> 2] >> (8 * (i & 3))) & 0xFFu) + 1);
-      }
-    } else {
-      for (uint32_t i = 0; i < cnt; i++) {
-        H[p0 + i] = hh;
-        hh = m.add(m.mul(hh, B), (uint64_t)T[p0 + i] + 1);
-      }
-    }
-    if (cnt && p0 + cnt == n) H[n] = hh;
-    if (threadIdx.x == blockDim.x - 1) C.carry = m.add(m.mul(carry, pw[blockDim.x]), incl);
     __syncthreads();
   }
 }
 
-// ---------------------------------------------------------------------------
-// One level.
-// ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
-// Selected grams: the anchors of the window scan on levels with long blocks.
-// A window's anchor is its first 16-byte gram whose hash is selected; a
-// window equal to a key has the key's anchor gram at the key's anchor offset,
-// so on those levels only the selected grams of the level's runs are read and
-// each proposes the windows that would have it as their anchor.  The grams
-// are selected once per document; a level looks them up in the list.
-// ---------------------------------------------------------------------------
-constexpr uint32_t kNoList = 0xFFFFFFFFu;        // the list overflowed: no anchors
-constexpr unsigned long long kNoAnchor = ~0ull;  // empty anchor-table entry
-
-__device__ __forceinline__ uint32_t gram_hash(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
-  uint32_t h = w0 * 0x9E3779B1u;
-  uint32_t t = w1 * 0x85EBCA77u;
-  h ^= __funnelshift_l(t, t, 13);
-  t = w2 * 0xC2B2AE3Du;
-  h ^= __funnelshift_l(t, t, 7);
-  t = w3 * 0x27D4EB2Fu;
-  h ^= __funnelshift_l(t, t, 19);
-  h ^= h >> 16;
-  h *= 0x7FEB352Du;
-  h ^= h >> 15;
-  h *= 0x846CA68Bu;
-  h ^= h >> 16;
-  return h;
-}
-
-// Bit of the shared-memory filter for a window's first 8 bytes (lo, hi as
-// little-endian words), the test of the blocks that have no selected gram.
-__device__ __forceinline__ uint32_t prefix_bit(uint32_t lo, uint32_t hi, uint32_t fshift) {
-  const uint32_t t = hi * 0x85EBCA77u;
-  return ((lo * 0x9E3779B1u) ^ __funnelshift_l(t, t, 15)) * 0xC2B2AE3Du >> fshift;
-}
-
-__device__ __forceinline__ uint32_t anchor_slot(uint32_t g, uint64_t mask) {
-  return (uint32_t)(((uint64_t)g * 0x9E3779B97F4A7C15ull >> 32) & mask);
+// H[p] for every p in [0, n] (levels of blocks too short for the list).
+template <class M>
+__device__ void expand_pass(const M& m, const uint8_t* T, uint64_t n, uint64_t B, const uint64_t* Hs, uint64_t* H) {
+  for (uint64_t j = threadIdx.x; j <= n / 32; j += blockDim.x) {
+    uint64_t h = Hs[j];
+    for (uint64_t p = 32 * j; p < 32 * j + 32 && p <= n; p++) {
+      H[p] = h;
+      if (p < n) h = m.add(m.mul(h, B), (uint64_t)T[p] + 1);
+    }
+  }
+  __syncthreads();
 }
 
 // Exclusive sum of one value per thread over the CTA; *total = the sum.
@@ -451,62 +402,81 @@ __device__ uint32_t cta_excl_u32(uint32_t v, Cta& C, uint32_t* total) {
   return r;
 }
 
-// The selected grams of T[0, n) in text order: positions and hashes, at most
-// cap of them (C.nsel = their number, or kNoList if there are more).  A
-// thread takes 32 consecutive positions of a tile, from 12 aligned words
-// (the text is followed by at least 48 readable bytes).
-__device__ void gram_list_pass(const uint8_t* __restrict__ T, uint64_t n, uint32_t* __restrict__ lpos,
-                               uint32_t* __restrict__ lhash, uint64_t cap, Cta& C) {
-  if (threadIdx.x == 0) C.nsel = 0;
+// The list of selected grams (bt_quick.cu): a thread takes 32 positions of a
+// tile, the entries' places come from a CTA scan, then the first-occurrence
+// table, the distances and the segment minima.
+__device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
+  const unsigned tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const uint64_t nw = n < kGramLen ? 0 : (n - kGramLen + 1 + 31) / 32, ns = (n + kSegBytes - 1) / kSegBytes,
+                 ns2 = (ns + 63) / 64;
+  uint32_t* idx = (uint32_t*)(scr + C.sl.idx);
+  uint32_t* x = (uint32_t*)(scr + C.sl.big);
+  uint32_t* D = x + ((n + 63) & ~63ull);
+  uint32_t* first = (uint32_t*)(scr + C.sl.first);
+  uint32_t* seg1 = (uint32_t*)(scr + C.sl.seg1);
+  uint32_t* seg2 = (uint32_t*)(scr + C.sl.seg2);
+  const uint32_t cmask = (uint32_t)(C.sl.cells - 1);
+  for (uint64_t i = tid; i < C.sl.cells; i += nt) first[i] = 0xFFFFFFFFu;
+  uint32_t total = 0;
+  for (uint64_t j0 = 0; j0 < nw; j0 += nt) {
+    const uint64_t j = j0 + tid;
+    uint32_t bits = 0;
+    if (j < nw) {
+      bits = half_mask(T, n, 32 * j) | half_mask(T, n, 32 * j + 16) << 16;
+      const uint64_t left = n - kGramLen + 1 - 32 * j;
+      if (left < 32) bits &= (1u << left) - 1u;
+    }
+    uint32_t sum;
+    uint32_t o = total + cta_excl_u32(__popc(bits), C, &sum);
+    if (j < nw) idx[j] = o;
+    for (; bits; bits &= bits - 1, o++) {
+      const uint32_t p = (uint32_t)(32 * j) + __ffs(bits) - 1, sh = 8 * (p & 3);
+      const uint32_t* w = (const uint32_t*)(T + (p & ~3u));
+      const uint32_t w0 = w[0], w1 = w[1], w2 = w[2], w3 = w[3], w4 = w[4];
+      x[o] = p;
+      D[o] = gram_cell(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh),
+                       __funnelshift_r(w3, w4, sh), cmask);
+    }
+    total += sum;
+  }
+  if (tid == 0) {
+    idx[nw] = total;
+    C.nsel = total;
+    C.list = QList{idx, x, D, seg1, seg2, nw};
+  }
   __syncthreads();
-  const uint64_t npos = n >= kGramW ? n - kGramW + 1 : 0;
-  const uint64_t tile = (uint64_t)blockDim.x * 32;
-  for (uint64_t t0 = 0; t0 < npos; t0 += tile) {
-    const uint64_t x0 = t0 + 32ull * threadIdx.x;
-    uint32_t w[12];
-    uint32_t mask = 0;
-    if (x0 < npos) {
-      const uint32_t* wp = (const uint32_t*)(T + x0);
+  for (uint32_t e = tid; e < total; e += 4 * nt) {
+    uint32_t c[4], f[4];
 #pragma unroll
-      for (int k = 0; k < 12; k++) w[k] = wp[k];
+    for (uint32_t u = 0; u < 4; u++) c[u] = e + u * nt < total ? D[e + u * nt] : 0;
 #pragma unroll
-      for (int i = 0; i < 32; i++) {
-        const int q = i >> 2, sh = 8 * (i & 3);
-        const uint32_t h = gram_hash(__funnelshift_r(w[q], w[q + 1], sh), __funnelshift_r(w[q + 1], w[q + 2], sh),
-                                     __funnelshift_r(w[q + 2], w[q + 3], sh), __funnelshift_r(w[q + 3], w[q + 4], sh));
-        if ((h >> kGramSelShift) == 0 && x0 + i < npos) mask |= 1u << i;
-      }
-    }
-    uint32_t total;
-    const uint32_t before = cta_excl_u32(__popc(mask), C, &total);
-    const uint32_t base = C.nsel;
-    if (base != kNoList && (uint64_t)base + total <= cap) {
-      uint32_t o = base + before;
+    for (uint32_t u = 0; u < 4; u++) f[u] = *(volatile uint32_t*)&first[c[u]];
 #pragma unroll
-      for (int i = 0; i < 32; i++) {
-        if (!((mask >> i) & 1u)) continue;
-        const int q = i >> 2, sh = 8 * (i & 3);
-        lpos[o] = (uint32_t)(x0 + i);
-        lhash[o] = gram_hash(__funnelshift_r(w[q], w[q + 1], sh), __funnelshift_r(w[q + 1], w[q + 2], sh),
-                             __funnelshift_r(w[q + 2], w[q + 3], sh), __funnelshift_r(w[q + 3], w[q + 4], sh));
-        o++;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) C.nsel = (base == kNoList || (uint64_t)base + total > cap) ? kNoList : base + total;
-    __syncthreads();
+    for (uint32_t u = 0; u < 4; u++)
+      if (e + u * nt < total && f[u] > x[e + u * nt]) atomicMin(&first[c[u]], x[e + u * nt]);
   }
-}
-
-// First index i of the sorted a[0, n) with a[i] >= x.
-__device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t* __restrict__ a, uint32_t n, uint64_t x) {
-  uint32_t lo = 0, hi = n;
-  while (lo < hi) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (a[mid] < x) lo = mid + 1;
-    else hi = mid;
+  __syncthreads();
+  for (uint32_t e = tid; e < total; e += 4 * nt) {
+    uint32_t f[4];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; u++) f[u] = e + u * nt < total ? *(volatile uint32_t*)&first[D[e + u * nt]] : 0;
+#pragma unroll
+    for (uint32_t u = 0; u < 4; u++)
+      if (e + u * nt < total) D[e + u * nt] = x[e + u * nt] - f[u];
   }
-  return lo;
+  __syncthreads();
+  for (uint64_t j = tid / 32; j < ns; j += nt / 32) {
+    const uint64_t w0 = j * (kSegBytes / 32), w1 = w0 + kSegBytes / 32 < nw ? w0 + kSegBytes / 32 : nw;
+    const uint32_t d = __reduce_min_sync(kFull, min_entries(D, idx[w0 < nw ? w0 : nw], idx[w1], lane, 32, kNoDist));
+    if (lane == 0) seg1[j] = d;
+  }
+  __syncthreads();
+  for (uint64_t j = tid; j < ns2; j += nt) {
+    uint32_t d = kNoDist;
+    for (uint64_t i = 64 * j; i < 64 * j + 64 && i < ns; i++) d = min(d, seg1[i]);
+    seg2[j] = d;
+  }
+  __syncthreads();
 }
 
 struct Work {
@@ -518,7 +488,6 @@ struct Work {
   BJob* jobs;
   BSlot* bt;
   PSlot* pt;
-  unsigned long long* at;  // anchor table: (gram hash << 32) | anchor offset
 };
 
 __device__ __forceinline__ char* carve(char*& p, uint64_t bytes) {
@@ -544,7 +513,6 @@ __device__ Work carve_level(char* temp, uint64_t c, uint64_t bcap, uint64_t pcap
   carve(p, c * 8 + 8);
   W.bt = (BSlot*)carve(p, bcap * 32);
   W.pt = (PSlot*)carve(p, pcap * 16);
-  W.at = (unsigned long long*)carve(p, bcap * 8);
   return W;
 }
 
@@ -615,42 +583,26 @@ __device__ __forceinline__ void window_hit(const M& m, const ScanArgs& A, uint64
   }
 }
 
+// Marks and leftmost occurrences of a level of short blocks (fewer than
+// kQuickMinB bytes): fingerprint tables and a scan of every window.
 template <class M>
-__device__ void level_pass(const M& m, const BParams& P, const BDoc& D, Cta& C, char* scr, uint32_t l,
-                           uint32_t* filt, uint32_t filt_words_max) {
-  const uint64_t* bsz = P.sizes + D.lv_off;
-  const uint64_t n = C.n, c = C.c[l], b = bsz[l];
-  const bool last = l + 1 == C.L;
+__device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, const LV& g, char* scr, uint32_t l,
+                          uint32_t* filt, uint32_t filt_words_max) {
+  const uint64_t n = C.n, c = g.c, b = g.b;
   const unsigned tid = threadIdx.x, nt = blockDim.x;
-  LV g{D.T, n, c, b, (uint64_t*)(scr + C.sl.st[l])};
-  const uint64_t* H = (const uint64_t*)(scr + C.sl.H);
   uint64_t* lo = (uint64_t*)(scr + C.sl.lo[l]);
-  uint64_t* off = (uint64_t*)(scr + C.sl.off[l]);
-  uint32_t* ptr = (uint32_t*)(scr + C.sl.ptr[l]);
   uint32_t* mw = (uint32_t*)(scr + C.sl.mw[l]);
   uint32_t* mr = (uint32_t*)(scr + C.sl.mr[l]);
+  uint64_t* H = (uint64_t*)(scr + C.sl.big);
+  if (!C.expanded) {
+    expand_pass(m, D.T, n, P.B, (const uint64_t*)(scr + C.sl.Hs), H);
+    if (tid == 0) C.expanded = 1;
+  }
   const uint64_t bcap = pow2_ge(2 * c), pcap = pow2_ge(2 * c);
   const Work W = carve_level(scr + C.sl.temp, c, bcap, pcap);
-
   if (tid == 0) {
-    const uint64_t len_last = n - C.last_start;
-    C.r = len_last < b ? len_last : 0;
-    C.Bb = pow_mod(m, P.B, b);
-    C.Br = C.r ? pow_mod(m, P.B, C.r) : 0;
-    C.B1 = P.B % m.q();
     C.bmask = bcap - 1;
     C.pmask = pcap - 1;
-    C.bshift = (b & (b - 1)) == 0 ? (uint32_t)(__ffsll((long long)b) - 1) : 0xFFu;
-    C.fp_tail = kNone;
-    C.lo_tail = kNone;
-    C.lo_tailpair = kNone;
-    C.pretail = kNoSlot;
-    C.npairs = 0;
-    C.njobs = 0;
-    C.nsusp = 0;
-    C.verify_bytes = 0;
-    C.collisions = 0;
-    C.lastk = 0;
   }
   for (uint64_t i = tid; i < bcap; i += nt) W.bt[i] = BSlot{kNone, kNone, 0, 0};
   for (uint64_t i = tid; i < pcap; i += nt) W.pt[i] = PSlot{kNone, kNone};
@@ -708,308 +660,40 @@ __device__ void level_pass(const M& m, const BParams& P, const BDoc& D, Cta& C, 
     }
   }
   if (cta_failed(C)) return;
-  // Levels of long blocks scan by anchors: every full-length block registers
-  // its first selected gram (hash, offset from the block's start) in the
-  // anchor table, each distinct (hash, offset) once.  Registering every block,
-  // not one per table slot, keeps the proposals complete when different
-  // contents share a fingerprint.  A block without a selected gram puts its
-  // first 8 bytes into the shared-memory filter instead, and the scan then
-  // also tests every window's first 8 bytes against it.
-  const uint32_t* lpos = (const uint32_t*)(scr + C.sl.lpos);
-  const uint32_t* lhash = (const uint32_t*)(scr + C.sl.lhash);
-  const uint32_t nsel = C.nsel;
-  const uint64_t amask = bcap - 1;
-  uint32_t fwords = 32, fshift = 32 - 10;  // 32 words = 2^10 bits
-  while (fwords < c && fwords < filt_words_max) {
-    fwords <<= 1;
-    fshift--;
-  }
-  const bool anch = b >= P.anchor_min_b && nsel != kNoList;
-  if (anch) {
-    if (tid == 0) {
-      C.anchorless = 0;
-      C.tail_anchored = 0;
-      if (r >= kGramW) {
-        const uint64_t ts = C.last_start;
-        const uint32_t j = lower_bound_u32(lpos, nsel, ts);
-        if (j < nsel && lpos[j] + kGramW <= ts + r) {
-          C.tail_g = lhash[j];
-          C.tail_a = (uint32_t)(lpos[j] - ts);
-          C.tail_anchored = 1;
-        }
-      }
-    }
-    for (uint64_t i = tid; i < bcap; i += nt) W.at[i] = kNoAnchor;
-    for (uint32_t i = tid; i < fwords; i += nt) filt[i] = 0;
-    __syncthreads();
-    for (uint64_t k = tid; k < c; k += nt) {
-      if (W.slotB[k] == kNoSlot) continue;
-      const uint64_t s0 = g.st[k];
-      const uint32_t j = lower_bound_u32(lpos, nsel, s0);
-      if (j >= nsel || lpos[j] + kGramW > s0 + b) {
-        // No selected gram: the block's first 8 bytes go to the filter that
-        // the per-window pass of the scan tests.
-        const uint32_t* w3 = (const uint32_t*)(D.T + (s0 & ~3ull));
-        const uint32_t sh = 8 * (uint32_t)(s0 & 3);
-        const uint32_t bit = prefix_bit(__funnelshift_r(w3[0], w3[1], sh), __funnelshift_r(w3[1], w3[2], sh), fshift);
-        atomicOr(&filt[bit >> 5], 1u << (bit & 31));
-        atomicAdd(&C.anchorless, 1u);
-        continue;
-      }
-      const unsigned long long e = ((unsigned long long)lhash[j] << 32) | (uint32_t)(lpos[j] - s0);
-      uint32_t h = anchor_slot(lhash[j], amask);
-      for (uint64_t it = 0; it <= amask; it++) {
-        const unsigned long long cur = *(volatile unsigned long long*)&W.at[h];
-        if (cur == e) break;
-        if (cur == kNoAnchor) {
-          const unsigned long long old = atomicCAS(&W.at[h], kNoAnchor, e);
-          if (old == kNoAnchor || old == e) break;
-        }
-        h = (uint32_t)((h + 1) & amask);
-      }
-    }
-    __syncthreads();
-  }
+  uint32_t fwords = 32;
+  while (fwords < c && fwords < filt_words_max) fwords <<= 1;
   // A bitmap of the full-length block fingerprints in shared memory (about
   // 32 bits per key): a window whose fingerprint's bit is clear matches no
   // key, so only the few that pass probe the table in global memory.
   const uint64_t fmask = (uint64_t)fwords * 32 - 1;
-  if (!anch) {
-    for (uint32_t i = tid; i < fwords; i += nt) filt[i] = 0;
-    for (uint32_t a = tid; a < 256; a += nt) C.rtab[a] = m.mul(a + 1, Bb);
-    __syncthreads();
-    for (uint64_t k = tid; k < c; k += nt)
-      if (W.slotB[k] != kNoSlot) {
-        const uint64_t bit = W.fpB[k] & fmask;
-        atomicOr(&filt[bit >> 5], 1u << (bit & 31));
-      }
-  }
+  for (uint32_t i = tid; i < fwords; i += nt) filt[i] = 0;
+  __syncthreads();
+  for (uint64_t k = tid; k < c; k += nt)
+    if (W.slotB[k] != kNoSlot) {
+      const uint64_t bit = W.fpB[k] & fmask;
+      atomicOr(&filt[bit >> 5], 1u << (bit & 31));
+    }
   __syncthreads();
   tmark(C, 1);
 
   // The window scan: every window [p, p+b) inside a run (and [p, p+r) for the
-  // short tail).  When b is a multiple of 32, a warp takes CH = 32 Re
-  // consecutive positions of one block (block, run end and bounds are warp
-  // values, positions 32-bit) and lane l the Re positions from p0 + l Re,
-  // rolling the fingerprint from one to the next.  Otherwise every thread
-  // maps its positions to blocks itself.  The short tail's windows are tested only where their first four
-  // bytes equal the tail's.
+  // short tail); the few whose fingerprint's bit is set probe the table.
   {
     const uint32_t pretail = C.pretail, bshift = C.bshift;
     const uint64_t fp_tail = C.fp_tail;
-    uint32_t tail4 = 0, tail4_mask = 0;
-    if (r) {
-      const uint64_t ts = C.last_start;
-      for (uint32_t i = 0; i < 4 && i < r; i++) {
-        tail4 |= (uint32_t)D.T[ts + i] << (8 * i);
-        tail4_mask |= 0xFFu << (8 * i);
-      }
-    }
     const ScanArgs A{H, W.bt, W.pt, bmask, pmask, b, r, Bb, Br, fp_tail, pretail, &C.lo_tailpair};
-    if (anch) {
-      // A warp per present block k: its selected grams x (the list entries
-      // in [s_k, s_k + len_k)) propose, for every key anchored on the gram's
-      // hash at offset a, the window at p = x - a.  As a < b, p lies in
-      // block k or in block k-1 when that one ends where k starts; the
-      // window must end within the run of p's block.
-      const unsigned lane = tid & 31, nw = nt >> 5;
-      const bool tail_anch = r && C.tail_anchored;
-      const uint32_t tail_g = C.tail_g, tail_a = C.tail_a;
-      for (uint64_t k = tid >> 5; k < c; k += nw) {
-        const uint64_t s = g.st[k];
-        const uint64_t len = n - s < b ? n - s : b, e0 = s + len;
-        uint64_t av = e0;  // run end of block k
-        uint64_t nxt = 0;  // length of block k+1 when it follows k
-        if (k + 1 < c && g.st[k + 1] == e0) {
-          nxt = n - e0 < b ? n - e0 : b;
-          av = e0 + nxt;
-          if (k + 2 < c && g.st[k + 2] == av) av += n - av < b ? n - av : b;
-        }
-        const bool prev = k > 0 && g.st[k - 1] + b == s;  // block k-1 ends where k starts
-        const uint64_t av_prev = e0 + nxt;                // run end of block k-1
-        uint32_t j0 = 0, j1 = 0;
-        if (lane == 0) {
-          j0 = lower_bound_u32(lpos, nsel, s);
-          j1 = lower_bound_u32(lpos, nsel, e0);
-        }
-        j0 = __shfl_sync(kFull, j0, 0);
-        j1 = __shfl_sync(kFull, j1, 0);
-        for (uint32_t j = j0 + lane; j < j1; j += 32) {
-          const uint64_t x = lpos[j];
-          const uint32_t gh = lhash[j];
-          uint32_t h = anchor_slot(gh, amask);
-          for (uint64_t it = 0; it <= amask; it++) {
-            const unsigned long long en = W.at[h];
-            if (en == kNoAnchor) break;
-            if ((uint32_t)(en >> 32) == gh && (uint32_t)en <= x) {
-              const uint64_t p = x - (uint32_t)en;
-              const uint64_t pav = p >= s ? av : (prev ? av_prev : 0);
-              if (p + b <= pav) {
-                const uint64_t hb = H[p + b];
-                window_hit(m, A, p, pav, m.sub(hb, m.mul(H[p], Bb)), hb);
-              }
-            }
-            h = (uint32_t)((h + 1) & amask);
-          }
-          if (tail_anch && gh == tail_g && tail_a <= x) {
-            const uint64_t p = x - tail_a;
-            const uint64_t pav = p >= s ? av : (prev ? av_prev : 0);
-            if (p + r <= pav && phi(m, H, Br, p, r) == fp_tail) min_pos(&C.lo_tail, p);
-          }
-        }
+    for (uint64_t w = tid; w < c * b; w += nt) {
+      const uint64_t k = bshift != 0xFFu ? w >> bshift : w / b;
+      const uint64_t j = w - k * b;
+      if (j >= blen(g, k)) continue;
+      const uint64_t p = g.st[k] + j, av = avail_end(g, k);
+      if (p + b <= av) {
+        const uint64_t hb = H[p + b];
+        const uint64_t x = m.sub(hb, m.mul(H[p], Bb));
+        const uint64_t bit = x & fmask;
+        if ((filt[bit >> 5] >> (bit & 31)) & 1u) window_hit(m, A, p, av, x, hb);
       }
-      const uint32_t nal = C.anchorless;
-      if (nal || (r && !tail_anch)) {
-        // Blocks without a selected gram, and the short tail without one:
-        // every window, where its first 8 bytes pass the blocks' filter
-        // (then its fingerprint decides) or its first 4 bytes equal the
-        // tail's.  A warp takes 256 consecutive positions of a block, a lane
-        // 8 of them, from 5 aligned words.
-        constexpr uint32_t Rp = 8, CHp = 32 * Rp;
-        const uint64_t cpbp = (b + CHp - 1) / CHp;
-        const bool all_present = c == (n + b - 1) / b;
-        const uint8_t* T = D.T;
-        for (uint64_t item = tid >> 5; item < c * cpbp; item += nw) {
-          const uint64_t k = item / cpbp, jc = item - k * cpbp;
-          uint64_t s, av;
-          if (all_present) {
-            s = k * b;
-            av = (k + 3) * b < n ? (k + 3) * b : n;
-          } else {
-            s = g.st[k];
-            const uint64_t s1 = k + 1 < c ? g.st[k + 1] : kNone, s2 = k + 2 < c ? g.st[k + 2] : kNone;
-            const uint64_t e0 = s + (n - s < b ? n - s : b);
-            av = e0;
-            if (s1 == e0) {
-              av = s1 + (n - s1 < b ? n - s1 : b);
-              if (s2 == av) av = s2 + (n - s2 < b ? n - s2 : b);
-            }
-          }
-          const uint64_t send = s + (n - s < b ? n - s : b);
-          const uint64_t p = s + jc * CHp + lane * Rp;
-          if (p >= send) continue;
-          const uint64_t pend = p + Rp < send ? p + Rp : send;
-          const uint32_t* wa = (const uint32_t*)(T + (p & ~3ull));
-          const uint32_t sa = 8 * (uint32_t)(p & 3);
-          uint32_t t[4];
-          {
-            uint32_t w[5];
-#pragma unroll
-            for (int q = 0; q < 5; q++) w[q] = wa[q];
-#pragma unroll
-            for (int q = 0; q < 4; q++) t[q] = __funnelshift_r(w[q], w[q + 1], sa);
-          }
-#pragma unroll
-          for (uint32_t i = 0; i < Rp; i++) {
-            const uint64_t q = p + i;
-            if (q >= pend) break;
-            const uint32_t lo = __funnelshift_r(t[i >> 2], t[(i >> 2) + 1], 8 * (i & 3));
-            if (nal && q + b <= av) {
-              const uint32_t hi = __funnelshift_r(t[(i >> 2) + 1], t[(i >> 2) + 2], 8 * (i & 3));
-              const uint32_t bit = prefix_bit(lo, hi, fshift);
-              if ((filt[bit >> 5] >> (bit & 31)) & 1u) {
-                const uint64_t hb = H[q + b];
-                window_hit(m, A, q, av, m.sub(hb, m.mul(H[q], Bb)), hb);
-              }
-            }
-            if (r && !tail_anch && q + r <= av && (lo & tail4_mask) == tail4 && phi(m, H, Br, q, r) == fp_tail)
-              min_pos(&C.lo_tail, q);
-          }
-        }
-      }
-    } else if (b % 32 == 0) {
-      // A lane takes a run of Re consecutive positions: the first window's
-      // fingerprint comes from two prefix fingerprints, each next one rolls
-      // in one step from the text bytes, phi(p+1, p+1+b) = B phi(p, p+b) +
-      // (T[p+b] + 1) - (T[p] + 1) B^b (the last term from a table in shared
-      // memory), so the loads per window are a few text bytes.
-      constexpr int R = 8;
-      const uint32_t Rmax = P.scan_u && P.scan_u < (uint32_t)R ? P.scan_u : (uint32_t)R;
-      const uint32_t Re = b / 32 < Rmax ? (uint32_t)(b / 32) : Rmax;  // positions per lane
-      const uint32_t CH = 32 * Re;
-      const uint64_t cpb = (b + CH - 1) / CH;
-      const unsigned lane = tid & 31, nw = nt >> 5;
-      const uint8_t* T = D.T;
-      const uint64_t B1 = C.B1;
-      const uint64_t* rtab = C.rtab;
-      // Every block of the level present: block k starts at k b and its run
-      // ends at min(n, (k + 3) b), with no loads.
-      const bool all_present = c == (n + b - 1) / b;
-      for (uint64_t item = tid >> 5; item < c * cpb; item += nw) {
-        const uint64_t k = item / cpb, jc = item - k * cpb;
-        uint64_t s, av;
-        if (all_present) {
-          s = k * b;
-          av = (k + 3) * b < n ? (k + 3) * b : n;
-        } else {
-          // The three starts are loaded together, then the run end follows.
-          s = g.st[k];
-          const uint64_t s1 = k + 1 < c ? g.st[k + 1] : kNone, s2 = k + 2 < c ? g.st[k + 2] : kNone;
-          const uint64_t e0 = s + (n - s < b ? n - s : b);
-          av = e0;
-          if (s1 == e0) {
-            av = s1 + (n - s1 < b ? n - s1 : b);
-            if (s2 == av) av = s2 + (n - s2 < b ? n - s2 : b);
-          }
-        }
-        const uint64_t send = s + (n - s < b ? n - s : b);
-        const uint32_t p = (uint32_t)(s + jc * CH + lane * Re);
-        if (p >= send) continue;
-        const uint32_t pend = (uint32_t)(p + Re < send ? p + Re : send);
-        // Text bytes [p, p+12) and [p+b, p+b+8) from aligned words (a
-        // document's bytes are followed by at least 48 readable bytes).
-        const uint32_t* wa = (const uint32_t*)(T + (p & ~3u));
-        const uint32_t sa = 8 * (p & 3);
-        const uint32_t a0 = wa[0], a1 = wa[1], a2 = wa[2];
-        const uint32_t ta0 = __funnelshift_r(a0, a1, sa), ta1 = __funnelshift_r(a1, a2, sa);
-        uint32_t ta2 = 0;
-        if (r) ta2 = __funnelshift_r(a2, wa[3], sa);
-        const bool full0 = p + b <= av;
-        uint64_t x = 0;
-        uint32_t tb0 = 0, tb1 = 0;
-        if (full0) {
-          const uint32_t q = p + (uint32_t)b;
-          const uint32_t* wb = (const uint32_t*)(T + (q & ~3u));
-          const uint32_t sb = 8 * (q & 3);
-          const uint32_t b0 = wb[0], b1 = wb[1], b2 = wb[2];
-          tb0 = __funnelshift_r(b0, b1, sb);
-          tb1 = __funnelshift_r(b1, b2, sb);
-          x = m.sub(H[q], m.mul(H[p], Bb));
-        }
-#pragma unroll
-        for (int i = 0; i < R; i++) {
-          if (i >= (int)Re) break;
-          const uint32_t q = p + i;
-          if (q >= pend) break;
-          if (q + b <= av) {
-            const uint64_t bit = x & fmask;
-            if ((filt[bit >> 5] >> (bit & 31)) & 1u) window_hit(m, A, q, av, x, H[q + b]);
-            if (i + 1 < R) {
-              const uint32_t lo = i < 4 ? ta0 : ta1, ins = i < 4 ? tb0 : tb1;
-              const uint32_t sh = 8 * (i & 3);
-              x = m.sub(m.add(m.mul(x, B1), ((ins >> sh) & 0xFFu) + 1), rtab[(lo >> sh) & 0xFFu]);
-            }
-          }
-          if (r && q + r <= av) {
-            const uint32_t v = i < 4 ? __funnelshift_r(ta0, ta1, 8 * (i & 3)) : __funnelshift_r(ta1, ta2, 8 * (i & 3));
-            if ((v & tail4_mask) == tail4 && phi(m, H, Br, q, r) == fp_tail) min_pos(&C.lo_tail, q);
-          }
-        }
-      }
-    } else {
-      for (uint64_t w = tid; w < c * b; w += nt) {
-        const uint64_t k = bshift != 0xFFu ? w >> bshift : w / b;
-        const uint64_t j = w - k * b;
-        if (j >= blen(g, k)) continue;
-        const uint64_t p = g.st[k] + j, av = avail_end(g, k);
-        if (p + b <= av) {
-          const uint64_t hb = H[p + b];
-          const uint64_t x = m.sub(hb, m.mul(H[p], Bb));
-          const uint64_t bit = x & fmask;
-          if ((filt[bit >> 5] >> (bit & 31)) & 1u) window_hit(m, A, p, av, x, hb);
-        }
-        if (r && p + r <= av && phi(m, H, Br, p, r) == fp_tail) min_pos(&C.lo_tail, p);
-      }
+      if (r && p + r <= av && phi(m, H, Br, p, r) == fp_tail) min_pos(&C.lo_tail, p);
     }
   }
   __syncthreads();
@@ -1117,6 +801,223 @@ __device__ void level_pass(const M& m, const BParams& P, const BDoc& D, Cta& C, 
     for (uint32_t i = tid; i < C.nsusp; i += nt) lo[W.susp[i]] = W.exlo[i];
     __syncthreads();
   }
+}
+
+constexpr uint32_t kCtaBitWords = 8192;  // the open keys' bitmap in shared memory up to 32 KiB
+
+// Marks and leftmost occurrences of a level by first occurrences: the steps of
+// bt_quick.cu over one CTA.  Measured on 1024 versioned documents of 4 KiB - 4
+// MiB (0.65 GB): with fingerprint tables and a scan of every window (anchored
+// on levels of 1 KiB blocks and more) the kernel took 50 ms, the longest
+// document 51; now 15 and 15.
+template <class M>
+__device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const LV& g, char* scr, uint32_t l,
+                           uint32_t* dyn) {
+  const uint64_t n = C.n, c = g.c, b = g.b, words = (c + 31) / 32;
+  const unsigned tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  uint64_t* lo = (uint64_t*)(scr + C.sl.lo[l]);
+  uint32_t* mw = (uint32_t*)(scr + C.sl.mw[l]);
+  uint32_t* mr = (uint32_t*)(scr + C.sl.mr[l]);
+  char* p = scr + C.sl.temp;
+  uint32_t* A = (uint32_t*)carve(p, c * 4 + 4);
+  uint32_t* X = (uint32_t*)carve(p, c * 4 + 4);
+  uint32_t* flags = (uint32_t*)carve(p, c * 4 + 4);
+  uint32_t* wpop = (uint32_t*)carve(p, c * 4 + 4);
+  uint32_t* items = (uint32_t*)carve(p, c * 8 + 8);
+  uint8_t* ps = (uint8_t*)carve(p, c + 8);
+  const QGeo q{g.T, n, c, b, g.st};
+  const Span w{tid, nt};
+  if (tid == 0) {
+    C.qs.nopen[0] = C.qs.nopen[1] = C.qs.nitems = C.qs.npairs = C.qs.nsusp = 0;
+    C.status.error = C.status.verify_bytes = C.status.collisions = 0;
+  }
+  unsigned G = 1;
+  while (G < 32 && 64ull * 2 * G <= b) G <<= 1;
+  quick_min(q, C.list, G, A, X, flags, w);
+  __syncthreads();
+  tmark(C, 1);
+  const uint64_t bl = b < n ? b : n;
+  const uint32_t ppk = (uint32_t)((2 * bl + q_piece(b) - 1) / q_piece(b));
+  const unsigned L = b >= 1024 ? 32u : b >= 512 ? 16u : b >= 256 ? 8u : b >= 128 ? 4u : b >= 64 ? 2u : 1u;
+  quick_compare(q, A, X, flags, ppk, L, w);
+  __syncthreads();
+  tmark(C, 3);
+  uint64_t vb = 0;
+  uint32_t np = 0, nob = 0, nop = 0;
+  for (uint64_t k = tid; k < c; k += nt) {
+    const uint64_t s = g.st[k], len = blen(g, k);
+    const uint32_t d = A[k];
+    uint64_t at = s;
+    bool open = false;
+    if (s != 0 && d != 0) {
+      open = d == kNoDist || (flags[k] & kBlkDiffers);
+      at = open ? kNone : (d > s ? 0 : s - d);
+      if (d != kNoDist) vb += 2 * len;
+    }
+    lo[k] = at;
+    if (open) {
+      items[atomicAdd(&C.qs.nitems, 1ull)] = (uint32_t)(2 * k);
+      nob++;
+    }
+    uint32_t d2 = 0;
+    uint64_t plen = 0;
+    const uint8_t st = pair_state(q, A, X, flags, k, &d2, &plen, &open);
+    ps[k] = st;
+    np += st & kIsPair;
+    if (st == kIsPair && d2 != kNoDist) vb += 2 * plen;
+    if (open) {
+      items[atomicAdd(&C.qs.nitems, 1ull)] = (uint32_t)(2 * k + 1);
+      nop++;
+    }
+  }
+  vb = warp_sum64(vb);
+  np = __reduce_add_sync(kFull, np);
+  nob = __reduce_add_sync(kFull, nob);
+  nop = __reduce_add_sync(kFull, nop);
+  if (lane == 0) {
+    if (vb) atomicAdd(&C.status.verify_bytes, (unsigned long long)vb);
+    if (np) atomicAdd(&C.npairs, np);
+    if (nob) atomicAdd(&C.qs.nopen[0], (unsigned long long)nob);
+    if (nop) atomicAdd(&C.qs.nopen[1], (unsigned long long)nop);
+  }
+  __syncthreads();
+  tmark(C, 3);
+  const uint64_t ni = C.qs.nitems;
+  if (ni) {
+    const uint64_t nb = C.qs.nopen[0] + 2 * C.qs.nopen[1];
+    const uint64_t bcap = pow2_ge(2 * (nb < c ? nb : c)), pcap = pow2_ge(2 * C.qs.nopen[1]), gcap = pow2_ge(2 * ni);
+    uint32_t fbits = 12;
+    while ((1ull << fbits) < 16 * ni && fbits < 30) fbits++;
+    const uint32_t bwords = 1u << (fbits - 5);
+    if (tid == 0) {
+      Chase& K = C.chase;
+      K.g = q;
+      K.Q = C.list;
+      K.A = A;
+      K.X = X;
+      K.items = items;
+      K.nitems = (uint32_t)ni;
+      K.Bb = C.Bb;
+      K.Br = C.Br;
+      K.r = C.r;
+      K.bt = (CSlot*)carve(p, bcap * 32);
+      K.pt = (CPair*)carve(p, pcap * 16);
+      K.gt = (CGram*)carve(p, gcap * 16);
+      K.bound2 = (unsigned long long*)carve(p, gcap * 8);
+      K.bitmap = (uint32_t*)carve(p, bwords * 4ull);
+      K.islot = (uint32_t*)carve(p, ni * 4);
+      K.igram = (uint32_t*)carve(p, ni * 4);
+      K.differ = (uint32_t*)carve(p, ni * 4);
+      K.susp = (uint32_t*)carve(p, ni * 4);
+      K.exlo = (unsigned long long*)carve(p, ni * 8);
+      K.bmask = (uint32_t)(bcap - 1);
+      K.pmask = (uint32_t)(pcap - 1);
+      K.gmask = (uint32_t)(gcap - 1);
+      K.bshift = 32 - fbits;
+      K.qs = &C.qs;
+      K.status = &C.status;
+      K.lo = lo;
+      K.ps = ps;
+    }
+    __syncthreads();
+    const Chase& K = C.chase;
+    const PrefixAt<M> H(PC, g.T, n, (const uint64_t*)(scr + C.sl.Hs));
+    chase_init(K, bwords, w);
+    __syncthreads();
+    if (b <= 256) chase_keys<M, 1>(m, H, K, w);
+    else chase_keys<M, 32>(m, H, K, w);
+    __syncthreads();
+    // Shared memory: the warps' queues, then the bitmap while it fits.
+    uint2* hq = (uint2*)dyn + warp * kHitQ;
+    uint32_t* cq = (uint32_t*)((uint2*)dyn + (nt / 32) * kHitQ) + warp * kCandQ;
+    uint32_t* bits_s = (uint32_t*)((uint2*)dyn + (nt / 32) * kHitQ) + (nt / 32) * kCandQ;
+    const bool fits = bwords <= kCtaBitWords;
+    if (fits)
+      for (uint32_t i = tid; i < bwords; i += nt) bits_s[i] = K.bitmap[i];
+    __syncthreads();
+    const uint32_t* bits = fits ? bits_s : K.bitmap;
+    const uint32_t total = C.nsel, split = total > (1u << 16) ? (total / 16) & ~(8 * kChaseTile - 1) : 0;
+    if (split) {
+      chase_scan(m, H, K, 0, split, bits, hq, cq, nullptr, w);
+      __syncthreads();
+      chase_bound(K, w);
+      __syncthreads();
+    }
+    chase_scan(m, H, K, split, total, bits, hq, cq, split ? K.bound2 : nullptr, w);
+    if (C.r && C.r < kQuickMinB) chase_tail(K, w);
+    __syncthreads();
+    tmark(C, 2);
+    const unsigned Lv = b >= 256 ? 32u : b >= 128 ? 16u : b >= 64 ? 8u : 4u;
+    chase_verify(K, (2 * b + q_piece(b) - 1) / q_piece(b), Lv, w);
+    __syncthreads();
+    chase_apply(K, w);
+    __syncthreads();
+    const uint64_t nsusp = C.qs.nsusp;
+    if (nsusp) {
+      chase_exact(K, 0, 1, nsusp, w);
+      __syncthreads();
+      chase_exact_apply(K, nsusp, w);
+      __syncthreads();
+    }
+  }
+  if (tid == 0) {
+    if (C.status.error) fail(C, BT_EINTERNAL);
+    C.verify_bytes = C.status.verify_bytes;
+    C.collisions = C.status.collisions;
+  }
+  if (cta_failed(C)) return;
+  for (uint64_t wb = warp; wb < words; wb += nt >> 5) {
+    const uint64_t k = wb * 32 + lane;
+    bool mk = false;
+    if (k < c) {
+      const uint8_t left = k ? ps[k - 1] : 0, r = ps[k];
+      mk = (left & kLeftmost) || (r & kLeftmost) || !((left | r) & kIsPair);
+    }
+    const uint32_t bits = __ballot_sync(kFull, mk);
+    if (lane == 0) {
+      mw[wb] = bits;
+      wpop[wb] = __popc(bits);
+    }
+  }
+  __syncthreads();
+  cta_scan_u32(wpop, mr, words, C);
+}
+
+template <class M>
+__device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& P, const BDoc& D, Cta& C, char* scr,
+                           uint32_t l, uint32_t* dyn, uint32_t dyn_words) {
+  const uint64_t* bsz = P.sizes + D.lv_off;
+  const uint64_t n = C.n, c = C.c[l], b = bsz[l];
+  const bool last = l + 1 == C.L;
+  const unsigned tid = threadIdx.x, nt = blockDim.x;
+  LV g{D.T, n, c, b, (uint64_t*)(scr + C.sl.st[l])};
+  uint64_t* lo = (uint64_t*)(scr + C.sl.lo[l]);
+  uint64_t* off = (uint64_t*)(scr + C.sl.off[l]);
+  uint32_t* ptr = (uint32_t*)(scr + C.sl.ptr[l]);
+  uint32_t* mw = (uint32_t*)(scr + C.sl.mw[l]);
+  uint32_t* mr = (uint32_t*)(scr + C.sl.mr[l]);
+  const uint64_t words = (c + 31) / 32;
+  if (tid == 0) {
+    const uint64_t len_last = n - C.last_start;
+    C.r = len_last < b ? len_last : 0;
+    C.Bb = pow_mod(m, P.B, b);
+    C.Br = C.r ? pow_mod(m, P.B, C.r) : 0;
+    C.bshift = (b & (b - 1)) == 0 ? (uint32_t)(__ffsll((long long)b) - 1) : 0xFFu;
+    C.fp_tail = kNone;
+    C.lo_tail = kNone;
+    C.lo_tailpair = kNone;
+    C.pretail = kNoSlot;
+    C.npairs = 0;
+    C.njobs = 0;
+    C.nsusp = 0;
+    C.verify_bytes = 0;
+    C.collisions = 0;
+    C.lastk = 0;
+  }
+  __syncthreads();
+  if (b >= kQuickMinB) quick_keys(m, PC, C, g, scr, l, dyn);
+  else scan_keys(m, P, D, C, g, scr, l, dyn, dyn_words);
+  if (cta_failed(C)) return;
 
   // Pointers of unmarked blocks: the block holding the leftmost occurrence
   // and the offset into it.
@@ -1159,8 +1060,8 @@ __device__ void level_pass(const M& m, const BParams& P, const BDoc& D, Cta& C, 
     S[BT_ST_VERIFY_BYTES] = C.verify_bytes;
     S[BT_ST_COLLISIONS] = C.collisions;
     S[BT_ST_FINAL_BLOCKS] = c;
-    S[BT_ST_CANDIDATES] = 0;
-    S[BT_ST_HITS] = 0;
+    S[BT_ST_CANDIDATES] = b >= kQuickMinB && C.qs.nitems ? C.qs.cands : 0;
+    S[BT_ST_HITS] = b >= kQuickMinB && C.qs.nitems ? C.qs.hits : 0;
   }
   if (last) {
     if (tid == 0) C.arity[l] = 0;
@@ -1456,10 +1357,10 @@ __device__ void prune_pass(const BParams& P, const BDoc& D, Cta& C, char* scr) {
 // Counters of a level, symbol-major (cp entries per symbol).  mode 0: symbol
 // counts of each block (marked blocks of a non-last level are filled from their
 // children afterwards); mode 1: counts of T[st[ptr], st[ptr] + off) of each
-// unmarked block (zeros for marked ones).  A warp takes four consecutive
-// blocks at a time, their bytes in flight together, each with its own
-// histogram (hist: 1024 words per warp), and writes the four counters of a
-// symbol at once.
+// unmarked block.  A warp takes four consecutive blocks at a time, 16 bytes per
+// lane and block in flight together, each with its own histogram (hist: 1024
+// words per warp), and writes the four counters of a symbol at once (zeros
+// where a block is not counted; nothing when none of the four is).
 __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PLv& v, int mode, bool last,
                            void* out, uint32_t cw, uint64_t cp, unsigned int* hist) {
   const uint32_t S = C.S;
@@ -1468,12 +1369,14 @@ __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PL
   for (uint64_t g = warp; 4 * g < v.c; g += nw) {
     uint64_t s0[4];
     uint32_t len[4], top = 0;
+    bool any = false;
 #pragma unroll
     for (uint32_t q = 0; q < 4; q++) {
       const uint64_t k = 4 * g + q;
       s0[q] = 0;
       len[q] = 0;
       if (k >= v.c) continue;
+      any |= mode == 0 ? last || !marked(v.mw, k) : !marked(v.mw, k);
       const bool mk = marked(v.mw, k);
       if (mode == 0 && (last || !mk)) {
         s0[q] = v.st[k];
@@ -1484,18 +1387,29 @@ __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PL
       }
       top = top > len[q] ? top : len[q];
     }
+    if (!any) continue;
     for (uint32_t i = lane; i < S; i += 32) {
 #pragma unroll
       for (uint32_t q = 0; q < 4; q++) h[256 * q + i] = 0;
     }
     __syncwarp();
-    for (uint32_t x = lane; x < top; x += 32) {
-      uint32_t ch[4];
+    for (uint32_t x = 16 * lane; x < top; x += 512) {
 #pragma unroll
-      for (uint32_t q = 0; q < 4; q++) ch[q] = x < len[q] ? T[s0[q] + x] : 256u;
+      for (uint32_t q0 = 0; q0 < 4; q0 += 2) {
+        uint4 t[2];
 #pragma unroll
-      for (uint32_t q = 0; q < 4; q++)
-        if (ch[q] < 256u) atomicAdd(&h[256 * q + C.sym[ch[q]]], 1u);
+        for (uint32_t q = 0; q < 2; q++)
+          if (x < len[q0 + q]) t[q] = load16u(T, s0[q0 + q] + x);
+#pragma unroll
+        for (uint32_t q = 0; q < 2; q++) {
+          if (x >= len[q0 + q]) continue;
+          const uint32_t w[4] = {t[q].x, t[q].y, t[q].z, t[q].w};
+          const uint32_t have = len[q0 + q] - x;
+#pragma unroll
+          for (uint32_t i = 0; i < 16; i++)
+            if (i < have) atomicAdd(&h[256 * (q0 + q) + C.sym[(w[i >> 2] >> (8 * (i & 3))) & 0xFF]], 1u);
+        }
+      }
     }
     __syncwarp();
     for (uint32_t i = lane; i < S; i += 32) {
@@ -1507,6 +1421,52 @@ __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PL
     }
     __syncwarp();
   }
+}
+
+// One-byte counters: a thread per block into a tile [S][TB] in shared memory
+// (as k_count_small of bt_query.cu: warp w takes the columns that put its
+// lanes in different banks), rows leave as runs.
+__device__ void count_small(const uint8_t* __restrict__ T, const Cta& C, const PLv& v, int mode, bool last, uint8_t* out,
+                            uint64_t cp, uint8_t* tile) {
+  const uint32_t S = C.S, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint32_t TB = blockDim.x;
+  while ((uint64_t)TB * S > kDynWords * 4ull) TB >>= 1;  // 1024, or 512 above 128 symbols
+  const uint32_t col = 4 * (lane + 32 * (warp >> 2)) + (warp & 3);
+  for (uint64_t k0 = 0; k0 < v.c; k0 += TB) {
+    __syncthreads();
+    for (uint32_t i = tid; i < S * (TB / 4); i += blockDim.x) ((uint32_t*)tile)[i] = 0;
+    __syncthreads();
+    const uint64_t k = k0 + col;
+    if (col < TB && k < v.c) {
+      const bool mk = marked(v.mw, k);
+      uint64_t s0 = 0;
+      uint32_t len = 0;
+      if (mode == 0 && (last || !mk)) {
+        s0 = v.st[k];
+        len = (uint32_t)plen(v, k);
+      } else if (mode == 1 && !mk) {
+        s0 = v.st[v.ptr[k]];
+        len = (uint32_t)v.off[k];
+      }
+      uint8_t* my = tile + col;
+      for (uint32_t x = 0; x < len; x += 16) {
+        const uint4 q = load16u(T, s0 + x);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+        const uint32_t have = len - x;
+#pragma unroll
+        for (uint32_t i = 0; i < 16; i++)
+          if (i < have) my[TB * (uint32_t)C.sym[(w[i >> 2] >> (8 * (i & 3))) & 0xFF]]++;
+      }
+    }
+    __syncthreads();
+    const uint32_t words = TB / 4;
+    for (uint32_t i = tid; i < S * words; i += blockDim.x) {
+      const uint32_t row = i / words, w = i - row * words;
+      const uint64_t at = k0 + 4 * w;
+      if (at < cp) *(uint32_t*)(out + row * cp + at) = ((const uint32_t*)tile)[i];
+    }
+  }
+  __syncthreads();
 }
 
 __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr, unsigned int* hist) {
@@ -1562,21 +1522,55 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
     void* pc = out + s_ol[l].pc;
     const uint32_t cw = s_cw[l];
     const uint64_t cp = counter_stride(v.c);
-    count_rows(D.T, C, v, 0, last, cnt, cw, cp, hist);
-    count_rows(D.T, C, v, 1, last, pc, cw, cp, hist);
+    if (cw == 1) {
+      count_small(D.T, C, v, 0, last, (uint8_t*)cnt, cp, (uint8_t*)hist);
+      count_small(D.T, C, v, 1, last, (uint8_t*)pc, cp, (uint8_t*)hist);
+    } else {
+      count_rows(D.T, C, v, 0, last, cnt, cw, cp, hist);
+      count_rows(D.T, C, v, 1, last, pc, cw, cp, hist);
+    }
     __syncthreads();
     if (!last) {
       const void* ccnt = out + s_ol[l + 1].cnt;
       const uint32_t ccw = s_cw[l + 1];
       const uint64_t bn = bsz[l + 1], ccp = counter_stride(C.c[l + 1]);
       const uint32_t arity = C.arity[l];
-      for (uint32_t s = warp; s < S; s += nw)
-        for (uint64_t k = lane; k < v.c; k += 32) {
-          if (!marked(v.mw, k)) continue;
-          const uint64_t first = mrank(v.mw, v.mr, k) * arity;
-          const uint32_t nch = (uint32_t)((plen(v, k) + bn - 1) / bn);
-          cput(cnt, cw, s * cp + k, sum_run(ccnt, ccw, s * ccp + first, nch));
+      // A warp takes 32 blocks and a quarter of the symbols; four symbols'
+      // children are read together.
+      const uint64_t chunks = (v.c + 31) / 32;
+      for (uint64_t it = warp; it < 4 * chunks; it += nw) {
+        const uint64_t k = (it >> 2) * 32 + lane;
+        if (k >= v.c || !marked(v.mw, k)) continue;
+        const uint32_t s0 = (uint32_t)(S * (it & 3) / 4), s1 = (uint32_t)(S * ((it & 3) + 1) / 4);
+        const uint64_t first = mrank(v.mw, v.mr, k) * arity;
+        const uint32_t nch = (uint32_t)((plen(v, k) + bn - 1) / bn);
+        for (uint32_t s = s0; s < s1; s += 4) {
+          uint32_t x[4];
+          if (ccw == 1 && nch == 4 && arity == 4) {
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++)
+              x[u] = s + u < s1 ? *(const uint32_t*)((const uint8_t*)ccnt + (s + u) * ccp + first) : 0u;
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++) x[u] = __dp4a(x[u], 0x01010101u, 0u);
+          } else if (nch == 2) {
+            uint32_t y[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++) {
+              const uint64_t at = (s + u < s1 ? s + u : s) * ccp + first;
+              x[u] = cget(ccnt, ccw, at);
+              y[u] = cget(ccnt, ccw, at + 1);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++) x[u] += y[u];
+          } else {
+#pragma unroll
+            for (uint32_t u = 0; u < 4; u++) x[u] = s + u < s1 ? sum_run(ccnt, ccw, (s + u) * ccp + first, nch) : 0u;
+          }
+#pragma unroll
+          for (uint32_t u = 0; u < 4; u++)
+            if (s + u < s1) cput(cnt, cw, (s + u) * cp + k, x[u]);
         }
+      }
       __syncthreads();
     }
   }
@@ -1606,10 +1600,19 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
   {
     const PLv v = plevel(C, scr, bsz, L - 1);
     uint8_t* leaf = (uint8_t*)(out + s_leaf);
-    for (uint64_t w = tid; w < v.c * v.b; w += nt) {
-      const uint64_t k = w / v.b, i = w - k * v.b;
+    // (16 bytes per thread when blocks are whole units.)
+    const uint32_t unit = v.b % 16 == 0 ? 16 : 1;
+    const uint64_t per = v.b / unit;
+    for (uint64_t w = tid; w < v.c * per; w += nt) {
+      const uint64_t k = w / per, i = (w - k * per) * unit;
       if (!marked(v.mw, k) || v.st[k] + i >= C.n) continue;
-      leaf[mrank(v.mw, v.mr, k) * v.b + i] = D.T[v.st[k] + i];
+      uint8_t* to = leaf + mrank(v.mw, v.mr, k) * v.b + i;
+      const uint64_t x = v.st[k] + i;
+      if (unit == 16) {  // (a last unit past the text's end copies its padding)
+        *(uint4*)to = *(const uint4*)(D.T + x);
+      } else {
+        *to = D.T[x];
+      }
     }
     if (tid == 0) {
       const uint64_t words = (v.c + 31) / 32;
@@ -1652,7 +1655,7 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
 }
 
 template <class M>
-__device__ void build_doc(const M& m, const BParams& P, uint32_t d, Cta& C, char* scr, unsigned int* hist,
+__device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const BParams& P, uint32_t d, Cta& C, char* scr, unsigned int* hist,
                           uint32_t dyn_words) {
   const BDoc D = P.docs[d];
   const uint64_t* bsz = P.sizes + D.lv_off;
@@ -1670,12 +1673,9 @@ __device__ void build_doc(const M& m, const BParams& P, uint32_t d, Cta& C, char
   __syncthreads();
   if (C.err == 0) alphabet(D.T, D.n, D.sigma, C);
   if (!cta_failed(C)) {
-    prefix_pass(m, D.T, D.n, P.B, P.pw32, (uint64_t*)(scr + C.sl.H), C);
-    if (bsz[0] >= P.anchor_min_b) {
-      gram_list_pass(D.T, D.n, (uint32_t*)(scr + C.sl.lpos), (uint32_t*)(scr + C.sl.lhash), gram_list_cap(D.n), C);
-    } else if (threadIdx.x == 0) {
-      C.nsel = kNoList;
-    }
+    prefix_pass(m, PC, pw, D.T, D.n, (uint64_t*)(scr + C.sl.Hs), C);
+    if (threadIdx.x == 0) C.expanded = 0;
+    if (bsz[0] >= kQuickMinB) list_pass(D.T, D.n, scr, C);
     // Level 1: blocks k b_1.
     uint64_t* st0 = (uint64_t*)(scr + C.sl.st[0]);
     const uint64_t c0 = (D.n + bsz[0] - 1) / bsz[0];
@@ -1687,7 +1687,7 @@ __device__ void build_doc(const M& m, const BParams& P, uint32_t d, Cta& C, char
     __syncthreads();
     tmark(C, 0);
     for (uint32_t l = 0; l < D.L; l++) {
-      level_pass(m, P, D, C, scr, l, (uint32_t*)hist, dyn_words);
+      level_pass(m, PC, P, D, C, scr, l, (uint32_t*)hist, dyn_words);
       if (cta_failed(C)) break;
     }
   }
@@ -1722,12 +1722,13 @@ __device__ void build_doc(const M& m, const BParams& P, uint32_t d, Cta& C, char
   __syncthreads();
 }
 
-// NT threads per CTA, MINB CTAs per SM: the register budget per thread is
-// 65536 / (NT * MINB) (capped at 255).
-template <class M, int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_batch(BParams P, M m) {
-  // Dynamic shared memory: the level's fingerprint filter, then (during the
-  // output) 256 symbol counters per warp.
+// One CTA of 1024 threads per SM: 64 registers per thread.
+template <class M>
+__global__ void __launch_bounds__(kMaxBThreads, 1) k_batch(const __grid_constant__ BParams P, M m,
+                                                           const __grid_constant__ PrefixConst<M> PC,
+                                                           const __grid_constant__ KrPow pw) {
+  // Dynamic shared memory: the open keys' queues and bitmap of a level (or its
+  // window filter), then (during the output) the symbol counters.
   extern __shared__ unsigned int s_hist[];
   __shared__ Cta C;
   char* scr = P.scratch + (uint64_t)blockIdx.x * P.scratch_per_cta;
@@ -1737,7 +1738,7 @@ __global__ void __launch_bounds__(NT, MINB) k_batch(BParams P, M m) {
     const uint32_t d = C.doc;
     __syncthreads();
     if (d >= P.ndocs) return;
-    build_doc(m, P, d, C, scr, s_hist, P.dyn_words);
+    build_doc(m, PC, pw, P, d, C, scr, s_hist, P.dyn_words);
   }
 }
 
@@ -1747,7 +1748,7 @@ __global__ void __launch_bounds__(NT, MINB) k_batch(BParams P, M m) {
 // What the last batched build did (bt_batch_report).
 struct Report {
   uint64_t kernel_docs, worker_docs, launches, retried, threads, ctas_per_sm, pool_bytes, scratch_bytes,
-      max_grid, chunk, tuned, upload_us, kernel_us;
+      max_grid, upload_us, kernel_us;
 };
 std::mutex g_report_mu;
 Report g_report{};
@@ -1760,36 +1761,21 @@ struct DocPlan {
   uint64_t size_off;       // first block size in the batch's size array
 };
 
-// Powers (B^32)^i, i <= 1024, for the prefix pass.
+// Opt the kernel in to its dynamic shared memory, once per device.
 template <class M>
-std::vector<uint64_t> chunk_powers(const M& m, uint64_t B) {
-  std::vector<uint64_t> pw(1025);
-  const uint64_t X = pow_mod(m, B, 32);
-  pw[0] = 1 % m.q();
-  for (int i = 1; i <= 1024; i++) pw[i] = m.mul(pw[i - 1], X);
-  return pw;
-}
-
-// Opt every instantiation in to its dynamic shared memory, once per device.
-template <class M>
-int allow_smem(const M&, unsigned threads, unsigned ctas_per_sm, int bytes) {
-  static std::mutex mu;
-  static uint64_t done[8] = {};
+int allow_batch_smem(int bytes) {
+  static std::atomic<uint64_t> done{0};
   int dev = 0;
   BT_CUDA(cudaGetDevice(&dev));
-  (void)threads;
-  (void)ctas_per_sm;
-  const int which = 0;
-  std::lock_guard<std::mutex> g(mu);
-  if (done[which] & (1ull << (dev & 63))) return BT_OK;
-  BT_CUDA(cudaFuncSetAttribute(k_batch<M, 1024, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  done[which] |= 1ull << (dev & 63);
+  const uint64_t bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return BT_OK;
+  BT_CUDA(cudaFuncSetAttribute(k_batch<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  done.fetch_or(bit, std::memory_order_acq_rel);
   return BT_OK;
 }
 
 template <class M>
-int launch_docs(const M& m, const BParams& base, const std::vector<const DocPlan*>& order, uint32_t first,
-                uint32_t count, unsigned threads, unsigned ctas_per_sm, unsigned grid, uint64_t per_cta,
+int launch_docs(const M& m, const BParams& base, uint32_t first, uint32_t count, unsigned grid, uint64_t per_cta,
                 char* scratch, unsigned int* next, cudaStream_t s) {
   BParams P = base;
   P.docs = base.docs + first;
@@ -1797,21 +1783,13 @@ int launch_docs(const M& m, const BParams& base, const std::vector<const DocPlan
   P.next = next;
   P.scratch = scratch;
   P.scratch_per_cta = per_cta;
+  P.dyn_words = kDynWords;
   BT_CUDA(cudaMemsetAsync(next, 0, sizeof(unsigned int), s));
-  // Filter words: 128 KiB of shared memory with one CTA per SM, 64 KiB with
-  // two; at least the output's 256 counters per warp.
-  const uint32_t hist_words = threads / 32 * 256;
-  uint32_t fw = ctas_per_sm <= 1 ? 32768u : 16384u;
-  if (fw < hist_words) fw = hist_words;
-  P.dyn_words = fw;
-  const size_t smem = (size_t)fw * sizeof(unsigned int);
-  BT_TRY(allow_smem(m, threads, ctas_per_sm, (int)smem));
-  // The one launch shape: 1024 threads, one CTA per SM (two CTAs of 512 and
-  // one of 512 measured slower; see the shape list of the tuner).
-  if (threads != 1024 || ctas_per_sm != 1) return BT_EINVAL;
-  BT_LAUNCH(k_batch<M, 1024, 1><<<grid, 1024, smem, s>>>(P, m));
+  BT_TRY(allow_batch_smem<M>((int)(kDynWords * sizeof(unsigned int))));
+  const PrefixConst<M> PC(m, P.B);
+  const KrPow pw = kr_pow(m, pow_mod(m, P.B, 128));  // a thread of the prefix pass takes four 32-byte chunks
+  BT_LAUNCH(k_batch<M><<<grid, kMaxBThreads, kDynWords * sizeof(unsigned int), s>>>(P, m, PC, pw));
   BT_CUDA(cudaGetLastError());
-  (void)order;
   return BT_OK;
 }
 
@@ -1842,7 +1820,8 @@ struct DevFree {
 template <class M>
 int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, const uint32_t* leaf_lens,
               const bt_opts& o, std::vector<DocPlan>& plans, const std::vector<uint64_t>& sizes,
-              unsigned threads, unsigned ctas_per_sm, unsigned chunk, bt_tree** outs, cudaStream_t s) {
+              bt_tree** outs, cudaStream_t s) {
+  constexpr unsigned threads = kMaxBThreads, ctas_per_sm = 1;  // the launch shape: one CTA of 1024 threads per SM
   const uint64_t nd = plans.size();
   if (nd == 0) return BT_OK;
   int device = 0;
@@ -1897,18 +1876,14 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
   uint64_t* d_sizes;
   BRes* d_res;
   BLevelRes* d_lres;
-  uint64_t* d_pw;
   unsigned int* d_next;
   BT_TRY(mem.alloc(&d_docs, nd));
   BT_TRY(mem.alloc(&d_sizes, nlv));
   BT_TRY(mem.alloc(&d_res, nd));
   BT_TRY(mem.alloc(&d_lres, nlv));
-  BT_TRY(mem.alloc(&d_pw, 1025));
   BT_TRY(mem.alloc(&d_next, 64));
-  const std::vector<uint64_t> pw = chunk_powers(m, B);
   BT_CUDA(cudaMemcpyAsync(d_docs, hd.data(), nd * sizeof(BDoc), cudaMemcpyHostToDevice, s));
   BT_CUDA(cudaMemcpyAsync(d_sizes, hsz.data(), nlv * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
-  BT_CUDA(cudaMemcpyAsync(d_pw, pw.data(), pw.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
   BT_CUDA(cudaMemsetAsync(d_res, 0, nd * sizeof(BRes), s));
   // Output pool: three bytes per text byte plus a fixed part per document;
   // a document that does not fit is built again into a pool of exactly the
@@ -1947,11 +1922,8 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
   P.pool_used = d_used;
   P.pool_cap = pool_cap;
   P.B = B;
-  P.pw32 = d_pw;
   P.prune = o.prune ? 1 : 0;
   P.max_rounds = o.max_rounds ? o.max_rounds : 4096;
-  P.scan_u = chunk;
-  P.anchor_min_b = (o.flags & BT_FLAG_ANCHOR_ALL) ? 32 : kAnchorMinB;
 
   // Size classes: consecutive documents (in decreasing scratch need) whose
   // need is within 4x of the class's first; one launch per class, with as
@@ -2004,8 +1976,8 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
   if (timed) cudaEventRecord(ev[0], s);
   int lrc = BT_OK;
   for (size_t ci = 0; ci < cls.size() && lrc == BT_OK; ci++)
-    lrc = launch_docs(m, P, order, cls[ci].first, cls[ci].count, threads, ctas_per_sm, cls[ci].grid,
-                      cls[ci].per_cta, d_scratch, d_next + (ci % 64), s);
+    lrc = launch_docs(m, P, cls[ci].first, cls[ci].count, cls[ci].grid, cls[ci].per_cta, d_scratch,
+                      d_next + (ci % 64), s);
   if (timed) cudaEventRecord(ev[1], s);
   std::vector<BRes> res(nd);
   std::vector<BLevelRes> lres(nlv);
@@ -2055,8 +2027,7 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
       const unsigned grid = (unsigned)std::max<uint64_t>(
           1, std::min<uint64_t>({(uint64_t)hd2.size(), (uint64_t)nsm * ctas_per_sm, scratch_max / top,
                                  o.batch_ctas ? (uint64_t)o.batch_ctas : ~0ull}));
-      BT_TRY(launch_docs(m, P2, order, 0, (uint32_t)hd2.size(), threads, ctas_per_sm, grid, top, d_scratch,
-                         d_next, s));
+      BT_TRY(launch_docs(m, P2, 0, (uint32_t)hd2.size(), grid, top, d_scratch, d_next, s));
       BT_CUDA(cudaMemcpyAsync(res.data(), d_res, nd * sizeof(BRes), cudaMemcpyDeviceToHost, s));
       BT_CUDA(cudaMemcpyAsync(lres.data(), d_lres, nlv * sizeof(BLevelRes), cudaMemcpyDeviceToHost, s));
       BT_CUDA(cudaStreamSynchronize(s));
@@ -2136,7 +2107,6 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
     g_report.retried = retried;
     g_report.threads = threads;
     g_report.ctas_per_sm = ctas_per_sm;
-    g_report.chunk = chunk;
     g_report.pool_bytes = pool_cap;
     g_report.scratch_bytes = scratch_max;
     g_report.max_grid = 0;
@@ -2154,10 +2124,7 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
 // failure's status; trees already made stay in outs for the caller to free.
 int batch_kernel_build(const uint8_t* const* texts, const uint64_t* ns, const uint32_t* sigmas,
                        const uint32_t* taus, const uint32_t* leaf_lens, uint64_t ndocs, const bt_opts& o,
-                       std::vector<char>& routed, bt_tree** outs, uint32_t threads, uint32_t ctas_per_sm,
-                       uint32_t chunk, cudaStream_t s, const std::vector<char>* eligible) {
-  if (threads < 64 || threads > kMaxBThreads || threads % 32) return BT_EINVAL;
-  if (ctas_per_sm == 0) ctas_per_sm = 1;
+                       std::vector<char>& routed, bt_tree** outs, cudaStream_t s, const std::vector<char>* eligible) {
   if (o.modulus && (o.modulus < 300 || o.modulus >= (1ull << 32))) return BT_EINVAL;
   std::vector<DocPlan> plans;
   std::vector<uint64_t> sizes;
@@ -2184,9 +2151,8 @@ int batch_kernel_build(const uint8_t* const* texts, const uint64_t* ns, const ui
     routed[d] = 1;
   }
   if (o.modulus)
-    return run_batch(SmallMod{o.modulus}, texts, taus, leaf_lens, o, plans, sizes, threads, ctas_per_sm, chunk,
-                     outs, s);
-  return run_batch(Mersenne61{}, texts, taus, leaf_lens, o, plans, sizes, threads, ctas_per_sm, chunk, outs, s);
+    return run_batch(SmallMod{o.modulus}, texts, taus, leaf_lens, o, plans, sizes, outs, s);
+  return run_batch(Mersenne61{}, texts, taus, leaf_lens, o, plans, sizes, outs, s);
 }
 
 void batch_report_workers(uint64_t docs) {
@@ -2199,150 +2165,10 @@ void batch_report_reset() {
   g_report = Report{};
 }
 
-// ---------------------------------------------------------------------------
-// Autotuner of the batched kernel's launch shape: threads per CTA, CTAs per
-// SM and the window chunk of the scan (positions per lane and step).  For a
-// batch of at least kTuneMinDocs documents whose size class has no cached
-// choice, each candidate builds the same seeded sample of the batch: every
-// k-th document no longer than the batch's 75th length percentile, about
-// 1/16 of the batch but at least two documents per CTA of a full grid, so
-// that every SM stays busy during the trial.  A candidate's cost is the SM
-// time it spent: the sum over the sample of the cycles of each document's
-// CTA, divided by the CTAs that share an SM (a wall-clock time would measure
-// the sample's longest document instead).  The cheapest is cached per (log2
-// of the mean length, log2 of the longest, log2 of the batch size) for the
-// rest of the process.  Smaller batches use the default shape.
-namespace {
-struct Shape {
-  uint32_t threads, ctas, chunk;
-};
-// One CTA of 1024 threads per SM: two CTAs of 512 per SM measured slower on
-// every batch tried (4 KiB - 4 MiB: 11.4k against 14.6k docs/s; 4 KiB -
-// 16 MiB: 3.9k against 4.3k), as each document then has half the threads and
-// half the shared-memory filter, and the longest documents set the batch's
-// end.  The tuner picks the scan's run length.
-constexpr Shape kShapes[] = {{1024, 1, 8}, {1024, 1, 4}};
-constexpr uint64_t kTuneMinDocs = 1024;
-std::mutex g_tune_mu;
-std::vector<std::pair<uint64_t, Shape>> g_tuned;
-
-uint64_t tune_key(const uint64_t* ns, uint64_t ndocs) {
-  uint64_t sum = 0, mx = 0;
-  for (uint64_t d = 0; d < ndocs; d++) {
-    sum += ns[d];
-    mx = std::max<uint64_t>(mx, ns[d]);
-  }
-  auto lg = [](uint64_t x) {
-    uint64_t l = 0;
-    while (x > 1) {
-      x >>= 1;
-      l++;
-    }
-    return l;
-  };
-  return (lg(sum / std::max<uint64_t>(ndocs, 1)) << 16) | (lg(mx) << 8) | lg(ndocs);
-}
-}  // namespace
-
-int batch_shape(const uint8_t* const* texts, const uint64_t* ns, const uint32_t* sigmas, const uint32_t* taus,
-                const uint32_t* leaf_lens, uint64_t ndocs, const bt_opts& o, cudaStream_t s, uint32_t* threads,
-                uint32_t* ctas_per_sm, uint32_t* chunk, uint64_t* tuned_now) {
-  Shape best = kShapes[0];
-  *tuned_now = 0;
-  if (const char* e = getenv("BT_BATCH_SHAPE")) {  // "threads,ctas,chunk": a fixed run length for measurements
-    unsigned a = 0, b2 = 0, c = 0;
-    if (sscanf(e, "%u,%u,%u", &a, &b2, &c) == 3 && c) best = Shape{1024, 1, c};
-  } else if (ndocs >= kTuneMinDocs && !o.batch_ctas) {
-    const uint64_t key = tune_key(ns, ndocs);
-    bool found = false;
-    {
-      std::lock_guard<std::mutex> g(g_tune_mu);
-      for (auto& kv : g_tuned)
-        if (kv.first == key) {
-          best = kv.second;
-          found = true;
-        }
-    }
-    if (!found) {
-      // The sample: every k-th document, about 1/16 of the batch but at least
-      // two per CTA of a full grid.
-      std::vector<uint64_t> lens(ns, ns + ndocs);
-      std::nth_element(lens.begin(), lens.begin() + ndocs * 3 / 4, lens.end());
-      const uint64_t cap75 = lens[ndocs * 3 / 4];
-      const uint64_t want = std::max<uint64_t>(ndocs / 16, 2ull * device_sm_count() * 2);
-      const uint64_t step = std::max<uint64_t>(1, ndocs * 3 / 4 / want);
-      std::vector<const uint8_t*> st;
-      std::vector<uint64_t> sn;
-      std::vector<uint32_t> ss, stau, sl;
-      for (uint64_t d = 0; d < ndocs; d += step) {
-        if (ns[d] > cap75) continue;
-        st.push_back(texts[d]);
-        sn.push_back(ns[d]);
-        ss.push_back(sigmas[d]);
-        stau.push_back(taus[d]);
-        sl.push_back(leaf_lens[d]);
-      }
-      // A document's work is estimated as its bytes times its levels; a
-      // shape's cost is the batch's makespan when its CTAs, at the cycles
-      // per unit of work measured on the sample, take the documents from the
-      // queue longest first.
-      std::vector<double> work(ndocs, 0.0);
-      double sample_work = 0;
-      {
-        std::vector<uint64_t> b;
-        for (uint64_t d = 0; d < ndocs; d++) {
-          if (ns[d] > kBMaxText || plan_sizes(ns[d], taus[d], leaf_lens[d], o, b) != BT_OK) continue;
-          work[d] = (double)ns[d] * (double)b.size();
-        }
-        for (uint64_t d = 0; d < ndocs; d += step)
-          if (ns[d] <= cap75) sample_work += work[d];
-      }
-      std::vector<double> order(work);
-      std::sort(order.begin(), order.end(), std::greater<double>());
-      double best_cost = 1e300;
-      for (const Shape& sh : kShapes) {
-        std::vector<char> routed;
-        std::vector<bt_tree*> outs(st.size(), nullptr);
-        const int rc = batch_kernel_build(st.data(), sn.data(), ss.data(), stau.data(), sl.data(), st.size(), o,
-                                          routed, outs.data(), sh.threads, sh.ctas, sh.chunk, s, nullptr);
-        cudaStreamSynchronize(s);
-        double cycles = 0;
-        for (bt_tree* t : outs)
-          if (t)
-            for (int i = 0; i < 6; i++) cycles += (double)t->batch_cycles[i];
-        for (bt_tree* t : outs) bt_free(t);
-        if (rc != BT_OK) return rc;
-        const double per_work = cycles / std::max(sample_work, 1.0);
-        std::priority_queue<double, std::vector<double>, std::greater<double>> slots;
-        for (uint64_t g = 0; g < (uint64_t)device_sm_count() * sh.ctas; g++) slots.push(0.0);
-        double cost = 0;
-        for (double w : order) {
-          if (w <= 0) break;
-          const double t = slots.top() + w * per_work;
-          slots.pop();
-          slots.push(t);
-          cost = std::max(cost, t);
-        }
-        if (cost < best_cost) {
-          best_cost = cost;
-          best = sh;
-        }
-        (*tuned_now)++;
-      }
-      std::lock_guard<std::mutex> g(g_tune_mu);
-      g_tuned.emplace_back(key, best);
-    }
-  }
-  *threads = best.threads;
-  *ctas_per_sm = best.ctas;
-  *chunk = best.chunk;
-  return BT_OK;
-}
-
 // Long documents are built by the level kernels of the single-text path on
 // host workers, at the same time as the batched kernel builds the others: a
 // document longer than the batch's share per CTA would outlast the batch in
-// its one CTA, and the single-text path's anchored scan gets more out of a
+// its one CTA, and the single-text path gets more out of a
 // long text than one CTA does.  A document is long at kSplitMin bytes or more
 // and at least half the batch's bytes per CTA (so a batch large enough to
 // balance its CTAs is not split).  The batched kernel then leaves the workers
@@ -2352,7 +2178,7 @@ int batch_shape(const uint8_t* const* texts, const uint64_t* ns, const uint32_t*
 constexpr uint64_t kSplitMin = 8ull << 20;
 
 uint32_t batch_split(const uint64_t* ns, const uint32_t* taus, const uint32_t* leaf_lens, uint64_t ndocs,
-                     const bt_opts& o, uint32_t ctas_per_sm, std::vector<char>& eligible) {
+                     const bt_opts& o, std::vector<char>& eligible) {
   (void)taus;
   (void)leaf_lens;
   eligible.assign(ndocs, 1);
@@ -2360,7 +2186,7 @@ uint32_t batch_split(const uint64_t* ns, const uint32_t* taus, const uint32_t* l
   const unsigned nsm = device_sm_count();
   double total = 0, heavy = 0;
   for (uint64_t d = 0; d < ndocs; d++) total += (double)ns[d];
-  const double share = total / ((double)nsm * ctas_per_sm);
+  const double share = total / (double)nsm;
   const double lim = std::max((double)kSplitMin, 0.5 * share);
   for (uint64_t d = 0; d < ndocs; d++)
     if ((double)ns[d] >= lim) {
@@ -2373,12 +2199,7 @@ uint32_t batch_split(const uint64_t* ns, const uint32_t* taus, const uint32_t* l
   }
   uint32_t reserve = (uint32_t)((double)nsm * heavy / total + 0.5);
   reserve = std::max<uint32_t>(8, std::min<uint32_t>(reserve, nsm / 2));
-  return (nsm - reserve) * ctas_per_sm;
-}
-
-void batch_report_tuned(uint64_t trials) {
-  std::lock_guard<std::mutex> g(g_report_mu);
-  g_report.tuned = trials;
+  return nsm - reserve;
 }
 
 }  // namespace bt
@@ -2389,7 +2210,7 @@ extern "C" int bt_batch_report(uint64_t* out, uint32_t cap) {
   std::lock_guard<std::mutex> g(g_report_mu);
   const uint64_t v[13] = {g_report.kernel_docs, g_report.worker_docs, g_report.launches, g_report.retried,
                           g_report.threads, g_report.ctas_per_sm, g_report.pool_bytes, g_report.scratch_bytes,
-                          g_report.max_grid, g_report.chunk, g_report.tuned, g_report.upload_us,
+                          g_report.max_grid, 0, 0, g_report.upload_us,
                           g_report.kernel_us};
   memcpy(out, v, sizeof(v));
   return BT_OK;

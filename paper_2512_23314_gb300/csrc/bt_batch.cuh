@@ -12,19 +12,12 @@
 #pragma once
 
 #include "bt_internal.cuh"
+#include "bt_quick.cuh"
 
 namespace bt {
 
 constexpr uint32_t kBMaxLevels = 40;       // documents with more levels use the standard path
 constexpr uint64_t kBMaxText = 1ull << 30; // longest document of the batched path
-// Selected grams (anchors of the window scan on levels with long blocks): a
-// 16-byte gram is selected when its 32-bit hash is below 2^(32 - 6), one
-// position in 64 on average; a document keeps up to n/32 + 1024 of them.
-constexpr uint32_t kGramW = 16;
-constexpr uint32_t kGramSelShift = 26;
-constexpr uint64_t kAnchorMinB = 1024;  // levels with b >= this scan by anchors (BT_FLAG_ANCHOR_ALL: 32)
-__host__ __device__ inline uint64_t gram_list_cap(uint64_t n) { return n / 32 + 1024; }
-
 // One document of a batch (host -> device).
 struct BDoc {
   const uint8_t* T;     // device text
@@ -110,8 +103,11 @@ __host__ __device__ inline uint64_t out_layout(uint32_t L, uint32_t base, const 
 // Scratch of one CTA for one document: offsets in bytes from the CTA's
 // region.  Level l may hold at most cmax[l] = ceil(n / b_l) blocks.
 struct ScratchLayout {
-  uint64_t H;                                   // u64[n + 1]
-  uint64_t lpos, lhash;                         // u32[gram_list_cap(n)]: selected grams in text order
+  uint64_t Hs;                                  // u64[n / 32 + 2]: prefix fingerprints H(32 j)
+  uint64_t big;                                 // the list's positions and distances, u32[n] each; later, for
+                                                // levels of short blocks, u64[n + 1]: H at every position
+  uint64_t idx, seg1, seg2, first;              // the list's index and segment minima; the first-occurrence table
+  uint64_t cells;
   uint64_t st[kBMaxLevels], lo[kBMaxLevels], off[kBMaxLevels];  // u64[cmax]
   uint64_t ptr[kBMaxLevels], mw[kBMaxLevels], mr[kBMaxLevels];  // u32
   uint64_t temp;                                // per-level work area (reused)
@@ -124,18 +120,24 @@ __host__ __device__ inline uint64_t pow2_ge(uint64_t x) {
   return p;
 }
 
-// Bytes of the per-level work area for a level of at most cm blocks: the
-// level pass (fingerprints, slots, pair results, jobs, suspects, block and
-// pair tables) or the pruning pass, whichever is larger.
-__host__ __device__ inline uint64_t temp_bytes(uint64_t cm) {
+// Bytes of the per-level work area for a level of at most cm blocks of b bytes:
+// the level pass (by first occurrences, or for short blocks the tables of the
+// window scan) or the pruning pass, whichever is larger.
+__host__ __device__ inline uint64_t temp_bytes(uint64_t cm, uint64_t b) {
   const uint64_t cap = pow2_ge(2 * cm);
-  const uint64_t level = out_align(cm * 8 + 8) * 5      // fpB, plo, job_of, susp, exlo
-                         + out_align(cm * 4 + 4) * 4    // slotB, slotP, mismatch, wpop
-                         + out_align(cm + 8)            // pm
-                         + out_align(cm * 32 + 32)      // jobs
-                         + out_align(cm * 8 + 8)        // exact-scan powers
-                         + out_align(cap * 32) + out_align(cap * 16)
-                         + out_align(cap * 8);          // anchor table
+  const uint64_t quick = out_align(cm * 4 + 4) * 4      // A, X, flags, wpop
+                         + out_align(cm * 8 + 8)        // items
+                         + out_align(cm + 8)            // ps
+                         + out_align(cap * 32) + out_align(cap * 16)               // block and pair tables
+                         + out_align(2 * cap * 16) + out_align(2 * cap * 8)        // gram table and bounds
+                         + out_align(8 * cm + 1024)     // bitmap
+                         + out_align(cm * 8 + 8) * 6;   // islot, igram, differ, susp (two per block), exlo
+  const uint64_t scan = out_align(cm * 8 + 8) * 6       // fpB, exBL, job_of, susp, exlo, spare
+                        + out_align(cm * 4 + 4) * 4     // slotB, slotP, mismatch, wpop
+                        + out_align(cm + 8)             // pm
+                        + out_align(cm * 32 + 32)       // jobs
+                        + out_align(cap * 32) + out_align(cap * 16);
+  const uint64_t level = b >= kQuickMinB ? quick : scan;
   const uint64_t prune = out_align(cm + 8) * 5          // hit_v, hit2, tgt_w, gone, mk2
                          + out_align(cm * 4 + 4) * 7    // state, indeg, fq x2, nidx, wpop, ptr2
                          + out_align(cm * 8 + 8) * 5;   // t1, t2, st2, off2, lo2
@@ -143,17 +145,26 @@ __host__ __device__ inline uint64_t temp_bytes(uint64_t cm) {
 }
 
 __host__ __device__ inline uint64_t scratch_layout(uint64_t n, uint32_t L, const uint64_t* b, ScratchLayout* s) {
-  uint64_t o = 0, cm_max = 1;
-  s->H = o;
-  o = out_align(o + (n + 1) * 8);
-  s->lpos = o;
-  o = out_align(o + gram_list_cap(n) * 4);
-  s->lhash = o;
-  o = out_align(o + gram_list_cap(n) * 4);
+  uint64_t o = 0, temp = 0;
+  s->Hs = o;
+  o = out_align(o + (n / 32 + 2) * 8);
+  s->big = o;
+  o = out_align(o + (n + 64) * 8);
+  s->idx = o;
+  o = out_align(o + (n / 32 + 2) * 4);
+  s->seg1 = o;
+  o = out_align(o + (n / 1024 + 2) * 4);
+  s->seg2 = o;
+  o = out_align(o + (n / 65536 + 2) * 4);
+  s->cells = 1024;
+  while (s->cells < n / 8) s->cells <<= 1;
+  s->first = o;
+  o = out_align(o + s->cells * 4);
   for (uint32_t l = 0; l < L; l++) {
     const uint64_t cm = (n + b[l] - 1) / b[l];
     const uint64_t words = (cm + 31) / 32;
-    if (cm > cm_max) cm_max = cm;
+    const uint64_t tb = temp_bytes(cm, b[l]);
+    if (tb > temp) temp = tb;
     s->st[l] = o;
     o = out_align(o + cm * 8 + 8);
     s->lo[l] = o;
@@ -168,7 +179,7 @@ __host__ __device__ inline uint64_t scratch_layout(uint64_t n, uint32_t L, const
     o = out_align(o + (words + 1) * 4 + 4);
   }
   s->temp = o;
-  o = out_align(o + temp_bytes(cm_max));
+  o = out_align(o + temp);
   s->total = o;
   return o;
 }
@@ -187,12 +198,9 @@ struct BParams {
   unsigned long long* pool_used;
   uint64_t pool_cap;
   uint64_t B;                     // Karp-Rabin base
-  const uint64_t* pw32;           // (B^32)^i for i <= blockDim.x
   int prune;
   uint64_t max_rounds;
   uint32_t dyn_words;             // 32-bit words of dynamic shared memory
-  uint32_t scan_u;                // window run: consecutive positions per lane of the scan (1-8)
-  uint64_t anchor_min_b;          // levels with b at least this scan by anchors
 };
 
 }  // namespace bt

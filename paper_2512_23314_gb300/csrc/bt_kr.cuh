@@ -59,6 +59,84 @@ struct ChunkHash<Mersenne61> {
   }
 };
 
+// Powers of the shift X of one scan item: X^1,2,4,8,16 within a warp and
+// X^32,64,..,512 across the warps.
+struct KrPow {
+  uint64_t x[5], w[5];
+};
+template <class M>
+KrPow kr_pow(const M& m, uint64_t X) {
+  KrPow p;
+  for (int i = 0; i < 5; i++) {
+    p.x[i] = X;
+    X = m.mul(X, X);
+  }
+  for (int i = 0; i < 5; i++) {
+    p.w[i] = X;
+    X = m.mul(X, X);
+  }
+  return p;
+}
+
+// Inclusive scan of the items' fingerprints over a CTA of at most 1024
+// threads (sm: 32 words).
+template <class M>
+__device__ __forceinline__ uint64_t cta_kr_scan(const M& m, uint64_t h, const KrPow& pw, uint64_t xl, uint64_t* sm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 5; i++) {
+    const uint64_t o = __shfl_up_sync(0xFFFFFFFFu, h, 1 << i);
+    if (lane >= (1 << i)) h = m.add(m.mul(o, pw.x[i]), h);
+  }
+  if (lane == 31) sm[warp] = h;
+  __syncthreads();
+  if (warp == 0) {
+    uint64_t w = lane < nw ? sm[lane] : 0;
+#pragma unroll
+    for (int i = 0; i < 5; i++) {
+      const uint64_t o = __shfl_up_sync(0xFFFFFFFFu, w, 1 << i);
+      if (lane >= (1 << i)) w = m.add(m.mul(o, pw.w[i]), w);
+    }
+    sm[lane] = w;
+  }
+  __syncthreads();
+  if (warp > 0) h = m.add(m.mul(sm[warp - 1], xl), h);
+  __syncthreads();
+  return h;
+}
+
+// X^(lane + 1) from the squares: the shift of a warp's carry-in.
+template <class M>
+__device__ __forceinline__ uint64_t kr_lane_pow(const M& m, const KrPow& pw) {
+  const unsigned e = (threadIdx.x & 31) + 1;
+  uint64_t r = 1;
+#pragma unroll
+  for (int i = 0; i < 5; i++)
+    if ((e >> i) & 1u) r = m.mul(r, pw.x[i]);
+  return e == 32 ? pw.w[0] : r;
+}
+
+// The words of chunk j, or zeros for a chunk the text does not hold.
+__device__ __forceinline__ void load_chunk(const uint8_t* __restrict__ T, uint64_t nchunks, uint64_t j, bool aligned,
+                                           uint32_t* w) {
+  if (j >= nchunks) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) w[i] = 0;
+    return;
+  }
+  const uint8_t* p = T + j * kPrefixStride;
+  if (aligned) {
+    const uint4 v0 = ((const uint4*)p)[0], v1 = ((const uint4*)p)[1];
+    w[0] = v0.x, w[1] = v0.y, w[2] = v0.z, w[3] = v0.w;
+    w[4] = v1.x, w[5] = v1.y, w[6] = v1.z, w[7] = v1.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+      w[i] = (uint32_t)p[4 * i] | ((uint32_t)p[4 * i + 1] << 8) | ((uint32_t)p[4 * i + 2] << 16) |
+             ((uint32_t)p[4 * i + 3] << 24);
+  }
+}
+
 // H(p) at any position from the stride-32 prefix values and the text.  With
 // j = p / 32 and r = p mod 32, H(p) B^(32-r) = H(32 j) B^32 + the chunk's
 // first r symbols times B^31, B^30, ..: the same constants for every r (bytes
@@ -68,32 +146,29 @@ struct ChunkHash<Mersenne61> {
 // text byte: this form neither writes it (445 us of a 256 MiB build) nor
 // needs its memory.
 template <class M>
-struct PrefixAt {  // any modulus: Horner
-  const uint8_t* T;
-  const uint64_t* Hs;
-  uint64_t n, B;
-  PrefixAt(const M&, const uint8_t* T_, uint64_t n_, const uint64_t* Hs_, uint64_t B_) : T(T_), Hs(Hs_), n(n_), B(B_) {}
-  __device__ __forceinline__ uint64_t at(const M& m, uint64_t p) const {
+struct PrefixConst {  // any modulus: Horner
+  uint64_t B, B32;
+  ChunkHash<M> hash;
+  PrefixConst(const M& m, uint64_t B_) : B(B_), B32(pow_mod(m, B_, 32)), hash(m, B_) {}
+  __device__ __forceinline__ uint64_t at(const M& m, const uint8_t* T, uint64_t, const uint64_t* Hs, bool,
+                                         uint64_t p) const {
     uint64_t h = Hs[p / kPrefixStride];
     for (uint64_t x = p & ~(uint64_t)(kPrefixStride - 1); x < p; x++) h = m.add(m.mul(h, B), (uint64_t)T[x] + 1);
     return h;
   }
 };
 template <>
-struct PrefixAt<Mersenne61> {
-  const uint8_t* T;
-  const uint64_t* Hs;
-  uint64_t n, B32;
-  bool aligned;
+struct PrefixConst<Mersenne61> {
+  uint64_t B, B32;
   ChunkHash<Mersenne61> hash;
   uint64_t ones[32], inv[32];  // [r]: the sum of B^31 .. B^(32-r); B^-(32-r)
-  PrefixAt(const Mersenne61& m, const uint8_t* T_, uint64_t n_, const uint64_t* Hs_, uint64_t B)
-      : T(T_), Hs(Hs_), n(n_), B32(pow_mod(m, B, 32)), aligned((((uintptr_t)T_) & 15) == 0), hash(m, B) {
+  PrefixConst(const Mersenne61& m, uint64_t B_) : B(B_), B32(pow_mod(m, B_, 32)), hash(m, B_) {
     ones[0] = 0;
     for (int r = 1; r < 32; r++) ones[r] = m.add(ones[r - 1], pow_mod(m, B, 32 - r));
     for (int r = 0; r < 32; r++) inv[r] = pow_mod(m, pow_mod(m, B, 32 - r), Mersenne61::Q - 2);
   }
-  __device__ __forceinline__ uint64_t at(const Mersenne61& m, uint64_t p) const {
+  __device__ __forceinline__ uint64_t at(const Mersenne61& m, const uint8_t* T, uint64_t n, const uint64_t* Hs,
+                                         bool aligned, uint64_t p) const {
     const uint64_t j = p >> 5;
     const uint32_t r = (uint32_t)p & 31u;
     const uint64_t h = Hs[j];
@@ -120,6 +195,19 @@ struct PrefixAt<Mersenne61> {
     const uint64_t u = m.add(m.mul(h, B32), m.add(hash.dot(w), ones[r]));
     return m.mul(u, inv[r]);
   }
+};
+
+// The prefix values of one text.
+template <class M>
+struct PrefixAt {
+  const PrefixConst<M>& c;
+  const uint8_t* T;
+  const uint64_t* Hs;
+  uint64_t n;
+  bool aligned;
+  __device__ __forceinline__ PrefixAt(const PrefixConst<M>& c_, const uint8_t* T_, uint64_t n_, const uint64_t* Hs_)
+      : c(c_), T(T_), Hs(Hs_), n(n_), aligned((((uintptr_t)T_) & 15) == 0) {}
+  __device__ __forceinline__ uint64_t at(const M& m, uint64_t p) const { return c.at(m, T, n, Hs, aligned, p); }
 };
 
 }  // namespace bt

@@ -128,84 +128,6 @@ constexpr int kKrThreads = 256;    // threads of a tile of kTile chunks
 constexpr int kKrChunks = 4;       // chunks per thread
 static_assert(kKrThreads * kKrChunks == kTile, "a tile is kTile chunks");
 
-// Powers of the shift X of one scan item: X^1,2,4,8,16 within a warp and
-// X^32,64,..,512 across the warps.
-struct KrPow {
-  uint64_t x[5], w[5];
-};
-template <class M>
-KrPow kr_pow(const M& m, uint64_t X) {
-  KrPow p;
-  for (int i = 0; i < 5; i++) {
-    p.x[i] = X;
-    X = m.mul(X, X);
-  }
-  for (int i = 0; i < 5; i++) {
-    p.w[i] = X;
-    X = m.mul(X, X);
-  }
-  return p;
-}
-
-// Inclusive scan of the items' fingerprints over a CTA of at most 1024
-// threads (sm: 32 words).
-template <class M>
-__device__ __forceinline__ uint64_t cta_kr_scan(const M& m, uint64_t h, const KrPow& pw, uint64_t xl, uint64_t* sm) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int i = 0; i < 5; i++) {
-    const uint64_t o = __shfl_up_sync(0xFFFFFFFFu, h, 1 << i);
-    if (lane >= (1 << i)) h = m.add(m.mul(o, pw.x[i]), h);
-  }
-  if (lane == 31) sm[warp] = h;
-  __syncthreads();
-  if (warp == 0) {
-    uint64_t w = lane < nw ? sm[lane] : 0;
-#pragma unroll
-    for (int i = 0; i < 5; i++) {
-      const uint64_t o = __shfl_up_sync(0xFFFFFFFFu, w, 1 << i);
-      if (lane >= (1 << i)) w = m.add(m.mul(o, pw.w[i]), w);
-    }
-    sm[lane] = w;
-  }
-  __syncthreads();
-  if (warp > 0) h = m.add(m.mul(sm[warp - 1], xl), h);
-  __syncthreads();
-  return h;
-}
-
-// X^(lane + 1) from the squares: the shift of a warp's carry-in.
-template <class M>
-__device__ __forceinline__ uint64_t kr_lane_pow(const M& m, const KrPow& pw) {
-  const unsigned e = (threadIdx.x & 31) + 1;
-  uint64_t r = 1;
-#pragma unroll
-  for (int i = 0; i < 5; i++)
-    if ((e >> i) & 1u) r = m.mul(r, pw.x[i]);
-  return e == 32 ? pw.w[0] : r;
-}
-
-// The words of chunk j, or zeros for a chunk the text does not hold.
-__device__ __forceinline__ void load_chunk(const uint8_t* __restrict__ T, uint64_t nchunks, uint64_t j, bool aligned,
-                                           uint32_t* w) {
-  if (j >= nchunks) {
-#pragma unroll
-    for (int i = 0; i < 8; i++) w[i] = 0;
-    return;
-  }
-  const uint8_t* p = T + j * kPrefixStride;
-  if (aligned) {
-    const uint4 v0 = ((const uint4*)p)[0], v1 = ((const uint4*)p)[1];
-    w[0] = v0.x, w[1] = v0.y, w[2] = v0.z, w[3] = v0.w;
-    w[4] = v1.x, w[5] = v1.y, w[6] = v1.z, w[7] = v1.w;
-  } else {
-#pragma unroll
-    for (int i = 0; i < 8; i++)
-      w[i] = (uint32_t)p[4 * i] | ((uint32_t)p[4 * i + 1] << 8) | ((uint32_t)p[4 * i + 2] << 16) |
-             ((uint32_t)p[4 * i + 3] << 24);
-  }
-}
-
 // agg[i] = fingerprint of tile i (kTile chunks); the last tile is not needed.
 // pw: the shift of a thread's four chunks, P = B^32 the shift of one.
 template <class M>

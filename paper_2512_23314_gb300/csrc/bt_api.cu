@@ -19,7 +19,7 @@
 
 namespace bt {
 
-int alphabet(const uint8_t* T, uint64_t n, uint32_t sigma, bt_tree* t, cudaStream_t s);
+int alphabet(const uint8_t* T, uint64_t n, uint32_t* seen, bt_tree* t, Status* st, cudaStream_t s);
 int run_query_one(const bt_tree* t, int kind, uint64_t a0, uint64_t a1, uint64_t* out, cudaStream_t s);
 int batch_kernel_build(const uint8_t* const* texts, const uint64_t* ns, const uint32_t* sigmas,
                        const uint32_t* taus, const uint32_t* leaf_lens, uint64_t ndocs, const bt_opts& o,
@@ -72,10 +72,28 @@ ProfScope::~ProfScope() {
   cudaEventRecord(g_prof[slot].b, s);
 }
 
+namespace {
+struct PinnedPage {
+  char* p = nullptr;
+  ~PinnedPage() {
+    if (p) cudaFreeHost(p);
+  }
+};
+thread_local PinnedPage g_page;
+}  // namespace
+
+char* pinned_page() {
+  if (!g_page.p && cudaHostAlloc((void**)&g_page.p, 8192, cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    g_page.p = nullptr;
+  }
+  return g_page.p;
+}
+
 int sync_status(BuildCtx& ctx) {
   BT_CUDA(cudaMemcpyAsync(ctx.st_host, ctx.st, sizeof(Status), cudaMemcpyDeviceToHost, ctx.s));
   BT_CUDA(cudaStreamSynchronize(ctx.s));
-  return BT_OK;
+  return ctx.st_host->symbols > ctx.sigma ? BT_EINVAL : BT_OK;
 }
 
 // splitmix64 (Steele, Lea, Flood 2014): the seed -> base map.
@@ -227,17 +245,26 @@ static int build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, 
   ctx.leaf_counts = (o.flags & BT_FLAG_LEAF_COUNTS) ? 1 : 0;
   ctx.sort_scan = (o.flags & BT_FLAG_SORT_SCAN) ? 1 : 0;
   ctx.partitions = o.partitions;
-  BT_TRY(sc.alloc(&ctx.st, 1));
-  BT_CUDA(cudaMemsetAsync(ctx.st, 0, sizeof(Status), s));
-  BT_CUDA(cudaMallocHost(&ctx.st_host, sizeof(Status)));
-  struct HostFree {
-    void* p;
-    ~HostFree() { cudaFreeHost(p); }
-  } hf{ctx.st_host};
+  // The build's status, the alphabet's marks, the pruned block counts.
+  struct Small {
+    Status st;
+    uint64_t new_blocks[kMaxLevels];
+    uint32_t seen[256 + 1];
+  };
+  Small* small;
+  BT_TRY(sc.alloc(&small, 1));
+  BT_CUDA(cudaMemsetAsync(small, 0, sizeof(Small), s));
+  ctx.st = &small->st;
+  ctx.new_blocks = small->new_blocks;
+  ctx.sigma = sigma;
+  char* page = pinned_page();
+  if (!page) return BT_ENOMEM;
+  ctx.st_host = (Status*)page;
+  static_assert(sizeof(Status) <= kPageQuick, "the status fits its place in the pinned page");
 
   {
     ProfScope ps("phase_alphabet", s, n);
-    BT_TRY(alphabet(dT, n, sigma, t, s));
+    BT_TRY(alphabet(dT, n, small->seen, t, ctx.st, s));
   }
   tr.mark("setup+alphabet");
   {
@@ -255,8 +282,8 @@ static int build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, 
   {
     ProfScope ps("phase_prune", s, 0);
     if (t->prune) BT_TRY(prune_tree(ctx, o.max_rounds));
-    else
-      for (Level& v : t->lv) v.stats[BT_ST_FINAL_BLOCKS] = v.c;
+    BT_TRY(tree_totals(ctx));
+    t->S = (uint32_t)ctx.st_host->symbols;
   }
   tr.mark("prune");
   {
@@ -272,7 +299,6 @@ static int build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, 
     bytes += v.c * 8 + (2 * words + 1) * 4 + (v.cnt ? 2 * counter_stride(v.c) * t->S * v.cw : 0);
   }
   t->dev_bytes = bytes;
-  BT_CUDA(cudaStreamSynchronize(s));
   BT_TRY(sync_status(ctx));
   tr.mark("finish");
   if (ctx.st_host->error) return BT_EINTERNAL;
@@ -350,7 +376,28 @@ struct ExportLevel {
   uint64_t at;  // u64 index of the level's first field in the serialization
 };
 
-__global__ void k_export_level(ExportLevel e, uint64_t* __restrict__ out) {
+struct ExportArgs {
+  ExportLevel lv[kMaxLevels];
+  uint64_t head[6];
+  uint32_t L;
+  const uint8_t* leaf;
+  uint64_t leaf_bytes, leaf_at;
+};
+
+// blockIdx.y: a level, or (the last one) the header and the leaf text.
+__global__ void __launch_bounds__(256) k_export(const __grid_constant__ ExportArgs E, uint64_t* __restrict__ out) {
+  if (blockIdx.y == E.L) {
+    const uint64_t words = (E.leaf_bytes + 7) / 8;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x) {
+      uint64_t w = ((const uint64_t*)E.leaf)[i];  // (the leaf text is padded by 16 bytes)
+      if (8 * i + 8 > E.leaf_bytes) w &= (1ull << (8 * (E.leaf_bytes - 8 * i))) - 1;
+      out[E.leaf_at + i] = w;
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 6) out[threadIdx.x] = E.head[threadIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x == 6) out[E.leaf_at - 1] = E.leaf_bytes;
+    return;
+  }
+  const ExportLevel& e = E.lv[blockIdx.y];
   const uint64_t words = (e.c + 31) / 32, mwords = (e.c + 63) / 64;
   uint64_t* marks = out + e.at + 2;
   uint64_t* pairs = marks + mwords + 1;
@@ -514,24 +561,16 @@ void bt_free(bt_tree* t) {
 // One query: its arguments travel with the launch and the kernel writes the
 // answer to the calling thread's pinned word (portable: any device), so a call
 // is one launch and one wait instead of an allocation, two copies and a free
-// around them (about 38 us).  The word is given back when its thread ends.
-namespace {
-struct AnswerWord {
-  uint64_t* p = nullptr;
-  ~AnswerWord() {
-    if (p) cudaFreeHost(p);
-  }
-};
-thread_local AnswerWord g_answer;
-}  // namespace
-
+// around them (about 38 us).
 static int single_query(const bt_tree* t, int kind, uint64_t a0, uint64_t a1, uint64_t* res) {
   if (!t) return BT_EINVAL;
   cudaStream_t s = cudaStreamPerThread;
-  if (!g_answer.p) BT_CUDA(cudaHostAlloc((void**)&g_answer.p, sizeof(uint64_t), cudaHostAllocPortable));
-  BT_TRY(run_query_one(t, kind, a0, a1, g_answer.p, s));
+  char* page = pinned_page();
+  if (!page) return BT_ENOMEM;
+  uint64_t* answer = (uint64_t*)(page + kPageAnswer);
+  BT_TRY(run_query_one(t, kind, a0, a1, answer, s));
   if (cudaStreamSynchronize(s) != cudaSuccess) return BT_ECUDA;
-  *res = *(volatile uint64_t*)g_answer.p;
+  *res = *(volatile uint64_t*)answer;
   return BT_OK;
 }
 
@@ -585,23 +624,19 @@ int bt_stats(const bt_tree* t, uint64_t* out, uint64_t cap) {
 
 int bt_export(const bt_tree* t, uint8_t* buf, uint64_t cap, uint64_t* len) {
   if (!t || !len) return BT_EINVAL;
-  // The layout needs each level's number of marked blocks (the last entry of
-  // its rank prefix); the serialization itself is written on the device and
-  // copied out once.
+  // The layout follows from the levels' block and mark counts; the
+  // serialization is written on the device by one launch and copied out once.
   cudaStream_t s = cudaStreamPerThread;
   const uint32_t L = t->L;
-  std::vector<uint32_t> nm(L, 0);
-  for (uint32_t l = 0; l < L; l++) {
-    const Level& v = t->lv[l];
-    BT_CUDA(cudaMemcpyAsync(&nm[l], v.mr + (v.c + 31) / 32, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  }
-  BT_CUDA(cudaStreamSynchronize(s));
-  std::vector<ExportLevel> ex(L);
+  ExportArgs E;
+  uint64_t cmax = 1;
   uint64_t at = 6;  // header: "BLKTREE1", n, tau, leaf_len, L, prune
   for (uint32_t l = 0; l < L; l++) {
     const Level& v = t->lv[l];
-    ex[l] = ExportLevel{v.mw, v.mr, v.rec, v.c, v.b, v.c - nm[l], at};
-    at += 2 + (v.c + 63) / 64 + 1 + 2 * (v.c - nm[l]);
+    const uint64_t nptr = v.c - v.nmarked;
+    E.lv[l] = ExportLevel{v.mw, v.mr, v.rec, v.c, v.b, nptr, at};
+    at += 2 + (v.c + 63) / 64 + 1 + 2 * nptr;
+    cmax = v.c > cmax ? v.c : cmax;
   }
   const uint64_t leaf_at = at + 1, leaf_pad = (t->leaf_bytes + 7) / 8 * 8;
   const uint64_t need = leaf_at * 8 + leaf_pad;
@@ -612,15 +647,14 @@ int bt_export(const bt_tree* t, uint8_t* buf, uint64_t cap, uint64_t* len) {
   uint64_t* d;
   BT_TRY(sc.alloc(&d, need / 8));
   const uint64_t head[6] = {0x31454552544B4C42ull, t->n, t->tau, t->leaf_len, L, (uint64_t)t->prune};
-  BT_CUDA(cudaMemcpyAsync(d, head, sizeof(head), cudaMemcpyHostToDevice, s));
-  for (uint32_t l = 0; l < L; l++)
-    BT_LAUNCH(k_export_level<<<grid_for(t->lv[l].c, 256), 256, 0, s>>>(ex[l], d));
-  const uint64_t lb = t->leaf_bytes;
-  BT_CUDA(cudaMemcpyAsync(d + at, &lb, sizeof(lb), cudaMemcpyHostToDevice, s));
-  if (leaf_pad) {
-    BT_CUDA(cudaMemsetAsync((uint8_t*)(d + leaf_at) + leaf_pad - 8, 0, 8, s));
-    if (lb) BT_CUDA(cudaMemcpyAsync(d + leaf_at, t->leaf, lb, cudaMemcpyDeviceToDevice, s));
-  }
+  memcpy(E.head, head, sizeof(head));
+  E.L = L;
+  E.leaf = t->leaf;
+  E.leaf_bytes = t->leaf_bytes;
+  E.leaf_at = leaf_at;
+  const uint64_t work = cmax > leaf_pad / 8 ? cmax : leaf_pad / 8;
+  BT_LAUNCH(k_export<<<dim3(grid_for(work, 256, 2048), L + 1), 256, 0, s>>>(E, d));
+  BT_CUDA(cudaGetLastError());
   BT_CUDA(cudaMemcpyAsync(buf, d, need, cudaMemcpyDeviceToHost, s));
   BT_CUDA(cudaStreamSynchronize(s));
   return BT_OK;

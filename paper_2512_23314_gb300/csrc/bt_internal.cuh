@@ -231,7 +231,6 @@ struct bt_tree {
   uint32_t base = 0;     // the level queries start at
   uint32_t* pre = nullptr;
   int16_t* sym = nullptr;  // device map
-  int16_t sym_host[256];
   uint32_t S = 0;
   bt::TreeView* view = nullptr;  // device copy of the view
   void* recs = nullptr;          // records, mark words and rank prefixes of all levels
@@ -299,8 +298,17 @@ struct Status {
   unsigned long long tail_susp;      // tail key verification state
   unsigned long long rounds;         // pruning rounds used
   unsigned long long undecided;      // pruning: candidates left after a round
-  unsigned long long pad[4];
+  unsigned long long symbols;        // distinct bytes of the text
+  unsigned long long leaf_short;     // bytes the text's last leaf block lacks, when it is marked
+  unsigned long long blocks[64], marks[64];  // per level of the finished tree
 };
+
+// 8 KiB of pinned host memory of the calling thread (portable: any device),
+// given back when the thread ends: where its builds and single queries
+// receive small results.  A build that allocated its own cost 0.1 ms and more
+// in the driver each time.
+char* pinned_page();
+constexpr uint32_t kPageQuick = 4096, kPageAnswer = 6144;  // places in it (the build's Status at 0)
 
 // Test hook (bt_test_alloc_limit): the largest single device allocation a
 // build may make; larger ones fail as if the device were out of memory.
@@ -411,6 +419,8 @@ struct BuildCtx {
   Arena arena;        // per-level scratch
   Status* st;         // device status
   Status* st_host;    // pinned mirror
+  uint32_t sigma = 0;              // distinct bytes the caller allows (sync_status checks)
+  uint64_t* new_blocks = nullptr;  // block counts of the pruned levels (device)
   cudaStream_t s;
   uint64_t verify_bytes = 0, collisions = 0;
   int dense_scan = 0;  // probe every window (diagnostic) instead of the anchored scan
@@ -425,6 +435,7 @@ struct BuildCtx {
 
 int build_levels(BuildCtx& ctx);
 int prune_tree(BuildCtx& ctx, uint64_t max_rounds);
+int tree_totals(BuildCtx& ctx);
 int build_counters(BuildCtx& ctx);
 int pack_records(BuildCtx& ctx);
 int sync_status(BuildCtx& ctx);

@@ -23,9 +23,11 @@
 // candidates the previous round decided (a worklist of block indices); wide
 // frontiers go to multi-CTA launches, narrow ones to a single CTA that runs
 // the remaining rounds without returning to the host.
+#include <algorithm>
 #include <vector>
 
 #include "bt_internal.cuh"
+#include "bt_prune_dev.cuh"
 
 namespace bt {
 
@@ -39,6 +41,9 @@ enum : uint32_t { UNDEC = 0, PRUNED = 1, KEPT = 2, NOTCAND = 3 };
 constexpr int kProg = 6, kTailFlag = 4, kTailRound = 5;
 // Worklists narrower than this run in the one-CTA tail.
 constexpr unsigned long long kTailFrontier = 4096;
+// A level with at most this many children goes to one CTA, with all above it.
+// Per level: about 50 us of launches against 15 us of one CTA at 4096 blocks.
+constexpr uint64_t kSmallPrune = 4096;
 
 struct PView {
   uint64_t n, c, b;
@@ -321,6 +326,51 @@ __global__ void k_pack_marks(const uint64_t* __restrict__ cnt, uint64_t cub, con
   }
 }
 
+// The levels from `top` up in one launch of one CTA: where a level and its
+// children are few, its twenty launches cost more than the work.
+struct SmallLevels {
+  PLv lv[kMaxLevels];
+  uint32_t arity[kMaxLevels];
+  int top;
+  int w_last;  // the children of `top` are the last level
+};
+__global__ void __launch_bounds__(1024) k_prune_small(const __grid_constant__ SmallLevels S, char* temp,
+                                                      uint64_t max_rounds, uint64_t* cnt, Status* status) {
+  __shared__ PruneShared Z;
+  for (int l = S.top; l >= 0; l--) {
+    const uint64_t c2 = prune_level(S.lv[l], S.lv[l + 1], S.w_last && l == S.top, S.arity[l], temp, max_rounds, Z);
+    if (c2 == kNone) {
+      if (threadIdx.x == 0) atomicExch(&status->error, 13ull);
+      return;
+    }
+    if (threadIdx.x == 0) cnt[l + 1] = c2;
+    __syncthreads();
+  }
+}
+
+// Block and mark counts of the finished levels, and how much the text's last
+// leaf block lacks.
+struct TotalsArgs {
+  uint64_t c[kMaxLevels];
+  const uint32_t* mr[kMaxLevels];
+  const uint32_t* mw;
+  const uint64_t* st;
+  uint64_t b, n;
+  uint32_t L;
+};
+__global__ void k_tree_totals(const __grid_constant__ TotalsArgs A, const uint64_t* cnt, Status* status) {
+  const uint32_t l = threadIdx.x;
+  if (l >= A.L) return;
+  const uint64_t c = cnt && l ? cnt[l] : A.c[l];
+  status->blocks[l] = c;
+  status->marks[l] = c <= A.c[l] ? A.mr[l][(c + 31) / 32] : 0;
+  if (l + 1 < A.L) return;
+  status->leaf_short = 0;
+  if (c == 0 || c > A.c[l]) return;
+  const uint64_t last = A.n - A.st[c - 1];
+  if (((A.mw[(c - 1) >> 5] >> ((c - 1) & 31)) & 1u) && last < A.b) status->leaf_short = A.b - last;
+}
+
 PView view_of(const bt_tree* t, const Level& v) {
   return PView{t->n, v.c, v.b, v.st, v.mw, v.mr, v.ptr, v.off, v.lo};
 }
@@ -334,17 +384,33 @@ int prune_tree(BuildCtx& ctx, uint64_t max_rounds) {
   if (max_rounds == 0) max_rounds = 4096;
   // New block counts of the compacted levels stay on the device until the
   // loop ends (no host round trip per level); cnt[l] for level l >= 1.
-  uint64_t* cnt = nullptr;
-  BT_CUDA(cudaMallocAsync((void**)&cnt, t->L * sizeof(uint64_t), s));
-  struct Release {
-    uint64_t* p;
-    cudaStream_t s;
-    ~Release() { cudaFreeAsync(p, s); }
-  } release{cnt, s};
+  uint64_t* cnt = ctx.new_blocks;
   BT_CUDA(cudaMemsetAsync(cnt, 0, t->L * sizeof(uint64_t), s));
   for (int l = (int)t->L - 2; l >= 0; l--) {
     Level& v = t->lv[l];
     Level& w = t->lv[l + 1];
+    if (w.c <= kSmallPrune) {
+      // This level and all above it (they have fewer blocks still).
+      SmallLevels S;
+      S.top = l;
+      S.w_last = l + 1 == (int)t->L - 1;
+      uint64_t bytes = 0;
+      for (int k = 0; k <= l + 1; k++) {
+        const Level& x = t->lv[k];
+        S.lv[k] = PLv{t->n, x.c, x.b, x.st, x.mw, x.mr, x.ptr, x.off, x.lo};
+        S.arity[k] = x.arity;
+        if (k) bytes = std::max<uint64_t>(bytes, (t->lv[k - 1].c + x.c) * 64 + (17 << 10));
+      }
+      Arena& A = ctx.arena;
+      char* temp = nullptr;
+      A.begin_dry();
+      A.take<char>(bytes);
+      BT_TRY(A.reserve());
+      temp = A.take<char>(bytes);
+      BT_LAUNCH(k_prune_small<<<1, 1024, 0, s>>>(S, temp, max_rounds, cnt, ctx.st));
+      BT_CUDA(cudaGetLastError());
+      break;
+    }
     // Multi-CTA rounds before the one-CTA tail; a level of at most 16 Ki
     // blocks goes to the one-CTA rounds at once (launches cost more there).
     const uint32_t multi_rounds = v.c <= (16u << 10) ? 0 : 8;
@@ -443,17 +509,35 @@ int prune_tree(BuildCtx& ctx, uint64_t max_rounds) {
       // this loop reads level l+1 again.
     }
   }
-  // One host round trip for the whole pass: the new counts and the status.
-  std::vector<uint64_t> c2(t->L, 0);
-  BT_CUDA(cudaMemcpyAsync(c2.data(), cnt, t->L * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+  return BT_OK;
+}
+
+// The counts of the finished levels, one host round trip for the whole pass.
+int tree_totals(BuildCtx& ctx) {
+  bt_tree* t = ctx.t;
+  TotalsArgs A;
+  for (uint32_t l = 0; l < t->L; l++) {
+    A.c[l] = t->lv[l].c;
+    A.mr[l] = t->lv[l].mr;
+  }
+  const Level& z = t->lv[t->L - 1];
+  A.mw = z.mw;
+  A.st = z.st;
+  A.b = z.b;
+  A.n = t->n;
+  A.L = t->L;
+  BT_LAUNCH(k_tree_totals<<<1, kMaxLevels, 0, ctx.s>>>(A, t->prune ? ctx.new_blocks : nullptr, ctx.st));
+  BT_CUDA(cudaGetLastError());
   BT_TRY(sync_status(ctx));
   if (ctx.st_host->error) return BT_EINTERNAL;
-  for (uint32_t l = 1; l < t->L; l++) {
-    if (c2[l] == 0 || c2[l] > t->lv[l].c) return BT_EINTERNAL;
-    t->lv[l].c = c2[l];
-    t->lv[l].stats[BT_ST_FINAL_BLOCKS] = c2[l];
+  for (uint32_t l = 0; l < t->L; l++) {
+    Level& v = t->lv[l];
+    const uint64_t c = ctx.st_host->blocks[l];
+    if (c == 0 || c > v.c) return BT_EINTERNAL;
+    v.c = c;
+    v.nmarked = ctx.st_host->marks[l];
+    v.stats[BT_ST_FINAL_BLOCKS] = c;
   }
-  t->lv[0].stats[BT_ST_FINAL_BLOCKS] = t->lv[0].c;
   return BT_OK;
 }
 

@@ -21,30 +21,54 @@ namespace bt {
 
 namespace {
 
-__global__ void k_histogram(const uint8_t* __restrict__ T, uint64_t n, unsigned long long* hist) {
-  __shared__ unsigned int h[256];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
+// Which bytes occur (seen[0, 256), all zero at first), and by the last CTA to
+// finish (seen[256] counts them) the dense symbol map.  Only presence matters:
+// after a CTA's first lines every mark is set, and looking costs no atomics and
+// no conflicts on frequent bytes.  Bound: the text's stream.
+__global__ void __launch_bounds__(256) k_alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t* seen,
+                                                  int16_t* __restrict__ sym, Status* status) {
+  __shared__ volatile uint32_t h[256];
+  __shared__ uint32_t s_last;
+  const unsigned tid = threadIdx.x;
+  h[tid] = 0;
   __syncthreads();
-  const uint64_t nv = n / 16;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  const uint64_t stride = (uint64_t)gridDim.x * 256, t0 = blockIdx.x * 256ull + tid;
   if (((uintptr_t)T & 15) == 0) {
     const uint4* V = (const uint4*)T;
-    for (uint64_t i = tid; i < nv; i += stride) {
-      uint4 q = V[i];
-      uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    for (uint64_t i = t0; i < n / 16; i += stride) {
+      const uint4 q = V[i];
+      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+      uint32_t f[16];
 #pragma unroll
-      for (int a = 0; a < 4; a++)
+      for (int a = 0; a < 16; a++) f[a] = h[(w[a >> 2] >> (8 * (a & 3))) & 0xFF];
 #pragma unroll
-        for (int b = 0; b < 4; b++) atomicAdd(&h[(w[a] >> (8 * b)) & 0xFF], 1u);
+      for (int a = 0; a < 16; a++)
+        if (!f[a]) h[(w[a >> 2] >> (8 * (a & 3))) & 0xFF] = 1;
     }
-    for (uint64_t i = nv * 16 + tid; i < n; i += stride) atomicAdd(&h[T[i]], 1u);
+    for (uint64_t i = n / 16 * 16 + t0; i < n; i += stride) h[T[i]] = 1;
   } else {
-    for (uint64_t i = tid; i < n; i += stride) atomicAdd(&h[T[i]], 1u);
+    for (uint64_t i = t0; i < n; i += stride) h[T[i]] = 1;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 256; i += blockDim.x)
-    if (h[i]) atomicAdd(&hist[i], (unsigned long long)h[i]);
+  if (h[tid]) atomicExch(&seen[tid], 1u);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&seen[256], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const bool mine = *(volatile uint32_t*)&seen[tid] != 0;
+  // Rank among the bytes that occur.
+  const unsigned bal = __ballot_sync(0xFFFFFFFFu, mine);
+  if ((tid & 31) == 0) h[tid >> 5] = __popc(bal);
+  __syncthreads();
+  uint32_t before = 0, all = 0;
+  for (uint32_t w = 0; w < 8; w++) {
+    if (w < tid >> 5) before += h[w];
+    all += h[w];
+  }
+  sym[tid] = mine ? (int16_t)(before + __popc(bal & ((1u << (tid & 31)) - 1u))) : (int16_t)-1;
+  if (tid == 0) status->symbols = all;
 }
 
 // Up to four counters of one symbol as read, and how many of them count:
@@ -835,22 +859,10 @@ __global__ void __launch_bounds__(256) k_pack_records(const __grid_constant__ Pa
 
 }  // namespace
 
-int alphabet(const uint8_t* T, uint64_t n, uint32_t sigma, bt_tree* t, cudaStream_t s) {
-  Scratch sc(s);
-  unsigned long long* hist;
-  BT_TRY(sc.alloc(&hist, 256));
-  BT_CUDA(cudaMemsetAsync(hist, 0, 256 * sizeof(unsigned long long), s));
-  BT_LAUNCH(k_histogram<<<grid_for(n / 16 + 1, 256, 152 * 8), 256, 0, s>>>(T, n, hist));
-  unsigned long long h[256];
-  BT_CUDA(cudaMemcpyAsync(h, hist, sizeof(h), cudaMemcpyDeviceToHost, s));
-  BT_CUDA(cudaStreamSynchronize(s));
-  uint32_t S = 0;
-  for (int i = 0; i < 256; i++) t->sym_host[i] = h[i] ? (int16_t)S++ : (int16_t)-1;
-  if (S > sigma) return BT_EINVAL;
-  t->S = S;
-  BT_CUDA(cudaMallocAsync(&t->sym, 256 * sizeof(int16_t), s));
-  BT_CUDA(cudaMemcpyAsync(t->sym, t->sym_host, 256 * sizeof(int16_t), cudaMemcpyHostToDevice, s));
-  BT_CUDA(cudaStreamSynchronize(s));
+int alphabet(const uint8_t* T, uint64_t n, uint32_t* seen, bt_tree* t, Status* st, cudaStream_t s) {
+  BT_CUDA(cudaMallocAsync((void**)&t->sym, 256 * sizeof(int16_t), s));
+  BT_LAUNCH(k_alphabet<<<grid_for(n / 16 + 1, 256, 152 * 8), 256, 0, s>>>(T, n, seen, t->sym, st));
+  BT_CUDA(cudaGetLastError());
   return BT_OK;
 }
 
@@ -947,28 +959,14 @@ int build_counters(BuildCtx& ctx) {
   BT_LAUNCH(k_base_prefix<<<S, r.c > 512 ? 1024 : 128, 0, s>>>(r.c, r.cnt, r.cw, counter_stride(r.c), t->pre));
   // Leaf text of the marked last-level blocks.
   const Level& z = t->lv[t->L - 1];
-  uint32_t nm = 0;
-  BT_CUDA(cudaMemcpyAsync(&nm, z.mr + (z.c + 31) / 32, sizeof(nm), cudaMemcpyDeviceToHost, s));
-  BT_CUDA(cudaStreamSynchronize(s));
-  t->leaf_bytes = (uint64_t)nm * z.b;
+  t->leaf_bytes = z.nmarked * z.b;
   BT_CUDA(cudaMallocAsync(&t->leaf, t->leaf_bytes + 16, s));
   if (z.b % 16 == 0 && ((uintptr_t)ctx.T & 15) == 0)
     BT_LAUNCH(k_leaf_text<true><<<grid_for(z.c * (z.b / 16), T), T, 0, s>>>(z.c, z.b, t->n, z.st, z.mw, z.mr, ctx.T, t->leaf));
   else
     BT_LAUNCH(k_leaf_text<false><<<grid_for(z.c * z.b, T), T, 0, s>>>(z.c, z.b, t->n, z.st, z.mw, z.mr, ctx.T, t->leaf));
   BT_CUDA(cudaGetLastError());
-  // Real leaf length: the tail block may be short.
-  uint64_t tail_short = 0;
-  if (nm) {
-    uint64_t last_st = 0;
-    BT_CUDA(cudaMemcpyAsync(&last_st, z.st + z.c - 1, sizeof(last_st), cudaMemcpyDeviceToHost, s));
-    uint32_t lastw = 0;
-    BT_CUDA(cudaMemcpyAsync(&lastw, z.mw + (z.c - 1) / 32, sizeof(lastw), cudaMemcpyDeviceToHost, s));
-    BT_CUDA(cudaStreamSynchronize(s));
-    bool last_marked = (lastw >> ((z.c - 1) & 31)) & 1u;
-    if (last_marked && t->n - last_st < z.b) tail_short = z.b - (t->n - last_st);
-  }
-  t->leaf_bytes -= tail_short;
+  t->leaf_bytes -= ctx.st_host->leaf_short;  // the text's last block may be short
   return BT_OK;
 }
 

@@ -561,7 +561,7 @@ int quick_list(BuildCtx& ctx, QuickBuild& qb) {
   qb.list = QList{qb.idx, qb.x, qb.D, qb.seg1, qb.seg2, nw};
   qb.ready = true;
   BT_TRY(qb.mem.alloc(&qb.qs, 1));
-  BT_CUDA(cudaMallocHost(&qb.qs_host, sizeof(QuickStatus)));
+  qb.qs_host = (QuickStatus*)(pinned_page() + kPageQuick);  // (the build made sure of the page)
   return BT_OK;
 }
 

@@ -39,13 +39,10 @@ struct QuickBuild {
   uint32_t *idx = nullptr, *x = nullptr, *D = nullptr, *seg1 = nullptr, *seg2 = nullptr;
   QList list{};
   QuickStatus* qs = nullptr;
-  QuickStatus* qs_host = nullptr;  // pinned
+  QuickStatus* qs_host = nullptr;  // in the thread's pinned page
   std::function<int(uint64_t)> resolve_exact;
   explicit QuickBuild(cudaStream_t s) : mem(s) { open.s = s; }
-  ~QuickBuild() {
-    open.release();
-    if (qs_host) cudaFreeHost(qs_host);
-  }
+  ~QuickBuild() { open.release(); }
 };
 
 int quick_list(BuildCtx& ctx, QuickBuild& qb);

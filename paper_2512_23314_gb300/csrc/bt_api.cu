@@ -24,6 +24,9 @@ int run_query_one(const bt_tree* t, int kind, uint64_t a0, uint64_t a1, uint64_t
 int batch_kernel_build(const uint8_t* const* texts, const uint64_t* ns, const uint32_t* sigmas,
                        const uint32_t* taus, const uint32_t* leaf_lens, uint64_t ndocs, const bt_opts& o,
                        std::vector<char>& routed, bt_tree** outs, cudaStream_t s, const std::vector<char>* eligible);
+int solo_build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, uint32_t leaf_len, const bt_opts& o,
+               const std::vector<uint64_t>& sizes, cudaStream_t s, bt_tree* t);
+bool solo_takes(uint64_t n, uint32_t sigma, const std::vector<uint64_t>& sizes);
 uint32_t batch_split(const uint64_t* ns, const uint32_t* taus, const uint32_t* leaf_lens, uint64_t ndocs,
                      const bt_opts& o, std::vector<char>& eligible);
 void batch_report_workers(uint64_t docs);
@@ -83,7 +86,7 @@ thread_local PinnedPage g_page;
 }  // namespace
 
 char* pinned_page() {
-  if (!g_page.p && cudaHostAlloc((void**)&g_page.p, 8192, cudaHostAllocPortable) != cudaSuccess) {
+  if (!g_page.p && cudaHostAlloc((void**)&g_page.p, kPageBytes, cudaHostAllocPortable) != cudaSuccess) {
     cudaGetLastError();
     g_page.p = nullptr;
   }
@@ -209,6 +212,19 @@ static int build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, 
   HostTrace tr;
   std::vector<uint64_t> sizes;
   BT_TRY(plan_sizes(n, tau, leaf, o, sizes));
+  // Short texts: one launch of the batched kernel.  The
+  // flags ask for variants of the path below, the profile for its phases; a
+  // device without room for the scratch in one piece takes it too.
+  constexpr uint32_t kVariants =
+      BT_FLAG_DENSE_SCAN | BT_FLAG_TINY_QUEUE | BT_FLAG_BATCH_WORKERS | BT_FLAG_LEAF_COUNTS | BT_FLAG_SORT_SCAN;
+  if (!(o.flags & kVariants) && !g_prof_on.load() && solo_takes(n, sigma, sizes)) {
+    int device = 0;
+    BT_CUDA(cudaGetDevice(&device));
+    keep_pool_memory(device);
+    const int rc = solo_build(text, n, sigma, tau, leaf, o, sizes, s, t);
+    tr.mark("one launch");
+    if (rc != BT_ENOMEM) return rc;
+  }
   t->n = n;
   t->tau = tau;
   t->leaf_len = leaf;

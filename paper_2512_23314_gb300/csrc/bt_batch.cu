@@ -1,7 +1,7 @@
 // bt_batch.cu -- batched construction: a persistent, level-synchronous kernel
 // with a per-document work queue.
 //
-// Each CTA of k_batch repeatedly takes the next document of the batch from a
+// Each CTA (or, for few long documents, each cluster of CTAs) of k_batch repeatedly takes the next document of the batch from a
 // device work queue (an atomic counter; the documents come in decreasing
 // expected work, length times levels) and builds its whole block tree by
 // itself:
@@ -74,10 +74,36 @@ struct BJob {
 };
 
 
-// Shared state of a CTA.
-struct Cta {
+constexpr uint32_t kMaxGroup = 16;  // CTAs of a cluster that share a document
+
+// State that all CTAs of a group change: in shared memory for one CTA, at the
+// start of a cluster's scratch otherwise (64-bit minima and maxima are no
+// native operations on another CTA's shared memory).
+struct Common {
   uint32_t doc;
   int err;
+  uint32_t seen[8];                 // which bytes occur
+  uint64_t part[kMaxGroup];         // one value per CTA (sums over its part of the text)
+  unsigned long long fp_tail, lo_tail, lo_tailpair;
+  uint32_t pretail;
+  unsigned int npairs, njobs, nsusp;
+  QuickStatus qs;
+  Status status;
+  unsigned long long verify_bytes, collisions;
+  unsigned long long lastk;
+  PruneShared prune;
+  unsigned long long out_off;
+};
+
+static_assert(sizeof(Common) <= kCommonBytes, "a cluster's common state fits its place in the scratch");
+
+// State of a CTA; what is not scratch of its own is the same in all CTAs of the
+// group, which each compute it from the same arrays.
+struct Cta {
+  Group grp;
+  Common* g;
+  Common own;
+  int bad;
   uint64_t n;
   uint32_t S, L;
   int16_t sym[256];
@@ -90,26 +116,16 @@ struct Cta {
   uint64_t last_start;
   // current level
   uint64_t r, Bb, Br;
-  uint64_t bmask, pmask;
   uint32_t bshift;
-  unsigned long long fp_tail, lo_tail, lo_tailpair;
-  uint32_t pretail;
-  unsigned int npairs, njobs, nsusp;
   uint32_t nsel;                      // entries of the list of selected grams
   int expanded;                       // H holds every position (the list is gone)
   QList list;
   Chase chase;
-  QuickStatus qs;
-  Status status;
-  unsigned long long verify_bytes, collisions;
-  unsigned long long lastk;
   // scans
-  uint32_t wtot[32];
+  uint32_t wtot[kScanWords];
   uint64_t wsum[32];
   uint64_t carry;
-  PruneShared prune;
   // output
-  char* out;
   uint64_t out_off, out_bytes;
   // phase timing (SM cycles)
   unsigned long long cyc[6];
@@ -126,8 +142,16 @@ __device__ __forceinline__ void tmark(Cta& C, int ph) {
   }
 }
 
-__device__ __forceinline__ bool cta_failed(Cta& C) { return __syncthreads_or(C.err != 0) != 0; }
-__device__ __forceinline__ void fail(Cta& C, int code) { atomicCAS(&C.err, 0, code); }
+__device__ __forceinline__ void fail(Cta& C, int code) { atomicCAS(&C.g->err, 0, code); }
+// Barrier of the group; has a step failed?  (Two barriers in a cluster: no
+// later step's failure may be seen by some of its CTAs only.)
+__device__ __forceinline__ bool failed(Cta& C) {
+  if (C.grp.size == 1) return __syncthreads_or(C.g->err != 0) != 0;
+  gsync(C.grp);
+  const int e = *(volatile int*)&C.g->err;
+  gsync(C.grp);
+  return e != 0;
+}
 
 __device__ __forceinline__ void min_pos(unsigned long long* a, uint64_t p) {
   if (*(volatile unsigned long long*)a > p) atomicMin(a, (unsigned long long)p);
@@ -230,12 +254,12 @@ __device__ __forceinline__ bool differs(const uint8_t* __restrict__ T, uint64_t 
 // Verify jobs[0, nj): mismatch[i] = 1 when the two ranges differ.  Groups of
 // G lanes (about len/16, a power of two up to 32) take one job each.
 __device__ void verify_jobs(const uint8_t* __restrict__ T, const BJob* jobs, uint32_t nj, uint64_t maxlen,
-                            unsigned int* mismatch) {
+                            unsigned int* mismatch, const Group& grp_) {
   unsigned G = 1;
   while (G < 32 && 16ull * G < maxlen) G <<= 1;
   const unsigned lane = threadIdx.x & 31, grp = lane / G, gl = lane % G, gpw = 32 / G;
   const unsigned gmask = (G == 32 ? kFull : ((1u << G) - 1u)) << (grp * G);
-  const unsigned nw = blockDim.x >> 5, warp = threadIdx.x >> 5;
+  const unsigned nw = grp_.threads() >> 5, warp = grp_.tid() >> 5;
   // Warp-uniform loop: every lane reaches every ballot.
   for (uint64_t base = (uint64_t)warp * gpw; base < nj; base += (uint64_t)nw * gpw) {
     const uint64_t j = base + grp;
@@ -256,10 +280,11 @@ __device__ void verify_jobs(const uint8_t* __restrict__ T, const BJob* jobs, uin
 // is set, and looking costs no atomics and no conflicts on frequent bytes.)
 __device__ void alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t sigma, Cta& C) {
   volatile unsigned int* seen = C.hist;
-  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) seen[i] = 0;
+  const unsigned tid = C.grp.tid(), nt = C.grp.threads(), t = threadIdx.x;
+  for (uint32_t i = t; i < 256; i += blockDim.x) seen[i] = 0;
   __syncthreads();
   const uint64_t nv = n / 16;
-  for (uint64_t i = threadIdx.x; i < nv; i += blockDim.x) {
+  for (uint64_t i = tid; i < nv; i += nt) {
     const uint4 q = ((const uint4*)T)[i];
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
     uint32_t f[16];
@@ -269,28 +294,43 @@ __device__ void alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t sig
     for (int a = 0; a < 16; a++)
       if (!f[a]) seen[(w[a >> 2] >> (8 * (a & 3))) & 0xFF] = 1;
   }
-  for (uint64_t i = nv * 16 + threadIdx.x; i < n; i += blockDim.x) seen[T[i]] = 1;
+  for (uint64_t i = nv * 16 + tid; i < n; i += nt) seen[T[i]] = 1;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t S = 0;
-    for (int i = 0; i < 256; i++) C.sym[i] = seen[i] ? (int16_t)S++ : (int16_t)-1;
-    C.S = S;
-    if (S > sigma) C.err = BT_EINVAL;
+  if (t < 256) {
+    const uint32_t bits = __ballot_sync(kFull, seen[t] != 0);
+    if ((t & 31) == 0 && bits) atomicOr(&C.g->seen[t >> 5], bits);
   }
-  __syncthreads();
+  gsync(C.grp);
+  if (t < 256) {
+    uint32_t before = 0, all = 0, mine = 0;
+    for (uint32_t w = 0; w < 8; w++) {
+      const uint32_t bits = *(volatile uint32_t*)&C.g->seen[w];
+      if (w < t >> 5) before += __popc(bits);
+      if (w == t >> 5) mine = bits;
+      all += __popc(bits);
+    }
+    C.sym[t] = (mine >> (t & 31)) & 1u ? (int16_t)(before + __popc(mine & ((1u << (t & 31)) - 1u))) : (int16_t)-1;
+    if (t == 0) {
+      C.S = all;
+      if (all > sigma) fail(C, BT_EINVAL);
+    }
+  }
 }
 
 // Hs[j] = H(32 j) for j <= n / 32: four chunks of 32 bytes per thread, their
 // byte dot products scanned over the CTA (as the prefix kernels of bt_scan.cu).
+// A CTA takes the chunks [j0, j1) after the ones whose fingerprint is `carry`;
+// returns (in C.carry) the fingerprint up to j1, a multiple of four chunks on,
+// or, with `store`, writes Hs.
 template <class M>
-__device__ void prefix_pass(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const uint8_t* T, uint64_t n,
-                            uint64_t* Hs, Cta& C) {
-  const uint64_t nchunks = n / 32;
-  if (threadIdx.x == 0) C.carry = 0;
+__device__ void prefix_range(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const uint8_t* T, uint64_t nchunks,
+                             uint64_t r0, uint64_t r1, uint64_t carry0, bool store, uint64_t* Hs, Cta& C) {
+  if (threadIdx.x == 0) C.carry = carry0;
   __syncthreads();
   const uint64_t xl = kr_lane_pow(m, pw);
-  for (uint64_t t0 = 0; t0 <= nchunks; t0 += 4ull * blockDim.x) {
+  for (uint64_t t0 = r0; t0 < r1; t0 += 4ull * blockDim.x) {
     const uint64_t j0 = t0 + 4ull * threadIdx.x;
+    const unsigned last = (unsigned)((r1 - t0 < 4ull * blockDim.x ? r1 - t0 : 4ull * blockDim.x) + 3) / 4 - 1;
     uint64_t c[4];
 #pragma unroll
     for (int i = 0; i < 4; i++) {
@@ -306,29 +346,56 @@ __device__ void prefix_pass(const M& m, const PrefixConst<M>& PC, const KrPow& p
     const uint64_t incl = cta_kr_scan(m, h, pw, xl, C.wsum);
     uint64_t up = __shfl_up_sync(kFull, incl, 1);
     if ((threadIdx.x & 31) == 31) C.wsum[threadIdx.x >> 5] = incl;
-    if (threadIdx.x == blockDim.x - 1) C.carry = incl;
+    if (threadIdx.x == last) C.carry = incl;
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) up = threadIdx.x ? C.wsum[(threadIdx.x >> 5) - 1] : carry;
+    if (store) {
+      if ((threadIdx.x & 31) == 0) up = threadIdx.x ? C.wsum[(threadIdx.x >> 5) - 1] : carry;
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-      if (j0 + i <= nchunks) Hs[j0 + i] = up;
-      up = m.add(m.mul(up, PC.B32), c[i]);
+      for (int i = 0; i < 4; i++) {
+        if (j0 + i < r1) Hs[j0 + i] = up;
+        up = m.add(m.mul(up, PC.B32), c[i]);
+      }
     }
     __syncthreads();
   }
 }
 
+// In a cluster each CTA takes an equal part of the text: its fingerprint, then
+// the parts before it, then its values.
+template <class M>
+__device__ void prefix_pass(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const uint8_t* T, uint64_t n,
+                            uint64_t* Hs, Cta& C) {
+  const uint64_t nchunks = n / 32, all = nchunks + 1;
+  if (C.grp.size == 1) {
+    prefix_range(m, PC, pw, T, nchunks, 0, all, 0, true, Hs, C);
+    return;
+  }
+  const uint64_t per = (all + 4 * C.grp.size - 1) / (4 * C.grp.size) * 4;
+  const uint64_t r0 = per * C.grp.rank < all ? per * C.grp.rank : all, r1 = r0 + per < all ? r0 + per : all;
+  prefix_range(m, PC, pw, T, nchunks, r0, r1, 0, false, Hs, C);
+  if (threadIdx.x == 0) C.g->part[C.grp.rank] = C.carry;
+  gsync(C.grp);
+  uint64_t carry = 0;
+  if (threadIdx.x == 0) {
+    const uint64_t x = pow_mod(m, PC.B32, per);
+    for (uint32_t k = 0; k < C.grp.rank; k++) carry = m.add(m.mul(carry, x), *(volatile uint64_t*)&C.g->part[k]);
+  }
+  prefix_range(m, PC, pw, T, nchunks, r0, r1, carry, true, Hs, C);
+  gsync(C.grp);
+}
+
 // H[p] for every p in [0, n] (levels of blocks too short for the list).
 template <class M>
-__device__ void expand_pass(const M& m, const uint8_t* T, uint64_t n, uint64_t B, const uint64_t* Hs, uint64_t* H) {
-  for (uint64_t j = threadIdx.x; j <= n / 32; j += blockDim.x) {
+__device__ void expand_pass(const M& m, const uint8_t* T, uint64_t n, uint64_t B, const uint64_t* Hs, uint64_t* H,
+                            const Group& grp) {
+  for (uint64_t j = grp.tid(); j <= n / 32; j += grp.threads()) {
     uint64_t h = Hs[j];
     for (uint64_t p = 32 * j; p < 32 * j + 32 && p <= n; p++) {
       H[p] = h;
       if (p < n) h = m.add(m.mul(h, B), (uint64_t)T[p] + 1);
     }
   }
-  __syncthreads();
+  gsync(grp);
 }
 
 // Exclusive sum of one value per thread over the CTA; *total = the sum.
@@ -360,9 +427,11 @@ __device__ uint32_t cta_excl_u32(uint32_t v, Cta& C, uint32_t* total) {
 
 // The list of selected grams (bt_quick.cu): a thread takes 32 positions of a
 // tile, the entries' places come from a CTA scan, then the first-occurrence
-// table, the distances and the segment minima.
+// table, the distances and the segment minima.  In a cluster each CTA takes an
+// equal part of the text: it marks and counts its entries first (the marks wait
+// in the first-occurrence table's place).
 __device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
-  const unsigned tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const unsigned tid = C.grp.tid(), nt = C.grp.threads(), lane = tid & 31;
   const uint64_t nw = n < kGramLen ? 0 : (n - kGramLen + 1 + 31) / 32, ns = (n + kSegBytes - 1) / kSegBytes,
                  ns2 = (ns + 63) / 64;
   uint32_t* idx = (uint32_t*)(scr + C.sl.idx);
@@ -372,19 +441,40 @@ __device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
   uint32_t* seg1 = (uint32_t*)(scr + C.sl.seg1);
   uint32_t* seg2 = (uint32_t*)(scr + C.sl.seg2);
   const uint32_t cmask = (uint32_t)(C.sl.cells - 1);
-  for (uint64_t i = tid; i < C.sl.cells; i += nt) first[i] = 0xFFFFFFFFu;
-  uint32_t total = 0;
-  for (uint64_t j0 = 0; j0 < nw; j0 += nt) {
-    const uint64_t j = j0 + tid;
-    uint32_t bits = 0;
-    if (j < nw) {
-      bits = half_mask(T, n, 32 * j) | half_mask(T, n, 32 * j + 16) << 16;
-      const uint64_t left = n - kGramLen + 1 - 32 * j;
-      if (left < 32) bits &= (1u << left) - 1u;
+  auto mask = [&](uint64_t j) {
+    uint32_t bits = half_mask(T, n, 32 * j) | half_mask(T, n, 32 * j + 16) << 16;
+    const uint64_t left = n - kGramLen + 1 - 32 * j;
+    if (left < 32) bits &= (1u << left) - 1u;
+    return bits;
+  };
+  const bool multi = C.grp.size > 1;
+  const uint64_t per = (nw + C.grp.size - 1) / C.grp.size, a0 = per * C.grp.rank < nw ? per * C.grp.rank : nw,
+                 a1 = a0 + per < nw ? a0 + per : nw;
+  uint32_t total = 0, all = 0;
+  if (multi) {
+    uint32_t mine = 0, sum;
+    for (uint64_t j = a0 + threadIdx.x; j < a1; j += blockDim.x) {
+      const uint32_t bits = mask(j);
+      first[j] = bits;
+      mine += __popc(bits);
     }
+    cta_excl_u32(mine, C, &sum);
+    if (threadIdx.x == 0) C.g->part[C.grp.rank] = sum;
+    gsync(C.grp);
+    for (uint32_t k = 0; k < C.grp.size; k++) {
+      const uint32_t x = (uint32_t)*(volatile uint64_t*)&C.g->part[k];
+      if (k < C.grp.rank) total += x;
+      all += x;
+    }
+  } else {
+    for (uint64_t i = tid; i < C.sl.cells; i += nt) first[i] = 0xFFFFFFFFu;
+  }
+  for (uint64_t j0 = a0; j0 < a1; j0 += blockDim.x) {
+    const uint64_t j = j0 + threadIdx.x;
+    uint32_t bits = j < a1 ? (multi ? first[j] : mask(j)) : 0u;
     uint32_t sum;
     uint32_t o = total + cta_excl_u32(__popc(bits), C, &sum);
-    if (j < nw) idx[j] = o;
+    if (j < a1) idx[j] = o;
     for (; bits; bits &= bits - 1, o++) {
       const uint32_t p = (uint32_t)(32 * j) + __ffs(bits) - 1, sh = 8 * (p & 3);
       const uint32_t* w = (const uint32_t*)(T + (p & ~3u));
@@ -395,12 +485,17 @@ __device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
     }
     total += sum;
   }
-  if (tid == 0) {
-    idx[nw] = total;
+  if (multi) {
+    gsync(C.grp);
+    for (uint64_t i = tid; i < C.sl.cells; i += nt) first[i] = 0xFFFFFFFFu;
+    total = all;
+  }
+  if (tid == 0) idx[nw] = total;
+  if (threadIdx.x == 0) {
     C.nsel = total;
     C.list = QList{idx, x, D, seg1, seg2, nw};
   }
-  __syncthreads();
+  gsync(C.grp);
   for (uint32_t e = tid; e < total; e += 4 * nt) {
     uint32_t c[4], f[4];
 #pragma unroll
@@ -411,7 +506,7 @@ __device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
     for (uint32_t u = 0; u < 4; u++)
       if (e + u * nt < total && f[u] > x[e + u * nt]) atomicMin(&first[c[u]], x[e + u * nt]);
   }
-  __syncthreads();
+  gsync(C.grp);
   for (uint32_t e = tid; e < total; e += 4 * nt) {
     uint32_t f[4];
 #pragma unroll
@@ -420,19 +515,19 @@ __device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
     for (uint32_t u = 0; u < 4; u++)
       if (e + u * nt < total) D[e + u * nt] = x[e + u * nt] - f[u];
   }
-  __syncthreads();
+  gsync(C.grp);
   for (uint64_t j = tid / 32; j < ns; j += nt / 32) {
     const uint64_t w0 = j * (kSegBytes / 32), w1 = w0 + kSegBytes / 32 < nw ? w0 + kSegBytes / 32 : nw;
     const uint32_t d = __reduce_min_sync(kFull, min_entries(D, idx[w0 < nw ? w0 : nw], idx[w1], lane, 32, kNoDist));
     if (lane == 0) seg1[j] = d;
   }
-  __syncthreads();
+  gsync(C.grp);
   for (uint64_t j = tid; j < ns2; j += nt) {
     uint32_t d = kNoDist;
     for (uint64_t i = 64 * j; i < 64 * j + 64 && i < ns; i++) d = min(d, seg1[i]);
     seg2[j] = d;
   }
-  __syncthreads();
+  gsync(C.grp);
 }
 
 struct Work {
@@ -472,9 +567,9 @@ __device__ Work carve_level(char* temp, uint64_t c, uint64_t bcap, uint64_t pcap
 template <class M>
 __device__ void exact_pass(const M& m, const LV& g, const uint64_t* H, const Work& W, int pair, uint64_t B,
                            Cta& C) {
-  const uint32_t ns = C.nsusp;
+  const uint32_t ns = C.g->nsusp;
   // Key fingerprint, length and B^length of each suspect (in the job array).
-  for (uint32_t i = threadIdx.x; i < ns; i += blockDim.x) {
+  for (uint32_t i = C.grp.tid(); i < ns; i += C.grp.threads()) {
     const uint64_t k = W.susp[i];
     uint64_t klen = blen(g, k), kfp = W.fpB[k];
     if (pair) {
@@ -484,9 +579,9 @@ __device__ void exact_pass(const M& m, const LV& g, const uint64_t* H, const Wor
     }
     W.jobs[i] = BJob{kfp, pow_mod(m, B, klen), klen, g.st[k]};
   }
-  __syncthreads();
+  gsync(C.grp);
   const uint64_t per = g.c * g.b;
-  for (uint64_t w = threadIdx.x; w < (uint64_t)ns * per; w += blockDim.x) {
+  for (uint64_t w = C.grp.tid(); w < (uint64_t)ns * per; w += C.grp.threads()) {
     const uint64_t i = w / per, rest = w - i * per;
     const uint64_t k = rest / g.b, j = rest - k * g.b;
     if (j >= blen(g, k)) continue;
@@ -499,7 +594,7 @@ __device__ void exact_pass(const M& m, const LV& g, const uint64_t* H, const Wor
     for (uint64_t x = 0; x < J.len && eq; x++) eq = g.T[p + x] == g.T[J.idx + x];
     if (eq) min_pos(&W.exlo[i], p);
   }
-  __syncthreads();
+  gsync(C.grp);
 }
 
 // A window of the scan whose fingerprint passed the filter: the block-table
@@ -539,27 +634,23 @@ template <class M>
 __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, const LV& g, char* scr, uint32_t l,
                           uint32_t* filt, uint32_t filt_words_max) {
   const uint64_t n = C.n, c = g.c, b = g.b;
-  const unsigned tid = threadIdx.x, nt = blockDim.x;
+  const unsigned tid = C.grp.tid(), nt = C.grp.threads();
   uint64_t* lo = (uint64_t*)(scr + C.sl.lo[l]);
   uint32_t* mw = (uint32_t*)(scr + C.sl.mw[l]);
   uint32_t* mr = (uint32_t*)(scr + C.sl.mr[l]);
   uint64_t* H = (uint64_t*)(scr + C.sl.big);
   if (!C.expanded) {
-    expand_pass(m, D.T, n, P.B, (const uint64_t*)(scr + C.sl.Hs), H);
-    if (tid == 0) C.expanded = 1;
+    expand_pass(m, D.T, n, P.B, (const uint64_t*)(scr + C.sl.Hs), H, C.grp);
+    if (threadIdx.x == 0) C.expanded = 1;
   }
   const uint64_t bcap = pow2_ge(2 * c), pcap = pow2_ge(2 * c);
   const Work W = carve_level(scr + C.sl.temp, c, bcap, pcap);
-  if (tid == 0) {
-    C.bmask = bcap - 1;
-    C.pmask = pcap - 1;
-  }
   for (uint64_t i = tid; i < bcap; i += nt) W.bt[i] = BSlot{kNone, kNone, 0, 0};
   for (uint64_t i = tid; i < pcap; i += nt) W.pt[i] = PSlot{kNone, kNone};
   for (uint64_t i = tid; i < c; i += nt) W.mismatch[i] = 0;
-  __syncthreads();
+  gsync(C.grp);
   tmark(C, 3);
-  const uint64_t r = C.r, Bb = C.Bb, Br = C.Br, bmask = C.bmask, pmask = C.pmask;
+  const uint64_t r = C.r, Bb = C.Bb, Br = C.Br, bmask = bcap - 1, pmask = pcap - 1;
 
   // Block fingerprints; full-length blocks into the block table (the slot's
   // leftmost window starts at the block's own start).
@@ -577,17 +668,17 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
       min_pos(&W.bt[slot].lo, s);
     } else {
       W.slotB[k] = kNoSlot;
-      C.fp_tail = fp;
-      atomicMin(&C.lo_tail, (unsigned long long)s);
+      C.g->fp_tail = fp;
+      atomicMin(&C.g->lo_tail, (unsigned long long)s);
     }
   }
-  if (cta_failed(C)) return;
+  if (failed(C)) return;
   // Pairs of consecutive blocks: one pair-table slot per (slot, slot); the
   // pair ending in the short tail is kept in the CTA's scalars.
   for (uint64_t k = tid; k + 1 < c; k += nt) {
     W.slotP[k] = kNoSlot;
     if (g.st[k + 1] != g.st[k] + b) continue;
-    atomicAdd(&C.npairs, 1u);
+    atomicAdd(&C.g->npairs, 1u);
     const uint32_t sk = W.slotB[k];
     if (sk == kNoSlot) {
       fail(C, BT_EINTERNAL);
@@ -597,8 +688,8 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
       atomicMax(&W.bt[sk].maxpst, (unsigned long long)g.st[k]);
     if (W.slotB[k + 1] == kNoSlot) {
       W.slotP[k] = kBTailPair;
-      C.pretail = sk;
-      atomicMin(&C.lo_tailpair, (unsigned long long)g.st[k]);
+      C.g->pretail = sk;
+      atomicMin(&C.g->lo_tailpair, (unsigned long long)g.st[k]);
     } else {
       const uint32_t sp = t_insert(W.pt, pmask, ((uint64_t)sk << 32) | W.slotB[k + 1]);
       W.slotP[k] = sp;
@@ -609,29 +700,30 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
       min_pos(&W.pt[sp].lo, g.st[k]);
     }
   }
-  if (cta_failed(C)) return;
+  if (failed(C)) return;
   uint32_t fwords = 32;
   while (fwords < c && fwords < filt_words_max) fwords <<= 1;
   // A bitmap of the full-length block fingerprints in shared memory (about
   // 32 bits per key): a window whose fingerprint's bit is clear matches no
   // key, so only the few that pass probe the table in global memory.
   const uint64_t fmask = (uint64_t)fwords * 32 - 1;
-  for (uint32_t i = tid; i < fwords; i += nt) filt[i] = 0;
+  // (every CTA has its own)
+  for (uint32_t i = threadIdx.x; i < fwords; i += blockDim.x) filt[i] = 0;
   __syncthreads();
-  for (uint64_t k = tid; k < c; k += nt)
+  for (uint64_t k = threadIdx.x; k < c; k += blockDim.x)
     if (W.slotB[k] != kNoSlot) {
       const uint64_t bit = W.fpB[k] & fmask;
       atomicOr(&filt[bit >> 5], 1u << (bit & 31));
     }
-  __syncthreads();
+  gsync(C.grp);
   tmark(C, 1);
 
   // The window scan: every window [p, p+b) inside a run (and [p, p+r) for the
   // short tail); the few whose fingerprint's bit is set probe the table.
   {
-    const uint32_t pretail = C.pretail, bshift = C.bshift;
-    const uint64_t fp_tail = C.fp_tail;
-    const ScanArgs A{H, W.bt, W.pt, bmask, pmask, b, r, Bb, Br, fp_tail, pretail, &C.lo_tailpair};
+    const uint32_t pretail = C.g->pretail, bshift = C.bshift;
+    const uint64_t fp_tail = C.g->fp_tail;
+    const ScanArgs A{H, W.bt, W.pt, bmask, pmask, b, r, Bb, Br, fp_tail, pretail, &C.g->lo_tailpair};
     for (uint64_t w = tid; w < c * b; w += nt) {
       const uint64_t k = bshift != 0xFFu ? w >> bshift : w / b;
       const uint64_t j = w - k * b;
@@ -643,10 +735,10 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
         const uint64_t bit = x & fmask;
         if ((filt[bit >> 5] >> (bit & 31)) & 1u) window_hit(m, A, p, av, x, hb);
       }
-      if (r && p + r <= av && phi(m, H, Br, p, r) == fp_tail) min_pos(&C.lo_tail, p);
+      if (r && p + r <= av && phi(m, H, Br, p, r) == fp_tail) min_pos(&C.g->lo_tail, p);
     }
   }
-  __syncthreads();
+  gsync(C.grp);
   tmark(C, 2);
 
   // Pairs: leftmost when the minimum is the pair's own start; otherwise the
@@ -656,36 +748,36 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
     W.job_of[k] = kNone;
     const uint32_t sp = W.slotP[k];
     if (sp == kNoSlot) continue;
-    const uint64_t lp = sp == kBTailPair ? C.lo_tailpair : W.pt[sp].lo;
+    const uint64_t lp = sp == kBTailPair ? C.g->lo_tailpair : W.pt[sp].lo;
     const uint64_t s = g.st[k];
     if (lp == s) {
       W.pm[k] = 1;
     } else if (lp < s) {
       const uint64_t len = b + blen(g, k + 1);
-      const uint32_t id = atomicAdd(&C.njobs, 1u);
+      const uint32_t id = atomicAdd(&C.g->njobs, 1u);
       W.jobs[id] = BJob{lp, s, len, k};
       W.job_of[k] = id;
-      atomicAdd(&C.verify_bytes, 2ull * len);
+      atomicAdd(&C.g->verify_bytes, 2ull * len);
     } else {
       fail(C, BT_EINTERNAL);  // the pair's own window was not seen
     }
   }
-  if (cta_failed(C)) return;
-  verify_jobs(g.T, W.jobs, C.njobs, 2 * b, W.mismatch);
-  __syncthreads();
+  if (failed(C)) return;
+  verify_jobs(g.T, W.jobs, C.g->njobs, 2 * b, W.mismatch, C.grp);
+  gsync(C.grp);
   for (uint64_t k = tid; k + 1 < c; k += nt) {
     const uint64_t id = W.job_of[k];
     if (id == kNone || !W.mismatch[id]) continue;
-    atomicAdd(&C.collisions, 1ull);
-    const uint32_t i = atomicAdd(&C.nsusp, 1u);
+    atomicAdd(&C.g->collisions, 1ull);
+    const uint32_t i = atomicAdd(&C.g->nsusp, 1u);
     W.susp[i] = k;
     W.exlo[i] = g.st[k];
   }
-  __syncthreads();
-  if (C.nsusp) {
+  gsync(C.grp);
+  if (C.g->nsusp) {
     exact_pass(m, g, H, W, 1, P.B, C);
-    for (uint32_t i = tid; i < C.nsusp; i += nt) W.pm[W.susp[i]] = W.exlo[i] == g.st[W.susp[i]];
-    __syncthreads();
+    for (uint32_t i = tid; i < C.g->nsusp; i += nt) W.pm[W.susp[i]] = W.exlo[i] == g.st[W.susp[i]];
+    gsync(C.grp);
   }
 
   // Marks: a block in a leftmost pair, or in no pair.
@@ -707,49 +799,50 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
       }
     }
   }
-  __syncthreads();
-  cta_scan_u32(W.wpop, mr, words, C.wtot);
+  gsync(C.grp);
+  if (C.grp.rank == 0) cta_scan_u32(W.wpop, mr, words, C.wtot);
+  if (C.grp.size > 1) gsync(C.grp);
 
   // Leftmost occurrence of every block that becomes a pointer (of every
   // block when pruning needs it), verified.
   if (tid == 0) {
-    C.njobs = 0;
-    C.nsusp = 0;
+    C.g->njobs = 0;
+    C.g->nsusp = 0;
   }
   for (uint64_t i = tid; i < c; i += nt) W.mismatch[i] = 0;
-  __syncthreads();
+  gsync(C.grp);
   for (uint64_t k = tid; k < c; k += nt) {
     W.job_of[k] = kNone;
     lo[k] = kNone;
     if (!P.prune && marked(mw, k)) continue;
     const uint64_t s = g.st[k], len = blen(g, k);
-    const uint64_t p = W.slotB[k] == kNoSlot ? C.lo_tail : W.bt[W.slotB[k]].lo;
+    const uint64_t p = W.slotB[k] == kNoSlot ? C.g->lo_tail : W.bt[W.slotB[k]].lo;
     lo[k] = p;
     if (p < s) {
-      const uint32_t id = atomicAdd(&C.njobs, 1u);
+      const uint32_t id = atomicAdd(&C.g->njobs, 1u);
       W.jobs[id] = BJob{p, s, len, k};
       W.job_of[k] = id;
-      atomicAdd(&C.verify_bytes, 2ull * len);
+      atomicAdd(&C.g->verify_bytes, 2ull * len);
     } else if (p > s) {
       fail(C, BT_EINTERNAL);
     }
   }
-  if (cta_failed(C)) return;
-  verify_jobs(g.T, W.jobs, C.njobs, b, W.mismatch);
-  __syncthreads();
+  if (failed(C)) return;
+  verify_jobs(g.T, W.jobs, C.g->njobs, b, W.mismatch, C.grp);
+  gsync(C.grp);
   for (uint64_t k = tid; k < c; k += nt) {
     const uint64_t id = W.job_of[k];
     if (id == kNone || !W.mismatch[id]) continue;
-    atomicAdd(&C.collisions, 1ull);
-    const uint32_t i = atomicAdd(&C.nsusp, 1u);
+    atomicAdd(&C.g->collisions, 1ull);
+    const uint32_t i = atomicAdd(&C.g->nsusp, 1u);
     W.susp[i] = k;
     W.exlo[i] = g.st[k];
   }
-  __syncthreads();
-  if (C.nsusp) {
+  gsync(C.grp);
+  if (C.g->nsusp) {
     exact_pass(m, g, H, W, 0, P.B, C);
-    for (uint32_t i = tid; i < C.nsusp; i += nt) lo[W.susp[i]] = W.exlo[i];
-    __syncthreads();
+    for (uint32_t i = tid; i < C.g->nsusp; i += nt) lo[W.susp[i]] = W.exlo[i];
+    gsync(C.grp);
   }
 }
 
@@ -764,7 +857,8 @@ template <class M>
 __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const LV& g, char* scr, uint32_t l,
                            uint32_t* dyn) {
   const uint64_t n = C.n, c = g.c, b = g.b, words = (c + 31) / 32;
-  const unsigned tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned tid = C.grp.tid(), nt = C.grp.threads(), lane = tid & 31, warp = threadIdx.x >> 5,
+                 nwarps = blockDim.x >> 5;
   uint64_t* lo = (uint64_t*)(scr + C.sl.lo[l]);
   uint32_t* mw = (uint32_t*)(scr + C.sl.mw[l]);
   uint32_t* mr = (uint32_t*)(scr + C.sl.mr[l]);
@@ -777,20 +871,16 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
   uint8_t* ps = (uint8_t*)carve(p, c + 8);
   const QGeo q{g.T, n, c, b, g.st};
   const Span w{tid, nt};
-  if (tid == 0) {
-    C.qs.nopen[0] = C.qs.nopen[1] = C.qs.nitems = C.qs.npairs = C.qs.nsusp = 0;
-    C.status.error = C.status.verify_bytes = C.status.collisions = 0;
-  }
   unsigned G = 1;
   while (G < 32 && 64ull * 2 * G <= b) G <<= 1;
   quick_min(q, C.list, G, A, X, flags, w);
-  __syncthreads();
+  gsync(C.grp);
   tmark(C, 1);
   const uint64_t bl = b < n ? b : n;
   const uint32_t ppk = (uint32_t)((2 * bl + q_piece(b) - 1) / q_piece(b));
   const unsigned L = b >= 1024 ? 32u : b >= 512 ? 16u : b >= 256 ? 8u : b >= 128 ? 4u : b >= 64 ? 2u : 1u;
   quick_compare(q, A, X, flags, ppk, L, w);
-  __syncthreads();
+  gsync(C.grp);
   tmark(C, 3);
   uint64_t vb = 0;
   uint32_t np = 0, nob = 0, nop = 0;
@@ -806,7 +896,7 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
     }
     lo[k] = at;
     if (open) {
-      items[atomicAdd(&C.qs.nitems, 1ull)] = (uint32_t)(2 * k);
+      items[atomicAdd(&C.g->qs.nitems, 1ull)] = (uint32_t)(2 * k);
       nob++;
     }
     uint32_t d2 = 0;
@@ -816,7 +906,7 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
     np += st & kIsPair;
     if (st == kIsPair && d2 != kNoDist) vb += 2 * plen;
     if (open) {
-      items[atomicAdd(&C.qs.nitems, 1ull)] = (uint32_t)(2 * k + 1);
+      items[atomicAdd(&C.g->qs.nitems, 1ull)] = (uint32_t)(2 * k + 1);
       nop++;
     }
   }
@@ -825,21 +915,21 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
   nob = __reduce_add_sync(kFull, nob);
   nop = __reduce_add_sync(kFull, nop);
   if (lane == 0) {
-    if (vb) atomicAdd(&C.status.verify_bytes, (unsigned long long)vb);
-    if (np) atomicAdd(&C.npairs, np);
-    if (nob) atomicAdd(&C.qs.nopen[0], (unsigned long long)nob);
-    if (nop) atomicAdd(&C.qs.nopen[1], (unsigned long long)nop);
+    if (vb) atomicAdd(&C.g->status.verify_bytes, (unsigned long long)vb);
+    if (np) atomicAdd(&C.g->npairs, np);
+    if (nob) atomicAdd(&C.g->qs.nopen[0], (unsigned long long)nob);
+    if (nop) atomicAdd(&C.g->qs.nopen[1], (unsigned long long)nop);
   }
-  __syncthreads();
+  gsync(C.grp);
   tmark(C, 3);
-  const uint64_t ni = C.qs.nitems;
+  const uint64_t ni = C.g->qs.nitems;
   if (ni) {
-    const uint64_t nb = C.qs.nopen[0] + 2 * C.qs.nopen[1];
-    const uint64_t bcap = pow2_ge(2 * (nb < c ? nb : c)), pcap = pow2_ge(2 * C.qs.nopen[1]), gcap = pow2_ge(2 * ni);
+    const uint64_t nb = C.g->qs.nopen[0] + 2 * C.g->qs.nopen[1];
+    const uint64_t bcap = pow2_ge(2 * (nb < c ? nb : c)), pcap = pow2_ge(2 * C.g->qs.nopen[1]), gcap = pow2_ge(2 * ni);
     uint32_t fbits = 12;
     while ((1ull << fbits) < 16 * ni && fbits < 30) fbits++;
     const uint32_t bwords = 1u << (fbits - 5);
-    if (tid == 0) {
+    if (threadIdx.x == 0) {
       Chase& K = C.chase;
       K.g = q;
       K.Q = C.list;
@@ -864,8 +954,8 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
       K.pmask = (uint32_t)(pcap - 1);
       K.gmask = (uint32_t)(gcap - 1);
       K.bshift = 32 - fbits;
-      K.qs = &C.qs;
-      K.status = &C.status;
+      K.qs = &C.g->qs;
+      K.status = &C.g->status;
       K.lo = lo;
       K.ps = ps;
     }
@@ -873,50 +963,45 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
     const Chase& K = C.chase;
     const PrefixAt<M> H(PC, g.T, n, (const uint64_t*)(scr + C.sl.Hs));
     chase_init(K, bwords, w);
-    __syncthreads();
+    gsync(C.grp);
     if (b <= 256) chase_keys<M, 1>(m, H, K, w);
     else chase_keys<M, 32>(m, H, K, w);
-    __syncthreads();
+    gsync(C.grp);
     // Shared memory: the warps' queues, then the bitmap while it fits.
     uint2* hq = (uint2*)dyn + warp * kHitQ;
-    uint32_t* cq = (uint32_t*)((uint2*)dyn + (nt / 32) * kHitQ) + warp * kCandQ;
-    uint32_t* bits_s = (uint32_t*)((uint2*)dyn + (nt / 32) * kHitQ) + (nt / 32) * kCandQ;
+    uint32_t* cq = (uint32_t*)((uint2*)dyn + nwarps * kHitQ) + warp * kCandQ;
+    uint32_t* bits_s = (uint32_t*)((uint2*)dyn + nwarps * kHitQ) + nwarps * kCandQ;
     const bool fits = bwords <= kCtaBitWords;
     if (fits)
-      for (uint32_t i = tid; i < bwords; i += nt) bits_s[i] = K.bitmap[i];
+      for (uint32_t i = threadIdx.x; i < bwords; i += blockDim.x) bits_s[i] = K.bitmap[i];
     __syncthreads();
     const uint32_t* bits = fits ? bits_s : K.bitmap;
     const uint32_t total = C.nsel, split = total > (1u << 16) ? (total / 16) & ~(8 * kChaseTile - 1) : 0;
     if (split) {
       chase_scan(m, H, K, 0, split, bits, hq, cq, nullptr, w);
-      __syncthreads();
+      gsync(C.grp);
       chase_bound(K, w);
-      __syncthreads();
+      gsync(C.grp);
     }
     chase_scan(m, H, K, split, total, bits, hq, cq, split ? K.bound2 : nullptr, w);
     if (C.r && C.r < kQuickMinB) chase_tail(K, w);
-    __syncthreads();
+    gsync(C.grp);
     tmark(C, 2);
     const unsigned Lv = b >= 256 ? 32u : b >= 128 ? 16u : b >= 64 ? 8u : 4u;
     chase_verify(K, (2 * b + q_piece(b) - 1) / q_piece(b), Lv, w);
-    __syncthreads();
+    gsync(C.grp);
     chase_apply(K, w);
-    __syncthreads();
-    const uint64_t nsusp = C.qs.nsusp;
+    gsync(C.grp);
+    const uint64_t nsusp = C.g->qs.nsusp;
     if (nsusp) {
       chase_exact(K, 0, 1, nsusp, w);
-      __syncthreads();
+      gsync(C.grp);
       chase_exact_apply(K, nsusp, w);
-      __syncthreads();
+      gsync(C.grp);
     }
   }
-  if (tid == 0) {
-    if (C.status.error) fail(C, BT_EINTERNAL);
-    C.verify_bytes = C.status.verify_bytes;
-    C.collisions = C.status.collisions;
-  }
-  if (cta_failed(C)) return;
-  for (uint64_t wb = warp; wb < words; wb += nt >> 5) {
+  if (tid == 0 && C.g->status.error) fail(C, BT_EINTERNAL);  // (the level goes on; the caller looks at the end)
+  for (uint64_t wb = tid >> 5; wb < words; wb += nt >> 5) {
     const uint64_t k = wb * 32 + lane;
     bool mk = false;
     if (k < c) {
@@ -929,8 +1014,9 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
       wpop[wb] = __popc(bits);
     }
   }
-  __syncthreads();
-  cta_scan_u32(wpop, mr, words, C.wtot);
+  gsync(C.grp);
+  if (C.grp.rank == 0) cta_scan_u32(wpop, mr, words, C.wtot);
+  if (C.grp.size > 1) gsync(C.grp);
 }
 
 template <class M>
@@ -939,7 +1025,7 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
   const uint64_t* bsz = P.sizes + D.lv_off;
   const uint64_t n = C.n, c = C.c[l], b = bsz[l];
   const bool last = l + 1 == C.L;
-  const unsigned tid = threadIdx.x, nt = blockDim.x;
+  const unsigned tid = C.grp.tid(), nt = C.grp.threads();
   LV g{D.T, n, c, b, (uint64_t*)(scr + C.sl.st[l])};
   uint64_t* lo = (uint64_t*)(scr + C.sl.lo[l]);
   uint64_t* off = (uint64_t*)(scr + C.sl.off[l]);
@@ -947,27 +1033,36 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
   uint32_t* mw = (uint32_t*)(scr + C.sl.mw[l]);
   uint32_t* mr = (uint32_t*)(scr + C.sl.mr[l]);
   const uint64_t words = (c + 31) / 32;
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     const uint64_t len_last = n - C.last_start;
     C.r = len_last < b ? len_last : 0;
     C.Bb = pow_mod(m, P.B, b);
     C.Br = C.r ? pow_mod(m, P.B, C.r) : 0;
     C.bshift = (b & (b - 1)) == 0 ? (uint32_t)(__ffsll((long long)b) - 1) : 0xFFu;
-    C.fp_tail = kNone;
-    C.lo_tail = kNone;
-    C.lo_tailpair = kNone;
-    C.pretail = kNoSlot;
-    C.npairs = 0;
-    C.njobs = 0;
-    C.nsusp = 0;
-    C.verify_bytes = 0;
-    C.collisions = 0;
-    C.lastk = 0;
   }
-  __syncthreads();
-  if (b >= kQuickMinB) quick_keys(m, PC, C, g, scr, l, dyn);
-  else scan_keys(m, P, D, C, g, scr, l, dyn, dyn_words);
-  if (cta_failed(C)) return;
+  if (tid == 0) {
+    Common& G = *C.g;
+    G.fp_tail = kNone;
+    G.lo_tail = kNone;
+    G.lo_tailpair = kNone;
+    G.pretail = kNoSlot;
+    G.npairs = 0;
+    G.njobs = 0;
+    G.nsusp = 0;
+    G.verify_bytes = 0;
+    G.collisions = 0;
+    G.lastk = 0;
+    G.qs.nopen[0] = G.qs.nopen[1] = G.qs.nitems = G.qs.npairs = G.qs.nsusp = 0;
+    G.status.error = G.status.verify_bytes = G.status.collisions = 0;
+  }
+  gsync(C.grp);
+  const bool quick = b >= kQuickMinB;
+  if (quick) {
+    quick_keys(m, PC, C, g, scr, l, dyn);
+  } else {
+    scan_keys(m, P, D, C, g, scr, l, dyn, dyn_words);
+    if (failed(C)) return;
+  }
 
   // Pointers of unmarked blocks: the block holding the leftmost occurrence
   // and the offset into it.
@@ -996,26 +1091,26 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
     ptr[k] = (uint32_t)j;
     off[k] = p - g.st[j];
   }
-  if (cta_failed(C)) return;
+  if (failed(C)) return;
 
   const uint64_t nm = mr[words];
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     C.nmarked[l] = nm;
     uint64_t* S = C.stats[l];
     S[BT_ST_NBLOCKS] = c;
     S[BT_ST_B] = b;
     S[BT_ST_COV] = (c - 1) * b + blen(g, c - 1);
     S[BT_ST_NMARKED] = nm;
-    S[BT_ST_NPAIRS] = C.npairs;
-    S[BT_ST_VERIFY_BYTES] = C.verify_bytes;
-    S[BT_ST_COLLISIONS] = C.collisions;
+    S[BT_ST_NPAIRS] = C.g->npairs;
+    S[BT_ST_VERIFY_BYTES] = quick ? C.g->status.verify_bytes : C.g->verify_bytes;
+    S[BT_ST_COLLISIONS] = quick ? C.g->status.collisions : C.g->collisions;
     S[BT_ST_FINAL_BLOCKS] = c;
-    S[BT_ST_CANDIDATES] = b >= kQuickMinB && C.qs.nitems ? C.qs.cands : 0;
-    S[BT_ST_HITS] = b >= kQuickMinB && C.qs.nitems ? C.qs.hits : 0;
+    S[BT_ST_CANDIDATES] = quick && C.g->qs.nitems ? C.g->qs.cands : 0;
+    S[BT_ST_HITS] = quick && C.g->qs.nitems ? C.g->qs.hits : 0;
   }
   if (last) {
-    if (tid == 0) C.arity[l] = 0;
-    __syncthreads();
+    if (threadIdx.x == 0) C.arity[l] = 0;
+    gsync(C.grp);
     tmark(C, 3);
     return;
   }
@@ -1024,22 +1119,26 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
   const uint32_t arity = (uint32_t)(b / bn);
   uint64_t* nst = (uint64_t*)(scr + C.sl.st[l + 1]);
   for (uint64_t wb = tid; wb < words; wb += nt)
-    if (mw[wb]) atomicMax(&C.lastk, (unsigned long long)(wb * 32 + 31 - __clz(mw[wb])));
-  __syncthreads();
-  if (tid == 0) {
+    if (mw[wb]) atomicMax(&C.g->lastk, (unsigned long long)(wb * 32 + 31 - __clz(mw[wb])));
+  gsync(C.grp);
+  if (threadIdx.x == 0) {
     C.arity[l] = arity;
-    const uint64_t lk = C.lastk;
-    if (nm == 0) {
-      C.err = BT_EINTERNAL;
-    } else {
+    const uint64_t lk = C.g->lastk;
+    C.bad = nm == 0;
+    if (nm != 0) {
       const uint64_t nch = (blen(g, lk) + bn - 1) / bn;
       const uint64_t nc = (nm - 1) * arity + nch;
-      if (nc > (n + bn - 1) / bn) C.err = BT_EINTERNAL;
+      C.bad = nc > (n + bn - 1) / bn;
       C.c[l + 1] = nc;
       C.last_start = g.st[lk] + (nch - 1) * bn;
     }
+    if (C.bad) fail(C, BT_EINTERNAL);
   }
-  if (cta_failed(C)) return;
+  __syncthreads();
+  if (C.bad) {  // (so in every CTA of the group)
+    gsync(C.grp);
+    return;
+  }
   for (uint64_t w = tid; w < c * arity; w += nt) {
     const uint64_t k = w / arity, i = w - k * arity;
     if (!marked(mw, k)) continue;
@@ -1047,7 +1146,7 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
     if (s >= g.st[k] + blen(g, k)) continue;
     nst[mrank(mw, mr, k) * arity + i] = s;
   }
-  __syncthreads();
+  gsync(C.grp);
   tmark(C, 3);
 }
 
@@ -1057,14 +1156,28 @@ __device__ PLv plevel(const Cta& C, char* scr, const uint64_t* bsz, uint32_t l) 
              (uint64_t*)(scr + C.sl.lo[l])};
 }
 
+// Levels with this few blocks are pruned by the leading CTA alone: some thirty
+// barriers of the cluster cost more than its help.
+constexpr uint64_t kLeaderPrune = 8192;
+
 __device__ void prune_pass(const BParams& P, const BDoc& D, Cta& C, char* scr) {
   const uint64_t* bsz = P.sizes + D.lv_off;
   for (int l = (int)C.L - 2; l >= 0; l--) {
     const PLv v = plevel(C, scr, bsz, (uint32_t)l), w = plevel(C, scr, bsz, (uint32_t)l + 1);
-    const uint64_t c2 = prune_level(v, w, l + 1 == (int)C.L - 1, C.arity[l], scr + C.sl.temp, P.max_rounds, C.prune);
-    if (c2 == kNone) {
-      if (threadIdx.x == 0) fail(C, BT_EINTERNAL);
-      __syncthreads();
+    const bool alone = v.c + w.c <= kLeaderPrune;
+    uint64_t c2 = 0;
+    if (!alone || C.grp.rank == 0)
+      c2 = prune_level(v, w, l + 1 == (int)C.L - 1, C.arity[l], scr + C.sl.temp, P.max_rounds, C.g->prune, C.wtot,
+                       alone ? Group{} : C.grp);
+    if (alone && C.grp.size > 1) {
+      if (C.grp.tid() == 0) C.g->part[0] = c2;
+      gsync(C.grp);
+      c2 = *(volatile uint64_t*)&C.g->part[0];
+      gsync(C.grp);
+    }
+    if (c2 == kNone) {  // (so in every CTA of the group)
+      if (C.grp.tid() == 0) fail(C, BT_EINTERNAL);
+      gsync(C.grp);
       return;
     }
     if (threadIdx.x == 0) {
@@ -1089,9 +1202,9 @@ __device__ void prune_pass(const BParams& P, const BDoc& D, Cta& C, char* scr) {
 __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PLv& v, int mode, bool last,
                            void* out, uint32_t cw, uint64_t cp, unsigned int* hist) {
   const uint32_t S = C.S;
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  unsigned int* h = hist + warp * 1024;
-  for (uint64_t g = warp; 4 * g < v.c; g += nw) {
+  const unsigned lane = threadIdx.x & 31, nw = C.grp.threads() >> 5;
+  unsigned int* h = hist + (threadIdx.x >> 5) * 1024;
+  for (uint64_t g = C.grp.tid() >> 5; 4 * g < v.c; g += nw) {
     uint64_t s0[4];
     uint32_t len[4], top = 0;
     bool any = false;
@@ -1157,7 +1270,7 @@ __device__ void count_small(const uint8_t* __restrict__ T, const Cta& C, const P
   uint32_t TB = blockDim.x;
   while ((uint64_t)TB * S > kDynWords * 4ull) TB >>= 1;  // 1024, or 512 above 128 symbols
   const uint32_t col = 4 * (lane + 32 * (warp >> 2)) + (warp & 3);
-  for (uint64_t k0 = 0; k0 < v.c; k0 += TB) {
+  for (uint64_t k0 = (uint64_t)C.grp.rank * TB; k0 < v.c; k0 += (uint64_t)C.grp.size * TB) {
     __syncthreads();
     for (uint32_t i = tid; i < S * (TB / 4); i += blockDim.x) ((uint32_t*)tile)[i] = 0;
     __syncthreads();
@@ -1196,13 +1309,13 @@ __device__ void count_small(const uint8_t* __restrict__ T, const Cta& C, const P
 
 __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr, unsigned int* hist) {
   const uint64_t* bsz = P.sizes + D.lv_off;
-  const unsigned tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  const unsigned tid = C.grp.tid(), nt = C.grp.threads(), lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   const uint32_t L = C.L, S = C.S;
   __shared__ OutLevel s_ol[kBMaxLevels];
   __shared__ uint32_t s_cw[kBMaxLevels];
   __shared__ uint64_t s_view, s_pre, s_leaf, s_sym;
   __shared__ uint32_t s_base;
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     for (uint32_t l = 0; l < L; l++) s_cw[l] = counter_width(bsz[l]);
     const uint64_t words = (C.c[L - 1] + 31) / 32;
     const uint32_t* mrl = (const uint32_t*)(scr + C.sl.mr[L - 1]);
@@ -1211,17 +1324,14 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
     s_base = out_base(L, C.c, bsz, C.n, S);
     const uint64_t need = out_layout(L, s_base, C.c, s_cw, S, leaf_alloc, s_ol, &s_view, &s_pre, &s_leaf, &s_sym);
     C.out_bytes = need;
-    const unsigned long long o = atomicAdd(P.pool_used, (unsigned long long)need);
-    if (o + need > P.pool_cap) {
-      C.err = BT_ENOMEM;
-      C.out = nullptr;
-    } else {
-      C.out_off = o;
-      C.out = P.pool + o;
+    if (tid == 0) {
+      const unsigned long long o = atomicAdd(P.pool_used, (unsigned long long)need);
+      C.g->out_off = C.out_off = o;
+      if (o + need > P.pool_cap) fail(C, BT_ENOMEM);
     }
   }
-  if (cta_failed(C)) return;
-  char* out = C.out;
+  if (failed(C)) return;
+  char* out = P.pool + C.g->out_off;
   const uint32_t bl = s_base;
   // Level arrays.
   for (uint32_t l = 0; l < L; l++) {
@@ -1238,7 +1348,7 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
       mr[i] = v.mr[i];
     }
   }
-  __syncthreads();
+  gsync(C.grp);
   // Counters, last level first (marked blocks sum their children's).
   for (int l = (int)L - 1; l >= (int)bl; l--) {
     const PLv v = plevel(C, scr, bsz, (uint32_t)l);
@@ -1254,7 +1364,7 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
       count_rows(D.T, C, v, 0, last, cnt, cw, cp, hist);
       count_rows(D.T, C, v, 1, last, pc, cw, cp, hist);
     }
-    __syncthreads();
+    gsync(C.grp);
     if (!last) {
       const void* ccnt = out + s_ol[l + 1].cnt;
       const uint32_t ccw = s_cw[l + 1];
@@ -1296,7 +1406,7 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
             if (s + u < s1) cput(cnt, cw, (s + u) * cp + k, x[u]);
         }
       }
-      __syncthreads();
+      gsync(C.grp);
     }
   }
   // Prefix counts of the base level, a warp per symbol.
@@ -1376,7 +1486,7 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
     tv->leaf = (const uint8_t*)(out + s_leaf);
     tv->sym = (const int16_t*)(out + s_sym);
   }
-  __syncthreads();
+  gsync(C.grp);
 }
 
 template <class M>
@@ -1385,55 +1495,57 @@ __device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw,
   const BDoc D = P.docs[d];
   const uint64_t* bsz = P.sizes + D.lv_off;
   if (threadIdx.x == 0) {
-    C.err = 0;
     C.n = D.n;
     C.L = D.L;
-    if (D.L == 0 || D.L > kBMaxLevels || scratch_layout(D.n, D.L, bsz, &C.sl) > P.scratch_per_cta)
-      C.err = BT_EINTERNAL;
+    C.bad = D.L == 0 || D.L > kBMaxLevels || scratch_layout(D.n, D.L, bsz, &C.sl) > P.scratch_per_cta;
+    if (C.grp.rank == 0) {
+      C.g->err = C.bad ? BT_EINTERNAL : 0;
+      for (uint32_t& x : C.g->seen) x = 0;
+    }
     C.out_off = 0;
     C.out_bytes = 0;
     for (int i = 0; i < 6; i++) C.cyc[i] = 0;
     C.t_mark = clock64();
   }
-  __syncthreads();
-  if (C.err == 0) alphabet(D.T, D.n, D.sigma, C);
-  if (!cta_failed(C)) {
+  gsync(C.grp);
+  if (!C.bad) alphabet(D.T, D.n, D.sigma, C);
+  if (!failed(C)) {
     prefix_pass(m, PC, pw, D.T, D.n, (uint64_t*)(scr + C.sl.Hs), C);
     if (threadIdx.x == 0) C.expanded = 0;
     if (bsz[0] >= kQuickMinB) list_pass(D.T, D.n, scr, C);
     // Level 1: blocks k b_1.
     uint64_t* st0 = (uint64_t*)(scr + C.sl.st[0]);
     const uint64_t c0 = (D.n + bsz[0] - 1) / bsz[0];
-    for (uint64_t k = threadIdx.x; k < c0; k += blockDim.x) st0[k] = k * bsz[0];
+    for (uint64_t k = C.grp.tid(); k < c0; k += C.grp.threads()) st0[k] = k * bsz[0];
     if (threadIdx.x == 0) {
       C.c[0] = c0;
       C.last_start = (c0 - 1) * bsz[0];
     }
-    __syncthreads();
+    gsync(C.grp);
     tmark(C, 0);
     for (uint32_t l = 0; l < D.L; l++) {
       level_pass(m, PC, P, D, C, scr, l, (uint32_t*)hist, dyn_words);
-      if (cta_failed(C)) break;
+      if (failed(C)) break;
     }
   }
-  if (!cta_failed(C) && P.prune) {
+  if (!failed(C) && P.prune) {
     prune_pass(P, D, C, scr);
     tmark(C, 4);
   }
-  if (!cta_failed(C)) write_output(P, D, C, scr, hist);
-  __syncthreads();
+  if (!failed(C)) write_output(P, D, C, scr, hist);
+  gsync(C.grp);
   tmark(C, 5);
-  // Results.
+  // Results, from the leading CTA.
+  if (C.grp.rank != 0) return;
   if (threadIdx.x == 0) {
     BRes& R = P.res[D.index];
-    R.status = C.err;
+    R.status = C.g->err;
     R.S = C.S;
     R.out_off = C.out_off;
     R.out_bytes = C.out_bytes;
     for (int i = 0; i < 6; i++) R.cycles[i] = C.cyc[i];
   }
-  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) P.res[D.index].sym[i] = C.sym[i];
-  if (C.err == 0) {
+  if (C.g->err == 0) {
     for (uint32_t l = threadIdx.x; l < D.L; l += blockDim.x) {
       BLevelRes& Lr = P.lres[D.lv_off + l];
       Lr.c = C.c[l];
@@ -1447,7 +1559,8 @@ __device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw,
   __syncthreads();
 }
 
-// One CTA of 1024 threads per SM: 64 registers per thread.
+// One CTA of 1024 threads per SM: 64 registers per thread.  A document belongs
+// to a CTA, or to a cluster of them.
 template <class M>
 __global__ void __launch_bounds__(kMaxBThreads, 1) k_batch(const __grid_constant__ BParams P, M m,
                                                            const __grid_constant__ PrefixConst<M> PC,
@@ -1456,12 +1569,18 @@ __global__ void __launch_bounds__(kMaxBThreads, 1) k_batch(const __grid_constant
   // window filter), then (during the output) the symbol counters.
   extern __shared__ unsigned int s_hist[];
   __shared__ Cta C;
-  char* scr = P.scratch + (uint64_t)blockIdx.x * P.scratch_per_cta;
+  const Group grp = this_cluster();
+  char* scr = P.scratch + (uint64_t)(blockIdx.x / grp.size) * P.scratch_per_cta;
+  if (threadIdx.x == 0) {
+    C.grp = grp;
+    C.g = grp.size == 1 ? &C.own : (Common*)scr;
+  }
+  __syncthreads();
   for (;;) {
-    if (threadIdx.x == 0) C.doc = atomicAdd(P.next, 1u);
-    __syncthreads();
-    const uint32_t d = C.doc;
-    __syncthreads();
+    if (grp.tid() == 0) C.g->doc = atomicAdd(P.next, 1u);
+    gsync(grp);
+    const uint32_t d = *(volatile uint32_t*)&C.g->doc;
+    gsync(grp);
     if (d >= P.ndocs) return;
     build_doc(m, PC, pw, P, d, C, scr, s_hist, P.dyn_words);
   }
@@ -1486,35 +1605,135 @@ struct DocPlan {
   uint64_t size_off;       // first block size in the batch's size array
 };
 
-// Opt the kernel in to its dynamic shared memory, once per device.
+// Opt the kernel in to its dynamic shared memory and to clusters of sixteen
+// CTAs, once per device; the largest cluster the device can hold.
 template <class M>
-int allow_batch_smem(int bytes) {
-  static std::atomic<uint64_t> done{0};
+int prepare_batch_kernel(int bytes, uint32_t* max_group) {
+  static std::atomic<uint32_t> most[64] = {};
   int dev = 0;
   BT_CUDA(cudaGetDevice(&dev));
-  const uint64_t bit = 1ull << (dev & 63);
-  if (done.load(std::memory_order_acquire) & bit) return BT_OK;
-  BT_CUDA(cudaFuncSetAttribute(k_batch<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  done.fetch_or(bit, std::memory_order_acq_rel);
+  uint32_t g = most[dev & 63].load(std::memory_order_acquire);
+  if (!g) {
+    BT_CUDA(cudaFuncSetAttribute(k_batch<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    g = 8;
+    if (cudaFuncSetAttribute(k_batch<M>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) g = 16;
+    for (; g > 1; g /= 2) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(g);
+      cfg.blockDim = dim3(kMaxBThreads);
+      cfg.dynamicSmemBytes = bytes;
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = g;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k_batch<M>, &cfg) == cudaSuccess && n > 0) break;
+    }
+    cudaGetLastError();
+    most[dev & 63].store(g, std::memory_order_release);
+  }
+  *max_group = g;
   return BT_OK;
 }
 
+// `groups` clusters of `group` CTAs, per_group bytes of scratch each.
 template <class M>
-int launch_docs(const M& m, const BParams& base, uint32_t first, uint32_t count, unsigned grid, uint64_t per_cta,
-                char* scratch, unsigned int* next, cudaStream_t s) {
+int launch_docs(const M& m, const BParams& base, uint32_t first, uint32_t count, unsigned groups, uint32_t group,
+                uint64_t per_group, char* scratch, unsigned int* next, cudaStream_t s) {
   BParams P = base;
   P.docs = base.docs + first;
   P.ndocs = count;
   P.next = next;
   P.scratch = scratch;
-  P.scratch_per_cta = per_cta;
+  P.scratch_per_cta = per_group;
   P.dyn_words = kDynWords;
-  BT_CUDA(cudaMemsetAsync(next, 0, sizeof(unsigned int), s));
-  BT_TRY(allow_batch_smem<M>((int)(kDynWords * sizeof(unsigned int))));
+  constexpr int smem = (int)(kDynWords * sizeof(unsigned int));
+  uint32_t most;
+  BT_TRY(prepare_batch_kernel<M>(smem, &most));
+  if (group > most) group = most;
   const PrefixConst<M> PC(m, P.B);
   const KrPow pw = kr_pow(m, pow_mod(m, P.B, 128));  // a thread of the prefix pass takes four 32-byte chunks
-  BT_LAUNCH(k_batch<M><<<grid, kMaxBThreads, kDynWords * sizeof(unsigned int), s>>>(P, m, PC, pw));
-  BT_CUDA(cudaGetLastError());
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(groups * group);
+  cfg.blockDim = dim3(kMaxBThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = group;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = group > 1 ? 1 : 0;
+  BT_LAUNCH(BT_CUDA(cudaLaunchKernelEx(&cfg, k_batch<M>, P, m, PC, pw)));
+  return BT_OK;
+}
+
+// Points a tree at the arrays that the kernel wrote to its pool.
+void tree_from(bt_tree* t, uint64_t n, uint32_t tau, uint32_t leaf_len, uint32_t L, const bt_opts& o, int device,
+               const BRes& R, const BLevelRes* lres, const std::shared_ptr<void>& pool) {
+  t->n = n;
+  t->tau = tau;
+  t->leaf_len = leaf_len;
+  t->L = L;
+  t->prune = o.prune ? 1 : 0;
+  t->seed = o.seed;
+  t->q = o.modulus ? o.modulus : Mersenne61::Q;
+  t->B = base_for(o.seed, t->q);
+  t->device = device;
+  t->S = R.S;
+  t->leaf_bytes = R.leaf_bytes;
+  t->slab = pool;
+  t->lv.resize(L);
+  uint64_t c[kBMaxLevels], bs[kBMaxLevels], o_view, o_pre, o_leaf, o_sym;
+  uint32_t cw[kBMaxLevels];
+  OutLevel ol[kBMaxLevels];
+  for (uint32_t l = 0; l < L; l++) {
+    c[l] = lres[l].c;
+    bs[l] = lres[l].b;
+    cw[l] = lres[l].cw;
+  }
+  const BLevelRes& last = lres[L - 1];
+  t->base = out_base(L, c, bs, n, R.S);
+  out_layout(L, t->base, c, cw, R.S, last.nmarked * last.b, ol, &o_view, &o_pre, &o_leaf, &o_sym);
+  char* base = (char*)pool.get() + R.out_off;
+  for (uint32_t l = 0; l < L; l++) {
+    Level& v = t->lv[l];
+    v.c = lres[l].c;
+    v.b = lres[l].b;
+    v.arity = lres[l].arity;
+    v.nmarked = lres[l].nmarked;
+    v.cw = lres[l].cw;
+    v.mw = (uint32_t*)(base + ol[l].mw);
+    v.mr = (uint32_t*)(base + ol[l].mr);
+    v.rec = (uint2*)(base + ol[l].rec);
+    v.cnt = l >= t->base ? base + ol[l].cnt : nullptr;
+    v.pc = l >= t->base ? base + ol[l].pc : nullptr;
+    memcpy(v.stats, lres[l].stats, sizeof(v.stats));
+  }
+  t->view = (TreeView*)(base + o_view);
+  t->pre = (uint32_t*)(base + o_pre);
+  t->leaf = (uint8_t*)(base + o_leaf);
+  t->sym = (int16_t*)(base + o_sym);
+  t->dev_bytes = R.out_bytes;
+}
+
+// A pool for finished trees, `cap` bytes.  It outlives the call: the memory
+// goes back to the device's stream-ordered pool when the last tree is freed (on
+// the freeing thread's stream; a tree is never freed while queries on it run).
+int make_pool(uint64_t cap, cudaStream_t s, std::shared_ptr<void>& out) {
+  void* p = nullptr;
+  if (!alloc_allowed(cap)) return BT_ENOMEM;
+  cudaError_t e = cudaMallocAsync(&p, cap, s);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? BT_ENOMEM : BT_ECUDA;
+  }
+  out = std::shared_ptr<void>(p, [](void* x) {
+    cudaFreeAsync(x, cudaStreamPerThread);
+    cudaStreamSynchronize(cudaStreamPerThread);
+  });
   return BT_OK;
 }
 
@@ -1615,25 +1834,8 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
   // size it reported.
   uint64_t pool_cap = 0;
   for (uint64_t k = 0; k < nd; k++) pool_cap += 3 * plans[k].n + (32u << 10);
-  // The pool outlives the call: it is returned to the device's stream-ordered
-  // pool when the last tree is freed (on the freeing thread's stream; a tree
-  // is never freed while queries on it run).
-  auto make_pool = [&](uint64_t cap, std::shared_ptr<void>& out) -> int {
-    void* p = nullptr;
-    if (!alloc_allowed(cap)) return BT_ENOMEM;
-    cudaError_t e = cudaMallocAsync(&p, cap, s);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return e == cudaErrorMemoryAllocation ? BT_ENOMEM : BT_ECUDA;
-    }
-    out = std::shared_ptr<void>(p, [](void* x) {
-      cudaFreeAsync(x, cudaStreamPerThread);
-      cudaStreamSynchronize(cudaStreamPerThread);
-    });
-    return BT_OK;
-  };
   std::shared_ptr<void> pool;
-  BT_TRY(make_pool(pool_cap, pool));
+  BT_TRY(make_pool(pool_cap, s, pool));
   unsigned long long* d_used;
   BT_TRY(mem.alloc(&d_used, 1));
   BT_CUDA(cudaMemsetAsync(d_used, 0, sizeof(unsigned long long), s));
@@ -1660,7 +1862,8 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
   struct Cls {
     uint32_t first, count;
     uint64_t per_cta;
-    unsigned grid;
+    unsigned grid;   // documents at a time
+    uint32_t group;  // CTAs for each
   };
   std::vector<Cls> cls;
   uint64_t scratch_max = 0;
@@ -1689,7 +1892,15 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
       grid = std::min<uint64_t>({(uint64_t)(e - r), budget / top, cap});
       if (grid == 0) grid = 1;
     }
-    cls.push_back(Cls{r, e - r, top, (unsigned)grid});
+    // Fewer documents than SMs: a cluster of CTAs for each (not with a bound
+    // on the CTAs, which leaves SMs to other work).  One document of DNA copies
+    // by 1, 4, 8, 16 CTAs: 16 KiB 559, 664, 665, 675 us, 256 KiB 1319, 1100,
+    // 1065, 1059, 1 MiB 3280, 1769, 1522, 1418 -- from 128 KiB a document on.
+    uint64_t bytes = 0;
+    for (uint32_t q2 = r; q2 < e; q2++) bytes += order[q2]->n;
+    uint32_t group = 1;
+    while (!o.batch_ctas && bytes >= (e - r) * (128ull << 10) && group < kMaxGroup && grid * group * 2 <= nsm) group *= 2;
+    cls.push_back(Cls{r, e - r, top, (unsigned)grid, group});
     scratch_max = std::max<uint64_t>(scratch_max, grid * top);
     r = e;
   }
@@ -1700,9 +1911,12 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
   const bool timed = cudaEventCreate(&ev[0]) == cudaSuccess && cudaEventCreate(&ev[1]) == cudaSuccess;
   if (timed) cudaEventRecord(ev[0], s);
   int lrc = BT_OK;
-  for (size_t ci = 0; ci < cls.size() && lrc == BT_OK; ci++)
-    lrc = launch_docs(m, P, cls[ci].first, cls[ci].count, cls[ci].grid, cls[ci].per_cta, d_scratch,
-                      d_next + (ci % 64), s);
+  for (size_t ci = 0; ci < cls.size() && lrc == BT_OK; ci++) {
+    unsigned int* next = d_next + (ci % 64);
+    lrc = cudaMemsetAsync(next, 0, sizeof(unsigned int), s) == cudaSuccess ? BT_OK : BT_ECUDA;
+    if (lrc == BT_OK)
+      lrc = launch_docs(m, P, cls[ci].first, cls[ci].count, cls[ci].grid, cls[ci].group, cls[ci].per_cta, d_scratch, next, s);
+  }
   if (timed) cudaEventRecord(ev[1], s);
   std::vector<BRes> res(nd);
   std::vector<BLevelRes> lres(nlv);
@@ -1733,7 +1947,7 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
       }
     if (!again.empty()) {
       std::shared_ptr<void> pool2;
-      BT_TRY(make_pool(cap2, pool2));
+      BT_TRY(make_pool(cap2, s, pool2));
       std::vector<BDoc> hd2;
       uint64_t top = 0;
       for (uint32_t k : again) {
@@ -1752,7 +1966,8 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
       const unsigned grid = (unsigned)std::max<uint64_t>(
           1, std::min<uint64_t>({(uint64_t)hd2.size(), (uint64_t)nsm * ctas_per_sm, scratch_max / top,
                                  o.batch_ctas ? (uint64_t)o.batch_ctas : ~0ull}));
-      BT_TRY(launch_docs(m, P2, 0, (uint32_t)hd2.size(), grid, top, d_scratch, d_next, s));
+      BT_CUDA(cudaMemsetAsync(d_next, 0, sizeof(unsigned int), s));
+      BT_TRY(launch_docs(m, P2, 0, (uint32_t)hd2.size(), grid, 1, top, d_scratch, d_next, s));
       BT_CUDA(cudaMemcpyAsync(res.data(), d_res, nd * sizeof(BRes), cudaMemcpyDeviceToHost, s));
       BT_CUDA(cudaMemcpyAsync(lres.data(), d_lres, nlv * sizeof(BLevelRes), cudaMemcpyDeviceToHost, s));
       BT_CUDA(cudaStreamSynchronize(s));
@@ -1772,54 +1987,7 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
     bt_tree* t = new (std::nothrow) bt_tree();
     if (!t) return BT_ENOMEM;
     outs[D.i] = t;
-    t->n = D.n;
-    t->tau = taus[D.i];
-    t->leaf_len = leaf_lens[D.i];
-    t->L = D.L;
-    t->prune = o.prune ? 1 : 0;
-    t->seed = o.seed;
-    t->q = q;
-    t->B = B;
-    t->device = device;
-    t->S = R.S;
-    t->leaf_bytes = R.leaf_bytes;
-    t->slab = pool_of[k];
-    t->lv.resize(D.L);
-    std::vector<uint64_t> c(D.L), bs(D.L);
-    std::vector<uint32_t> cw(D.L);
-    for (uint32_t l = 0; l < D.L; l++) {
-      const BLevelRes& Lr = lres[lv_off[k] + l];
-      c[l] = Lr.c;
-      bs[l] = Lr.b;
-      cw[l] = Lr.cw;
-    }
-    const BLevelRes& last = lres[lv_off[k] + D.L - 1];
-    std::vector<OutLevel> ol(D.L);
-    uint64_t o_view, o_pre, o_leaf, o_sym;
-    t->base = out_base(D.L, c.data(), bs.data(), D.n, R.S);
-    out_layout(D.L, t->base, c.data(), cw.data(), R.S, last.nmarked * last.b, ol.data(), &o_view, &o_pre, &o_leaf,
-               &o_sym);
-    char* base = (char*)t->slab.get() + R.out_off;
-    for (uint32_t l = 0; l < D.L; l++) {
-      const BLevelRes& Lr = lres[lv_off[k] + l];
-      Level& v = t->lv[l];
-      v.c = Lr.c;
-      v.b = Lr.b;
-      v.arity = Lr.arity;
-      v.nmarked = Lr.nmarked;
-      v.cw = Lr.cw;
-      v.mw = (uint32_t*)(base + ol[l].mw);
-      v.mr = (uint32_t*)(base + ol[l].mr);
-      v.rec = (uint2*)(base + ol[l].rec);
-      v.cnt = l >= t->base ? base + ol[l].cnt : nullptr;
-      v.pc = l >= t->base ? base + ol[l].pc : nullptr;
-      memcpy(v.stats, Lr.stats, sizeof(v.stats));
-    }
-    t->view = (TreeView*)(base + o_view);
-    t->pre = (uint32_t*)(base + o_pre);
-    t->leaf = (uint8_t*)(base + o_leaf);
-    t->sym = (int16_t*)(base + o_sym);
-    t->dev_bytes = R.out_bytes;
+    tree_from(t, D.n, taus[D.i], leaf_lens[D.i], D.L, o, device, R, &lres[lv_off[k]], pool_of[k]);
     for (int i = 0; i < 6; i++) t->batch_cycles[i] = R.cycles[i];
   }
   {
@@ -1834,12 +2002,142 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
     g_report.pool_bytes = pool_cap;
     g_report.scratch_bytes = scratch_max;
     g_report.max_grid = 0;
-    for (const Cls& c2 : cls) g_report.max_grid = std::max<uint64_t>(g_report.max_grid, c2.grid);
+    for (const Cls& c2 : cls) g_report.max_grid = std::max<uint64_t>(g_report.max_grid, (uint64_t)c2.grid * c2.group);
   }
   return BT_OK;
 }
 
+// Texts up to this long are built by one CTA in one launch: at 4 KiB and four
+// levels it takes 240 us, some fifty launches and four round trips 350 us.  The
+// line lies where one CTA is too slow for the counters of many symbols: random
+// bytes take about as long both ways at 16 KiB (DNA copies still half at 64 KiB).
+constexpr uint64_t kSoloText = 16u << 10;
+constexpr uint64_t kSoloOut = 64u << 20;  // most room for its tree
+
+// What a single build sends (to the start of its scratch) and receives (in the
+// thread's pinned page, written by the kernel).
+struct SoloHead {
+  BDoc doc;
+  uint64_t sizes[kBMaxLevels];
+  unsigned long long used;
+  unsigned int next;
+};
+struct SoloPage {
+  SoloHead head;
+  BRes res;
+  BLevelRes lres[kBMaxLevels];
+};
+static_assert(sizeof(SoloPage) <= kPageBytes - kPageSolo, "a document fits its place in the pinned page");
+
+// Moves a finished tree to memory of its own: the arrays as they are, the view's
+// pointers moved along.
+__global__ void __launch_bounds__(256) k_move_tree(const char* from, char* to, uint64_t bytes) {
+  for (uint64_t i = 16 * (blockIdx.x * 256ull + threadIdx.x); i < bytes; i += 16 * 256ull * gridDim.x) {
+    if (i >= sizeof(TreeView)) *(uint4*)(to + i) = *(const uint4*)(from + i);
+  }
+  if (blockIdx.x) return;
+  // (The view, one thread per level: the rest of its 16-byte unit is padding.)
+  const TreeView* a = (const TreeView*)from;
+  TreeView* b = (TreeView*)to;
+  auto moved = [&](const void* p) { return p ? to + ((const char*)p - from) : nullptr; };
+  const uint32_t l = threadIdx.x;
+  if (l < a->L) {
+    LevelView v = a->lv[l];
+    v.rec = (const uint2*)moved(v.rec);
+    v.cnt = moved(v.cnt);
+    v.pc = moved(v.pc);
+    b->lv[l] = v;
+  }
+  if (l == 255) {
+    b->n = a->n;
+    b->L = a->L;
+    b->S = a->S;
+    b->base = a->base;
+    b->pre = (const uint32_t*)moved(a->pre);
+    b->leaf = (const uint8_t*)moved(a->leaf);
+    b->sym = (const int16_t*)moved(a->sym);
+  }
+}
+
+// The most a text's tree can take (no level pruned, all symbols).
+uint64_t most_out(uint64_t n, uint32_t sigma, const std::vector<uint64_t>& b) {
+  const uint32_t L = (uint32_t)b.size();
+  uint64_t c[kBMaxLevels], x;
+  uint32_t cw[kBMaxLevels];
+  OutLevel ol[kBMaxLevels];
+  for (uint32_t l = 0; l < L; l++) {
+    c[l] = (n + b[l] - 1) / b[l];
+    cw[l] = counter_width(b[l]);
+  }
+  const uint32_t S = (uint32_t)std::min<uint64_t>(std::min<uint64_t>(sigma, 256), n);
+  // The prefix table is the largest at the level with the most blocks.
+  return out_layout(L, 0, c, cw, S, c[L - 1] * b[L - 1], ol, &x, &x, &x, &x) + (c[L - 1] + 1) * (uint64_t)S * 4;
+}
+
+template <class M>
+int run_solo(const M& m, const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, uint32_t leaf_len,
+             const bt_opts& o, const std::vector<uint64_t>& sizes, cudaStream_t s, bt_tree* t) {
+  char* page = pinned_page();
+  if (!page) return BT_ENOMEM;
+  SoloPage* S = (SoloPage*)(page + kPageSolo);
+  const uint32_t L = (uint32_t)sizes.size();
+  int device = 0;
+  BT_CUDA(cudaGetDevice(&device));
+  ScratchLayout sl;
+  const uint64_t need = scratch_layout(n, L, sizes.data(), &sl), head = out_align(sizeof(SoloHead)),
+                 room = out_align(n + 64), cap = out_align(most_out(n, sigma, sizes));
+  DevFree mem;
+  mem.s = s;
+  char* d;
+  BT_TRY(mem.alloc(&d, head + room + need + cap));
+  SoloHead* dh = (SoloHead*)d;
+  char* out = d + head + room + need;
+  BT_CUDA(cudaMemcpyAsync(d + head, text, n, cudaMemcpyDefault, s));
+  S->head.doc = BDoc{(const uint8_t*)(d + head), n, sigma, L, 0, 0};
+  for (uint32_t l = 0; l < L; l++) S->head.sizes[l] = sizes[l];
+  S->head.used = 0;
+  S->head.next = 0;
+  S->res.status = BT_ECUDA;
+  BT_CUDA(cudaMemcpyAsync(dh, &S->head, sizeof(SoloHead), cudaMemcpyHostToDevice, s));
+  BParams P{};
+  P.docs = &dh->doc;
+  P.sizes = dh->sizes;
+  P.res = &S->res;
+  P.lres = S->lres;
+  P.pool = out;
+  P.pool_used = &dh->used;
+  P.pool_cap = cap;
+  P.B = base_for(o.seed, o.modulus ? o.modulus : Mersenne61::Q);
+  P.prune = o.prune ? 1 : 0;
+  P.max_rounds = o.max_rounds ? o.max_rounds : 4096;
+  BT_TRY(launch_docs(m, P, 0, 1, 1, 1, need, d + head + room, &dh->next, s));
+  BT_CUDA(cudaStreamSynchronize(s));
+  const int rc = *(volatile int*)&S->res.status;
+  if (rc == BT_ENOMEM) return BT_EINTERNAL;  // (the room was the most it can take)
+  if (rc != BT_OK) return rc;
+  std::shared_ptr<void> own;
+  const uint64_t bytes = out_align16(S->res.out_bytes);
+  BT_TRY(make_pool(bytes, s, own));
+  BT_LAUNCH(k_move_tree<<<(unsigned)std::min<uint64_t>(152, bytes / 4096 + 1), 256, 0, s>>>(out, (char*)own.get(), bytes));
+  BT_CUDA(cudaGetLastError());
+  BT_CUDA(cudaStreamSynchronize(s));
+  tree_from(t, n, tau, leaf_len, L, o, device, S->res, S->lres, own);
+  return BT_OK;
+}
+
 }  // namespace
+
+// One short text by one CTA.  BT_ENOMEM leaves the tree untouched: the caller's
+// other path needs no memory in one piece.
+int solo_build(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau, uint32_t leaf_len, const bt_opts& o,
+               const std::vector<uint64_t>& sizes, cudaStream_t s, bt_tree* t) {
+  if (!o.modulus) return run_solo(Mersenne61{}, text, n, sigma, tau, leaf_len, o, sizes, s, t);
+  return run_solo(SmallMod{o.modulus}, text, n, sigma, tau, leaf_len, o, sizes, s, t);
+}
+
+bool solo_takes(uint64_t n, uint32_t sigma, const std::vector<uint64_t>& sizes) {
+  return n <= kSoloText && sizes.size() <= kBMaxLevels && most_out(n, sigma, sizes) <= kSoloOut;
+}
 
 // Builds, with the persistent kernel, every document it can take (at most
 // kBMaxText bytes and kBMaxLevels levels): routed[d] = 1 and outs[d] holds

@@ -45,7 +45,6 @@ struct BRes {
   // fingerprints), tables (block and pair fingerprints), window scan,
   // verification / marks / pointers / split, pruning, output and counters.
   unsigned long long cycles[6];
-  int16_t sym[256];
 };
 
 // Where the arrays of a finished tree lie in its pool region, in bytes from
@@ -100,7 +99,9 @@ __host__ __device__ inline uint64_t out_layout(uint32_t L, uint32_t base, const 
   return o;
 }
 
-// Scratch of one CTA for one document: offsets in bytes from the CTA's
+constexpr uint32_t kCommonBytes = 4096;  // first of all: what a cluster's CTAs share
+
+// Scratch of one CTA (or cluster) for one document: offsets in bytes from its
 // region.  Level l may hold at most cmax[l] = ceil(n / b_l) blocks.
 struct ScratchLayout {
   uint64_t Hs;                                  // u64[n / 32 + 2]: prefix fingerprints H(32 j)
@@ -145,7 +146,7 @@ __host__ __device__ inline uint64_t temp_bytes(uint64_t cm, uint64_t b) {
 }
 
 __host__ __device__ inline uint64_t scratch_layout(uint64_t n, uint32_t L, const uint64_t* b, ScratchLayout* s) {
-  uint64_t o = 0, temp = 0;
+  uint64_t o = kCommonBytes, temp = 0;
   s->Hs = o;
   o = out_align(o + (n / 32 + 2) * 8);
   s->big = o;

@@ -303,12 +303,13 @@ struct Status {
   unsigned long long blocks[64], marks[64];  // per level of the finished tree
 };
 
-// 8 KiB of pinned host memory of the calling thread (portable: any device),
+// 16 KiB of pinned host memory of the calling thread (portable: any device),
 // given back when the thread ends: where its builds and single queries
 // receive small results.  A build that allocated its own cost 0.1 ms and more
 // in the driver each time.
 char* pinned_page();
-constexpr uint32_t kPageQuick = 4096, kPageAnswer = 6144;  // places in it (the build's Status at 0)
+constexpr uint32_t kPageBytes = 16384;
+constexpr uint32_t kPageQuick = 4096, kPageAnswer = 6144, kPageSolo = 8192;  // places in it (a build's Status at 0)
 
 // Test hook (bt_test_alloc_limit): the largest single device allocation a
 // build may make; larger ones fail as if the device were out of memory.

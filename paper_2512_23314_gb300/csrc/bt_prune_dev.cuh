@@ -1,10 +1,38 @@
-// bt_prune_dev.cuh -- one level of the pruning pass by one CTA, for the batched
-// kernel (bt_batch.cu) and the small levels of a single text (bt_prune.cu).
+// bt_prune_dev.cuh -- one level of the pruning pass by one CTA or a cluster of
+// CTAs, for the batched kernel (bt_batch.cu) and the small levels of a single
+// text (bt_prune.cu).
 #pragma once
+
+#include <cooperative_groups.h>
 
 #include "bt_internal.cuh"
 
 namespace bt {
+
+// The CTAs that share a document: one, or a thread-block cluster.  Every thread
+// of the group reaches every gsync.
+struct Group {
+  uint32_t rank = 0, size = 1;
+  __device__ unsigned tid() const { return rank * blockDim.x + threadIdx.x; }
+  __device__ unsigned threads() const { return size * blockDim.x; }
+};
+
+__device__ __forceinline__ Group this_cluster() {
+  const cooperative_groups::cluster_group c = cooperative_groups::this_cluster();
+  Group g;
+  g.rank = c.block_rank();
+  g.size = c.num_blocks();
+  return g;
+}
+
+// Barrier of the group; what its threads wrote before is seen by all after.
+__device__ __forceinline__ void gsync(const Group& g) {
+  if (g.size == 1) {
+    __syncthreads();
+  } else {
+    cooperative_groups::this_cluster().sync();
+  }
+}
 
 enum : uint32_t { P_UNDEC = 0, P_PRUNED = 1, P_KEPT = 2, P_NOTCAND = 3 };
 constexpr uint32_t kFull = 0xFFFFFFFFu;
@@ -21,14 +49,17 @@ __device__ __forceinline__ char* carve(char*& p, uint64_t bytes) {
 }
 
 // Exclusive prefix sum of in[0, n) into out[0, n]; out[n] = total.  in and
-// out may be the same array.
+// out may be the same array.  Four elements per thread and round.
 __device__ inline void cta_scan_u32(const uint32_t* in, uint32_t* out, uint64_t n, uint32_t* wtot) {
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint32_t carry = 0;
-  for (uint64_t base = 0; base < n; base += blockDim.x) {
-    const uint64_t i = base + threadIdx.x;
-    const uint32_t v = i < n ? in[i] : 0u;
-    uint32_t x = v;
+  for (uint64_t base = 0; base < n; base += 4 * blockDim.x) {
+    const uint64_t i = base + 4 * threadIdx.x;
+    uint32_t v[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) v[u] = i + u < n ? in[i + u] : 0u;
+    const uint32_t sum = v[0] + v[1] + v[2] + v[3];
+    uint32_t x = sum;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, x, d);
@@ -46,11 +77,14 @@ __device__ inline void cta_scan_u32(const uint32_t* in, uint32_t* out, uint64_t 
       wtot[lane] = w;
     }
     __syncthreads();
-    const uint32_t before = warp ? wtot[warp - 1] : 0u;
-    if (i < n) out[i] = carry + before + x - v;
-    const uint32_t tot = wtot[nw - 1];
+    uint32_t o = carry + (warp ? wtot[warp - 1] : 0u) + x - sum;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      if (i + u < n) out[i + u] = o;
+      o += v[u];
+    }
+    carry += wtot[nw - 1];
     __syncthreads();
-    carry += tot;
   }
   if (threadIdx.x == 0) out[n] = carry;
   __syncthreads();
@@ -67,6 +101,9 @@ __device__ inline void cta_scan_u32(const uint32_t* in, uint32_t* out, uint64_t 
 // right targets it, resolved by frontier rounds (then right to left for what
 // the round bound leaves).
 // ---------------------------------------------------------------------------
+// Shared-memory words of one CTA's scans.
+constexpr uint32_t kScanWords = 32;
+
 struct PrW {
   uint8_t *hit_v, *hit2, *tgt_w, *gone, *mk2;
   uint32_t *state, *indeg, *fq0, *fq1, *nidx, *wpop, *ptr2;
@@ -111,16 +148,16 @@ __device__ __forceinline__ uint64_t plen(const PLv& v, uint64_t k) {
   return v.n - s < v.b ? v.n - s : v.b;
 }
 
-// Shared state of a CTA that prunes.
+// Shared state of a group that prunes (a CTA's in shared memory, a cluster's
+// in global memory).
 struct PruneShared {
   unsigned int wl[3];  // lengths of the rounds' worklists
   unsigned long long undecided;
-  uint32_t wtot[32];
   int err;
 };
 
-__device__ inline void flag_targets(const PLv& v, uint8_t* flag) {
-  for (uint64_t u = threadIdx.x; u < v.c; u += blockDim.x) {
+__device__ inline void flag_targets(const PLv& v, uint8_t* flag, const Group& G) {
+  for (uint64_t u = G.tid(); u < v.c; u += G.threads()) {
     if (marked(v.mw, u)) continue;
     const uint64_t j = v.ptr[u];
     flag[j] = 1;
@@ -132,9 +169,15 @@ __device__ inline void flag_targets(const PLv& v, uint8_t* flag) {
 // device check failed).  v's marks, ranks, pointers and offsets are updated, w
 // is compacted in place.
 __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, uint32_t arity, char* temp,
-                                       uint64_t max_rounds, PruneShared& Z) {
-  const unsigned tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, nw = nt >> 5;
-  if (tid == 0) Z.err = 0;
+                                       uint64_t max_rounds, PruneShared& Z, uint32_t* wtot, const Group& G) {
+  const unsigned tid = G.tid(), nt = G.threads(), lane = tid & 31, nw = nt >> 5;
+  // A check that failed anywhere: everyone's to know before anyone goes on.
+  auto failed = [&]() {
+    gsync(G);
+    const int e = *(volatile int*)&Z.err;
+    gsync(G);
+    return e != 0;
+  };
   const PrW R = carve_prune(temp, v.c, w.c);
   for (uint64_t i = tid; i <= v.c; i += nt) {
     R.hit_v[i] = 0;
@@ -148,11 +191,12 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
   if (tid == 0) {
     Z.wl[0] = Z.wl[1] = Z.wl[2] = 0;
     Z.undecided = 0;
+    Z.err = 0;
   }
-  __syncthreads();
-  flag_targets(v, R.hit_v);
-  flag_targets(w, R.tgt_w);
-  __syncthreads();
+  gsync(G);
+  flag_targets(v, R.hit_v, G);
+  flag_targets(w, R.tgt_w, G);
+  gsync(G);
   // Candidates and their target blocks.
   for (uint64_t k = tid; k < v.c; k += nt) {
     R.state[k] = P_NOTCAND;
@@ -182,29 +226,29 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
     R.t2[k] = (lo + len > v.st[j] + plen(v, j)) ? j + 1 : kNone;
     R.state[k] = P_UNDEC;
   }
-  if (__syncthreads_or(Z.err)) return kNone;
+  if (failed()) return kNone;
   for (uint64_t k = tid; k < v.c; k += nt) {
     if (R.state[k] != P_UNDEC) continue;
     if (R.state[R.t1[k]] != P_NOTCAND) atomicAdd(&R.indeg[R.t1[k]], 1u);
     if (R.t2[k] != kNone && R.state[R.t2[k]] != P_NOTCAND) atomicAdd(&R.indeg[R.t2[k]], 1u);
   }
-  __syncthreads();
+  gsync(G);
   // Round 0: candidates nothing targets are pruned.
   for (uint64_t k = tid; k < v.c; k += nt)
     if (R.state[k] == P_UNDEC && R.indeg[k] == 0) {
       R.state[k] = P_PRUNED;
       R.fq0[atomicAdd(&Z.wl[0], 1u)] = (uint32_t)k;
     }
-  __syncthreads();
+  gsync(G);
   // Rounds: the candidates decided in the previous round inform their
   // targets (a pruned attacker keeps its target; the last kept attacker of
   // a target prunes it).
   uint64_t r = 1;
   for (; r < max_rounds; r++) {
-    const uint32_t m = Z.wl[(r - 1) % 3];
+    const uint32_t m = *(volatile uint32_t*)&Z.wl[(r - 1) % 3];
     if (m == 0) break;
     if (tid == 0) Z.wl[r % 3] = 0;
-    __syncthreads();
+    gsync(G);
     const uint32_t* qin = (r - 1) & 1 ? R.fq1 : R.fq0;
     uint32_t* qout = r & 1 ? R.fq1 : R.fq0;
     for (uint32_t i = tid; i < m; i += nt) {
@@ -220,13 +264,13 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
           qout[atomicAdd(&Z.wl[r % 3], 1u)] = (uint32_t)t;
       }
     }
-    __syncthreads();
+    gsync(G);
   }
   // Right-to-left finish of the candidates the round bound left undecided.
   for (uint64_t k = tid; k < v.c; k += nt)
     if (R.state[k] == P_UNDEC) atomicAdd(&Z.undecided, 1ull);
-  __syncthreads();
-  if (Z.undecided && tid == 0) {
+  gsync(G);
+  if (tid == 0 && Z.undecided) {
     for (uint64_t k = v.c; k-- > 0;) {
       uint32_t s = R.state[k];
       if (s == P_UNDEC) {
@@ -239,7 +283,7 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
       }
     }
   }
-  __syncthreads();
+  gsync(G);
   // Apply: pruned blocks lose their children and become pointers.
   for (uint64_t k = tid; k < v.c; k += nt) {
     if (R.state[k] != P_PRUNED) continue;
@@ -248,7 +292,7 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
     v.ptr[k] = (uint32_t)R.t1[k];
     v.off[k] = v.lo[k] - v.st[R.t1[k]];
   }
-  __syncthreads();
+  gsync(G);
   const uint64_t words = (v.c + 31) / 32;
   for (uint64_t wb = tid >> 5; wb < words; wb += nw) {
     const uint64_t k = wb * 32 + lane;
@@ -258,12 +302,13 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
     __syncwarp();
     if (lane == 0) v.mw[wb] = bits;
   }
-  __syncthreads();
-  cta_scan_u32(R.wpop, v.mr, words, Z.wtot);
+  gsync(G);
+  if (G.rank == 0) cta_scan_u32(R.wpop, v.mr, words, wtot);
   // Compact level l+1 without the deleted children.
   for (uint64_t k = tid; k < w.c; k += nt) R.nidx[k] = R.gone[k] ? 0u : 1u;
-  __syncthreads();
-  cta_scan_u32(R.nidx, R.nidx, w.c, Z.wtot);
+  gsync(G);
+  if (G.rank == 0) cta_scan_u32(R.nidx, R.nidx, w.c, wtot);
+  if (G.size > 1) gsync(G);
   for (uint64_t k = tid; k < w.c; k += nt) {
     if (R.gone[k]) continue;
     const uint64_t i = R.nidx[k];
@@ -280,7 +325,7 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
       R.ptr2[i] = R.nidx[j];
     }
   }
-  if (__syncthreads_or(Z.err)) return kNone;
+  if (failed()) return kNone;
   const uint64_t c2 = R.nidx[w.c];
   const uint64_t words2 = (c2 + 31) / 32;
   for (uint64_t i = tid; i < c2; i += nt) {
@@ -297,8 +342,9 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
       R.wpop[wb] = __popc(bits);
     }
   }
-  __syncthreads();
-  cta_scan_u32(R.wpop, w.mr, words2, Z.wtot);
+  gsync(G);
+  if (G.rank == 0) cta_scan_u32(R.wpop, w.mr, words2, wtot);
+  if (G.size > 1) gsync(G);
   return c2;
 }
 

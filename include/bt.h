@@ -262,7 +262,7 @@ int bt_prefix_fingerprints(const uint8_t* d_text, uint64_t n, uint64_t seed, uin
  *
  * Same arguments, results and stream semantics as bt_prefix_fingerprints.
  * The caller still provides d_text and d_out.  The scratch (per-tile
- * totals) is a fixed 512 KiB array in device memory, which every GPU that
+ * totals) is a fixed 256 KiB array in device memory, which every GPU that
  * loads the library holds until the process exits.  The entry point
  * calls no cudaMalloc, cudaFree or allocating library routine.
  *  - n may be at most 2^31 (2 GiB); larger texts return BT_ERANGE before any

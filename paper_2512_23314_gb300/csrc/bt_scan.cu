@@ -14,6 +14,7 @@
 //    only its squares.  Tile totals, a single-CTA scan of them, then a pass
 //    that computes every chunk's prefix from its tile's.
 #include <cstdio>
+#include <algorithm>
 #include <mutex>
 
 #include "bt_internal.cuh"
@@ -109,59 +110,93 @@ int scan_sum(const T* in, T* out, uint64_t n, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // Karp-Rabin all-prefix.
 //
-// Bound: the text once per pass (twice in all) and n/4 bytes written.  A
-// Horner step is a 61-bit product (about 20 instructions) per byte; instead a
-// 32-byte chunk is the dot product of its bytes with the powers B^31 .. B^0,
-// whose eight 8-bit limbs are constants: two 4-way byte products (__dp4a)
-// per byte and one reduction per chunk.  A thread takes four chunks, so that
-// the scan's products (about eight per thread) are shared by 128 bytes.  The
-// CTA totals come from a pass of their own and the text is read again: the
-// pass that writes then writes final values, instead of local ones that a
-// third pass reads, corrects and writes once more.  The second pass takes
-// the tiles from the last to the first, so that it starts with the text the
-// first pass left in L2.
-// Measured on 256 MiB + 77, the whole call: 548 us with a Horner pass that
-// wrote local values (454), their totals (33) and a correcting pass (32); 169
-// us now.
+// Bound: the text read and n/4 bytes written once (60 us on 256 MiB); in fact
+// the issue of the first pass's integer instructions.  A Horner step is a 61-bit
+// product (about 20 instructions) per byte; instead a 32-byte chunk is the dot
+// product of its bytes with the powers B^31 .. B^0, whose eight 8-bit limbs are
+// constants: two 4-way byte products (__dp4a) per byte and one reduction per
+// chunk.  A thread takes eight chunks, so that the scan's products (about seven
+// per thread) are shared by 256 bytes, and leaves values local to its chunks,
+// which the last pass moves along by one product each: it reads and writes the
+// n/4 bytes once more, mostly in the L2, where a second pass over the text for
+// final values took twice the first one's instructions.
+// Measured on 256 MiB + 77, the whole call: 548 us with a Horner pass, 169 with
+// dot products in two passes over the text, 110 now
+// (68, 9 and 27).
 // ---------------------------------------------------------------------------
-constexpr int kKrThreads = 256;    // threads of a tile of kTile chunks
-constexpr int kKrChunks = 4;       // chunks per thread
-static_assert(kKrThreads * kKrChunks == kTile, "a tile is kTile chunks");
+constexpr int kKrThreads = 256;    // threads of a tile
+constexpr int kKrChunks = 8;       // chunks per thread
+constexpr int kKrTile = kKrThreads * kKrChunks;
 
-// agg[i] = fingerprint of tile i (kTile chunks); the last tile is not needed.
-// pw: the shift of a thread's four chunks, P = B^32 the shift of one.
+// X^(lane + 1) for a thread's shift X, by lane.
+struct KrLane {
+  uint64_t x[32];
+};
+
+// First pass, a tile of kKrTile chunks per CTA, kKrChunks per thread: of a
+// thread's chunks j0 .. the fingerprint of the tile's chunks before j0 goes to
+// Hs[j0], that of chunks j0 .. j - 1 to Hs[j] (j <= nchunks), and every tile's but the
+// last to agg.
 template <class M>
-__global__ void __launch_bounds__(kKrThreads) k_kr_totals(M m, const uint8_t* __restrict__ T, uint64_t nchunks,
-                                                          const ChunkHash<M> hash, uint64_t P, KrPow pw,
-                                                          uint64_t* __restrict__ agg) {
+__global__ void __launch_bounds__(kKrThreads) k_kr_local(M m, const uint8_t* __restrict__ T, uint64_t nchunks,
+                                                         const __grid_constant__ ChunkHash<M> hash, uint64_t P,
+                                                         const __grid_constant__ KrPow pw,
+                                                         const __grid_constant__ KrLane xl, uint64_t* __restrict__ agg,
+                                                         uint64_t* __restrict__ Hs) {
   __shared__ uint64_t sm[kKrThreads / 32];
+  __shared__ uint64_t val[kKrTile + kKrTile / kKrChunks];  // (one word more per thread: no bank conflicts)
   const bool aligned = (((uintptr_t)T) & 15) == 0;
-  const uint64_t j0 = (uint64_t)blockIdx.x * kTile + (uint64_t)threadIdx.x * kKrChunks;
-  uint32_t w[kKrChunks][8];
-#pragma unroll
-  for (int i = 0; i < kKrChunks; i++) load_chunk(T, nchunks, j0 + i, aligned, w[i]);
-  uint64_t h = hash(m, w[0]);
-#pragma unroll
-  for (int i = 1; i < kKrChunks; i++) h = m.add(m.mul(h, P), hash(m, w[i]));
-  // Ordered tree over the warp, then over the warps.
+  const uint64_t tile0 = (uint64_t)blockIdx.x * kKrTile;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // Chunks in the order of the threads (coalesced), then each thread its own.
 #pragma unroll
-  for (int i = 0; i < 5; i++) h = m.add(m.mul(h, pw.x[i]), __shfl_down_sync(0xFFFFFFFFu, h, 1 << i));
-  if (lane == 0) sm[warp] = h;
+  for (int q = 0; q < kKrChunks; q += 4) {
+    uint32_t w[4][8];
+#pragma unroll
+    for (int i = 0; i < 4; i++) load_chunk(T, nchunks, tile0 + (q + i) * kKrThreads + threadIdx.x, aligned, w[i]);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const uint32_t at = (q + i) * kKrThreads + threadIdx.x;
+      val[at + at / kKrChunks] = hash(m, w[i]);
+    }
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    h = sm[0];
+  uint64_t* mine = val + threadIdx.x * (kKrChunks + 1);
+  uint64_t o[kKrChunks], h = mine[0];
 #pragma unroll
-    for (int i = 1; i < kKrThreads / 32; i++) h = m.add(m.mul(h, pw.w[0]), sm[i]);
-    agg[blockIdx.x] = h;
+  for (int i = 1; i < kKrChunks; i++) {
+    o[i] = h;
+    h = m.add(m.mul(h, P), mine[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < 5; i++) {
+    const uint64_t u = __shfl_up_sync(0xFFFFFFFFu, h, 1 << i);
+    if (lane >= (1 << i)) h = m.add(m.mul(u, pw.x[i]), h);
+  }
+  if (lane == 31) sm[warp] = h;
+  __syncthreads();
+  uint64_t before = 0;  // the warps before this one
+  for (int k = 0; k < warp; k++) before = k ? m.add(m.mul(before, pw.w[0]), sm[k]) : sm[0];
+  const uint64_t up = __shfl_up_sync(0xFFFFFFFFu, h, 1);
+  if (threadIdx.x == kKrThreads - 1 && blockIdx.x + 1 < gridDim.x) agg[blockIdx.x] = m.add(m.mul(before, pw.w[0]), h);
+  mine[0] = lane ? m.add(m.mul(before, xl.x[lane - 1]), up) : before;
+#pragma unroll
+  for (int i = 1; i < kKrChunks; i++) mine[i] = o[i];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kKrChunks; i++) {
+    const uint32_t at = i * kKrThreads + threadIdx.x;
+    if (tile0 + at <= nchunks) Hs[tile0 + at] = val[at + at / kKrChunks];
   }
 }
 
 // agg[i] = fingerprint of tiles 0 .. i, by one CTA: a thread folds `per`
 // consecutive tiles (all loads first, eight at a time), then the threads are
 // scanned.  Y: the shift of a tile; pw: the shift of a thread's tiles.
+constexpr int kAggThreads = 512;
+
 template <class M>
-__global__ void __launch_bounds__(kTile) k_kr_aggs(M m, uint64_t* __restrict__ agg, uint64_t na, uint64_t per,
+__global__ void __launch_bounds__(kAggThreads) k_kr_aggs(M m, uint64_t* __restrict__ agg, uint64_t na, uint64_t per,
                                                    uint64_t Y, KrPow pw) {
   __shared__ uint64_t sm[32];
   const uint64_t i0 = threadIdx.x * per;
@@ -179,71 +214,86 @@ __global__ void __launch_bounds__(kTile) k_kr_aggs(M m, uint64_t* __restrict__ a
   if ((threadIdx.x & 31) == 31) sm[threadIdx.x >> 5] = incl;
   __syncthreads();
   if ((threadIdx.x & 31) == 0) up = threadIdx.x ? sm[(threadIdx.x >> 5) - 1] : 0;
-  for (uint64_t i = 0; i < per && i0 + i < na; i++) {
-    up = m.add(m.mul(up, Y), agg[i0 + i]);
-    agg[i0 + i] = up;
+  for (uint64_t i = 0; i < per; i += 8) {
+    uint64_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) v[u] = i + u < per && i0 + i + u < na ? agg[i0 + i + u] : 0;
+#pragma unroll
+    for (int u = 0; u < 8; u++)
+      if (i + u < per && i0 + i + u < na) {
+        up = m.add(m.mul(up, Y), v[u]);
+        agg[i0 + i + u] = up;
+      }
   }
 }
 
-// Hs[j] = H(32 j) for j <= nchunks: every thread's four chunks again, scanned
-// over the tile with the tile's prefix as the first item's carry-in.
+// Last pass: with c = the text before a thread's chunks (the tiles before, the
+// tile's chunks before them), Hs[j0] = c and Hs[j] = c P^(j - j0) + Hs[j].  The last
+// tiles first: what the first pass wrote last is in the L2.  pw: the shift of a
+// thread's chunks.
+struct KrShift {
+  uint64_t p[kKrChunks];  // P^i
+};
+constexpr int kShiftThreads = 256, kShiftPairs = kKrTile / 2 / kShiftThreads;  // pairs of values per thread
 template <class M>
-__global__ void __launch_bounds__(kKrThreads) k_kr_write(M m, const uint8_t* __restrict__ T, uint64_t nchunks,
-                                                         const ChunkHash<M> hash, uint64_t P, KrPow pw,
-                                                         const uint64_t* __restrict__ agg, uint64_t* __restrict__ Hs) {
-  __shared__ uint64_t sm[32];
-  const bool aligned = (((uintptr_t)T) & 15) == 0;
-  const uint64_t tile = gridDim.x - 1 - blockIdx.x;
-  const uint64_t j0 = tile * kTile + (uint64_t)threadIdx.x * kKrChunks;
-  uint64_t c[kKrChunks];
-  {
-    uint32_t w[kKrChunks][8];
+__global__ void __launch_bounds__(kShiftThreads) k_kr_shift(M m, uint64_t nchunks, uint64_t tiles,
+                                                            const __grid_constant__ KrShift S,
+                                                            const __grid_constant__ KrPow pw,
+                                                            const uint64_t* __restrict__ agg, uint64_t* __restrict__ Hs) {
+  constexpr int kPer = kKrChunks / 2;  // threads that hold a first-pass thread's values
+  const unsigned t = threadIdx.x, r = 2 * (t % kPer);
+  uint64_t x[kShiftPairs] = {1};  // the shift of the tile's chunks before the values' first-pass thread
 #pragma unroll
-    for (int i = 0; i < kKrChunks; i++) load_chunk(T, nchunks, j0 + i, aligned, w[i]);
+  for (int i = 0; i < 6; i++)
+    if ((t / kPer >> i) & 1u) x[0] = m.mul(x[0], i < 5 ? pw.x[i] : pw.w[0]);
 #pragma unroll
-    for (int i = 0; i < kKrChunks; i++) c[i] = hash(m, w[i]);
-  }
-  uint64_t h = c[0];
+  for (int u = 1; u < kShiftPairs; u++) x[u] = m.mul(x[u - 1], pw.w[1]);
+  const uint64_t p0 = S.p[r], p1 = S.p[r + 1];
+  const bool aligned = (((uintptr_t)Hs) & 15) == 0;
+  for (uint64_t tile = tiles - 1 - blockIdx.x; tile < tiles; tile -= gridDim.x) {
+    const uint64_t carry = tile ? agg[tile - 1] : 0;
+    ulonglong2 v[kShiftPairs];
 #pragma unroll
-  for (int i = 1; i < kKrChunks; i++) h = m.add(m.mul(h, P), c[i]);
-  const uint64_t carry = threadIdx.x == 0 && tile ? agg[tile - 1] : 0;
-  if (threadIdx.x == 0) h = m.add(m.mul(carry, pw.x[0]), h);
-  const uint64_t incl = cta_kr_scan(m, h, pw, kr_lane_pow(m, pw), sm);
-  uint64_t up = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
-  if ((threadIdx.x & 31) == 31) sm[threadIdx.x >> 5] = incl;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) up = threadIdx.x ? sm[(threadIdx.x >> 5) - 1] : carry;
-  // up = H(32 j0); the four values are one aligned 32-byte sector.
-  uint64_t o[kKrChunks];
+    for (int u = 0; u < kShiftPairs; u++) {
+      const uint64_t j = tile * kKrTile + 2 * (t + u * kShiftThreads);
+      if (aligned && j + 1 <= nchunks) v[u] = *(const ulonglong2*)(Hs + j);
+      else v[u] = make_ulonglong2(j <= nchunks ? Hs[j] : 0, j + 1 <= nchunks ? Hs[j + 1] : 0);
+    }
 #pragma unroll
-  for (int i = 0; i < kKrChunks; i++) {
-    o[i] = up;
-    up = m.add(m.mul(up, P), c[i]);
-  }
-  if (j0 + kKrChunks - 1 <= nchunks && (((uintptr_t)Hs) & 15) == 0) {
-    ((ulonglong2*)(Hs + j0))[0] = make_ulonglong2(o[0], o[1]);
-    ((ulonglong2*)(Hs + j0))[1] = make_ulonglong2(o[2], o[3]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < kKrChunks; i++)
-      if (j0 + i <= nchunks) Hs[j0 + i] = o[i];
+    for (int u = 0; u < kShiftPairs; u++) {
+      const uint64_t j = tile * kKrTile + 2 * (t + u * kShiftThreads);
+      const uint64_t c = m.add(m.mul(carry, x[u]), __shfl_sync(0xFFFFFFFFu, v[u].x, (t & 31) & ~(kPer - 1)));
+      const uint64_t a = r ? m.add(m.mul(c, p0), v[u].x) : c, b = m.add(m.mul(c, p1), v[u].y);
+      if (aligned && j + 1 <= nchunks) {
+        *(ulonglong2*)(Hs + j) = make_ulonglong2(a, b);
+      } else {
+        if (j <= nchunks) Hs[j] = a;
+        if (j + 1 <= nchunks) Hs[j + 1] = b;
+      }
+    }
   }
 }
+static_assert(kShiftThreads / (kKrChunks / 2) == 64, "a round of pairs is those of 64 first-pass threads");
 
-// The three launches; agg holds nchunks / kTile entries.
+// The three launches; agg holds nchunks / kKrTile entries.
 template <class M>
 int kr_launch(const M& m, const uint8_t* T, uint64_t n, uint64_t B, uint64_t* Hs, uint64_t* agg, cudaStream_t s) {
   const uint64_t nchunks = n / kPrefixStride;
-  const uint64_t tiles = nchunks / kTile + 1, na = tiles - 1;  // the last tile writes Hs[nchunks]
+  const uint64_t tiles = nchunks / kKrTile + 1, na = tiles - 1;  // the last tile writes Hs[nchunks]
   const uint64_t P = pow_mod(m, B, kPrefixStride);
-  const KrPow pw = kr_pow(m, pow_mod(m, P, kKrChunks));
+  const uint64_t X = pow_mod(m, P, kKrChunks);
+  const KrPow pw = kr_pow(m, X);
   const ChunkHash<M> hash(m, B);
+  KrLane xl;
+  KrShift S;
+  for (int i = 0; i < 32; i++) xl.x[i] = i ? m.mul(xl.x[i - 1], X) : X;
+  for (int i = 0; i < kKrChunks; i++) S.p[i] = i ? m.mul(S.p[i - 1], P) : 1;
+  BT_LAUNCH(k_kr_local<M><<<(unsigned)tiles, kKrThreads, 0, s>>>(m, T, nchunks, hash, P, pw, xl, agg, Hs));
   if (na) {
-    BT_LAUNCH(k_kr_totals<M><<<(unsigned)na, kKrThreads, 0, s>>>(m, T, nchunks, hash, P, pw, agg));
-    const uint64_t per = (na + kTile - 1) / kTile, Y = pow_mod(m, P, kTile);
-    BT_LAUNCH(k_kr_aggs<M><<<1, kTile, 0, s>>>(m, agg, na, per, Y, kr_pow(m, pow_mod(m, Y, per))));
+    const uint64_t per = (na + kAggThreads - 1) / kAggThreads, Y = pow_mod(m, P, kKrTile);
+    BT_LAUNCH(k_kr_aggs<M><<<1, kAggThreads, 0, s>>>(m, agg, na, per, Y, kr_pow(m, pow_mod(m, Y, per))));
   }
-  BT_LAUNCH(k_kr_write<M><<<(unsigned)tiles, kKrThreads, 0, s>>>(m, T, nchunks, hash, P, pw, agg, Hs));
+  BT_LAUNCH(k_kr_shift<M><<<(unsigned)std::min<uint64_t>(tiles, 152 * 8), kShiftThreads, 0, s>>>(m, nchunks, tiles, S, pw, agg, Hs));
   BT_CUDA(cudaGetLastError());
   return BT_OK;
 }
@@ -257,7 +307,7 @@ int kr_prefix(const M& m, const uint8_t* T, uint64_t n, uint64_t B, uint64_t* Hs
   }
   Scratch sc(s);
   uint64_t* agg = nullptr;
-  if (nchunks >= kTile) BT_TRY(sc.alloc(&agg, nchunks / kTile));
+  if (nchunks >= kKrTile) BT_TRY(sc.alloc(&agg, nchunks / kKrTile));
   ProfScope ps("prefix_fingerprint", s, n);
   return kr_launch(m, T, n, B, Hs, agg, s);
 }
@@ -364,11 +414,11 @@ int expand_prefix(const uint8_t* T, uint64_t n, uint64_t B, uint64_t q, const ui
 namespace {
 
 constexpr uint64_t kNoAllocMaxN = 1ull << 31;  // largest text accepted (2 GiB)
-constexpr uint64_t kNoAllocAggs = (kNoAllocMaxN / kPrefixStride + kTile - 1) / kTile;
-constexpr uint64_t kNoAllocWords = kNoAllocAggs;  // 65536 u64, 512 KiB
+constexpr uint64_t kNoAllocAggs = (kNoAllocMaxN / kPrefixStride + kKrTile - 1) / kKrTile;
+constexpr uint64_t kNoAllocWords = kNoAllocAggs;  // 32768 u64, 256 KiB
 constexpr int kNoAllocDevices = 64;
 // The array holds exactly the tile totals of the largest text.
-static_assert(kNoAllocAggs == 65536, "one aggregate per 1024 chunks of 32 bytes of a 2 GiB text");
+static_assert(kNoAllocAggs == 32768, "one aggregate per 2048 chunks of 32 bytes of a 2 GiB text");
 
 static __device__ __align__(256) uint64_t g_noalloc_scratch[kNoAllocWords];
 

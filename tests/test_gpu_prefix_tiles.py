@@ -27,3 +27,25 @@ def test_every_prefix(n, shift, q, noalloc):
         if i % 32 == 0:
             want.append(h)
     assert out.cpu().numpy().tolist() == want
+
+
+@pytest.mark.parametrize("n", [2 * TILE - 33, 2 * TILE - 1, 2 * TILE, 2 * TILE + 32, 6 * TILE + 31, 8 * TILE, 2 * TILE * 511 + 5,
+                               2 * TILE * 513, 2 * TILE * 8200 + 77])
+@pytest.mark.parametrize("q", [0, 331])
+def test_steps_of_large_tiles(n, q):
+    """Tiles of 2048 chunks, up to more of them than the threads that add them up: each value from the one before, at
+    every edge of a tile and of a thread's chunks nearby and at random."""
+    text = workloads.random_bytes(n, 256, n % 1000)
+    out = torch.full((n // 32 + 2,), -1, dtype=torch.int64, device="cuda")
+    bt.bt_prefix_fingerprints(torch.from_numpy(text).cuda(), n, 7, q, 32, out[1:])  # (an odd place)
+    h, B, Q = out.cpu().numpy()[1:], oracle.base(7, q), q or (1 << 61) - 1
+    last = n // 32
+    js = np.random.default_rng(n).integers(0, last, 500).tolist()
+    js += [t + d for t in range(0, last, 2048) for d in (-2, -1, 0, 7, 8)][-4000:] + [last - 1]
+    assert h[0] == 0
+    for j in js:
+        if 0 <= j < last:
+            x = int(h[j])
+            for c in text[32 * j:32 * j + 32].tolist():
+                x = (x * B + c + 1) % Q
+            assert x == h[j + 1], j

@@ -972,16 +972,23 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
     uint32_t* cq = (uint32_t*)((uint2*)dyn + nwarps * kHitQ) + warp * kCandQ;
     uint32_t* bits_s = (uint32_t*)((uint2*)dyn + nwarps * kHitQ) + nwarps * kCandQ;
     const bool fits = bwords <= kCtaBitWords;
-    if (fits)
-      for (uint32_t i = threadIdx.x; i < bwords; i += blockDim.x) bits_s[i] = K.bitmap[i];
-    __syncthreads();
+    auto fetch = [&]() {
+      if (fits)
+        for (uint32_t i = threadIdx.x; i < bwords; i += blockDim.x) bits_s[i] = K.bitmap[i];
+      __syncthreads();
+    };
+    fetch();
     const uint32_t* bits = fits ? bits_s : K.bitmap;
     const uint32_t total = C.nsel, split = total > (1u << 16) ? (total / 16) & ~(8 * kChaseTile - 1) : 0;
     if (split) {
       chase_scan(m, H, K, 0, split, bits, hq, cq, nullptr, w);
       gsync(C.grp);
       chase_bound(K, w);
+      for (uint32_t i = tid; i < bwords; i += nt) K.bitmap[i] = 0;
       gsync(C.grp);
+      chase_live(K, split, w);
+      gsync(C.grp);
+      fetch();
     }
     chase_scan(m, H, K, split, total, bits, hq, cq, split ? K.bound2 : nullptr, w);
     if (C.r && C.r < kQuickMinB) chase_tail(K, w);

@@ -237,6 +237,8 @@ __global__ void __launch_bounds__(kT, 4) k_chase_scan(M m, const __grid_constant
 
 __global__ void __launch_bounds__(kT) k_chase_bound(Chase C) { chase_bound(C, grid_span()); }
 
+__global__ void __launch_bounds__(kT) k_chase_live(Chase C, uint32_t split) { chase_live(C, split, grid_span()); }
+
 __global__ void __launch_bounds__(kT) k_chase_tail(Chase C) { chase_tail(C, grid_span()); }
 
 __global__ void __launch_bounds__(kT) k_chase_verify(Chase C, uint64_t ppk, unsigned L) { chase_verify(C, ppk, L, grid_span()); }
@@ -628,6 +630,8 @@ static int chase(const M& m, BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint6
     if (split) {
       BT_LAUNCH(k_chase_scan<M><<<grid(split), kT, sw * 4, s>>>(m, P, ctx.Hs, C, 0, split, sw, nullptr));
       BT_LAUNCH(k_chase_bound<<<grid_for(ni, kT), kT, 0, s>>>(C));
+      BT_CUDA(cudaMemsetAsync(C.bitmap, 0, bwords * 4, s));
+      BT_LAUNCH(k_chase_live<<<grid_for(gcap, kT), kT, 0, s>>>(C, split));
     }
     if (total)
       BT_LAUNCH(k_chase_scan<M><<<grid(total - split), kT, sw * 4, s>>>(m, P, ctx.Hs, C, split, total, sw,

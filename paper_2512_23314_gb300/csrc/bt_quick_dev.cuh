@@ -644,6 +644,22 @@ __device__ __forceinline__ void chase_bound(const Chase& C, Span w) {
   }
 }
 
+// After chase_bound, into a cleared bitmap: the grams that entries from `split` on
+// can still propose a window for.  The copies' content is settled by then, and
+// its grams, most of the list's hits, are left out.
+__device__ __forceinline__ void chase_live(const Chase& C, uint32_t split, Span w) {
+  const uint32_t xs = C.Q.x[split];
+  auto set = [&](uint32_t F) {
+    const uint32_t bit = c_bit(C, F), one = 1u << (bit & 31);
+    if (!(*(volatile uint32_t*)&C.bitmap[bit >> 5] & one)) atomicOr(&C.bitmap[bit >> 5], one);
+  };
+  for (uint64_t i = w.tid; i <= C.gmask; i += w.n) {
+    const unsigned long long key = C.gt[i].key;
+    if (key != kNone && C.bound2[i] + (uint32_t)key > xs) set((uint32_t)(key >> 32));
+  }
+  if (w.tid == 0 && C.qs->tail_F != 0xFFFFFFFFu) set(C.qs->tail_F);
+}
+
 // The short last block when it has no selected gram (at most 26 bytes): every
 // position before it, 16 per thread, filtered by its first bytes.
 __device__ __forceinline__ void chase_tail(const Chase& C, Span w) {

@@ -550,42 +550,47 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
     cn -= n;
     __syncwarp();
   };
-  // 32 gram hits (fewer at the end): every offset of the gram proposes.
-  auto take_hits = [&]() {
-    const uint32_t n = hn < 32 ? hn : 32;
+  // One step of the lanes' walks: a lane whose walk has ended takes the next
+  // gram hit, every lane looks at one slot of the table, and a slot that holds
+  // its gram proposes a window.  (Walks end: half the slots are empty.)
+  bool live = false;
+  uint2 hit = make_uint2(0, 0);
+  uint32_t s = 0;
+  auto walk = [&]() {
     __syncwarp();
-    const bool mine = lane < n;
-    const uint2 h = mine ? hq[hn - n + lane] : make_uint2(0, 0);
-    hn -= n;
-    if (mine && h.y == tail_F && tail_off <= h.x) {
-      const uint64_t p = h.x - tail_off;
-      if (p + C.r < C.g.n && p < *(volatile unsigned long long*)&C.qs->lo_tail &&
-          m.sub(H.at(m, p + C.r), m.mul(H.at(m, p), C.Br)) == fp_tail)
-        c_min(&C.qs->lo_tail, p);
+    const unsigned idle = __ballot_sync(0xFFFFFFFFu, !live);
+    const uint32_t k = __popc(idle & lt), free = __popc(idle);
+    if (!live && k < hn) {
+      hit = hq[hn - 1 - k];
+      s = c_gram_home(hit.y, C.gmask);
+      live = true;
+      if (hit.y == tail_F && tail_off <= hit.x) {
+        const uint64_t p = hit.x - tail_off;
+        if (p + C.r < C.g.n && p < *(volatile unsigned long long*)&C.qs->lo_tail &&
+            m.sub(H.at(m, p + C.r), m.mul(H.at(m, p), C.Br)) == fp_tail)
+          c_min(&C.qs->lo_tail, p);
+      }
     }
-    bool live = mine;
-    uint32_t s = c_gram_home(h.y, C.gmask);
-    for (uint32_t it = 0; it <= C.gmask && __any_sync(0xFFFFFFFFu, live); it++) {
-      bool want = false;
-      uint32_t p = 0;
-      if (live) {
-        const ulonglong2 en = *(const ulonglong2*)&C.gt[s];
-        if (en.x == kNone) {
-          live = false;
-        } else if ((uint32_t)(en.x >> 32) == h.y) {
-          const uint32_t off = (uint32_t)en.x;
-          p = h.x - off;
-          want = off <= h.x && p < (bound2 ? bound2[s] : en.y);
-        }
-        s = (s + 1) & C.gmask;
+    hn -= free < hn ? free : hn;
+    bool want = false;
+    uint32_t p = 0;
+    if (live) {
+      const ulonglong2 en = *(const ulonglong2*)&C.gt[s];
+      if (en.x == kNone) {
+        live = false;
+      } else if ((uint32_t)(en.x >> 32) == hit.y) {
+        const uint32_t off = (uint32_t)en.x;
+        p = hit.x - off;
+        want = off <= hit.x && p < (bound2 ? bound2[s] : en.y);
       }
-      const unsigned bal = __ballot_sync(0xFFFFFFFFu, want);
-      if (bal) {
-        if (want) cq[cn + __popc(bal & lt)] = p;
-        cn += __popc(bal);
-        if (lane == 0) ncand += __popc(bal);
-        if (cn >= 32) take_cands();
-      }
+      s = (s + 1) & C.gmask;
+    }
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, want);
+    if (bal) {
+      if (want) cq[cn + __popc(bal & lt)] = p;
+      cn += __popc(bal);
+      if (lane == 0) ncand += __popc(bal);
+      if (cn >= 32) take_cands();
     }
   };
   for (uint64_t t0 = e0 + w.tid / 32 * kChaseTile; t0 < e1; t0 += w.n / 32 * kChaseTile) {
@@ -622,9 +627,9 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
       if (ok) hq[hn + __popc(bal & lt)] = make_uint2(x[u], F[u]);
       hn += __popc(bal);
     }
-    while (hn >= 32) take_hits();
+    while (hn >= 32) walk();  // (unfinished walks go on with the next tile's)
   }
-  while (hn) take_hits();
+  while (hn || __any_sync(0xFFFFFFFFu, live)) walk();
   while (cn) take_cands();
   ncand = __reduce_add_sync(0xFFFFFFFFu, ncand);
   nhit = __reduce_add_sync(0xFFFFFFFFu, nhit);

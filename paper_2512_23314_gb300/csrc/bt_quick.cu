@@ -136,13 +136,24 @@ __global__ void __launch_bounds__(kT) k_list_write(const uint8_t* __restrict__ T
   }
 }
 
-// first[cell] = the least position of an entry with that cell (read first:
+// The list's leading part, whose first occurrences are found before the rest:
+// in a repetitive text most later entries meet a cell that has one of those,
+// which is final, so one read of the table settles them.  In one part, DNA 2
+// GiB took 5.0 + 4.9 ms for the two passes; now 0.4 + 5.6 + 0.3.  Lists of up to
+// 2^22 entries stay whole: the third launch costs what the second read does
+// (text 20 MB: 1.63 and 1.66 ms).
+constexpr uint32_t kWholeList = 1u << 22;
+__host__ __device__ inline uint64_t list_split(uint32_t total) {
+  return total > kWholeList ? (total / 16) & ~127ull : total;
+}
+
+// first[cell] = the least position of a leading entry with that cell (read first:
 // after a gram's first copies have been seen nobody writes).  A pass of its
 // own: inside k_list_write, between that kernel's barriers, the same random
 // reads took 400 us of a 256 MiB build instead of 180.
 __global__ void __launch_bounds__(kT) k_list_first(const uint32_t* __restrict__ total_p, const uint32_t* __restrict__ x,
                                                    const uint32_t* __restrict__ cell, uint32_t* first) {
-  const uint64_t total = *total_p;
+  const uint64_t total = list_split(*total_p);
   for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; 4 * i < total; i += (uint64_t)gridDim.x * kT) {
     if (4 * i + 4 <= total) {
       const uint4 X = ((const uint4*)x)[i], C = ((const uint4*)cell)[i];
@@ -158,17 +169,67 @@ __global__ void __launch_bounds__(kT) k_list_first(const uint32_t* __restrict__ 
   }
 }
 
-// D[e] = x[e] - F, in place of the cell.  Four entries per thread: the random
-// reads of the table are in flight together.
+// Distances of the entries whose cell has a position of the leading part; the
+// others lower their cell and are marked in `open` (a bit per entry, from the
+// split on).
 __global__ void __launch_bounds__(kT) k_list_dist(const uint32_t* __restrict__ total_p, const uint32_t* __restrict__ x,
-                                                  uint32_t* __restrict__ D, const uint32_t* __restrict__ first) {
-  const uint64_t total = *total_p;
-  for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; 4 * i < total; i += (uint64_t)gridDim.x * kT) {
+                                                  uint32_t* __restrict__ D, uint32_t* first, uint32_t* __restrict__ open) {
+  const uint64_t total = *total_p, split = list_split((uint32_t)total);
+  const uint32_t xs = split < total ? x[split] : 0xFFFFFFFFu;
+  // Whole warps: eight threads put their bits together.
+  for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; 4 * (i & ~31ull) < total; i += (uint64_t)gridDim.x * kT) {
+    uint32_t bits = 0;
     if (4 * i + 4 <= total) {
-      const uint4 X = ((const uint4*)x)[i], C = ((const uint4*)D)[i];
-      ((uint4*)D)[i] = make_uint4(X.x - first[C.x], X.y - first[C.y], X.z - first[C.z], X.w - first[C.w]);
+      const uint4 X = ((const uint4*)x)[i];
+      uint4 C = ((const uint4*)D)[i];
+      const uint32_t f0 = *(volatile uint32_t*)&first[C.x], f1 = *(volatile uint32_t*)&first[C.y],
+                     f2 = *(volatile uint32_t*)&first[C.z], f3 = *(volatile uint32_t*)&first[C.w];
+      auto one = [&](uint32_t p, uint32_t& c, uint32_t f, uint32_t bit) {
+        if (f < xs) {
+          c = p - f;
+        } else {
+          if (f > p) atomicMin(&first[c], p);
+          bits |= bit;
+        }
+      };
+      one(X.x, C.x, f0, 1);
+      one(X.y, C.y, f1, 2);
+      one(X.z, C.z, f2, 4);
+      one(X.w, C.w, f3, 8);
+      ((uint4*)D)[i] = C;
     } else {
-      for (uint64_t e = 4 * i; e < total; e++) D[e] = x[e] - first[D[e]];
+      for (uint64_t e = 4 * i; e < total; e++) {
+        const uint32_t c = D[e], f = *(volatile uint32_t*)&first[c];
+        if (f < xs) {
+          D[e] = x[e] - f;
+        } else {
+          atomicMin(&first[c], x[e]);
+          bits |= 1u << (e & 3);
+        }
+      }
+    }
+    if (split == total) continue;
+    bits <<= 4 * (threadIdx.x & 7);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) bits |= __shfl_xor_sync(0xFFFFFFFFu, bits, o);
+    if ((threadIdx.x & 7) == 0 && 4 * i < total) open[i / 8] = bits;
+  }
+}
+
+// Distances of the marked entries, a warp per 32.
+__global__ void __launch_bounds__(kT) k_list_rest(const uint32_t* __restrict__ total_p, const uint32_t* __restrict__ x,
+                                                  uint32_t* __restrict__ D, const uint32_t* __restrict__ first,
+                                                  const uint32_t* __restrict__ open) {
+  const uint64_t total = *total_p, split = list_split((uint32_t)total), words = (total + 31) / 32;
+  if (split == total) return;
+  const unsigned lane = threadIdx.x & 31;
+  for (uint64_t w0 = split / 32 + (blockIdx.x * (uint64_t)kT + threadIdx.x) / 32 * 32; w0 < words;
+       w0 += (uint64_t)gridDim.x * kT) {
+    const uint32_t mine = w0 + lane < words ? open[w0 + lane] : 0u;
+    for (unsigned left = __ballot_sync(0xFFFFFFFFu, mine != 0); left; left &= left - 1) {
+      const unsigned src = __ffs(left) - 1;
+      const uint64_t e = 32 * (w0 + src) + lane;
+      if ((__shfl_sync(0xFFFFFFFFu, mine, src) >> lane) & 1u) D[e] = x[e] - first[D[e]];
     }
   }
 }
@@ -556,7 +617,11 @@ int quick_list(BuildCtx& ctx, QuickBuild& qb) {
     BT_LAUNCH(k_list_write<<<(unsigned)std::min<uint64_t>((nw + kT - 1) / kT, 152 * 16), kT, 0, s>>>(
         ctx.T, n, nw, mask, qb.idx, qb.x, qb.D, (uint32_t)(cells - 1)));
   BT_LAUNCH(k_list_first<<<grid_for(cap / 4 + 1, kT, 152 * 16), kT, 0, s>>>(qb.idx + nw, qb.x, qb.D, first));
-  BT_LAUNCH(k_list_dist<<<grid_for(cap / 4 + 1, kT, 152 * 16), kT, 0, s>>>(qb.idx + nw, qb.x, qb.D, first));
+  uint32_t* open = mask;  // (not read any more, and as long: a list has no more entries than grams)
+  const bool parts = cap > kWholeList;
+  BT_LAUNCH(k_list_dist<<<grid_for(cap / 4 + 1, kT, 152 * 16), kT, 0, s>>>(qb.idx + nw, qb.x, qb.D, first, open));
+  if (parts)
+    BT_LAUNCH(k_list_rest<<<grid_for(cap / 32 + 1, kT, 152 * 8), kT, 0, s>>>(qb.idx + nw, qb.x, qb.D, first, open));
   BT_LAUNCH(k_list_seg1<<<grid_for(ns * 32, kT), kT, 0, s>>>(nw, qb.idx, qb.D, ns, qb.seg1));
   BT_LAUNCH(k_list_seg2<<<grid_for(ns2, kT), kT, 0, s>>>(ns, qb.seg1, ns2, qb.seg2));
   BT_CUDA(cudaGetLastError());
@@ -584,7 +649,7 @@ static int chase(const M& m, BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint6
   C.r = len_last < g.b ? len_last : 0;
   C.Bb = pow_mod(m, t->B, g.b);
   C.Br = C.r ? pow_mod(m, t->B, C.r) : 0;
-  const uint64_t bcap = pow2_from(2 * (nb + 2 * np)), pcap = pow2_from(2 * np), gcap = pow2_from(2 * ni);
+  const uint64_t bcap = pow2_from(2 * (nb + 2 * np)), pcap = pow2_from(2 * np), gcap = pow2_from(4 * ni);  // (2 ni: DNA 2 GiB 41.5 ms, not 40.8)
   uint32_t fbits = 12;
   while ((1ull << fbits) < 16 * ni && fbits < 30) fbits++;
   const uint32_t bwords = 1u << (fbits - 5);

@@ -72,3 +72,15 @@ def test_shared_cells_and_repeats():
         text = np.frombuffer(bytes(out), np.uint8).copy()
         check(text, 2, leaf)
         check(text, 4, leaf, prune=False, two_phase=True)
+
+
+@pytest.mark.parametrize("n", [28 << 20, (33 << 20) + 77])
+def test_lists_in_two_parts(n):
+    """More than 2^22 list entries: distances of repeats, of grams that are new after the leading part, of both; the
+    tree is that of the scan of every window."""
+    half = workloads.random_bytes(n // 2, 256, 1)
+    for text in (workloads.random_bytes(n, 256, n % 97), np.concatenate([half, half[::-1], half])[:n],
+                 workloads.dna_genome(n=n, genome_len=n // 3, snp_rate=1e-2, indel_rate=1e-3, seed=2)):
+        d = torch.from_numpy(np.ascontiguousarray(text)).cuda()
+        blob = bt.Tree(d, 256, 4, 64).export()
+        assert blob == bt.Tree(d, 256, 4, 64, bt.BuildOptions(dense_scan=True)).export()

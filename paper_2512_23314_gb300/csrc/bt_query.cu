@@ -27,23 +27,27 @@ namespace {
 // no conflicts on frequent bytes.  Bound: the text's stream.
 __global__ void __launch_bounds__(256) k_alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t* seen,
                                                   int16_t* __restrict__ sym, Status* status) {
-  __shared__ volatile uint32_t h[256];
-  __shared__ uint32_t s_last;
+  __shared__ volatile uint8_t h[256];  // (a byte each: the letters of a text share a few words, which are broadcast)
+  __shared__ uint32_t s_last, count[8];
   const unsigned tid = threadIdx.x;
   h[tid] = 0;
   __syncthreads();
   const uint64_t stride = (uint64_t)gridDim.x * 256, t0 = blockIdx.x * 256ull + tid;
   if (((uintptr_t)T & 15) == 0) {
     const uint4* V = (const uint4*)T;
-    for (uint64_t i = t0; i < n / 16; i += stride) {
-      const uint4 q = V[i];
-      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-      uint32_t f[16];
+    const uint64_t units = n / 16;
+    for (uint64_t i = t0; i < units; i += 2 * stride) {
+      const uint4 q[2] = {V[i], V[i + stride < units ? i + stride : i]};
 #pragma unroll
-      for (int a = 0; a < 16; a++) f[a] = h[(w[a >> 2] >> (8 * (a & 3))) & 0xFF];
+      for (int u = 0; u < 2; u++) {
+        const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+        uint32_t f = 1;
 #pragma unroll
-      for (int a = 0; a < 16; a++)
-        if (!f[a]) h[(w[a >> 2] >> (8 * (a & 3))) & 0xFF] = 1;
+        for (int a = 0; a < 16; a++) f &= h[(w[a >> 2] >> (8 * (a & 3))) & 0xFF];
+        if (f) continue;
+#pragma unroll
+        for (int a = 0; a < 16; a++) h[(w[a >> 2] >> (8 * (a & 3))) & 0xFF] = 1;
+      }
     }
     for (uint64_t i = n / 16 * 16 + t0; i < n; i += stride) h[T[i]] = 1;
   } else {
@@ -60,12 +64,12 @@ __global__ void __launch_bounds__(256) k_alphabet(const uint8_t* __restrict__ T,
   const bool mine = *(volatile uint32_t*)&seen[tid] != 0;
   // Rank among the bytes that occur.
   const unsigned bal = __ballot_sync(0xFFFFFFFFu, mine);
-  if ((tid & 31) == 0) h[tid >> 5] = __popc(bal);
+  if ((tid & 31) == 0) count[tid >> 5] = __popc(bal);
   __syncthreads();
   uint32_t before = 0, all = 0;
   for (uint32_t w = 0; w < 8; w++) {
-    if (w < tid >> 5) before += h[w];
-    all += h[w];
+    if (w < tid >> 5) before += count[w];
+    all += count[w];
   }
   sym[tid] = mine ? (int16_t)(before + __popc(bal & ((1u << (tid & 31)) - 1u))) : (int16_t)-1;
   if (tid == 0) status->symbols = all;

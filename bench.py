@@ -117,7 +117,7 @@ def summarize_launches(path: str, builds: int) -> None:
     for k, v in sorted(agg.items(), key=lambda x: -x[1][1])[:40]:
         print(f"{k:44s} {v[0]:8d} {v[1] / builds:9.3f} {100 * v[1] / tot:6.2f}%")
     for k in per:
-        if any(s in k for s in ("k_scan_stream", "k_scan_list", "k_scan_anchor", "k_hits", "k_candidates<")):
+        if any(s in k for s in ("k_chase_scan", "k_quick_compare", "k_scan_anchor", "k_hits", "k_candidates<")):
             n = len(per[k]) // builds
             lo = n if builds > 1 else 0
             print(k, "per level:", " ".join(f"{x:.3f}" for x in per[k][lo:lo + n]))
@@ -431,8 +431,7 @@ def measure_batch(ndocs: int = 8192, min_len: int = 4 << 10, max_len: int = 16 <
             bt.bt_free(h)
         return dt, blobs, rep, cyc
 
-    # Warm-up on the whole batch: the first call of a size class also runs the
-    # autotuner's trials (cached for the process), outside the timed call.
+    # Warm-up on the whole batch (the first call maps its memory).
     warm = bt.bt_build_batch(*args, o_kernel, nworkers=nworkers)
     tuning = bt.bt_batch_report()
     for h in warm:
@@ -579,8 +578,8 @@ def scan_roofline(prof: dict, step_ms_total: float, traffic_ratio: float | None)
     achieved = scan["bytes"] / (scan["ms"] / 1e3) / 1e9 if scan["ms"] > 0 else None
     per_launch_bytes = scan["bytes"] / max(1, scan["launches"])
     return {
-        "kernel": "window scan of a level (k_scan_stream or k_scan_list, k_scan_anchor, k_hits, "
-                  "k_candidates, and the tail-key k_scan)",
+        "kernel": "window search of a level (k_chase_scan and its bounds; k_scan_anchor, k_hits and "
+                  "k_candidates on levels of blocks under 27 bytes)",
         "bound": "hbm",
         "achieved": achieved,
         "peak": hbm if hbm else 6800.0,

@@ -98,7 +98,9 @@ typedef struct {
  * blocks always work this way on texts with more than 2^20 selected grams. */
 /* BT_FLAG_BATCH_WORKERS makes bt_build_batch build every document with
  * bt_build_ex on host worker threads instead of the persistent batched kernel
- * (the comparison arm of the batched build; the same trees). */
+ * (the comparison arm of the batched build; the same trees).  bt_build_ex builds
+ * texts of at most 16 KiB with the batched kernel too, unless this flag or one
+ * of the diagnostic and layout flags asks for the path of longer texts. */
 /* BT_FLAG_LEAF_COUNTS: space-efficient rank/select support (the paper's
  * section 6 names the auxiliary space of rank and select as future work).
  * The last level, which holds most blocks, stores no per-block symbol

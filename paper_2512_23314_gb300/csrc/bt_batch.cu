@@ -1,10 +1,10 @@
 // bt_batch.cu -- batched construction: a persistent, level-synchronous kernel
 // with a per-document work queue.
 //
-// Each CTA (or, for few long documents, each cluster of CTAs) of k_batch repeatedly takes the next document of the batch from a
-// device work queue (an atomic counter; the documents come in decreasing
-// expected work, length times levels) and builds its whole block tree by
-// itself:
+// Each CTA (or, for few long documents, each cluster of CTAs) of k_batch
+// repeatedly takes the next document of the batch from a device work queue (an
+// atomic counter; the documents come in decreasing expected work, length times
+// levels) and builds its whole block tree by itself:
 //
 //   1. alphabet (byte histogram -> dense symbol map, sigma check);
 //   2. Karp-Rabin prefix fingerprints H(32 j) (section 2, the all-prefix form of
@@ -26,8 +26,8 @@
 //      with the tree's arrays into a region of the batch's output pool taken
 //      with one atomic add.
 //
-// Between steps the CTA meets at a barrier; nothing waits on another CTA, on
-// another launch or on the host.  The tree of every document is the one
+// Between steps the CTA (or cluster) meets at a barrier; nothing waits on
+// another document's CTAs, on another launch or on the host.  The tree of every document is the one
 // bt_build_ex builds for it alone: the same readings of the paper, the same
 // sizing, marking, pointer and pruning rules, every match verified.
 #include <algorithm>

@@ -42,7 +42,7 @@ struct BRes {
   uint64_t leaf_bytes;     // bytes of leaf text
   uint64_t out_off;        // the tree's arrays: pool + out_off
   uint64_t out_bytes;      // bytes taken from the pool (or needed, with BT_ENOMEM)
-  // SM clock cycles the CTA spent per phase: set-up (alphabet, prefix
+  // SM clock cycles the CTA (a cluster's leading one) spent per phase: set-up (alphabet, prefix
   // fingerprints), tables (block and pair fingerprints), window scan,
   // verification / marks / pointers / split, pruning, output and counters.
   unsigned long long cycles[6];

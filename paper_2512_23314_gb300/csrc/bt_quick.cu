@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(kT) k_list_first(const uint32_t* __restrict__ 
   }
 }
 
-// Distances of the entries whose cell has a position of the leading part; the
+// D[e] = x[e] - F in place of the cell, four entries per thread (their random
+// reads are in flight together), for the entries whose cell has a position of the leading part; the
 // others lower their cell and are marked in `open` (a bit per entry, from the
 // split on).
 __global__ void __launch_bounds__(kT) k_list_dist(const uint32_t* __restrict__ total_p, const uint32_t* __restrict__ x,
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(kT) k_list_dist(const uint32_t* __restrict__ t
   }
 }
 
-// Distances of the marked entries, a warp per 32.
+// The marked entries' distances, a warp per 32.
 __global__ void __launch_bounds__(kT) k_list_rest(const uint32_t* __restrict__ total_p, const uint32_t* __restrict__ x,
                                                   uint32_t* __restrict__ D, const uint32_t* __restrict__ first,
                                                   const uint32_t* __restrict__ open) {

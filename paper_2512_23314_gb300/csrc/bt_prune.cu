@@ -41,9 +41,13 @@ enum : uint32_t { UNDEC = 0, PRUNED = 1, KEPT = 2, NOTCAND = 3 };
 constexpr int kProg = 6, kTailFlag = 4, kTailRound = 5;
 // Worklists narrower than this run in the one-CTA tail.
 constexpr unsigned long long kTailFrontier = 4096;
-// A level with at most this many children goes to one CTA, with all above it.
-// With 1024, 4096, 16384: DNA 1 MiB 2.36, 2.20, 2.00 ms, text 20 MB 1.77, 1.69,
-// 1.63 ms, text 256 MiB 7.05, 6.97, 6.89 ms.
+// Levels of at most this many blocks each go to one CTA, from the lowest one
+// that has no longer level among or above its children on.  With 1024, 4096,
+// 16384: DNA 1 MiB 2.36, 2.20, 2.00 ms, text 20 MB 1.77, 1.69, 1.63 ms, text
+// 256 MiB 7.05, 6.97, 6.89 ms.  Levels need not grow downwards (few distinct
+// short blocks: 64-byte records from four values, tau 4, leaf 32, have 65536
+// blocks over 736), so the children's number alone says nothing of the levels
+// above: a level of 2 M blocks in one CTA took 16 of 43 ms of a 256 MiB build.
 constexpr uint64_t kSmallPrune = 16384;
 
 struct PView {
@@ -388,11 +392,14 @@ int prune_tree(BuildCtx& ctx, uint64_t max_rounds) {
   // loop ends (no host round trip per level); cnt[l] for level l >= 1.
   uint64_t* cnt = ctx.new_blocks;
   BT_CUDA(cudaMemsetAsync(cnt, 0, t->L * sizeof(uint64_t), s));
+  // The levels [0, small) have at most kSmallPrune blocks each.
+  uint32_t small = 0;
+  while (small < t->L && t->lv[small].c <= kSmallPrune) small++;
   for (int l = (int)t->L - 2; l >= 0; l--) {
     Level& v = t->lv[l];
     Level& w = t->lv[l + 1];
-    if (w.c <= kSmallPrune) {
-      // This level and all above it (they have fewer blocks still).
+    if ((uint32_t)l + 1 < small) {
+      // This level and all above it.
       SmallLevels S;
       S.top = l;
       S.w_last = l + 1 == (int)t->L - 1;

@@ -180,9 +180,9 @@ int bt_build_batch(const uint8_t* const* texts, const uint64_t* ns, const uint32
  * u64: documents built by the batched kernel, documents built by host
  * workers, kernel launches, documents built a second time because the output
  * pool ran out, threads per CTA, CTAs per SM, output pool bytes, CTA scratch
- * bytes, the largest grid, two zeros (formerly
- * the tuned window run and the trial builds: the kernel has one launch shape
- * and nothing to tune), the microseconds the host spent issuing the texts'
+ * bytes, the largest grid, two zeros (formerly the tuned window run and the
+ * trial builds: the shape follows from the documents' number and lengths,
+ * nothing is tuned), the microseconds the host spent issuing the texts'
  * copies to the device (the copies themselves when the texts are in pageable
  * memory) and the microseconds of device time of the batched kernel's
  * launches.  bt_batch_cycles: for a tree from the batched

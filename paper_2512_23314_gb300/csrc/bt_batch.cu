@@ -60,8 +60,9 @@ namespace {
 constexpr uint32_t kBTailPair = 0xFFFFFFFEu;
 constexpr uint32_t kMaxBThreads = 1024;
 // 32-bit words of dynamic shared memory: the open keys' queues and bitmap, the
-// window filter, the counters' histograms and tiles, one after the other.
-constexpr uint32_t kDynWords = 32768;
+// window filter, the counters' histograms (1024 words a warp) and tiles, one
+// after the other.
+constexpr uint32_t dyn_words_of(uint32_t threads) { return 32 * threads; }
 
 struct __align__(32) BSlot {
   unsigned long long key, lo, maxpst, pad;
@@ -76,9 +77,7 @@ struct BJob {
 
 constexpr uint32_t kMaxGroup = 16;  // CTAs of a cluster that share a document
 
-// State that all CTAs of a group change: in shared memory for one CTA, at the
-// start of a cluster's scratch otherwise (64-bit minima and maxima are no
-// native operations on another CTA's shared memory).
+// State that all CTAs of a group change.
 struct Common {
   uint32_t doc;
   int err;
@@ -97,12 +96,27 @@ struct Common {
 
 static_assert(sizeof(Common) <= kCommonBytes, "a cluster's common state fits its place in the scratch");
 
+// Where it is: in shared memory for one CTA, at the start of a cluster's scratch
+// otherwise (64-bit minima and maxima are no native operations on another CTA's
+// shared memory).
+template <class GRP>
+struct CommonOf;
+template <>
+struct CommonOf<One> {
+  Common own;
+  __device__ Common& common() { return own; }
+};
+template <>
+struct CommonOf<Cluster> {
+  Common* g;
+  __device__ Common& common() { return *g; }
+};
+
 // State of a CTA; what is not scratch of its own is the same in all CTAs of the
 // group, which each compute it from the same arrays.
-struct Cta {
-  Group grp;
-  Common* g;
-  Common own;
+template <class GRP>
+struct Cta : CommonOf<GRP> {
+  GRP grp;
   int bad;
   uint64_t n;
   uint32_t S, L;
@@ -134,7 +148,8 @@ struct Cta {
 
 // Adds the cycles since the last mark to phase `ph` (thread 0; call right
 // after a barrier).
-__device__ __forceinline__ void tmark(Cta& C, int ph) {
+template <class GRP>
+__device__ __forceinline__ void tmark(Cta<GRP>& C, int ph) {
   if (threadIdx.x == 0) {
     const long long t = clock64();
     C.cyc[ph] += (unsigned long long)(t - C.t_mark);
@@ -142,13 +157,15 @@ __device__ __forceinline__ void tmark(Cta& C, int ph) {
   }
 }
 
-__device__ __forceinline__ void fail(Cta& C, int code) { atomicCAS(&C.g->err, 0, code); }
+template <class GRP>
+__device__ __forceinline__ void fail(Cta<GRP>& C, int code) { atomicCAS(&C.common().err, 0, code); }
 // Barrier of the group; has a step failed?  (Two barriers in a cluster: no
 // later step's failure may be seen by some of its CTAs only.)
-__device__ __forceinline__ bool failed(Cta& C) {
-  if (C.grp.size == 1) return __syncthreads_or(C.g->err != 0) != 0;
+template <class GRP>
+__device__ __forceinline__ bool failed(Cta<GRP>& C) {
+  if (!GRP::many) return __syncthreads_or(C.common().err != 0) != 0;
   gsync(C.grp);
-  const int e = *(volatile int*)&C.g->err;
+  const int e = *(volatile int*)&C.common().err;
   gsync(C.grp);
   return e != 0;
 }
@@ -253,8 +270,9 @@ __device__ __forceinline__ bool differs(const uint8_t* __restrict__ T, uint64_t 
 
 // Verify jobs[0, nj): mismatch[i] = 1 when the two ranges differ.  Groups of
 // G lanes (about len/16, a power of two up to 32) take one job each.
+template <class GRP>
 __device__ void verify_jobs(const uint8_t* __restrict__ T, const BJob* jobs, uint32_t nj, uint64_t maxlen,
-                            unsigned int* mismatch, const Group& grp_) {
+                            unsigned int* mismatch, const GRP& grp_) {
   unsigned G = 1;
   while (G < 32 && 16ull * G < maxlen) G <<= 1;
   const unsigned lane = threadIdx.x & 31, grp = lane / G, gl = lane % G, gpw = 32 / G;
@@ -278,7 +296,8 @@ __device__ void verify_jobs(const uint8_t* __restrict__ T, const BJob* jobs, uin
 // ---------------------------------------------------------------------------
 // (Only which bytes occur matters: after a document's first lines every mark
 // is set, and looking costs no atomics and no conflicts on frequent bytes.)
-__device__ void alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t sigma, Cta& C) {
+template <class GRP>
+__device__ void alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t sigma, Cta<GRP>& C) {
   volatile unsigned int* seen = C.hist;
   const unsigned tid = C.grp.tid(), nt = C.grp.threads(), t = threadIdx.x;
   for (uint32_t i = t; i < 256; i += blockDim.x) seen[i] = 0;
@@ -298,13 +317,13 @@ __device__ void alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t sig
   __syncthreads();
   if (t < 256) {
     const uint32_t bits = __ballot_sync(kFull, seen[t] != 0);
-    if ((t & 31) == 0 && bits) atomicOr(&C.g->seen[t >> 5], bits);
+    if ((t & 31) == 0 && bits) atomicOr(&C.common().seen[t >> 5], bits);
   }
   gsync(C.grp);
   if (t < 256) {
     uint32_t before = 0, all = 0, mine = 0;
     for (uint32_t w = 0; w < 8; w++) {
-      const uint32_t bits = *(volatile uint32_t*)&C.g->seen[w];
+      const uint32_t bits = *(volatile uint32_t*)&C.common().seen[w];
       if (w < t >> 5) before += __popc(bits);
       if (w == t >> 5) mine = bits;
       all += __popc(bits);
@@ -322,9 +341,9 @@ __device__ void alphabet(const uint8_t* __restrict__ T, uint64_t n, uint32_t sig
 // A CTA takes the chunks [j0, j1) after the ones whose fingerprint is `carry`;
 // returns (in C.carry) the fingerprint up to j1, a multiple of four chunks on,
 // or, with `store`, writes Hs.
-template <class M>
+template <class M, class GRP>
 __device__ void prefix_range(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const uint8_t* T, uint64_t nchunks,
-                             uint64_t r0, uint64_t r1, uint64_t carry0, bool store, uint64_t* Hs, Cta& C) {
+                             uint64_t r0, uint64_t r1, uint64_t carry0, bool store, uint64_t* Hs, Cta<GRP>& C) {
   if (threadIdx.x == 0) C.carry = carry0;
   __syncthreads();
   const uint64_t xl = kr_lane_pow(m, pw);
@@ -362,32 +381,32 @@ __device__ void prefix_range(const M& m, const PrefixConst<M>& PC, const KrPow& 
 
 // In a cluster each CTA takes an equal part of the text: its fingerprint, then
 // the parts before it, then its values.
-template <class M>
+template <class M, class GRP>
 __device__ void prefix_pass(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const uint8_t* T, uint64_t n,
-                            uint64_t* Hs, Cta& C) {
+                            uint64_t* Hs, Cta<GRP>& C) {
   const uint64_t nchunks = n / 32, all = nchunks + 1;
-  if (C.grp.size == 1) {
+  if constexpr (!GRP::many) {
     prefix_range(m, PC, pw, T, nchunks, 0, all, 0, true, Hs, C);
-    return;
+  } else {
+    const uint64_t per = (all + 4 * C.grp.size - 1) / (4 * C.grp.size) * 4;
+    const uint64_t r0 = per * C.grp.rank < all ? per * C.grp.rank : all, r1 = r0 + per < all ? r0 + per : all;
+    prefix_range(m, PC, pw, T, nchunks, r0, r1, 0, false, Hs, C);
+    if (threadIdx.x == 0) C.common().part[C.grp.rank] = C.carry;
+    gsync(C.grp);
+    uint64_t carry = 0;
+    if (threadIdx.x == 0) {
+      const uint64_t x = pow_mod(m, PC.B32, per);
+      for (uint32_t k = 0; k < C.grp.rank; k++) carry = m.add(m.mul(carry, x), *(volatile uint64_t*)&C.common().part[k]);
+    }
+    prefix_range(m, PC, pw, T, nchunks, r0, r1, carry, true, Hs, C);
+    gsync(C.grp);
   }
-  const uint64_t per = (all + 4 * C.grp.size - 1) / (4 * C.grp.size) * 4;
-  const uint64_t r0 = per * C.grp.rank < all ? per * C.grp.rank : all, r1 = r0 + per < all ? r0 + per : all;
-  prefix_range(m, PC, pw, T, nchunks, r0, r1, 0, false, Hs, C);
-  if (threadIdx.x == 0) C.g->part[C.grp.rank] = C.carry;
-  gsync(C.grp);
-  uint64_t carry = 0;
-  if (threadIdx.x == 0) {
-    const uint64_t x = pow_mod(m, PC.B32, per);
-    for (uint32_t k = 0; k < C.grp.rank; k++) carry = m.add(m.mul(carry, x), *(volatile uint64_t*)&C.g->part[k]);
-  }
-  prefix_range(m, PC, pw, T, nchunks, r0, r1, carry, true, Hs, C);
-  gsync(C.grp);
 }
 
 // H[p] for every p in [0, n] (levels of blocks too short for the list).
-template <class M>
+template <class M, class GRP>
 __device__ void expand_pass(const M& m, const uint8_t* T, uint64_t n, uint64_t B, const uint64_t* Hs, uint64_t* H,
-                            const Group& grp) {
+                            const GRP& grp) {
   for (uint64_t j = grp.tid(); j <= n / 32; j += grp.threads()) {
     uint64_t h = Hs[j];
     for (uint64_t p = 32 * j; p < 32 * j + 32 && p <= n; p++) {
@@ -399,7 +418,8 @@ __device__ void expand_pass(const M& m, const uint8_t* T, uint64_t n, uint64_t B
 }
 
 // Exclusive sum of one value per thread over the CTA; *total = the sum.
-__device__ uint32_t cta_excl_u32(uint32_t v, Cta& C, uint32_t* total) {
+template <class GRP>
+__device__ uint32_t cta_excl_u32(uint32_t v, Cta<GRP>& C, uint32_t* total) {
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint32_t x = v;
 #pragma unroll
@@ -430,7 +450,8 @@ __device__ uint32_t cta_excl_u32(uint32_t v, Cta& C, uint32_t* total) {
 // table, the distances and the segment minima.  In a cluster each CTA takes an
 // equal part of the text: it marks and counts its entries first (the marks wait
 // in the first-occurrence table's place).
-__device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
+template <class GRP>
+__device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta<GRP>& C) {
   const unsigned tid = C.grp.tid(), nt = C.grp.threads(), lane = tid & 31;
   const uint64_t nw = n < kGramLen ? 0 : (n - kGramLen + 1 + 31) / 32, ns = (n + kSegBytes - 1) / kSegBytes,
                  ns2 = (ns + 63) / 64;
@@ -447,11 +468,11 @@ __device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
     if (left < 32) bits &= (1u << left) - 1u;
     return bits;
   };
-  const bool multi = C.grp.size > 1;
+  constexpr bool multi = GRP::many;
   const uint64_t per = (nw + C.grp.size - 1) / C.grp.size, a0 = per * C.grp.rank < nw ? per * C.grp.rank : nw,
                  a1 = a0 + per < nw ? a0 + per : nw;
   uint32_t total = 0, all = 0;
-  if (multi) {
+  if constexpr (multi) {
     uint32_t mine = 0, sum;
     for (uint64_t j = a0 + threadIdx.x; j < a1; j += blockDim.x) {
       const uint32_t bits = mask(j);
@@ -459,10 +480,10 @@ __device__ void list_pass(const uint8_t* T, uint64_t n, char* scr, Cta& C) {
       mine += __popc(bits);
     }
     cta_excl_u32(mine, C, &sum);
-    if (threadIdx.x == 0) C.g->part[C.grp.rank] = sum;
+    if (threadIdx.x == 0) C.common().part[C.grp.rank] = sum;
     gsync(C.grp);
     for (uint32_t k = 0; k < C.grp.size; k++) {
-      const uint32_t x = (uint32_t)*(volatile uint64_t*)&C.g->part[k];
+      const uint32_t x = (uint32_t)*(volatile uint64_t*)&C.common().part[k];
       if (k < C.grp.rank) total += x;
       all += x;
     }
@@ -564,10 +585,10 @@ __device__ Work carve_level(char* temp, uint64_t c, uint64_t bcap, uint64_t pcap
 // Exact leftmost occurrence of every suspect key (a fingerprint collision
 // was found by verification): every window before the key's start, inside a
 // run, whose fingerprint equals the key's is compared byte by byte.
-template <class M>
+template <class M, class GRP>
 __device__ void exact_pass(const M& m, const LV& g, const uint64_t* H, const Work& W, int pair, uint64_t B,
-                           Cta& C) {
-  const uint32_t ns = C.g->nsusp;
+                           Cta<GRP>& C) {
+  const uint32_t ns = C.common().nsusp;
   // Key fingerprint, length and B^length of each suspect (in the job array).
   for (uint32_t i = C.grp.tid(); i < ns; i += C.grp.threads()) {
     const uint64_t k = W.susp[i];
@@ -630,8 +651,8 @@ __device__ __forceinline__ void window_hit(const M& m, const ScanArgs& A, uint64
 
 // Marks and leftmost occurrences of a level of short blocks (fewer than
 // kQuickMinB bytes): fingerprint tables and a scan of every window.
-template <class M>
-__device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, const LV& g, char* scr, uint32_t l,
+template <class M, class GRP>
+__device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta<GRP>& C, const LV& g, char* scr, uint32_t l,
                           uint32_t* filt, uint32_t filt_words_max) {
   const uint64_t n = C.n, c = g.c, b = g.b;
   const unsigned tid = C.grp.tid(), nt = C.grp.threads();
@@ -668,8 +689,8 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
       min_pos(&W.bt[slot].lo, s);
     } else {
       W.slotB[k] = kNoSlot;
-      C.g->fp_tail = fp;
-      atomicMin(&C.g->lo_tail, (unsigned long long)s);
+      C.common().fp_tail = fp;
+      atomicMin(&C.common().lo_tail, (unsigned long long)s);
     }
   }
   if (failed(C)) return;
@@ -678,7 +699,7 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
   for (uint64_t k = tid; k + 1 < c; k += nt) {
     W.slotP[k] = kNoSlot;
     if (g.st[k + 1] != g.st[k] + b) continue;
-    atomicAdd(&C.g->npairs, 1u);
+    atomicAdd(&C.common().npairs, 1u);
     const uint32_t sk = W.slotB[k];
     if (sk == kNoSlot) {
       fail(C, BT_EINTERNAL);
@@ -688,8 +709,8 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
       atomicMax(&W.bt[sk].maxpst, (unsigned long long)g.st[k]);
     if (W.slotB[k + 1] == kNoSlot) {
       W.slotP[k] = kBTailPair;
-      C.g->pretail = sk;
-      atomicMin(&C.g->lo_tailpair, (unsigned long long)g.st[k]);
+      C.common().pretail = sk;
+      atomicMin(&C.common().lo_tailpair, (unsigned long long)g.st[k]);
     } else {
       const uint32_t sp = t_insert(W.pt, pmask, ((uint64_t)sk << 32) | W.slotB[k + 1]);
       W.slotP[k] = sp;
@@ -721,9 +742,9 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
   // The window scan: every window [p, p+b) inside a run (and [p, p+r) for the
   // short tail); the few whose fingerprint's bit is set probe the table.
   {
-    const uint32_t pretail = C.g->pretail, bshift = C.bshift;
-    const uint64_t fp_tail = C.g->fp_tail;
-    const ScanArgs A{H, W.bt, W.pt, bmask, pmask, b, r, Bb, Br, fp_tail, pretail, &C.g->lo_tailpair};
+    const uint32_t pretail = C.common().pretail, bshift = C.bshift;
+    const uint64_t fp_tail = C.common().fp_tail;
+    const ScanArgs A{H, W.bt, W.pt, bmask, pmask, b, r, Bb, Br, fp_tail, pretail, &C.common().lo_tailpair};
     for (uint64_t w = tid; w < c * b; w += nt) {
       const uint64_t k = bshift != 0xFFu ? w >> bshift : w / b;
       const uint64_t j = w - k * b;
@@ -735,7 +756,7 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
         const uint64_t bit = x & fmask;
         if ((filt[bit >> 5] >> (bit & 31)) & 1u) window_hit(m, A, p, av, x, hb);
       }
-      if (r && p + r <= av && phi(m, H, Br, p, r) == fp_tail) min_pos(&C.g->lo_tail, p);
+      if (r && p + r <= av && phi(m, H, Br, p, r) == fp_tail) min_pos(&C.common().lo_tail, p);
     }
   }
   gsync(C.grp);
@@ -748,35 +769,35 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
     W.job_of[k] = kNone;
     const uint32_t sp = W.slotP[k];
     if (sp == kNoSlot) continue;
-    const uint64_t lp = sp == kBTailPair ? C.g->lo_tailpair : W.pt[sp].lo;
+    const uint64_t lp = sp == kBTailPair ? C.common().lo_tailpair : W.pt[sp].lo;
     const uint64_t s = g.st[k];
     if (lp == s) {
       W.pm[k] = 1;
     } else if (lp < s) {
       const uint64_t len = b + blen(g, k + 1);
-      const uint32_t id = atomicAdd(&C.g->njobs, 1u);
+      const uint32_t id = atomicAdd(&C.common().njobs, 1u);
       W.jobs[id] = BJob{lp, s, len, k};
       W.job_of[k] = id;
-      atomicAdd(&C.g->verify_bytes, 2ull * len);
+      atomicAdd(&C.common().verify_bytes, 2ull * len);
     } else {
       fail(C, BT_EINTERNAL);  // the pair's own window was not seen
     }
   }
   if (failed(C)) return;
-  verify_jobs(g.T, W.jobs, C.g->njobs, 2 * b, W.mismatch, C.grp);
+  verify_jobs(g.T, W.jobs, C.common().njobs, 2 * b, W.mismatch, C.grp);
   gsync(C.grp);
   for (uint64_t k = tid; k + 1 < c; k += nt) {
     const uint64_t id = W.job_of[k];
     if (id == kNone || !W.mismatch[id]) continue;
-    atomicAdd(&C.g->collisions, 1ull);
-    const uint32_t i = atomicAdd(&C.g->nsusp, 1u);
+    atomicAdd(&C.common().collisions, 1ull);
+    const uint32_t i = atomicAdd(&C.common().nsusp, 1u);
     W.susp[i] = k;
     W.exlo[i] = g.st[k];
   }
   gsync(C.grp);
-  if (C.g->nsusp) {
+  if (C.common().nsusp) {
     exact_pass(m, g, H, W, 1, P.B, C);
-    for (uint32_t i = tid; i < C.g->nsusp; i += nt) W.pm[W.susp[i]] = W.exlo[i] == g.st[W.susp[i]];
+    for (uint32_t i = tid; i < C.common().nsusp; i += nt) W.pm[W.susp[i]] = W.exlo[i] == g.st[W.susp[i]];
     gsync(C.grp);
   }
 
@@ -801,13 +822,13 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
   }
   gsync(C.grp);
   if (C.grp.rank == 0) cta_scan_u32(W.wpop, mr, words, C.wtot);
-  if (C.grp.size > 1) gsync(C.grp);
+  if (GRP::many) gsync(C.grp);
 
   // Leftmost occurrence of every block that becomes a pointer (of every
   // block when pruning needs it), verified.
   if (tid == 0) {
-    C.g->njobs = 0;
-    C.g->nsusp = 0;
+    C.common().njobs = 0;
+    C.common().nsusp = 0;
   }
   for (uint64_t i = tid; i < c; i += nt) W.mismatch[i] = 0;
   gsync(C.grp);
@@ -816,46 +837,44 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta& C, c
     lo[k] = kNone;
     if (!P.prune && marked(mw, k)) continue;
     const uint64_t s = g.st[k], len = blen(g, k);
-    const uint64_t p = W.slotB[k] == kNoSlot ? C.g->lo_tail : W.bt[W.slotB[k]].lo;
+    const uint64_t p = W.slotB[k] == kNoSlot ? C.common().lo_tail : W.bt[W.slotB[k]].lo;
     lo[k] = p;
     if (p < s) {
-      const uint32_t id = atomicAdd(&C.g->njobs, 1u);
+      const uint32_t id = atomicAdd(&C.common().njobs, 1u);
       W.jobs[id] = BJob{p, s, len, k};
       W.job_of[k] = id;
-      atomicAdd(&C.g->verify_bytes, 2ull * len);
+      atomicAdd(&C.common().verify_bytes, 2ull * len);
     } else if (p > s) {
       fail(C, BT_EINTERNAL);
     }
   }
   if (failed(C)) return;
-  verify_jobs(g.T, W.jobs, C.g->njobs, b, W.mismatch, C.grp);
+  verify_jobs(g.T, W.jobs, C.common().njobs, b, W.mismatch, C.grp);
   gsync(C.grp);
   for (uint64_t k = tid; k < c; k += nt) {
     const uint64_t id = W.job_of[k];
     if (id == kNone || !W.mismatch[id]) continue;
-    atomicAdd(&C.g->collisions, 1ull);
-    const uint32_t i = atomicAdd(&C.g->nsusp, 1u);
+    atomicAdd(&C.common().collisions, 1ull);
+    const uint32_t i = atomicAdd(&C.common().nsusp, 1u);
     W.susp[i] = k;
     W.exlo[i] = g.st[k];
   }
   gsync(C.grp);
-  if (C.g->nsusp) {
+  if (C.common().nsusp) {
     exact_pass(m, g, H, W, 0, P.B, C);
-    for (uint32_t i = tid; i < C.g->nsusp; i += nt) lo[W.susp[i]] = W.exlo[i];
+    for (uint32_t i = tid; i < C.common().nsusp; i += nt) lo[W.susp[i]] = W.exlo[i];
     gsync(C.grp);
   }
 }
-
-constexpr uint32_t kCtaBitWords = 8192;  // the open keys' bitmap in shared memory up to 32 KiB
 
 // Marks and leftmost occurrences of a level by first occurrences: the steps of
 // bt_quick.cu over one CTA.  Measured on 1024 versioned documents of 4 KiB - 4
 // MiB (0.65 GB): with fingerprint tables and a scan of every window (anchored
 // on levels of 1 KiB blocks and more) the kernel took 50 ms, the longest
 // document 51; now 15 and 15.
-template <class M>
-__device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const LV& g, char* scr, uint32_t l,
-                           uint32_t* dyn) {
+template <class M, class GRP>
+__device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, const LV& g, char* scr, uint32_t l,
+                           uint32_t* dyn, uint32_t dyn_words) {
   const uint64_t n = C.n, c = g.c, b = g.b, words = (c + 31) / 32;
   const unsigned tid = C.grp.tid(), nt = C.grp.threads(), lane = tid & 31, warp = threadIdx.x >> 5,
                  nwarps = blockDim.x >> 5;
@@ -896,7 +915,7 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
     }
     lo[k] = at;
     if (open) {
-      items[atomicAdd(&C.g->qs.nitems, 1ull)] = (uint32_t)(2 * k);
+      items[atomicAdd(&C.common().qs.nitems, 1ull)] = (uint32_t)(2 * k);
       nob++;
     }
     uint32_t d2 = 0;
@@ -906,7 +925,7 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
     np += st & kIsPair;
     if (st == kIsPair && d2 != kNoDist) vb += 2 * plen;
     if (open) {
-      items[atomicAdd(&C.g->qs.nitems, 1ull)] = (uint32_t)(2 * k + 1);
+      items[atomicAdd(&C.common().qs.nitems, 1ull)] = (uint32_t)(2 * k + 1);
       nop++;
     }
   }
@@ -915,17 +934,17 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
   nob = __reduce_add_sync(kFull, nob);
   nop = __reduce_add_sync(kFull, nop);
   if (lane == 0) {
-    if (vb) atomicAdd(&C.g->status.verify_bytes, (unsigned long long)vb);
-    if (np) atomicAdd(&C.g->npairs, np);
-    if (nob) atomicAdd(&C.g->qs.nopen[0], (unsigned long long)nob);
-    if (nop) atomicAdd(&C.g->qs.nopen[1], (unsigned long long)nop);
+    if (vb) atomicAdd(&C.common().status.verify_bytes, (unsigned long long)vb);
+    if (np) atomicAdd(&C.common().npairs, np);
+    if (nob) atomicAdd(&C.common().qs.nopen[0], (unsigned long long)nob);
+    if (nop) atomicAdd(&C.common().qs.nopen[1], (unsigned long long)nop);
   }
   gsync(C.grp);
   tmark(C, 3);
-  const uint64_t ni = C.g->qs.nitems;
+  const uint64_t ni = C.common().qs.nitems;
   if (ni) {
-    const uint64_t nb = C.g->qs.nopen[0] + 2 * C.g->qs.nopen[1];
-    const uint64_t bcap = pow2_ge(2 * (nb < c ? nb : c)), pcap = pow2_ge(2 * C.g->qs.nopen[1]), gcap = pow2_ge(2 * ni);
+    const uint64_t nb = C.common().qs.nopen[0] + 2 * C.common().qs.nopen[1];
+    const uint64_t bcap = pow2_ge(2 * (nb < c ? nb : c)), pcap = pow2_ge(2 * C.common().qs.nopen[1]), gcap = pow2_ge(2 * ni);
     uint32_t fbits = 12;
     while ((1ull << fbits) < 16 * ni && fbits < 30) fbits++;
     const uint32_t bwords = 1u << (fbits - 5);
@@ -954,8 +973,8 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
       K.pmask = (uint32_t)(pcap - 1);
       K.gmask = (uint32_t)(gcap - 1);
       K.bshift = 32 - fbits;
-      K.qs = &C.g->qs;
-      K.status = &C.g->status;
+      K.qs = &C.common().qs;
+      K.status = &C.common().status;
       K.lo = lo;
       K.ps = ps;
     }
@@ -971,7 +990,7 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
     uint2* hq = (uint2*)dyn + warp * kHitQ;
     uint32_t* cq = (uint32_t*)((uint2*)dyn + nwarps * kHitQ) + warp * kCandQ;
     uint32_t* bits_s = (uint32_t*)((uint2*)dyn + nwarps * kHitQ) + nwarps * kCandQ;
-    const bool fits = bwords <= kCtaBitWords;
+    const bool fits = bwords <= dyn_words - nwarps * (2 * kHitQ + kCandQ);
     auto fetch = [&]() {
       if (fits)
         for (uint32_t i = threadIdx.x; i < bwords; i += blockDim.x) bits_s[i] = K.bitmap[i];
@@ -999,7 +1018,7 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
     gsync(C.grp);
     chase_apply(K, w);
     gsync(C.grp);
-    const uint64_t nsusp = C.g->qs.nsusp;
+    const uint64_t nsusp = C.common().qs.nsusp;
     if (nsusp) {
       chase_exact(K, 0, 1, nsusp, w);
       gsync(C.grp);
@@ -1007,7 +1026,7 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
       gsync(C.grp);
     }
   }
-  if (tid == 0 && C.g->status.error) fail(C, BT_EINTERNAL);  // (the level goes on; the caller looks at the end)
+  if (tid == 0 && C.common().status.error) fail(C, BT_EINTERNAL);  // (the level goes on; the caller looks at the end)
   for (uint64_t wb = tid >> 5; wb < words; wb += nt >> 5) {
     const uint64_t k = wb * 32 + lane;
     bool mk = false;
@@ -1023,11 +1042,11 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta& C, const L
   }
   gsync(C.grp);
   if (C.grp.rank == 0) cta_scan_u32(wpop, mr, words, C.wtot);
-  if (C.grp.size > 1) gsync(C.grp);
+  if (GRP::many) gsync(C.grp);
 }
 
-template <class M>
-__device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& P, const BDoc& D, Cta& C, char* scr,
+template <class M, class GRP>
+__device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& P, const BDoc& D, Cta<GRP>& C, char* scr,
                            uint32_t l, uint32_t* dyn, uint32_t dyn_words) {
   const uint64_t* bsz = P.sizes + D.lv_off;
   const uint64_t n = C.n, c = C.c[l], b = bsz[l];
@@ -1048,7 +1067,7 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
     C.bshift = (b & (b - 1)) == 0 ? (uint32_t)(__ffsll((long long)b) - 1) : 0xFFu;
   }
   if (tid == 0) {
-    Common& G = *C.g;
+    Common& G = C.common();
     G.fp_tail = kNone;
     G.lo_tail = kNone;
     G.lo_tailpair = kNone;
@@ -1065,7 +1084,7 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
   gsync(C.grp);
   const bool quick = b >= kQuickMinB;
   if (quick) {
-    quick_keys(m, PC, C, g, scr, l, dyn);
+    quick_keys(m, PC, C, g, scr, l, dyn, dyn_words);
   } else {
     scan_keys(m, P, D, C, g, scr, l, dyn, dyn_words);
     if (failed(C)) return;
@@ -1108,12 +1127,12 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
     S[BT_ST_B] = b;
     S[BT_ST_COV] = (c - 1) * b + blen(g, c - 1);
     S[BT_ST_NMARKED] = nm;
-    S[BT_ST_NPAIRS] = C.g->npairs;
-    S[BT_ST_VERIFY_BYTES] = quick ? C.g->status.verify_bytes : C.g->verify_bytes;
-    S[BT_ST_COLLISIONS] = quick ? C.g->status.collisions : C.g->collisions;
+    S[BT_ST_NPAIRS] = C.common().npairs;
+    S[BT_ST_VERIFY_BYTES] = quick ? C.common().status.verify_bytes : C.common().verify_bytes;
+    S[BT_ST_COLLISIONS] = quick ? C.common().status.collisions : C.common().collisions;
     S[BT_ST_FINAL_BLOCKS] = c;
-    S[BT_ST_CANDIDATES] = quick && C.g->qs.nitems ? C.g->qs.cands : 0;
-    S[BT_ST_HITS] = quick && C.g->qs.nitems ? C.g->qs.hits : 0;
+    S[BT_ST_CANDIDATES] = quick && C.common().qs.nitems ? C.common().qs.cands : 0;
+    S[BT_ST_HITS] = quick && C.common().qs.nitems ? C.common().qs.hits : 0;
   }
   if (last) {
     if (threadIdx.x == 0) C.arity[l] = 0;
@@ -1126,11 +1145,11 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
   const uint32_t arity = (uint32_t)(b / bn);
   uint64_t* nst = (uint64_t*)(scr + C.sl.st[l + 1]);
   for (uint64_t wb = tid; wb < words; wb += nt)
-    if (mw[wb]) atomicMax(&C.g->lastk, (unsigned long long)(wb * 32 + 31 - __clz(mw[wb])));
+    if (mw[wb]) atomicMax(&C.common().lastk, (unsigned long long)(wb * 32 + 31 - __clz(mw[wb])));
   gsync(C.grp);
   if (threadIdx.x == 0) {
     C.arity[l] = arity;
-    const uint64_t lk = C.g->lastk;
+    const uint64_t lk = C.common().lastk;
     C.bad = nm == 0;
     if (nm != 0) {
       const uint64_t nch = (blen(g, lk) + bn - 1) / bn;
@@ -1157,7 +1176,8 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
   tmark(C, 3);
 }
 
-__device__ PLv plevel(const Cta& C, char* scr, const uint64_t* bsz, uint32_t l) {
+template <class GRP>
+__device__ PLv plevel(const Cta<GRP>& C, char* scr, const uint64_t* bsz, uint32_t l) {
   return PLv{C.n, C.c[l], bsz[l], (uint64_t*)(scr + C.sl.st[l]), (uint32_t*)(scr + C.sl.mw[l]),
              (uint32_t*)(scr + C.sl.mr[l]), (uint32_t*)(scr + C.sl.ptr[l]), (uint64_t*)(scr + C.sl.off[l]),
              (uint64_t*)(scr + C.sl.lo[l])};
@@ -1167,19 +1187,23 @@ __device__ PLv plevel(const Cta& C, char* scr, const uint64_t* bsz, uint32_t l) 
 // barriers of the cluster cost more than its help.
 constexpr uint64_t kLeaderPrune = 8192;
 
-__device__ void prune_pass(const BParams& P, const BDoc& D, Cta& C, char* scr) {
+template <class GRP>
+__device__ void prune_pass(const BParams& P, const BDoc& D, Cta<GRP>& C, char* scr) {
   const uint64_t* bsz = P.sizes + D.lv_off;
   for (int l = (int)C.L - 2; l >= 0; l--) {
     const PLv v = plevel(C, scr, bsz, (uint32_t)l), w = plevel(C, scr, bsz, (uint32_t)l + 1);
     const bool alone = v.c + w.c <= kLeaderPrune;
     uint64_t c2 = 0;
-    if (!alone || C.grp.rank == 0)
-      c2 = prune_level(v, w, l + 1 == (int)C.L - 1, C.arity[l], scr + C.sl.temp, P.max_rounds, C.g->prune, C.wtot,
-                       alone ? Group{} : C.grp);
-    if (alone && C.grp.size > 1) {
-      if (C.grp.tid() == 0) C.g->part[0] = c2;
+    const bool w_last = l + 1 == (int)C.L - 1;
+    char* temp = scr + C.sl.temp;
+    if (!GRP::many || (alone && C.grp.rank == 0))
+      c2 = prune_level(v, w, w_last, C.arity[l], temp, P.max_rounds, C.common().prune, C.wtot, One{});
+    else if (!alone)
+      c2 = prune_level(v, w, w_last, C.arity[l], temp, P.max_rounds, C.common().prune, C.wtot, C.grp);
+    if (GRP::many && alone) {
+      if (C.grp.tid() == 0) C.common().part[0] = c2;
       gsync(C.grp);
-      c2 = *(volatile uint64_t*)&C.g->part[0];
+      c2 = *(volatile uint64_t*)&C.common().part[0];
       gsync(C.grp);
     }
     if (c2 == kNone) {  // (so in every CTA of the group)
@@ -1202,27 +1226,30 @@ __device__ void prune_pass(const BParams& P, const BDoc& D, Cta& C, char* scr) {
 // Counters of a level, symbol-major (cp entries per symbol).  mode 0: symbol
 // counts of each block (marked blocks of a non-last level are filled from their
 // children afterwards); mode 1: counts of T[st[ptr], st[ptr] + off) of each
-// unmarked block.  A warp takes four consecutive blocks at a time, 16 bytes per
+// unmarked block.  A warp takes BLOCKS consecutive blocks at a time, 16 bytes per
 // lane and block in flight together, each with its own histogram (hist: 1024
-// words per warp), and writes the four counters of a symbol at once (zeros
-// where a block is not counted; nothing when none of the four is).
-__device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PLv& v, int mode, bool last,
+// words per warp).  Four of them write the four counters of a symbol at once
+// (zeros where a block is not counted; nothing when none of the four is); one, on
+// levels with too few blocks to give every warp four, writes single counters.
+template <uint32_t BLOCKS, class GRP>
+__device__ void count_rows(const uint8_t* __restrict__ T, const Cta<GRP>& C, const PLv& v, int mode, bool last,
                            void* out, uint32_t cw, uint64_t cp, unsigned int* hist) {
+  constexpr uint32_t IN_FLIGHT = BLOCKS < 2 ? BLOCKS : 2;
   const uint32_t S = C.S;
   const unsigned lane = threadIdx.x & 31, nw = C.grp.threads() >> 5;
   unsigned int* h = hist + (threadIdx.x >> 5) * 1024;
-  for (uint64_t g = C.grp.tid() >> 5; 4 * g < v.c; g += nw) {
-    uint64_t s0[4];
-    uint32_t len[4], top = 0;
+  for (uint64_t g = C.grp.tid() >> 5; BLOCKS * g < v.c; g += nw) {
+    uint64_t s0[BLOCKS];
+    uint32_t len[BLOCKS], top = 0;
     bool any = false;
 #pragma unroll
-    for (uint32_t q = 0; q < 4; q++) {
-      const uint64_t k = 4 * g + q;
+    for (uint32_t q = 0; q < BLOCKS; q++) {
+      const uint64_t k = BLOCKS * g + q;
       s0[q] = 0;
       len[q] = 0;
       if (k >= v.c) continue;
-      any |= mode == 0 ? last || !marked(v.mw, k) : !marked(v.mw, k);
       const bool mk = marked(v.mw, k);
+      any |= mode == 0 ? last || !mk : !mk;
       if (mode == 0 && (last || !mk)) {
         s0[q] = v.st[k];
         len[q] = (uint32_t)plen(v, k);
@@ -1235,18 +1262,18 @@ __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PL
     if (!any) continue;
     for (uint32_t i = lane; i < S; i += 32) {
 #pragma unroll
-      for (uint32_t q = 0; q < 4; q++) h[256 * q + i] = 0;
+      for (uint32_t q = 0; q < BLOCKS; q++) h[256 * q + i] = 0;
     }
     __syncwarp();
     for (uint32_t x = 16 * lane; x < top; x += 512) {
 #pragma unroll
-      for (uint32_t q0 = 0; q0 < 4; q0 += 2) {
-        uint4 t[2];
+      for (uint32_t q0 = 0; q0 < BLOCKS; q0 += IN_FLIGHT) {
+        uint4 t[IN_FLIGHT];
 #pragma unroll
-        for (uint32_t q = 0; q < 2; q++)
+        for (uint32_t q = 0; q < IN_FLIGHT; q++)
           if (x < len[q0 + q]) t[q] = load16u(T, s0[q0 + q] + x);
 #pragma unroll
-        for (uint32_t q = 0; q < 2; q++) {
+        for (uint32_t q = 0; q < IN_FLIGHT; q++) {
           if (x >= len[q0 + q]) continue;
           const uint32_t w[4] = {t[q].x, t[q].y, t[q].z, t[q].w};
           const uint32_t have = len[q0 + q] - x;
@@ -1258,11 +1285,15 @@ __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PL
     }
     __syncwarp();
     for (uint32_t i = lane; i < S; i += 32) {
-      const uint32_t a = h[i], b = h[256 + i], c = h[512 + i], d = h[768 + i];
-      const uint64_t at = i * cp + 4 * g;
-      if (cw == 1) *(uint32_t*)((uint8_t*)out + at) = a | (b << 8) | (c << 16) | (d << 24);
-      else if (cw == 2) *(uint2*)((uint16_t*)out + at) = make_uint2(a | (b << 16), c | (d << 16));
-      else *(uint4*)((uint32_t*)out + at) = make_uint4(a, b, c, d);
+      const uint64_t at = i * cp + BLOCKS * g;
+      if constexpr (BLOCKS == 1) {
+        cput(out, cw, at, h[i]);
+      } else {
+        const uint32_t a = h[i], b = h[256 + i], c = h[512 + i], d = h[768 + i];
+        if (cw == 1) *(uint32_t*)((uint8_t*)out + at) = a | (b << 8) | (c << 16) | (d << 24);
+        else if (cw == 2) *(uint2*)((uint16_t*)out + at) = make_uint2(a | (b << 16), c | (d << 16));
+        else *(uint4*)((uint32_t*)out + at) = make_uint4(a, b, c, d);
+      }
     }
     __syncwarp();
   }
@@ -1271,11 +1302,16 @@ __device__ void count_rows(const uint8_t* __restrict__ T, const Cta& C, const PL
 // One-byte counters: a thread per block into a tile [S][TB] in shared memory
 // (as k_count_small of bt_query.cu: warp w takes the columns that put its
 // lanes in different banks), rows leave as runs.
-__device__ void count_small(const uint8_t* __restrict__ T, const Cta& C, const PLv& v, int mode, bool last, uint8_t* out,
-                            uint64_t cp, uint8_t* tile) {
+template <class GRP>
+__device__ void count_small(const uint8_t* __restrict__ T, const Cta<GRP>& C, const PLv& v, int mode, bool last, uint8_t* out,
+                            uint64_t cp, uint8_t* tile, uint32_t tile_words) {
   const uint32_t S = C.S, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  uint32_t TB = blockDim.x;
-  while ((uint64_t)TB * S > kDynWords * 4ull) TB >>= 1;  // 1024, or 512 above 128 symbols
+  // As wide as the level, while the tile has room: at 128 blocks of 256 symbols
+  // a tile of 512 was cleared and written mostly for nothing.
+  uint32_t shift = 31 - __clz(blockDim.x);
+  while (((uint64_t)S << shift) > tile_words * 4ull) shift--;
+  while (shift > 7 && (1ull << (shift - 1)) >= v.c) shift--;
+  const uint32_t TB = 1u << shift;
   const uint32_t col = 4 * (lane + 32 * (warp >> 2)) + (warp & 3);
   for (uint64_t k0 = (uint64_t)C.grp.rank * TB; k0 < v.c; k0 += (uint64_t)C.grp.size * TB) {
     __syncthreads();
@@ -1304,9 +1340,8 @@ __device__ void count_small(const uint8_t* __restrict__ T, const Cta& C, const P
       }
     }
     __syncthreads();
-    const uint32_t words = TB / 4;
-    for (uint32_t i = tid; i < S * words; i += blockDim.x) {
-      const uint32_t row = i / words, w = i - row * words;
+    for (uint32_t i = tid; i < S * (TB / 4); i += blockDim.x) {
+      const uint32_t row = i >> (shift - 2), w = i & (TB / 4 - 1);
       const uint64_t at = k0 + 4 * w;
       if (at < cp) *(uint32_t*)(out + row * cp + at) = ((const uint32_t*)tile)[i];
     }
@@ -1314,7 +1349,8 @@ __device__ void count_small(const uint8_t* __restrict__ T, const Cta& C, const P
   __syncthreads();
 }
 
-__device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr, unsigned int* hist) {
+template <class GRP>
+__device__ void write_output(const BParams& P, const BDoc& D, Cta<GRP>& C, char* scr, unsigned int* hist) {
   const uint64_t* bsz = P.sizes + D.lv_off;
   const unsigned tid = C.grp.tid(), nt = C.grp.threads(), lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   const uint32_t L = C.L, S = C.S;
@@ -1333,12 +1369,12 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
     C.out_bytes = need;
     if (tid == 0) {
       const unsigned long long o = atomicAdd(P.pool_used, (unsigned long long)need);
-      C.g->out_off = C.out_off = o;
+      C.common().out_off = C.out_off = o;
       if (o + need > P.pool_cap) fail(C, BT_ENOMEM);
     }
   }
   if (failed(C)) return;
-  char* out = P.pool + C.g->out_off;
+  char* out = P.pool + C.common().out_off;
   const uint32_t bl = s_base;
   // Level arrays.
   for (uint32_t l = 0; l < L; l++) {
@@ -1365,11 +1401,13 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
     const uint32_t cw = s_cw[l];
     const uint64_t cp = counter_stride(v.c);
     if (cw == 1) {
-      count_small(D.T, C, v, 0, last, (uint8_t*)cnt, cp, (uint8_t*)hist);
-      count_small(D.T, C, v, 1, last, (uint8_t*)pc, cp, (uint8_t*)hist);
+      count_small(D.T, C, v, 0, last, (uint8_t*)cnt, cp, (uint8_t*)hist, P.dyn_words);
+      count_small(D.T, C, v, 1, last, (uint8_t*)pc, cp, (uint8_t*)hist, P.dyn_words);
     } else {
-      count_rows(D.T, C, v, 0, last, cnt, cw, cp, hist);
-      count_rows(D.T, C, v, 1, last, pc, cw, cp, hist);
+      for (int mode = 0; mode < 2; mode++) {
+        if (v.c >= 4 * nw) count_rows<4>(D.T, C, v, mode, last, mode ? pc : cnt, cw, cp, hist);
+        else count_rows<1>(D.T, C, v, mode, last, mode ? pc : cnt, cw, cp, hist);
+      }
     }
     gsync(C.grp);
     if (!last) {
@@ -1377,13 +1415,18 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
       const uint32_t ccw = s_cw[l + 1];
       const uint64_t bn = bsz[l + 1], ccp = counter_stride(C.c[l + 1]);
       const uint32_t arity = C.arity[l];
-      // A warp takes 32 blocks and a quarter of the symbols; four symbols'
-      // children are read together.
-      const uint64_t chunks = (v.c + 31) / 32;
-      for (uint64_t it = warp; it < 4 * chunks; it += nw) {
-        const uint64_t k = (it >> 2) * 32 + lane;
+      // A warp takes 32 blocks and a part of the symbols -- a quarter, or fewer
+      // where the level has too few blocks for all warps, down to four (with
+      // quarters a document of 4 KiB and 256 symbols took 160 thousand cycles
+      // here, a third of its build); four symbols' children are read together.
+      const uint32_t chunks = (uint32_t)((v.c + 31) / 32);
+      uint32_t parts = 4;
+      while (parts * chunks < nw && 4 * parts < S) parts *= 2;
+      for (uint32_t it = warp; it < parts * chunks; it += nw) {
+        const uint32_t part = it & (parts - 1);
+        const uint64_t k = (uint64_t)(it / parts) * 32 + lane;
         if (k >= v.c || !marked(v.mw, k)) continue;
-        const uint32_t s0 = (uint32_t)(S * (it & 3) / 4), s1 = (uint32_t)(S * ((it & 3) + 1) / 4);
+        const uint32_t s0 = S * part / parts, s1 = S * (part + 1) / parts;
         const uint64_t first = mrank(v.mw, v.mr, k) * arity;
         const uint32_t nch = (uint32_t)((plen(v, k) + bn - 1) / bn);
         for (uint32_t s = s0; s < s1; s += 4) {
@@ -1496,8 +1539,8 @@ __device__ void write_output(const BParams& P, const BDoc& D, Cta& C, char* scr,
   gsync(C.grp);
 }
 
-template <class M>
-__device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const BParams& P, uint32_t d, Cta& C, char* scr, unsigned int* hist,
+template <class M, class GRP>
+__device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw, const BParams& P, uint32_t d, Cta<GRP>& C, char* scr, unsigned int* hist,
                           uint32_t dyn_words) {
   const BDoc D = P.docs[d];
   const uint64_t* bsz = P.sizes + D.lv_off;
@@ -1506,8 +1549,8 @@ __device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw,
     C.L = D.L;
     C.bad = D.L == 0 || D.L > kBMaxLevels || scratch_layout(D.n, D.L, bsz, &C.sl) > P.scratch_per_cta;
     if (C.grp.rank == 0) {
-      C.g->err = C.bad ? BT_EINTERNAL : 0;
-      for (uint32_t& x : C.g->seen) x = 0;
+      C.common().err = C.bad ? BT_EINTERNAL : 0;
+      for (uint32_t& x : C.common().seen) x = 0;
     }
     C.out_off = 0;
     C.out_bytes = 0;
@@ -1546,13 +1589,13 @@ __device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw,
   if (C.grp.rank != 0) return;
   if (threadIdx.x == 0) {
     BRes& R = P.res[D.index];
-    R.status = C.g->err;
+    R.status = C.common().err;
     R.S = C.S;
     R.out_off = C.out_off;
     R.out_bytes = C.out_bytes;
     for (int i = 0; i < 6; i++) R.cycles[i] = C.cyc[i];
   }
-  if (C.g->err == 0) {
+  if (C.common().err == 0) {
     for (uint32_t l = threadIdx.x; l < D.L; l += blockDim.x) {
       BLevelRes& Lr = P.lres[D.lv_off + l];
       Lr.c = C.c[l];
@@ -1566,27 +1609,32 @@ __device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw,
   __syncthreads();
 }
 
-// One CTA of 1024 threads per SM: 64 registers per thread.  A document belongs
-// to a CTA, or to a cluster of them.
-template <class M>
+// 64 registers per thread: one CTA of 1024 threads per SM, or several narrower
+// ones (launch_shape).  A document belongs to a CTA, or to a cluster of them.
+// Compiled apart for the two: one kernel for both spilled 2000 bytes of stores and
+// 4160 of loads (-Xptxas -v), these 344 and 780 (one CTA), 972 and 2524 (cluster).
+template <class M, class GRP>
 __global__ void __launch_bounds__(kMaxBThreads, 1) k_batch(const __grid_constant__ BParams P, M m,
                                                            const __grid_constant__ PrefixConst<M> PC,
                                                            const __grid_constant__ KrPow pw) {
   // Dynamic shared memory: the open keys' queues and bitmap of a level (or its
   // window filter), then (during the output) the symbol counters.
   extern __shared__ unsigned int s_hist[];
-  __shared__ Cta C;
-  const Group grp = this_cluster();
+  __shared__ Cta<GRP> C;
+  GRP grp;
+  if constexpr (GRP::many) grp = this_cluster();
   char* scr = P.scratch + (uint64_t)(blockIdx.x / grp.size) * P.scratch_per_cta;
-  if (threadIdx.x == 0) {
-    C.grp = grp;
-    C.g = grp.size == 1 ? &C.own : (Common*)scr;
+  if constexpr (GRP::many) {
+    if (threadIdx.x == 0) {
+      C.grp = grp;
+      C.g = (Common*)scr;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   for (;;) {
-    if (grp.tid() == 0) C.g->doc = atomicAdd(P.next, 1u);
+    if (grp.tid() == 0) C.common().doc = atomicAdd(P.next, 1u);
     gsync(grp);
-    const uint32_t d = *(volatile uint32_t*)&C.g->doc;
+    const uint32_t d = *(volatile uint32_t*)&C.common().doc;
     gsync(grp);
     if (d >= P.ndocs) return;
     build_doc(m, PC, pw, P, d, C, scr, s_hist, P.dyn_words);
@@ -1612,7 +1660,7 @@ struct DocPlan {
   uint64_t size_off;       // first block size in the batch's size array
 };
 
-// Opt the kernel in to its dynamic shared memory and to clusters of sixteen
+// Opt the kernels in to their dynamic shared memory and to clusters of sixteen
 // CTAs, once per device; the largest cluster the device can hold.
 template <class M>
 int prepare_batch_kernel(int bytes, uint32_t* max_group) {
@@ -1621,9 +1669,10 @@ int prepare_batch_kernel(int bytes, uint32_t* max_group) {
   BT_CUDA(cudaGetDevice(&dev));
   uint32_t g = most[dev & 63].load(std::memory_order_acquire);
   if (!g) {
-    BT_CUDA(cudaFuncSetAttribute(k_batch<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    BT_CUDA(cudaFuncSetAttribute(k_batch<M, One>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    BT_CUDA(cudaFuncSetAttribute(k_batch<M, Cluster>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     g = 8;
-    if (cudaFuncSetAttribute(k_batch<M>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) g = 16;
+    if (cudaFuncSetAttribute(k_batch<M, Cluster>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) g = 16;
     for (; g > 1; g /= 2) {
       cudaLaunchConfig_t cfg{};
       cfg.gridDim = dim3(g);
@@ -1636,7 +1685,7 @@ int prepare_batch_kernel(int bytes, uint32_t* max_group) {
       cfg.attrs = &at;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k_batch<M>, &cfg) == cudaSuccess && n > 0) break;
+      if (cudaOccupancyMaxActiveClusters(&n, k_batch<M, Cluster>, &cfg) == cudaSuccess && n > 0) break;
     }
     cudaGetLastError();
     most[dev & 63].store(g, std::memory_order_release);
@@ -1648,23 +1697,23 @@ int prepare_batch_kernel(int bytes, uint32_t* max_group) {
 // `groups` clusters of `group` CTAs, per_group bytes of scratch each.
 template <class M>
 int launch_docs(const M& m, const BParams& base, uint32_t first, uint32_t count, unsigned groups, uint32_t group,
-                uint64_t per_group, char* scratch, unsigned int* next, cudaStream_t s) {
+                uint64_t per_group, char* scratch, unsigned int* next, uint32_t threads, cudaStream_t s) {
   BParams P = base;
   P.docs = base.docs + first;
   P.ndocs = count;
   P.next = next;
   P.scratch = scratch;
   P.scratch_per_cta = per_group;
-  P.dyn_words = kDynWords;
-  constexpr int smem = (int)(kDynWords * sizeof(unsigned int));
+  P.dyn_words = dyn_words_of(threads);
+  const int smem = (int)(P.dyn_words * sizeof(unsigned int));
   uint32_t most;
-  BT_TRY(prepare_batch_kernel<M>(smem, &most));
+  BT_TRY(prepare_batch_kernel<M>((int)(dyn_words_of(kMaxBThreads) * sizeof(unsigned int)), &most));
   if (group > most) group = most;
   const PrefixConst<M> PC(m, P.B);
   const KrPow pw = kr_pow(m, pow_mod(m, P.B, 128));  // a thread of the prefix pass takes four 32-byte chunks
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(groups * group);
-  cfg.blockDim = dim3(kMaxBThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at{};
@@ -1673,7 +1722,8 @@ int launch_docs(const M& m, const BParams& base, uint32_t first, uint32_t count,
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = group > 1 ? 1 : 0;
-  BT_LAUNCH(BT_CUDA(cudaLaunchKernelEx(&cfg, k_batch<M>, P, m, PC, pw)));
+  if (group > 1) BT_LAUNCH(BT_CUDA(cudaLaunchKernelEx(&cfg, k_batch<M, Cluster>, P, m, PC, pw)));
+  else BT_LAUNCH(BT_CUDA(cudaLaunchKernelEx(&cfg, k_batch<M, One>, P, m, PC, pw)));
   return BT_OK;
 }
 
@@ -1768,13 +1818,41 @@ struct DevFree {
   }
 };
 
+// Threads of a CTA and CTAs per SM.  A short document leaves most of 1024 threads
+// idle between barriers that wait for all of them, so several narrow CTAs share
+// an SM where the documents are short enough and enough to fill them.  Kernel
+// time of versioned texts (DNA copies, random bytes), us, with 1 x 1024, 2 x 512
+// and 4 x 256 threads per SM:
+//    64 of   4 KiB   152  124  123   (193  170  155;   163   163   199)
+//   512 of   4 KiB   475  244  160   (643  332  213;   459   287   244)
+//  2048 of  32 KiB  3414 1890 1401  (4529 2830 2478;  2951  1870  1666)
+//   512 of  64 KiB  1260  750  574  (1563 1080 1104;  1014   734  1104)
+//  1024 of 128 KiB  5050 4094 4319  (5355 4489 5074;  2952  2295  2562)
+//   256 of 512 KiB  4923 4273 5822  (3830 3424 5191;  2710  3726  6470)
+// A document much longer than the others would outlast them in a narrow CTA; a
+// caller's bound on the CTAs counts whole SMs.
+struct Shape {
+  unsigned threads, ctas_per_sm;
+};
+Shape launch_shape(uint64_t docs, uint64_t mean, uint64_t longest, bool bounded) {
+  const unsigned nsm = device_sm_count();
+  if (bounded) return Shape{kMaxBThreads, 1};
+  if (docs > nsm && mean <= (32u << 10) && longest <= (128u << 10)) return Shape{256, 4};
+  if (docs > 2 * nsm && mean <= (128u << 10) && longest <= (512u << 10)) return Shape{512, 2};
+  if (docs <= nsm && longest <= (8u << 10)) return Shape{512, 1};
+  return Shape{kMaxBThreads, 1};
+}
+
 template <class M>
 int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, const uint32_t* leaf_lens,
               const bt_opts& o, std::vector<DocPlan>& plans, const std::vector<uint64_t>& sizes,
               bt_tree** outs, cudaStream_t s) {
-  constexpr unsigned threads = kMaxBThreads, ctas_per_sm = 1;  // the launch shape: one CTA of 1024 threads per SM
   const uint64_t nd = plans.size();
   if (nd == 0) return BT_OK;
+  uint64_t bytes_all = 0, longest = 0;
+  for (const DocPlan& d : plans) bytes_all += d.n, longest = std::max(longest, d.n);
+  const Shape shape = launch_shape(nd, bytes_all / nd, longest, o.batch_ctas != 0);
+  const unsigned threads = shape.threads, ctas_per_sm = shape.ctas_per_sm;
   int device = 0;
   BT_CUDA(cudaGetDevice(&device));
   const uint64_t q = o.modulus ? o.modulus : Mersenne61::Q;
@@ -1922,7 +2000,7 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
     unsigned int* next = d_next + (ci % 64);
     lrc = cudaMemsetAsync(next, 0, sizeof(unsigned int), s) == cudaSuccess ? BT_OK : BT_ECUDA;
     if (lrc == BT_OK)
-      lrc = launch_docs(m, P, cls[ci].first, cls[ci].count, cls[ci].grid, cls[ci].group, cls[ci].per_cta, d_scratch, next, s);
+      lrc = launch_docs(m, P, cls[ci].first, cls[ci].count, cls[ci].grid, cls[ci].group, cls[ci].per_cta, d_scratch, next, threads, s);
   }
   if (timed) cudaEventRecord(ev[1], s);
   std::vector<BRes> res(nd);
@@ -1974,7 +2052,7 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
           1, std::min<uint64_t>({(uint64_t)hd2.size(), (uint64_t)nsm * ctas_per_sm, scratch_max / top,
                                  o.batch_ctas ? (uint64_t)o.batch_ctas : ~0ull}));
       BT_CUDA(cudaMemsetAsync(d_next, 0, sizeof(unsigned int), s));
-      BT_TRY(launch_docs(m, P2, 0, (uint32_t)hd2.size(), grid, 1, top, d_scratch, d_next, s));
+      BT_TRY(launch_docs(m, P2, 0, (uint32_t)hd2.size(), grid, 1, top, d_scratch, d_next, threads, s));
       BT_CUDA(cudaMemcpyAsync(res.data(), d_res, nd * sizeof(BRes), cudaMemcpyDeviceToHost, s));
       BT_CUDA(cudaMemcpyAsync(lres.data(), d_lres, nlv * sizeof(BLevelRes), cudaMemcpyDeviceToHost, s));
       BT_CUDA(cudaStreamSynchronize(s));
@@ -2117,7 +2195,7 @@ int run_solo(const M& m, const uint8_t* text, uint64_t n, uint32_t sigma, uint32
   P.B = base_for(o.seed, o.modulus ? o.modulus : Mersenne61::Q);
   P.prune = o.prune ? 1 : 0;
   P.max_rounds = o.max_rounds ? o.max_rounds : 4096;
-  BT_TRY(launch_docs(m, P, 0, 1, 1, 1, need, d + head + room, &dh->next, s));
+  BT_TRY(launch_docs(m, P, 0, 1, 1, 1, need, d + head + room, &dh->next, kMaxBThreads, s));
   BT_CUDA(cudaStreamSynchronize(s));
   const int rc = *(volatile int*)&S->res.status;
   if (rc == BT_ENOMEM) return BT_EINTERNAL;  // (the room was the most it can take)

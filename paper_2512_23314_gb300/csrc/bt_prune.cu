@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(1024) k_prune_small(const __grid_constant__ Sm
   __shared__ PruneShared Z;
   __shared__ uint32_t wtot[kScanWords];
   for (int l = S.top; l >= 0; l--) {
-    const uint64_t c2 = prune_level(S.lv[l], S.lv[l + 1], S.w_last && l == S.top, S.arity[l], temp, max_rounds, Z, wtot, Group{});
+    const uint64_t c2 = prune_level(S.lv[l], S.lv[l + 1], S.w_last && l == S.top, S.arity[l], temp, max_rounds, Z, wtot, One{});
     if (c2 == kNone) {
       if (threadIdx.x == 0) atomicExch(&status->error, 13ull);
       return;

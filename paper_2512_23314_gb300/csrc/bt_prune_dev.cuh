@@ -9,30 +9,35 @@
 
 namespace bt {
 
-// The CTAs that share a document: one, or a thread-block cluster.  Every thread
-// of the group reaches every gsync.
-struct Group {
-  uint32_t rank = 0, size = 1;
+// The CTAs that share a document: one (One), or a thread-block cluster (Cluster).
+// Every thread of the group reaches every gsync.  Which of the two is known when
+// the code is compiled: with the choice made at every barrier, and the shared
+// state reached through a pointer that could lead to shared or global memory, a
+// short document took 1.4 times as long in one CTA.
+struct One {
+  static constexpr bool many = false;
+  static constexpr uint32_t rank = 0, size = 1;
+  __device__ unsigned tid() const { return threadIdx.x; }
+  __device__ unsigned threads() const { return blockDim.x; }
+};
+struct Cluster {
+  static constexpr bool many = true;
+  uint32_t rank, size;
   __device__ unsigned tid() const { return rank * blockDim.x + threadIdx.x; }
   __device__ unsigned threads() const { return size * blockDim.x; }
 };
 
-__device__ __forceinline__ Group this_cluster() {
+__device__ __forceinline__ Cluster this_cluster() {
   const cooperative_groups::cluster_group c = cooperative_groups::this_cluster();
-  Group g;
+  Cluster g;
   g.rank = c.block_rank();
   g.size = c.num_blocks();
   return g;
 }
 
 // Barrier of the group; what its threads wrote before is seen by all after.
-__device__ __forceinline__ void gsync(const Group& g) {
-  if (g.size == 1) {
-    __syncthreads();
-  } else {
-    cooperative_groups::this_cluster().sync();
-  }
-}
+__device__ __forceinline__ void gsync(const One&) { __syncthreads(); }
+__device__ __forceinline__ void gsync(const Cluster&) { cooperative_groups::this_cluster().sync(); }
 
 enum : uint32_t { P_UNDEC = 0, P_PRUNED = 1, P_KEPT = 2, P_NOTCAND = 3 };
 constexpr uint32_t kFull = 0xFFFFFFFFu;
@@ -156,7 +161,8 @@ struct PruneShared {
   int err;
 };
 
-__device__ inline void flag_targets(const PLv& v, uint8_t* flag, const Group& G) {
+template <class GRP>
+__device__ inline void flag_targets(const PLv& v, uint8_t* flag, const GRP& G) {
   for (uint64_t u = G.tid(); u < v.c; u += G.threads()) {
     if (marked(v.mw, u)) continue;
     const uint64_t j = v.ptr[u];
@@ -168,8 +174,9 @@ __device__ inline void flag_targets(const PLv& v, uint8_t* flag, const Group& G)
 // Level l = v, its children w; returns the blocks of w that stay (kNone: a
 // device check failed).  v's marks, ranks, pointers and offsets are updated, w
 // is compacted in place.
+template <class GRP>
 __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, uint32_t arity, char* temp,
-                                       uint64_t max_rounds, PruneShared& Z, uint32_t* wtot, const Group& G) {
+                                       uint64_t max_rounds, PruneShared& Z, uint32_t* wtot, const GRP& G) {
   const unsigned tid = G.tid(), nt = G.threads(), lane = tid & 31, nw = nt >> 5;
   // A check that failed anywhere: everyone's to know before anyone goes on.
   auto failed = [&]() {
@@ -308,7 +315,7 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
   for (uint64_t k = tid; k < w.c; k += nt) R.nidx[k] = R.gone[k] ? 0u : 1u;
   gsync(G);
   if (G.rank == 0) cta_scan_u32(R.nidx, R.nidx, w.c, wtot);
-  if (G.size > 1) gsync(G);
+  if (GRP::many) gsync(G);
   for (uint64_t k = tid; k < w.c; k += nt) {
     if (R.gone[k]) continue;
     const uint64_t i = R.nidx[k];
@@ -344,7 +351,7 @@ __device__ inline uint64_t prune_level(const PLv& v, const PLv& w, bool w_last, 
   }
   gsync(G);
   if (G.rank == 0) cta_scan_u32(R.wpop, w.mr, words2, wtot);
-  if (G.size > 1) gsync(G);
+  if (GRP::many) gsync(G);
   return c2;
 }
 

@@ -596,11 +596,14 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
       if (cn >= 32) take_cands();
     }
   };
-  for (uint64_t t0 = e0 + w.tid / 32 * kChaseTile; t0 < e1; t0 += w.n / 32 * kChaseTile) {
+  // (A short list is dealt out one entry a lane: eight would leave most warps
+  // without and the others with eight times the steps one after the other.)
+  const uint32_t per = e1 - e0 <= w.n ? 1 : kChaseTile / 32;
+  for (uint64_t t0 = e0 + w.tid / 32 * (32 * per); t0 < e1; t0 += w.n / 32 * (32 * per)) {
     uint32_t x[8], F[8];
     uint32_t pass = 0;
-    const uint64_t e = t0 + 8ull * lane;
-    if (e + 8 <= e1) {
+    const uint64_t e = t0 + (uint64_t)per * lane;
+    if (per == 8 && e + 8 <= e1) {
 #pragma unroll
       for (int q = 0; q < 2; q++) {
         const uint4 a = ((const uint4*)(C.Q.x + e))[q], d = ((const uint4*)(C.Q.D + e))[q];
@@ -616,7 +619,7 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
 #pragma unroll
       for (int u = 0; u < 8; u++) {
         x[u] = F[u] = 0;
-        if (e + u >= e1) continue;
+        if (u >= (int)per || e + u >= e1) continue;
         x[u] = C.Q.x[e + u];
         F[u] = x[u] - C.Q.D[e + u];
         const uint32_t bit = c_bit(C, F[u]);

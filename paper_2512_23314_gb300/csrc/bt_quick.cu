@@ -509,7 +509,10 @@ __device__ __forceinline__ bool qmark(const uint32_t* __restrict__ mw, uint64_t 
 // Back-pointers of the unmarked blocks (the block that holds the leftmost
 // occurrence and the offset into it; the copied window must lie in one or two
 // marked blocks and end before the block) and the children of the marked
-// ones: the block of mark rank r puts its children at r arity + i.
+// ones: the block of mark rank r puts its children at r arity + i.  The host
+// reads the status one step later, after the next level or the pruning has run
+// on these pointers: a block whose occurrence fails the check still gets one that
+// lies in the level.
 __global__ void __launch_bounds__(kT) k_quick_points(QGeo g, const uint32_t* __restrict__ mw, const uint32_t* __restrict__ mr,
                                                      const uint64_t* __restrict__ lo, uint32_t* __restrict__ ptr,
                                                      uint64_t* __restrict__ off, uint32_t arity, uint64_t bn,
@@ -528,7 +531,7 @@ __global__ void __launch_bounds__(kT) k_quick_points(QGeo g, const uint32_t* __r
     }
     const uint64_t p = lo[k];
     uint64_t j;
-    bool ok = p + len <= s;
+    bool ok = p < s && len <= s - p;
     if (all_present) {
       j = ok ? p / g.b : 0;
     } else {
@@ -546,6 +549,8 @@ __global__ void __launch_bounds__(kT) k_quick_points(QGeo g, const uint32_t* __r
       ok = j + 1 < g.c && g.st[j + 1] == g.st[j] + qblen(g, j) && qmark(mw, j + 1);
     if (!ok) {
       atomicExch(&status->error, 5ull);
+      ptr[k] = 0;
+      off[k] = 0;
       continue;
     }
     ptr[k] = (uint32_t)j;

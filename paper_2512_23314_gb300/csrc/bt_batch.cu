@@ -650,7 +650,8 @@ __device__ __forceinline__ void window_hit(const M& m, const ScanArgs& A, uint64
 }
 
 // Marks and leftmost occurrences of a level of short blocks (fewer than
-// kQuickMinB bytes): fingerprint tables and a scan of every window.
+// kQuickMinB bytes), or of one whose search by grams was given up: fingerprint
+// tables and a scan of every window.
 template <class M, class GRP>
 __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta<GRP>& C, const LV& g, char* scr, uint32_t l,
                           uint32_t* filt, uint32_t filt_words_max) {
@@ -666,6 +667,7 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta<GRP>&
   }
   const uint64_t bcap = pow2_ge(2 * c), pcap = pow2_ge(2 * c);
   const Work W = carve_level(scr + C.sl.temp, c, bcap, pcap);
+  if (tid == 0) C.common().npairs = 0;  // (a search that was given up counted them)
   for (uint64_t i = tid; i < bcap; i += nt) W.bt[i] = BSlot{kNone, kNone, 0, 0};
   for (uint64_t i = tid; i < pcap; i += nt) W.pt[i] = PSlot{kNone, kNone};
   for (uint64_t i = tid; i < c; i += nt) W.mismatch[i] = 0;
@@ -872,8 +874,9 @@ __device__ void scan_keys(const M& m, const BParams& P, const BDoc& D, Cta<GRP>&
 // MiB (0.65 GB): with fingerprint tables and a scan of every window (anchored
 // on levels of 1 KiB blocks and more) the kernel took 50 ms, the longest
 // document 51; now 15 and 15.
+// False, the same for all threads: given up, the level goes by scan_keys.
 template <class M, class GRP>
-__device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, const LV& g, char* scr, uint32_t l,
+__device__ bool quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, const LV& g, char* scr, uint32_t l,
                            uint32_t* dyn, uint32_t dyn_words) {
   const uint64_t n = C.n, c = g.c, b = g.b, words = (c + 31) / 32;
   const unsigned tid = C.grp.tid(), nt = C.grp.threads(), lane = tid & 31, warp = threadIdx.x >> 5,
@@ -950,6 +953,8 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, co
     const uint32_t bwords = 1u << (fbits - 5);
     if (threadIdx.x == 0) {
       Chase& K = C.chase;
+      K.first = false;
+      K.probes = probes_most(ni);
       K.g = q;
       K.Q = C.list;
       K.A = A;
@@ -981,35 +986,75 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, co
     __syncthreads();
     const Chase& K = C.chase;
     const PrefixAt<M> H(PC, g.T, n, (const uint64_t*)(scr + C.sl.Hs));
-    chase_init(K, bwords, w);
-    gsync(C.grp);
-    if (b <= 256) chase_keys<M, 1>(m, H, K, w);
-    else chase_keys<M, 32>(m, H, K, w);
-    gsync(C.grp);
     // Shared memory: the warps' queues, then the bitmap while it fits.
     uint2* hq = (uint2*)dyn + warp * kHitQ;
-    uint32_t* cq = (uint32_t*)((uint2*)dyn + nwarps * kHitQ) + warp * kCandQ;
-    uint32_t* bits_s = (uint32_t*)((uint2*)dyn + nwarps * kHitQ) + nwarps * kCandQ;
-    const bool fits = bwords <= dyn_words - nwarps * (2 * kHitQ + kCandQ);
-    auto fetch = [&]() {
+    uint32_t* queues = (uint32_t*)((uint2*)dyn + nwarps * kHitQ);
+    uint32_t* cq = queues + warp * kCandQ;
+    uint8_t* gq = (uint8_t*)(queues + nwarps * kCandQ) + warp * kHitQ;
+    uint32_t* bits_s = queues + nwarps * (kCandQ + kHitQ / 4);
+    const bool fits = bwords <= dyn_words - nwarps * (2 * kHitQ + kCandQ + kHitQ / 4);
+    const uint32_t* bits = fits ? bits_s : K.bitmap;
+    // As for a single text (bt_quick.cu): the sample by newest grams, perhaps by
+    // first grams too, then the rest by one of them, or every window.
+    enum { kBySample, kByBoth, kByRest };
+    const uint32_t total = C.nsel, split = total > (1u << 16) ? (total / 16) & ~(8 * kChaseTile - 1) : 0;
+    const uint64_t few = split ? work_few(n) : work_most(n, false);
+    uint64_t limit = work_most(n, split != 0), newest = 0, before = 0;
+    uint32_t step = kBySample;
+    bool enter = true;
+    for (bool again = false;; again = true) {
+      const bool rest = step == kByRest;
+      if (enter) {
+        chase_init(K, bwords, again, w);
+        gsync(C.grp);
+        if (b <= 256) chase_keys<M, 1>(m, H, K, w);
+        else chase_keys<M, 32>(m, H, K, w);
+        gsync(C.grp);
+      }
+      if (rest) {
+        chase_bound(K, w);
+        for (uint32_t i = tid; i < bwords; i += nt) K.bitmap[i] = 0;
+        gsync(C.grp);
+        chase_live(K, split, w);
+        gsync(C.grp);
+      }
       if (fits)
         for (uint32_t i = threadIdx.x; i < bwords; i += blockDim.x) bits_s[i] = K.bitmap[i];
       __syncthreads();
-    };
-    fetch();
-    const uint32_t* bits = fits ? bits_s : K.bitmap;
-    const uint32_t total = C.nsel, split = total > (1u << 16) ? (total / 16) & ~(8 * kChaseTile - 1) : 0;
-    if (split) {
-      chase_scan(m, H, K, 0, split, bits, hq, cq, nullptr, w);
+      chase_scan(m, H, K, K.first, rest ? split : 0, rest || !split ? total : split, bits, hq, gq, cq, rest ? K.bound2 : nullptr, limit,
+                 kGiveUp, w);
       gsync(C.grp);
-      chase_bound(K, w);
-      for (uint32_t i = tid; i < bwords; i += nt) K.bitmap[i] = 0;
+      const bool over = *(volatile unsigned int*)&K.qs->redo != kSearchDone;
+      const uint64_t seen = *(volatile unsigned long long*)&K.qs->work;
+      bool first = K.first;
       gsync(C.grp);
-      chase_live(K, split, w);
-      gsync(C.grp);
-      fetch();
+      if (step == kBySample && !over && (!split || seen <= work_sample(n))) {
+        if (!split) break;
+        step = kByRest;
+        enter = false;
+      } else if (step == kBySample) {
+        step = kByBoth;
+        newest = over ? ~0ull : seen;
+        first = enter = true;
+      } else if (step == kByBoth) {
+        const uint64_t by_first = over ? ~0ull : seen - before;
+        if ((newest < by_first ? newest : by_first) > few) return false;
+        if (!split) break;
+        step = kByRest;
+        enter = newest < by_first;
+        first = !enter;
+      } else {
+        if (over) return false;
+        break;
+      }
+      before = seen;
+      limit = seen + (step == kByBoth ? few : work_most(n, false));
+      if (threadIdx.x == 0) {
+        C.chase.first = first;
+        C.chase.probes = ~0ull;
+      }
+      __syncthreads();
     }
-    chase_scan(m, H, K, split, total, bits, hq, cq, split ? K.bound2 : nullptr, w);
     if (C.r && C.r < kQuickMinB) chase_tail(K, w);
     gsync(C.grp);
     tmark(C, 2);
@@ -1043,6 +1088,7 @@ __device__ void quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, co
   gsync(C.grp);
   if (C.grp.rank == 0) cta_scan_u32(wpop, mr, words, C.wtot);
   if (GRP::many) gsync(C.grp);
+  return true;
 }
 
 template <class M, class GRP>
@@ -1082,10 +1128,10 @@ __device__ void level_pass(const M& m, const PrefixConst<M>& PC, const BParams& 
     G.status.error = G.status.verify_bytes = G.status.collisions = 0;
   }
   gsync(C.grp);
-  const bool quick = b >= kQuickMinB;
-  if (quick) {
-    quick_keys(m, PC, C, g, scr, l, dyn, dyn_words);
-  } else {
+  // (The scan's H takes the place of the list.)
+  bool quick = b >= kQuickMinB && !C.expanded;
+  if (quick) quick = quick_keys(m, PC, C, g, scr, l, dyn, dyn_words);
+  if (!quick) {
     scan_keys(m, P, D, C, g, scr, l, dyn, dyn_words);
     if (failed(C)) return;
   }

@@ -107,7 +107,7 @@ constexpr uint32_t kCommonBytes = 4096;  // first of all: what a cluster's CTAs 
 struct ScratchLayout {
   uint64_t Hs;                                  // u64[n / 32 + 2]: prefix fingerprints H(32 j)
   uint64_t big;                                 // the list's positions and distances, u32[n] each; later, for
-                                                // levels of short blocks, u64[n + 1]: H at every position
+                                                // levels by the window scan, u64[n + 1]: H at every position
   uint64_t idx, seg1, seg2, first;              // the list's index and segment minima; the first-occurrence table
   uint64_t cells;
   uint64_t st[kBMaxLevels], lo[kBMaxLevels], off[kBMaxLevels];  // u64[cmax]
@@ -139,7 +139,7 @@ __host__ __device__ inline uint64_t temp_bytes(uint64_t cm, uint64_t b) {
                         + out_align(cm + 8)             // pm
                         + out_align(cm * 32 + 32)       // jobs
                         + out_align(cap * 32) + out_align(cap * 16);
-  const uint64_t level = b >= kQuickMinB ? quick : scan;
+  const uint64_t level = b >= kQuickMinB && quick > scan ? quick : scan;  // (the first may end up as the second)
   const uint64_t prune = out_align(cm + 8) * 5          // hit_v, hit2, tgt_w, gone, mk2
                          + out_align(cm * 4 + 4) * 7    // state, indeg, fq x2, nidx, wpop, ptr2
                          + out_align(cm * 8 + 8) * 5;   // t1, t2, st2, off2, lo2

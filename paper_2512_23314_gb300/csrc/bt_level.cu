@@ -1824,8 +1824,9 @@ int sort_minima(const M& m, const Geo& g, LevelWork& W, uint64_t c, uint64_t b, 
   return BT_OK;
 }
 
+// `dense`: by the scan of every window.
 template <class M>
-int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
+int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start, bool dense) {
   bt_tree* t = ctx.t;
   Level& v = t->lv[l];
   cudaStream_t s = ctx.s;
@@ -1853,7 +1854,7 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
   const unsigned T = 256;
   const unsigned gc = grid_for(c, T);
   const uint64_t words = (c + 31) / 32;
-  const bool anchored = !ctx.dense_scan && !ctx.sort_scan;
+  const bool anchored = !dense && !ctx.sort_scan;
   const GramP gp = choose_gram(b, r, c);
   const uint64_t acap = anchored ? pow2_at_least(2 * (c + 2)) : 0;
   GramP gq = gp;
@@ -1937,7 +1938,7 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start) {
   BT_TRY(A.reserve());
   carve();
 
-  BT_TRY(alloc_level_arrays(v, words, s));
+  if (!v.mw) BT_TRY(alloc_level_arrays(v, words, s));
 
   InitArgs ia{W.bt, bcap, W.pt, pcap, W.mismatch, c,
               atab, acap, bitmap, bwords, secbits, qn, W.ld};
@@ -2078,16 +2079,20 @@ int all_levels(const M& m, BuildCtx& ctx) {
   QuickBuild qb(ctx.s);
   Scratch hm(ctx.s);
   if (!ctx.dense_scan && !ctx.sort_scan && r.b >= kQuickMinB) BT_TRY(quick_list(ctx, qb));
+  qb.expand = [&]() -> int {
+    if (ctx.H) return BT_OK;
+    BT_TRY(hm.alloc(&ctx.H, t->n + 1));
+    return expand_prefix(ctx.T, t->n, t->B, t->q, ctx.Hs, ctx.H, ctx.s);
+  };
   for (uint32_t l = 0; l < t->L; l++) {
     auto h0 = std::chrono::steady_clock::now();
-    if (qb.ready && t->lv[l].b >= kQuickMinB) {
-      BT_TRY(quick_level(ctx, qb, l, last_start));
+    const bool quick = qb.ready && t->lv[l].b >= kQuickMinB;
+    const int rc = quick ? quick_level(ctx, qb, l, last_start) : kEveryWindow;
+    if (rc == kEveryWindow) {
+      BT_TRY(qb.expand());
+      BT_TRY(level_pass(m, ctx, l, last_start, quick || ctx.dense_scan));
     } else {
-      if (!ctx.H) {
-        BT_TRY(hm.alloc(&ctx.H, t->n + 1));
-        BT_TRY(expand_prefix(ctx.T, t->n, t->B, t->q, ctx.Hs, ctx.H, ctx.s));
-      }
-      BT_TRY(level_pass(m, ctx, l, last_start));
+      BT_TRY(rc);
     }
     last_start = ctx.st_host->last_start;
     if (trace) {

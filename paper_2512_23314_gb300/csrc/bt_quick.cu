@@ -40,6 +40,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdio>
+#include <type_traits>
 
 #include "bt_quick_dev.cuh"
 
@@ -266,6 +267,7 @@ __global__ void __launch_bounds__(kT) k_quick_min(QGeo g, QList Q, unsigned G, u
                                                   QuickStatus* qs) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     qs->nopen[0] = qs->nopen[1] = qs->npairs = qs->nsusp = qs->nitems = 0;
+    qs->redo = kSearchDone;
     qs->total = Q.idx[Q.nw];
   }
   quick_min(g, Q, G, A, X, flags, grid_span());
@@ -276,28 +278,36 @@ __global__ void __launch_bounds__(kT) k_quick_compare(QGeo g, const uint32_t* __
   quick_compare(g, A, X, flags, ppk, L, grid_span());
 }
 
-__global__ void __launch_bounds__(kT) k_chase_init(Chase C, uint32_t bwords) { chase_init(C, bwords, grid_span()); }
+__global__ void __launch_bounds__(kT) k_chase_init(Chase C, uint32_t bwords, bool again) { chase_init(C, bwords, again, grid_span()); }
 
 template <class M, unsigned G>
 __global__ void __launch_bounds__(kT) k_chase_keys(M m, const __grid_constant__ PrefixConst<M> P, const uint64_t* Hs, Chase C) {
   chase_keys<M, G>(m, PrefixAt<M>(P, C.g.T, C.g.n, Hs), C, grid_span());
 }
 
-template <class M>
+template <class M, class FIRST>
 __global__ void __launch_bounds__(kT, 4) k_chase_scan(M m, const __grid_constant__ PrefixConst<M> P, const uint64_t* Hs,
                                                       const __grid_constant__ Chase C, uint32_t e0, uint32_t e1,
-                                                      uint32_t smem_words, const unsigned long long* __restrict__ bound2) {
+                                                      uint32_t smem_words, const unsigned long long* __restrict__ bound2,
+                                                      unsigned long long limit, ChaseState verdict) {
   extern __shared__ uint32_t bits_s[];
   __shared__ uint2 hit_q[kT / 32][kHitQ];
+  __shared__ uint8_t gap_q[FIRST::value ? kT / 32 : 1][kHitQ];
   __shared__ uint32_t cand_q[kT / 32][kCandQ];
   for (uint32_t i = threadIdx.x; i < smem_words; i += kT) bits_s[i] = C.bitmap[i];
   __syncthreads();
   const unsigned warp = threadIdx.x >> 5;
-  chase_scan(m, PrefixAt<M>(P, C.g.T, C.g.n, Hs), C, e0, e1, smem_words ? bits_s : C.bitmap, hit_q[warp], cand_q[warp],
-             bound2, grid_span());
+  chase_scan(m, PrefixAt<M>(P, C.g.T, C.g.n, Hs), C, FIRST{}, e0, e1, smem_words ? bits_s : C.bitmap, hit_q[warp],
+             gap_q[FIRST::value ? warp : 0], cand_q[warp], bound2, limit, verdict, grid_span());
 }
 
-__global__ void __launch_bounds__(kT) k_chase_bound(Chase C) { chase_bound(C, grid_span()); }
+// (After the sample: too much work in it?)
+__global__ void __launch_bounds__(kT) k_chase_bound(Chase C, unsigned long long most) {
+  const uint64_t work = C.qs->work;
+  const uint32_t redo = C.qs->redo;
+  chase_bound(C, grid_span());
+  if (blockIdx.x == 0 && threadIdx.x == 0 && redo == kSearchDone && work > most) C.qs->redo = kCompare;
+}
 
 __global__ void __launch_bounds__(kT) k_chase_live(Chase C, uint32_t split) { chase_live(C, split, grid_span()); }
 
@@ -305,7 +315,10 @@ __global__ void __launch_bounds__(kT) k_chase_tail(Chase C) { chase_tail(C, grid
 
 __global__ void __launch_bounds__(kT) k_chase_verify(Chase C, uint64_t ppk, unsigned L) { chase_verify(C, ppk, L, grid_span()); }
 
-__global__ void __launch_bounds__(kT) k_chase_apply(Chase C) { chase_apply(C, grid_span()); }
+// (What a search that was given up has found is not the answer.)
+__global__ void __launch_bounds__(kT) k_chase_apply(Chase C) {
+  if (C.qs->redo == kSearchDone) chase_apply(C, grid_span());
+}
 
 __global__ void __launch_bounds__(kT) k_chase_exact(Chase C, uint64_t nsusp) {
   chase_exact(C, blockIdx.y, gridDim.y, nsusp, grid_span());
@@ -638,14 +651,120 @@ int quick_list(BuildCtx& ctx, QuickBuild& qb) {
   return BT_OK;
 }
 
+// The search of a level's open keys: its tables, the list's two parts (the first
+// sixteenth, then the rest against the bounds it lowered: most copies' content is
+// first seen early; short lists have one part), and the launches of its steps.
+struct SearchRun {
+  Chase C;
+  uint64_t ni, gcap, top;
+  uint32_t bwords, total, split;
+};
+
 template <class M>
-static int chase(const M& m, BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint64_t last_start, const uint32_t* A,
-                 const uint32_t* X, const uint32_t* items, uint64_t* lo, uint8_t* ps) {
+struct Search {
+  const M& m;
+  BuildCtx& ctx;
+  QuickBuild& qb;
+  SearchRun& R;
+  const PrefixConst<M> P;
+  cudaStream_t s;
+  const uint64_t n;
+  Search(const M& m_, BuildCtx& ctx_, QuickBuild& qb_, SearchRun& R_)
+      : m(m_), ctx(ctx_), qb(qb_), R(R_), P(m_, ctx_.t->B), s(ctx_.s), n(ctx_.t->n) {}
+
+  static constexpr unsigned long long kAny = ~0ull;
+
+  int keys(bool first, bool again, unsigned long long probes = kAny) {
+    R.C.first = first;
+    R.C.probes = probes;
+    BT_LAUNCH(k_chase_init<<<grid_for(R.top, kT), kT, 0, s>>>(R.C, R.bwords, again));
+    if (R.C.g.b <= 256) BT_LAUNCH(k_chase_keys<M, 1><<<grid_for(R.ni, kT), kT, 0, s>>>(m, P, ctx.Hs, R.C));
+    else BT_LAUNCH(k_chase_keys<M, 32><<<grid_for(R.ni * 32, kT), kT, 0, s>>>(m, P, ctx.Hs, R.C));
+    return BT_OK;
+  }
+  int scan(uint32_t e0, uint32_t e1, bool bounded, unsigned long long limit, ChaseState verdict) {
+    if (e1 <= e0) return BT_OK;
+    const uint32_t sw = R.bwords <= kChaseBitWords ? R.bwords : 0;
+    const unsigned grid = (unsigned)std::min<uint64_t>((e1 - e0 + 8ull * kChaseTile - 1) / (8 * kChaseTile), 152 * 4);
+    auto launch = [&](auto kernel) {
+      BT_LAUNCH(kernel<<<grid, kT, sw * 4, s>>>(m, P, ctx.Hs, R.C, e0, e1, sw, bounded ? R.C.bound2 : nullptr, limit, verdict));
+    };
+    if (R.C.first) launch(k_chase_scan<M, std::true_type>);
+    else launch(k_chase_scan<M, std::false_type>);
+    return BT_OK;
+  }
+  // The second part against the bounds of what was found so far, unless that
+  // was more work than `most`.
+  int rest(unsigned long long most, unsigned long long limit) {
+    BT_LAUNCH(k_chase_bound<<<grid_for(R.ni, kT), kT, 0, s>>>(R.C, most));
+    BT_CUDA(cudaMemsetAsync(R.C.bitmap, 0, R.bwords * 4, s));
+    BT_LAUNCH(k_chase_live<<<grid_for(R.gcap, kT), kT, 0, s>>>(R.C, R.split));
+    return scan(R.split, R.total, true, limit, kGiveUp);
+  }
+  int finish() {
+    const QGeo& g = R.C.g;
+    if (R.C.r && R.C.r < kQuickMinB) BT_LAUNCH(k_chase_tail<<<grid_for(n / 16 + 1, kT, 152 * 8), kT, 0, s>>>(R.C));
+    const uint64_t ppk = (2 * g.b + q_piece(g.b) - 1) / q_piece(g.b);
+    const unsigned L = g.b >= 256 ? 32u : g.b >= 128 ? 16u : g.b >= 64 ? 8u : 4u;
+    BT_LAUNCH(k_chase_verify<<<grid_for(R.ni * ppk * L, kT), kT, 0, s>>>(R.C, ppk, L));
+    BT_LAUNCH(k_chase_apply<<<grid_for(R.ni, kT, 152 * 4), kT, 0, s>>>(R.C));
+    BT_CUDA(cudaGetLastError());
+    return BT_OK;
+  }
+  int wait() {
+    BT_CUDA(cudaGetLastError());
+    BT_CUDA(cudaMemcpyAsync(qb.qs_host, qb.qs, sizeof(QuickStatus), cudaMemcpyDeviceToHost, s));
+    BT_CUDA(cudaStreamSynchronize(s));
+    return BT_OK;
+  }
+
+  // By newest grams, all steps without a look at the host.
+  int newest() {
+    BT_TRY((allow_smem<k_chase_scan<M, std::false_type>>(kChaseBitWords * 4)));
+    BT_TRY((allow_smem<k_chase_scan<M, std::true_type>>(kChaseBitWords * 4)));
+    BT_TRY(keys(false, false, probes_most(R.ni)));
+    {
+      ProfScope prof("window_scan", s, 0);  // (the level's bytes are counted by its first part)
+      BT_TRY(scan(0, R.split ? R.split : R.total, false, work_most(n, R.split != 0), kTryFirst));
+      if (R.split) BT_TRY(rest(work_sample(n), work_most(n, false)));
+    }
+    return finish();
+  }
+  // What the host does when the status says that the search is not done;
+  // kEveryWindow: that is the better way.
+  int others() {
+    const QuickStatus* q = qb.qs_host;
+    if (q->redo == kGiveUp) return kEveryWindow;
+    ProfScope prof("window_scan", s, 0);
+    const unsigned long long few = R.split ? work_few(n) : work_most(n, false);
+    const unsigned long long by_newest = q->redo == kCompare ? q->work : kAny, before = q->work;
+    BT_TRY(keys(true, true));
+    BT_TRY(scan(0, R.split ? R.split : R.total, false, before + few, kGiveUp));
+    BT_TRY(wait());
+    const unsigned long long by_first = q->redo ? kAny : q->work - before;
+    if (std::min(by_newest, by_first) > few) return kEveryWindow;
+    if (R.split) {
+      if (by_newest < by_first) BT_TRY(keys(false, true));
+      BT_TRY(rest(kAny, q->work + work_most(n, false)));
+      BT_TRY(wait());
+      if (q->redo) return kEveryWindow;
+    }
+    return finish();
+  }
+  // Without memory for the scan of every window: whatever it takes.
+  int all() {
+    BT_TRY(keys(false, true));
+    BT_TRY(scan(0, R.total, false, kAny, kGiveUp));
+    return finish();
+  }
+};
+
+static int search_tables(BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint64_t last_start, const uint32_t* A,
+                         const uint32_t* X, const uint32_t* items, uint64_t* lo, uint8_t* ps, SearchRun& R) {
   bt_tree* t = ctx.t;
-  cudaStream_t s = ctx.s;
   const uint64_t nb = qb.qs_host->nopen[0], np = qb.qs_host->nopen[1], ni = nb + np;
   const uint64_t len_last = g.n - last_start;
-  Chase C;
+  Chase& C = R.C;
   C.g = g;
   C.Q = qb.list;
   C.A = A;
@@ -653,12 +772,13 @@ static int chase(const M& m, BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint6
   C.items = items;
   C.nitems = (uint32_t)ni;
   C.r = len_last < g.b ? len_last : 0;
-  C.Bb = pow_mod(m, t->B, g.b);
-  C.Br = C.r ? pow_mod(m, t->B, C.r) : 0;
+  auto power = [&](uint64_t e) { return t->q == Mersenne61::Q ? pow_mod(Mersenne61{}, t->B, e) : pow_mod(SmallMod{t->q}, t->B, e); };
+  C.Bb = power(g.b);
+  C.Br = C.r ? power(C.r) : 0;
   const uint64_t bcap = pow2_from(2 * (nb + 2 * np)), pcap = pow2_from(2 * np), gcap = pow2_from(4 * ni);  // (2 ni: DNA 2 GiB 41.5 ms, not 40.8)
   uint32_t fbits = 12;
   while ((1ull << fbits) < 16 * ni && fbits < 30) fbits++;
-  const uint32_t bwords = 1u << (fbits - 5);
+  R.bwords = 1u << (fbits - 5);
   C.bmask = (uint32_t)(bcap - 1);
   C.pmask = (uint32_t)(pcap - 1);
   C.gmask = (uint32_t)(gcap - 1);
@@ -667,60 +787,50 @@ static int chase(const M& m, BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint6
   C.status = ctx.st;
   C.lo = lo;
   C.ps = ps;
-  Arena& R = qb.open;
+  Arena& A2 = qb.open;
   auto carve = [&]() {
-    C.bt = R.take<CSlot>(bcap);
-    C.pt = R.take<CPair>(pcap);
-    C.gt = R.take<CGram>(gcap);
-    C.bound2 = R.take<unsigned long long>(gcap);
-    C.bitmap = R.take<uint32_t>(bwords);
-    C.islot = R.take<uint32_t>(ni);
-    C.igram = R.take<uint32_t>(ni);
-    C.differ = R.take<uint32_t>(ni);
-    C.susp = R.take<uint32_t>(ni);
-    C.exlo = R.take<unsigned long long>(ni);
+    C.bt = A2.take<CSlot>(bcap);
+    C.pt = A2.take<CPair>(pcap);
+    C.gt = A2.take<CGram>(gcap);
+    C.bound2 = A2.take<unsigned long long>(gcap);
+    C.bitmap = A2.take<uint32_t>(R.bwords);
+    C.islot = A2.take<uint32_t>(ni);
+    C.igram = A2.take<uint32_t>(ni);
+    C.differ = A2.take<uint32_t>(ni);
+    C.susp = A2.take<uint32_t>(ni);
+    C.exlo = A2.take<unsigned long long>(ni);
   };
-  R.begin_dry();
+  A2.begin_dry();
   carve();
-  BT_TRY(R.reserve());
+  BT_TRY(A2.reserve());
   carve();
-  const PrefixConst<M> P(m, t->B);
-  BT_TRY(allow_smem<k_chase_scan<M>>(kChaseBitWords * 4));
-  const uint64_t top = std::max<uint64_t>(std::max(bcap, pcap), std::max<uint64_t>(gcap, bwords));
-  BT_LAUNCH(k_chase_init<<<grid_for(top, kT), kT, 0, s>>>(C, bwords));
-  if (g.b <= 256) BT_LAUNCH(k_chase_keys<M, 1><<<grid_for(ni, kT), kT, 0, s>>>(m, P, ctx.Hs, C));
-  else BT_LAUNCH(k_chase_keys<M, 32><<<grid_for(ni * 32, kT), kT, 0, s>>>(m, P, ctx.Hs, C));
-  {
-    ProfScope prof("window_scan", s, 0);  // (the level's bytes are counted by its first part)
-    // Two halves: the first sixteenth of the list, then the rest against the
-    // bounds it lowered (most copies' content is first seen early).
-    const uint32_t total = qb.qs_host->total;
-    const uint32_t split = total > (1u << 20) ? (total / 16) & ~(8 * kChaseTile - 1) : 0;
-    const uint32_t sw = bwords <= kChaseBitWords ? bwords : 0;
-    auto grid = [](uint64_t n) { return (unsigned)std::min<uint64_t>((n + 8 * kChaseTile - 1) / (8 * kChaseTile), 152 * 4); };
-    if (split) {
-      BT_LAUNCH(k_chase_scan<M><<<grid(split), kT, sw * 4, s>>>(m, P, ctx.Hs, C, 0, split, sw, nullptr));
-      BT_LAUNCH(k_chase_bound<<<grid_for(ni, kT), kT, 0, s>>>(C));
-      BT_CUDA(cudaMemsetAsync(C.bitmap, 0, bwords * 4, s));
-      BT_LAUNCH(k_chase_live<<<grid_for(gcap, kT), kT, 0, s>>>(C, split));
-    }
-    if (total)
-      BT_LAUNCH(k_chase_scan<M><<<grid(total - split), kT, sw * 4, s>>>(m, P, ctx.Hs, C, split, total, sw,
-                                                                       split ? C.bound2 : nullptr));
-    if (C.r && C.r < 27) BT_LAUNCH(k_chase_tail<<<grid_for(g.n / 16 + 1, kT, 152 * 8), kT, 0, s>>>(C));
-  }
-  const uint64_t ppk = (2 * g.b + q_piece(g.b) - 1) / q_piece(g.b);
-  const unsigned L = g.b >= 256 ? 32u : g.b >= 128 ? 16u : g.b >= 64 ? 8u : 4u;
-  BT_LAUNCH(k_chase_verify<<<grid_for(ni * ppk * L, kT), kT, 0, s>>>(C, ppk, L));
-  BT_LAUNCH(k_chase_apply<<<grid_for(ni, kT, 152 * 4), kT, 0, s>>>(C));
+  R.ni = ni;
+  R.gcap = gcap;
+  R.top = std::max<uint64_t>(std::max(bcap, pcap), std::max<uint64_t>(gcap, R.bwords));
+  R.total = qb.qs_host->total;
+  R.split = R.total > (1u << 20) ? (R.total / 16) & ~(8 * kChaseTile - 1) : 0;
+  return BT_OK;
+}
+
+enum class How { kNewest, kOthers, kAll };
+
+template <class M>
+static int search_as(const M& m, BuildCtx& ctx, QuickBuild& qb, SearchRun& R, How how) {
+  Search<M> S(m, ctx, qb, R);
+  return how == How::kNewest ? S.newest() : how == How::kOthers ? S.others() : S.all();
+}
+
+static int search_open(BuildCtx& ctx, QuickBuild& qb, SearchRun& R, How how) {
+  const uint64_t q = ctx.t->q;
+  return q == Mersenne61::Q ? search_as(Mersenne61{}, ctx, qb, R, how) : search_as(SmallMod{q}, ctx, qb, R, how);
+}
+
+// Exact leftmost occurrences of the keys whose fingerprint match was false.
+static int search_exact(BuildCtx& ctx, const SearchRun& R, uint64_t nsusp) {
+  const dim3 grid(grid_for(R.C.g.n, kT, 1024), (unsigned)std::min<uint64_t>(nsusp, 1024));
+  BT_LAUNCH(k_chase_exact<<<grid, kT, 0, ctx.s>>>(R.C, nsusp));
+  BT_LAUNCH(k_chase_exact_apply<<<grid_for(nsusp, kT), kT, 0, ctx.s>>>(R.C, nsusp));
   BT_CUDA(cudaGetLastError());
-  qb.resolve_exact = [=](uint64_t nsusp) -> int {
-    const dim3 grid(grid_for(g.n, kT, 1024), (unsigned)std::min<uint64_t>(nsusp, 1024));
-    BT_LAUNCH(k_chase_exact<<<grid, kT, 0, s>>>(C, nsusp));
-    BT_LAUNCH(k_chase_exact_apply<<<grid_for(nsusp, kT), kT, 0, s>>>(C, nsusp));
-    BT_CUDA(cudaGetLastError());
-    return BT_OK;
-  };
   return BT_OK;
 }
 
@@ -778,14 +888,32 @@ int quick_level(BuildCtx& ctx, QuickBuild& qb, uint32_t l, uint64_t last_start) 
   BT_TRY(rank_and_wait());
   const QuickStatus q0 = *qb.qs_host;
   if (q0.nitems) {
-    if (t->q == Mersenne61::Q) BT_TRY(chase(Mersenne61{}, ctx, qb, g, last_start, A, X, items, v.lo, ps));
-    else BT_TRY(chase(SmallMod{t->q}, ctx, qb, g, last_start, A, X, items, v.lo, ps));
-    BT_LAUNCH(k_quick_remark<<<grid_for(words * 32, kT), kT, 0, s>>>(c, ps, v.mw, wpop));
-    BT_TRY(rank_and_wait());
-    if (qb.qs_host->nsusp) {
-      BT_TRY(qb.resolve_exact(qb.qs_host->nsusp));
+    SearchRun run;
+    BT_TRY(search_tables(ctx, qb, g, last_start, A, X, items, v.lo, ps, run));
+    auto remark = [&]() -> int {
       BT_LAUNCH(k_quick_remark<<<grid_for(words * 32, kT), kT, 0, s>>>(c, ps, v.mw, wpop));
-      BT_TRY(rank_and_wait());
+      return rank_and_wait();
+    };
+    BT_TRY(search_open(ctx, qb, run, How::kNewest));
+    BT_TRY(remark());
+    if (qb.qs_host->redo) {
+      int rc = search_open(ctx, qb, run, How::kOthers);
+      if (rc == kEveryWindow) {
+        rc = qb.expand();
+        if (rc == BT_OK) {
+          qb.open.release();  // (room for the scan's tables)
+          return kEveryWindow;
+        }
+        if (rc != BT_ENOMEM) return rc;
+        cudaGetLastError();
+        rc = search_open(ctx, qb, run, How::kAll);
+      }
+      BT_TRY(rc);
+      BT_TRY(remark());
+    }
+    if (qb.qs_host->nsusp) {
+      BT_TRY(search_exact(ctx, run, qb.qs_host->nsusp));
+      BT_TRY(remark());
     }
   }
   uint64_t* next_st = nullptr;

@@ -28,8 +28,11 @@ struct QuickStatus {
   unsigned long long nitems, npairs, nmarked, nsusp;
   unsigned long long fp_tail, lo_tail, lo_tailpair;  // keys that end in the short last block
   unsigned long long cands, hits;
+  unsigned long long work;    // of the search of the open keys (kWalkWork, kTestWork)
+  unsigned long long probes;  // slots passed by the long walks of their registration
   unsigned int pretail, tail_F, tail_off;
   unsigned int total;  // entries of the list
+  unsigned int redo;   // how far the search of the open keys is (ChaseState)
 };
 
 struct QuickBuild {
@@ -40,10 +43,13 @@ struct QuickBuild {
   QList list{};
   QuickStatus* qs = nullptr;
   QuickStatus* qs_host = nullptr;  // in the thread's pinned page
-  std::function<int(uint64_t)> resolve_exact;
+  std::function<int()> expand;  // ctx.H for the scan of every window
   explicit QuickBuild(cudaStream_t s) : mem(s) { open.s = s; }
   ~QuickBuild() { open.release(); }
 };
+
+// Returned by quick_level: this level goes by the scan of every window.
+constexpr int kEveryWindow = -1;
 
 int quick_list(BuildCtx& ctx, QuickBuild& qb);
 int quick_level(BuildCtx& ctx, QuickBuild& qb, uint32_t l, uint64_t last_start);

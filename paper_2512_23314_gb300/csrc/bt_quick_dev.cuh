@@ -294,6 +294,16 @@ __device__ __forceinline__ uint8_t pair_state(const QGeo& g, const uint32_t* A, 
 // last start of a key with that pair, and a proposed window's fingerprint is
 // looked up among the open blocks (and, joined with the one at p + b, among
 // the open pairs).  A gram is named by its first position F.
+//
+// Where few grams make up the text (records from few values, words in any order,
+// two letters), many keys have the same newest gram, each at an offset of its
+// own, and a window is proposed once for every gram it holds: up to hundreds of
+// windows per text position.  Two other ways are tried then.  The keys go by their
+// *first* gram: of any 12 consecutive grams one is selected, so its offset is at
+// most 11, and the first gram of a window is the list's next entry, so an entry at
+// x proposes only windows after the entry before it, each window once.  That is
+// little where keys start at few places of the grams (records), and a window per
+// position where they start anywhere; then every window is scanned.
 // ---------------------------------------------------------------------------
 struct __align__(32) CSlot {  // a block fingerprint: leftmost window, last start of an open pair beginning with it
   unsigned long long key, lo, maxpst, pad;
@@ -305,7 +315,31 @@ struct __align__(16) CGram {  // F << 32 | offset; windows from `bound` on are o
   unsigned long long key, bound;
 };
 
+// When a search is given up.  Its work is counted in steps of a warp's walk over
+// the gram table (about 0.45 ns each with the whole GPU), and six for testing 32
+// windows (2.9 ns); the scan of every window costs about n / 26 of these (4.6 ms on
+// 256 MiB).  With a list long enough for two parts the first sixteenth is a
+// sample: above n / 512 there (versions and copies stay below n / 800), or given up
+// at n / 64, first grams are tried on the same sixteenth, and the better way takes
+// the rest unless both are above n / 256.  No search goes on beyond n / 16.  The
+// registration is given up too: keys that share a gram stand in one run of slots,
+// which each passes (80 ns a slot: 4 M keys of two-letter text took 30 ms).
+enum ChaseState : uint32_t {
+  kSearchDone = 0,
+  kCompare = 1,   // the sample is done, and much work
+  kTryFirst = 2,  // registration or sample given up
+  kGiveUp = 3,
+};
+constexpr uint32_t kWalkWork = 1, kTestWork = 6;
+__host__ __device__ inline uint64_t work_sample(uint64_t n) { return n / 512; }
+__host__ __device__ inline uint64_t work_few(uint64_t n) { return n / 256 + 4096; }
+__host__ __device__ inline uint64_t work_most(uint64_t n, bool sample) { return (sample ? n / 64 : n / 16) + 4096; }
+constexpr uint32_t kLongProbe = 64;  // slots; a walk counts from there on
+__host__ __device__ inline uint64_t probes_most(uint64_t nitems) { return 4 * nitems + (1u << 16); }
+
 struct Chase {
+  bool first;              // keys go by their first gram (otherwise by their newest)
+  uint64_t probes;         // most slots passed by long walks before the registration is given up
   QGeo g;
   QList Q;
   const uint32_t* A;
@@ -370,38 +404,48 @@ __device__ __forceinline__ void c_min(unsigned long long* a, uint64_t p) {
   if (*(volatile unsigned long long*)a > p) atomicMin(a, (unsigned long long)p);
 }
 
-__device__ __forceinline__ void chase_init(const Chase& C, uint32_t bwords, Span w) {
+// `again`: the gram table alone (the keys' tables and what was found stay).
+__device__ __forceinline__ void chase_init(const Chase& C, uint32_t bwords, bool again, Span w) {
   uint64_t top = (uint64_t)C.bmask + 1;
   top = top > (uint64_t)C.pmask + 1 ? top : (uint64_t)C.pmask + 1;
   top = top > (uint64_t)C.gmask + 1 ? top : (uint64_t)C.gmask + 1;
   top = top > bwords ? top : bwords;
   for (uint64_t i = w.tid; i < top; i += w.n) {
-    if (i <= C.bmask) C.bt[i] = CSlot{kNone, kNone, 0, 0};
-    if (i <= C.pmask) C.pt[i] = CPair{kNone, kNone};
+    if (i <= C.bmask && !again) C.bt[i] = CSlot{kNone, kNone, 0, 0};
+    if (i <= C.pmask && !again) C.pt[i] = CPair{kNone, kNone};
     if (i <= C.gmask) {
       C.gt[i] = CGram{kNone, 0};
       C.bound2[i] = 0;
     }
     if (i < bwords) C.bitmap[i] = 0;
-    if (i < C.nitems) C.differ[i] = 0;
+    if (i < C.nitems) {
+      C.differ[i] = 0;
+      C.igram[i] = C.islot[i] = kNoSlot;  // (a registration that is given up leaves some)
+    }
     if (i == 0) {
+      C.qs->tail_F = C.qs->tail_off = 0xFFFFFFFFu;
+      C.qs->redo = kSearchDone;
+      C.qs->probes = 0;
+    }
+    if (i == 0 && !again) {
       C.qs->fp_tail = C.qs->lo_tail = C.qs->lo_tailpair = kNone;
       C.qs->pretail = kNoSlot;
-      C.qs->tail_F = C.qs->tail_off = 0xFFFFFFFFu;
-      C.qs->cands = C.qs->hits = 0;
+      C.qs->cands = C.qs->hits = C.qs->work = 0;
     }
   }
 }
 
 // G lanes per open key (one when blocks are short, else a warp): the list entry
-// with the key's min D, then (one lane) the tables.  A pair enters both of its
-// blocks.
+// with the key's min D (or its first entry), then (one lane) the tables.  A pair
+// enters both of its blocks.
 template <class M, unsigned G>
 __device__ __forceinline__ void chase_keys(const M& m, const PrefixAt<M>& H, const Chase& C, Span w) {
   const unsigned gl = threadIdx.x % G;
   const QGeo& g = C.g;
   for (uint64_t i = w.tid / G; i < C.nitems; i += w.n / G) {
     const uint32_t it = C.items[i];
+    const bool given_up = *(volatile unsigned int*)&C.qs->redo != kSearchDone;
+    if (G == 1 ? given_up : __any_sync(0xFFFFFFFFu, given_up)) return;  // (a warp's lanes together: they vote below)
     const uint64_t k = it >> 1;
     const bool pair = it & 1;
     const uint64_t s = g.st[k], len = g.n - s < g.b ? g.n - s : g.b;
@@ -414,24 +458,22 @@ __device__ __forceinline__ void chase_keys(const M& m, const PrefixAt<M>& H, con
       const uint32_t e1 = list_at(C.Q, (end + 31) / 32);
       for (uint32_t e0 = list_at(C.Q, s / 32); e0 < e1 && !found; e0 += G) {
         const uint32_t e = e0 + gl;
-        const uint32_t x = e < e1 ? C.Q.x[e] : 0;
-        const bool hit = e < e1 && C.Q.D[e] == d && x >= s && x < end;
+        const uint32_t x = e < e1 ? C.Q.x[e] : 0, D = e < e1 ? C.Q.D[e] : 0;
+        const bool hit = e < e1 && x >= s && x < end && (C.first || D == d);
         if (G == 1) {
           found = hit;
-          if (hit) F = x - d, off = (uint32_t)(x - s);
+          if (hit) F = x - D, off = (uint32_t)(x - s);
         } else {
           const unsigned bal = __ballot_sync(0xFFFFFFFFu, hit);
           found = bal != 0;
           if (found) {
             const uint32_t fx = __shfl_sync(0xFFFFFFFFu, x, __ffs(bal) - 1);
-            F = fx - d, off = (uint32_t)(fx - s);
+            F = fx - __shfl_sync(0xFFFFFFFFu, D, __ffs(bal) - 1), off = (uint32_t)(fx - s);
           }
         }
       }
     }
     if (gl) continue;
-    C.igram[i] = kNoSlot;
-    C.islot[i] = kNoSlot;
     const bool tail = !pair && len != g.b;
     if (found && !tail) {
       uint32_t h = c_gram_home(F, C.gmask);
@@ -442,11 +484,16 @@ __device__ __forceinline__ void chase_keys(const M& m, const PrefixAt<M>& H, con
         if (old == kNone) old = atomicCAS(&C.gt[h].key, (unsigned long long)kNone, key);
         if (old == kNone || old == key) placed = true;
         else h = (h + 1) & C.gmask;
+        if (q % kLongProbe == kLongProbe - 1 && !placed &&
+            atomicAdd(&C.qs->probes, (unsigned long long)kLongProbe) >= C.probes) {
+          C.qs->redo = kTryFirst;
+          break;
+        }
       }
       if (placed) {
         atomicMax(&C.gt[h].bound, (unsigned long long)s);
         C.igram[i] = h;
-      } else {
+      } else if (!C.qs->redo) {
         atomicExch(&C.status->error, 21ull);
       }
     }
@@ -534,17 +581,31 @@ __device__ __forceinline__ void chase_test(const M& m, const PrefixAt<M>& H, con
 constexpr uint32_t kChaseTile = 256;                 // entries per warp and step, eight per lane
 constexpr uint32_t kHitQ = kChaseTile + 32, kCandQ = 64;
 constexpr uint32_t kChaseBitWords = 4096;            // bitmap kept in shared memory up to 16 KiB
+constexpr uint32_t kChaseReport = 256;               // work of a warp before it adds it to the level's
 
-// hq, cq: the warp's queues; bits: the bitmap (shared or global memory).
-template <class M>
-__device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, const Chase& C, uint32_t e0, uint32_t e1,
-                                           const uint32_t* bits, uint2* hq, uint32_t* cq,
-                                           const unsigned long long* bound2, Span w) {
+// hq, cq: the warp's queues; gq: for first grams, the distance of each hit to
+// the entry before it; bits: the bitmap (shared or global memory).  Above a work of
+// `limit` on the level in all it stops and leaves `verdict` in C.qs->redo.  first:
+// as C.first, or that value as a type.
+template <class M, class FIRST>
+__device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, const Chase& C, FIRST first, uint32_t e0, uint32_t e1,
+                                           const uint32_t* bits, uint2* hq, uint8_t* gq, uint32_t* cq,
+                                           const unsigned long long* bound2, unsigned long long limit,
+                                           ChaseState verdict, Span w) {
   const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
   uint32_t hn = 0, cn = 0;  // warp-uniform
   const uint32_t tail_F = C.qs->tail_F, tail_off = C.qs->tail_off, pretail = C.qs->pretail;
   const uint64_t fp_tail = C.qs->fp_tail;
-  uint32_t ncand = 0, nhit = 0;
+  const uint32_t given_up = *(volatile unsigned int*)&C.qs->redo;  // (before, or just now: looked at with the first tile)
+  uint32_t ncand = 0, nhit = 0, work = 0;  // ncand, work (since the last report): warp-uniform
+  bool stop = false;
+  auto report = [&]() {
+    unsigned long long all = 0;
+    if (lane == 0) all = atomicAdd(&C.qs->work, (unsigned long long)work) + work;
+    work = 0;
+    stop = __shfl_sync(0xFFFFFFFFu, all > limit, 0);
+    if (stop && lane == 0) C.qs->redo = verdict;
+  };
   // 32 proposed windows (fewer at the end).
   auto take_cands = [&]() {
     const uint32_t n = cn < 32 ? cn : 32;
@@ -558,13 +619,14 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
   // its gram proposes a window.  (Walks end: half the slots are empty.)
   bool live = false;
   uint2 hit = make_uint2(0, 0);
-  uint32_t s = 0;
+  uint32_t s = 0, gap = 0xFFFFFFFFu;
   auto walk = [&]() {
     __syncwarp();
     const unsigned idle = __ballot_sync(0xFFFFFFFFu, !live);
     const uint32_t k = __popc(idle & lt), free = __popc(idle);
     if (!live && k < hn) {
       hit = hq[hn - 1 - k];
+      if (first) gap = gq[hn - 1 - k];
       s = c_gram_home(hit.y, C.gmask);
       live = true;
       if (hit.y == tail_F && tail_off <= hit.x) {
@@ -584,7 +646,7 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
       } else if ((uint32_t)(en.x >> 32) == hit.y) {
         const uint32_t off = (uint32_t)en.x;
         p = hit.x - off;
-        want = off <= hit.x && p < (bound2 ? bound2[s] : en.y);
+        want = off <= hit.x && (!first || off < gap) && p < (bound2 ? bound2[s] : en.y);
       }
       s = (s + 1) & C.gmask;
     }
@@ -592,14 +654,22 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
     if (bal) {
       if (want) cq[cn + __popc(bal & lt)] = p;
       cn += __popc(bal);
-      if (lane == 0) ncand += __popc(bal);
-      if (cn >= 32) take_cands();
+      ncand += __popc(bal);
+      if (cn >= 32) {
+        take_cands();
+        work += kTestWork;
+      }
+    }
+    work += kWalkWork;
+    if (work >= kChaseReport) {
+      report();
+      if (stop) live = false, hn = cn = 0;
     }
   };
   // (A short list is dealt out one entry a lane: eight would leave most warps
   // without and the others with eight times the steps one after the other.)
   const uint32_t per = e1 - e0 <= w.n ? 1 : kChaseTile / 32;
-  for (uint64_t t0 = e0 + w.tid / 32 * (32 * per); t0 < e1; t0 += w.n / 32 * (32 * per)) {
+  for (uint64_t t0 = e0 + w.tid / 32 * (32 * per); t0 < e1 && !stop; t0 += w.n / 32 * (32 * per)) {
     uint32_t x[8], F[8];
     uint32_t pass = 0;
     const uint64_t e = t0 + (uint64_t)per * lane;
@@ -626,19 +696,25 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
         pass |= ((bits[bit >> 5] >> (bit & 31)) & 1u) << u;
       }
     }
+    if (__any_sync(0xFFFFFFFFu, given_up)) break;
 #pragma unroll
     for (int u = 0; u < 8; u++) {
       const bool ok = (pass >> u) & 1u;
       const unsigned bal = __ballot_sync(0xFFFFFFFFu, ok);
-      if (ok) hq[hn + __popc(bal & lt)] = make_uint2(x[u], F[u]);
+      if (ok) {
+        const uint32_t at = hn + __popc(bal & lt);
+        hq[at] = make_uint2(x[u], F[u]);
+        // (The text's first entry proposes every window before it: 255 is more than any offset of a first gram.)
+        if (first) gq[at] = e + u ? (uint8_t)min(x[u] - (u ? x[u ? u - 1 : 0] : C.Q.x[e - 1]), 255u) : (uint8_t)255;
+      }
       hn += __popc(bal);
     }
     while (hn >= 32) walk();  // (unfinished walks go on with the next tile's)
   }
   while (hn || __any_sync(0xFFFFFFFFu, live)) walk();
   while (cn) take_cands();
-  ncand = __reduce_add_sync(0xFFFFFFFFu, ncand);
   nhit = __reduce_add_sync(0xFFFFFFFFu, nhit);
+  if (lane == 0 && work) atomicAdd(&C.qs->work, (unsigned long long)work);
   if (lane == 0 && ncand) atomicAdd(&C.qs->cands, (unsigned long long)ncand);
   if (lane == 0 && nhit) atomicAdd(&C.qs->hits, (unsigned long long)nhit);
 }

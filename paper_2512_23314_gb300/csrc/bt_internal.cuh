@@ -205,6 +205,22 @@ __device__ __forceinline__ uint32_t sum_run(const void* cnt, uint32_t w, uint64_
   return acc;
 }
 
+// The last nonzero one of the mark words, from their exclusive prefix popcounts
+// mr (total = mr[words] > 0): the last word, or a search for the last prefix below
+// the total.  Where only a text's first blocks are marked, walking down from the end
+// took 2 ms on a level of 4 M blocks.
+__device__ __forceinline__ uint64_t last_marked_word(const uint32_t* mw, const uint32_t* mr, uint64_t words,
+                                                     uint64_t total) {
+  if (mw[words - 1]) return words - 1;
+  uint64_t a = 0, z = words;  // mr[a] < total, mr[z] = total
+  while (z - a > 1) {
+    const uint64_t mid = (a + z) / 2;
+    if (mr[mid] < total) a = mid;
+    else z = mid;
+  }
+  return a;
+}
+
 constexpr int kMaxLevels = 64;
 
 struct TreeView {

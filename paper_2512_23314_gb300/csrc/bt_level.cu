@@ -1492,18 +1492,12 @@ __global__ void k_level_finish(Geo g, const uint32_t* __restrict__ mw, const uin
                                uint32_t arity, uint64_t bn, Status* status) {
   const uint64_t words = (g.c + 31) / 32;
   uint64_t nmarked = mr[words];
-  uint64_t last = kNone;
-  for (uint64_t w = words; w-- > 0;) {
-    if (mw[w]) {
-      last = w * 32 + 31 - __clz(mw[w]);
-      break;
-    }
-  }
-  if (last == kNone || arity == 0) {
+  if (nmarked == 0 || arity == 0) {
     status->next_c = 0;
     status->last_start = 0;
     return;
   }
+  const uint64_t w = last_marked_word(mw, mr, words, nmarked), last = w * 32 + 31 - __clz(mw[w]);
   uint64_t len = blen(g, last), nch = (len + bn - 1) / bn;
   status->next_c = (nmarked - 1) * arity + nch;
   status->last_start = g.st[last] + (nch - 1) * bn;

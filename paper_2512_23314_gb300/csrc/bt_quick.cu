@@ -445,27 +445,24 @@ __global__ void __launch_bounds__(kT) k_quick_remark(uint64_t c, const uint8_t* 
 }
 
 // Size of the next level and the start of its last block (one thread).
-__device__ void level_end(const QGeo& g, const uint32_t* mw, uint64_t words, uint64_t nmarked, uint32_t arity, uint64_t bn,
-                          Status* status, QuickStatus* qs) {
+__device__ void level_end(const QGeo& g, const uint32_t* mw, const uint32_t* mr, uint64_t words, uint64_t nmarked,
+                          uint32_t arity, uint64_t bn, Status* status, QuickStatus* qs) {
   qs->nmarked = nmarked;
   status->next_c = 0;
   status->last_start = 0;
-  if (arity == 0) return;
-  for (uint64_t w = words; w-- > 0;) {
-    if (!mw[w]) continue;
-    const uint64_t last = w * 32 + 31 - __clz(mw[w]);
-    const uint64_t len = qblen(g, last), nch = (len + bn - 1) / bn;
-    status->next_c = (nmarked - 1) * arity + nch;
-    status->last_start = g.st[last] + (nch - 1) * bn;
-    return;
-  }
+  if (arity == 0 || nmarked == 0) return;
+  const uint64_t w = last_marked_word(mw, mr, words, nmarked);
+  const uint64_t last = w * 32 + 31 - __clz(mw[w]);
+  const uint64_t len = qblen(g, last), nch = (len + bn - 1) / bn;
+  status->next_c = (nmarked - 1) * arity + nch;
+  status->last_start = g.st[last] + (nch - 1) * bn;
 }
 
 // Rank prefix of a level of at most kRankWords mark words and the level's end,
 // by one CTA (eight words per thread and step).
 constexpr uint64_t kRankWords = 16384;
 __global__ void __launch_bounds__(1024) k_quick_rank(QGeo g, const uint32_t* __restrict__ mw, const uint32_t* __restrict__ wpop,
-                                                     uint32_t* __restrict__ mr, uint32_t arity, uint64_t bn, Status* status,
+                                                     uint32_t* mr, uint32_t arity, uint64_t bn, Status* status,
                                                      QuickStatus* qs) {
   __shared__ uint32_t sm[32];
   const uint64_t words = (g.c + 31) / 32;
@@ -508,13 +505,13 @@ __global__ void __launch_bounds__(1024) k_quick_rank(QGeo g, const uint32_t* __r
   }
   if (threadIdx.x == 0) {
     mr[words] = carry;
-    level_end(g, mw, words, carry, arity, bn, status, qs);
+    level_end(g, mw, mr, words, carry, arity, bn, status, qs);
   }
 }
 __global__ void k_quick_end(QGeo g, const uint32_t* mw, const uint32_t* mr, uint32_t arity, uint64_t bn, Status* status,
                             QuickStatus* qs) {
   const uint64_t words = (g.c + 31) / 32;
-  level_end(g, mw, words, mr[words], arity, bn, status, qs);
+  level_end(g, mw, mr, words, mr[words], arity, bn, status, qs);
 }
 
 __device__ __forceinline__ bool qmark(const uint32_t* __restrict__ mw, uint64_t k) { return (mw[k >> 5] >> (k & 31)) & 1u; }

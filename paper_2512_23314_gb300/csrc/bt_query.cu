@@ -464,72 +464,78 @@ __device__ __forceinline__ uint32_t div_b(uint32_t x, const LevelView& v) {
   return v.bshift != 0xFFu ? x >> v.bshift : x / v.b;
 }
 
-// Occurrences of byte c in p[0, o): 16 bytes per load from a 16-byte aligned
-// start (a per-byte compare, __vcmpeq4, then a population count), four bytes
-// per step otherwise.
-__device__ __forceinline__ uint32_t leaf_count(const uint8_t* p, uint32_t o, uint32_t c) {
-  uint32_t x = 0, acc = 0;
-  const uint32_t cc = c * 0x01010101u;
-  if ((((uintptr_t)p) & 15) == 0) {
-    // (The leaf text is followed by 16 bytes, so the last unit is readable.)
-    for (; x < o; x += 16) {
-      const uint4 v = *(const uint4*)(p + x);
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-      const uint32_t left = o - x;
+// The bytes of one aligned 16-byte unit that equal c, 0xFF each, those before
+// byte `from` and from byte `to` on cleared.
+struct Eq16 {
+  uint32_t e[4];
+};
+__device__ __forceinline__ Eq16 unit_equals(const uint8_t* p, uint32_t cc, uint32_t from, uint32_t to) {
+  const uint4 v = *(const uint4*)p;
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  Eq16 r;
 #pragma unroll
-      for (uint32_t q = 0; q < 4; q++) {
-        uint32_t eq = __vcmpeq4(w[q], cc);
-        if (left < 4 * q + 4) eq = left <= 4 * q ? 0u : eq & ((1u << (8 * (left - 4 * q))) - 1u);
-        acc += __popc(eq);
-      }
-    }
-    return acc >> 3;
+  for (uint32_t q = 0; q < 4; q++) {
+    r.e[q] = __vcmpeq4(w[q], cc);
+    if (from > 4 * q) r.e[q] = from >= 4 * q + 4 ? 0u : r.e[q] & (0xFFFFFFFFu << (8 * (from - 4 * q)));
+    if (to < 4 * q + 4) r.e[q] = to <= 4 * q ? 0u : r.e[q] & ((1u << (8 * (to - 4 * q))) - 1u);
   }
-  for (; x < o && (((uintptr_t)(p + x)) & 3); x++) acc += p[x] == c;  // up to an aligned word
-  const uint32_t* w = (const uint32_t*)(p + x);
-  for (uint32_t i = 0; x + 4 <= o; x += 4, i++) acc += __popc(__vcmpeq4(w[i], cc)) >> 3;
-  for (; x < o; x++) acc += p[x] == c;
+  return r;
+}
+__device__ __forceinline__ uint32_t matches(const Eq16& r) {
+  return (__popc(r.e[0]) + __popc(r.e[1]) + __popc(r.e[2]) + __popc(r.e[3])) >> 3;
+}
+
+// Occurrences of byte c in p[0, o): aligned 16-byte units whatever p's alignment,
+// four in flight on long stretches.  (The leaf text starts at such a unit and is
+// followed by 16 bytes, so the first and the last one are readable.)  When only
+// aligned starts took whole units, the lanes of a warp did both loops one after the
+// other: 300 k ranks on DNA copies with leaves of 200 bytes and no stored leaf
+// counters took 343 us, now 117.
+__device__ __forceinline__ uint32_t leaf_count(const uint8_t* p, uint32_t o, uint32_t c) {
+  if (o == 0) return 0;
+  const uint32_t d = (uint32_t)((uintptr_t)p & 15), end = d + o, cc = c * 0x01010101u;
+  const uint8_t* u = p - d;
+  uint32_t acc = matches(unit_equals(u, cc, d, end)), y = 16;
+  for (; y + 64 <= end; y += 64) {
+    const uint4* q = (const uint4*)(u + y);
+    const uint4 v[4] = {q[0], q[1], q[2], q[3]};
+    uint32_t a = 0;
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+      a += __popc(__vcmpeq4(v[i].x, cc)) + __popc(__vcmpeq4(v[i].y, cc)) + __popc(__vcmpeq4(v[i].z, cc)) +
+           __popc(__vcmpeq4(v[i].w, cc));
+    acc += a >> 3;
+  }
+  for (; y < end; y += 16) acc += matches(unit_equals(u + y, cc, 0, end - y));
   return acc;
 }
 
 // Position of the j-th occurrence (j >= 1) of byte c in p[0, len), or kNoSlot.
 __device__ __forceinline__ uint32_t leaf_find(const uint8_t* p, uint32_t len, uint32_t c, uint32_t j) {
-  uint32_t x = 0;
-  const uint32_t cc = c * 0x01010101u;
-  if ((((uintptr_t)p) & 15) == 0) {
-    for (; x < len; x += 16) {
-      const uint4 v = *(const uint4*)(p + x);
-      const uint32_t e[4] = {__vcmpeq4(v.x, cc), __vcmpeq4(v.y, cc), __vcmpeq4(v.z, cc), __vcmpeq4(v.w, cc)};
-      const uint32_t k = (__popc(e[0]) + __popc(e[1]) + __popc(e[2]) + __popc(e[3])) >> 3;
-      if (k < j) {
-        j -= k;
+  const uint32_t d = (uint32_t)((uintptr_t)p & 15), end = d + len, cc = c * 0x01010101u;
+  const uint8_t* u = p - d;
+  for (uint32_t y = 0; y < end; y += 16) {
+    const uint4 v = *(const uint4*)(u + y);
+    Eq16 r{{__vcmpeq4(v.x, cc), __vcmpeq4(v.y, cc), __vcmpeq4(v.z, cc), __vcmpeq4(v.w, cc)}};
+    if (y < d) r = unit_equals(u, cc, d, 16);  // (the bytes before p)
+    const uint32_t k = matches(r);
+    if (k < j) {
+      j -= k;
+      continue;
+    }
+#pragma unroll
+    for (uint32_t q = 0; q < 4; q++) {
+      const uint32_t kq = __popc(r.e[q]) >> 3;
+      if (j > kq) {
+        j -= kq;
         continue;
       }
-#pragma unroll
-      for (uint32_t q = 0; q < 4; q++) {
-        const uint32_t kq = __popc(e[q]) >> 3;
-        if (j > kq) {
-          j -= kq;
-          continue;
-        }
-        uint32_t m = e[q] & 0x01010101u;
-        for (; j > 1; j--) m &= m - 1;
-        const uint32_t at = x + 4 * q + (__ffs(m) - 1) / 8;
-        return at < len ? at : kNoSlot;
-      }
-    }
-    return kNoSlot;
-  }
-  if ((((uintptr_t)p) & 3) == 0) {
-    const uint32_t* w = (const uint32_t*)p;
-    for (; x + 4 <= len; x += 4) {
-      const uint32_t k = __popc(__vcmpeq4(w[x >> 2], cc)) >> 3;
-      if (k >= j) break;  // the j-th is in this word: bytes below
-      j -= k;
+      uint32_t m = r.e[q] & 0x01010101u;
+      for (; j > 1; j--) m &= m - 1;
+      const uint32_t at = y + 4 * q + (__ffs(m) - 1) / 8 - d;
+      return at < len ? at : kNoSlot;
     }
   }
-  for (; x < len; x++)
-    if (p[x] == c && --j == 0) return x;
   return kNoSlot;
 }
 
@@ -541,13 +547,13 @@ __device__ __forceinline__ uint32_t leaf_find(const uint8_t* p, uint32_t len, ui
 __device__ __noinline__ uint32_t leaf_block_count(const uint8_t* leaf, const LevelView& v, uint32_t k, uint32_t c) {
   const uint32_t len = qlen(v, k);
   const uint2 r = v.rec[k];
-  if (r.x == kMarkedRec) return leaf_count(leaf + (uint64_t)r.y * v.b, len, c);
-  const uint32_t lj = qlen(v, r.x);
-  const uint32_t first = r.y + len <= lj ? len : lj - r.y;
-  const uint32_t rank = v.rec[r.x].y;  // the targets are marked: ranks rank, rank + 1
-  uint32_t acc = leaf_count(leaf + (uint64_t)rank * v.b + r.y, first, c);
-  if (first < len) acc += leaf_count(leaf + (uint64_t)(rank + 1) * v.b, len - first, c);
-  return acc;
+  // The two blocks have ranks r and r + 1, so that their text is one stretch of the
+  // leaf text, and the lanes of a warp, some at marked blocks and some at copies,
+  // count together: 1 M ranks on 64 MiB of DNA copies, leaves of 64 bytes, 336 us with
+  // up to three stretches, 250 now.
+  const uint8_t* p = leaf + (uint64_t)r.y * v.b;
+  if (r.x != kMarkedRec) p = leaf + (uint64_t)v.rec[r.x].y * v.b + r.y;
+  return leaf_count(p, len, c);
 }
 
 // Counts of byte c in the target of an unmarked last-level block before the window.

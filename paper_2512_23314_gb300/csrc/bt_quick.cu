@@ -772,7 +772,8 @@ static int search_tables(BuildCtx& ctx, QuickBuild& qb, const QGeo& g, uint64_t 
   auto power = [&](uint64_t e) { return t->q == Mersenne61::Q ? pow_mod(Mersenne61{}, t->B, e) : pow_mod(SmallMod{t->q}, t->B, e); };
   C.Bb = power(g.b);
   C.Br = C.r ? power(C.r) : 0;
-  const uint64_t bcap = pow2_from(2 * (nb + 2 * np)), pcap = pow2_from(2 * np), gcap = pow2_from(4 * ni);  // (2 ni: DNA 2 GiB 41.5 ms, not 40.8)
+  // (No more blocks are open, or halves of open pairs, than there are.)
+  const uint64_t bcap = pow2_from(2 * std::min(nb + 2 * np, g.c)), pcap = pow2_from(2 * np), gcap = pow2_from(4 * ni);  // (2 ni: DNA 2 GiB 41.5 ms, not 40.8)
   uint32_t fbits = 12;
   while ((1ull << fbits) < 16 * ni && fbits < 30) fbits++;
   R.bwords = 1u << (fbits - 5);

@@ -2044,7 +2044,8 @@ int level_pass(const M& m, BuildCtx& ctx, uint32_t l, uint64_t last_start, bool 
   v.stats[BT_ST_VERIFY_BYTES] = ctx.st_host->verify_bytes - ctx.verify_bytes;
   v.stats[BT_ST_COLLISIONS] = ctx.st_host->collisions - ctx.collisions;
   v.stats[BT_ST_CANDIDATES] = ldh.cands;
-  ctx.prev_cands = ldh.cands;
+  // (The scan of every window proposes none: room for a quarter of the windows.)
+  ctx.prev_cands = dense ? cov_l / 64 : ldh.cands;
   v.stats[BT_ST_HITS] = ldh.hits;
   ctx.verify_bytes = ctx.st_host->verify_bytes;
   ctx.collisions = ctx.st_host->collisions;

@@ -940,6 +940,7 @@ int quick_level(BuildCtx& ctx, QuickBuild& qb, uint32_t l, uint64_t last_start) 
   v.stats[BT_ST_COLLISIONS] = ctx.st_host->collisions - ctx.collisions;
   v.stats[BT_ST_CANDIDATES] = q0.nitems ? qb.qs_host->cands : 0;
   v.stats[BT_ST_HITS] = q0.nitems ? qb.qs_host->hits : 0;
+  ctx.prev_cands = v.stats[BT_ST_CANDIDATES];  // (a level of short blocks sizes its queue by it)
   ctx.verify_bytes = ctx.st_host->verify_bytes;
   ctx.collisions = ctx.st_host->collisions;
   if (ctx.st_host->error) {

@@ -319,9 +319,9 @@ struct __align__(16) CGram {  // F << 32 | offset; windows from `bound` on are o
 // the gram table (about 0.45 ns each with the whole GPU), and six for testing 32
 // windows (2.9 ns); the scan of every window costs about n / 26 of these (4.6 ms on
 // 256 MiB).  With a list long enough for two parts the first sixteenth is a
-// sample: above n / 512 there (versions and copies stay below n / 800), or given up
+// sample: above n / 700 there (versions and copies stay below n / 800), or given up
 // at n / 64, first grams are tried on the same sixteenth, and the better way takes
-// the rest unless both are above n / 256.  No search goes on beyond n / 16.  The
+// the rest unless both are above n / 256.  No search goes on beyond n / 32.  The
 // registration is given up too: keys that share a gram stand in one run of slots,
 // which each passes (80 ns a slot: 4 M keys of two-letter text took 30 ms).
 enum ChaseState : uint32_t {
@@ -331,9 +331,9 @@ enum ChaseState : uint32_t {
   kGiveUp = 3,
 };
 constexpr uint32_t kWalkWork = 1, kTestWork = 6;
-__host__ __device__ inline uint64_t work_sample(uint64_t n) { return n / 512; }
+__host__ __device__ inline uint64_t work_sample(uint64_t n) { return n / 700; }
 __host__ __device__ inline uint64_t work_few(uint64_t n) { return n / 256 + 4096; }
-__host__ __device__ inline uint64_t work_most(uint64_t n, bool sample) { return (sample ? n / 64 : n / 16) + 4096; }
+__host__ __device__ inline uint64_t work_most(uint64_t n, bool sample) { return (sample ? n / 64 : n / 32) + 4096; }
 constexpr uint32_t kLongProbe = 64;  // slots; a walk counts from there on
 __host__ __device__ inline uint64_t probes_most(uint64_t nitems) { return 4 * nitems + (1u << 16); }
 
@@ -581,7 +581,9 @@ __device__ __forceinline__ void chase_test(const M& m, const PrefixAt<M>& H, con
 constexpr uint32_t kChaseTile = 256;                 // entries per warp and step, eight per lane
 constexpr uint32_t kHitQ = kChaseTile + 32, kCandQ = 64;
 constexpr uint32_t kChaseBitWords = 4096;            // bitmap kept in shared memory up to 16 KiB
-constexpr uint32_t kChaseReport = 256;               // work of a warp before it adds it to the level's
+// Work of a warp before it adds it to the level's: often enough that what all warps
+// do meanwhile is no more than the limit, or 64.
+constexpr uint32_t kChaseReport = 256, kChaseReportOften = 64;
 
 // hq, cq: the warp's queues; gq: for first grams, the distance of each hit to
 // the entry before it; bits: the bitmap (shared or global memory).  Above a work of
@@ -598,6 +600,7 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
   const uint64_t fp_tail = C.qs->fp_tail;
   const uint32_t given_up = *(volatile unsigned int*)&C.qs->redo;  // (before, or just now: looked at with the first tile)
   uint32_t ncand = 0, nhit = 0, work = 0;  // ncand, work (since the last report): warp-uniform
+  const uint32_t every = limit >= kChaseReport * (w.n / 32) ? kChaseReport : kChaseReportOften;
   bool stop = false;
   auto report = [&]() {
     unsigned long long all = 0;
@@ -661,7 +664,7 @@ __device__ __forceinline__ void chase_scan(const M& m, const PrefixAt<M>& H, con
       }
     }
     work += kWalkWork;
-    if (work >= kChaseReport) {
+    if (work >= every) {
       report();
       if (stop) live = false, hn = cn = 0;
     }

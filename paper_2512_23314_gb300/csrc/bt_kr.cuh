@@ -173,10 +173,17 @@ struct PrefixConst<Mersenne61> {
   uint64_t B, B32;
   ChunkHash<Mersenne61> hash;
   uint64_t ones[32], inv[32];  // [r]: the sum of B^31 .. B^(32-r); B^-(32-r)
+  // (One inverse and products: a build makes this once per level, and again where
+  // a search is given up; 32 inverses took 10 us of host time.)
   PrefixConst(const Mersenne61& m, uint64_t B_) : B(B_), B32(pow_mod(m, B_, 32)), hash(m, B_) {
+    uint64_t power[32];
+    power[0] = 1;
+    for (int i = 1; i < 32; i++) power[i] = m.mul(power[i - 1], B);
     ones[0] = 0;
-    for (int r = 1; r < 32; r++) ones[r] = m.add(ones[r - 1], pow_mod(m, B, 32 - r));
-    for (int r = 0; r < 32; r++) inv[r] = pow_mod(m, pow_mod(m, B, 32 - r), Mersenne61::Q - 2);
+    for (int r = 1; r < 32; r++) ones[r] = m.add(ones[r - 1], power[32 - r]);
+    const uint64_t step = pow_mod(m, B, Mersenne61::Q - 2);
+    inv[31] = step;
+    for (int r = 30; r >= 0; r--) inv[r] = m.mul(inv[r + 1], step);
   }
   __device__ __forceinline__ uint64_t at(const Mersenne61& m, const uint8_t* T, uint64_t n, const uint64_t* Hs,
                                          bool aligned, uint64_t p) const {

@@ -998,8 +998,13 @@ __device__ bool quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, co
     // first grams too, then the rest by one of them, or every window.
     enum { kBySample, kByBoth, kByRest };
     const uint32_t total = C.nsel, split = total > (1u << 16) ? (total / 16) & ~(8 * kChaseTile - 1) : 0;
-    const uint64_t few = split ? work_few(n) : work_most(n, false);
-    uint64_t limit = work_most(n, split != 0), newest = 0, before = 0;
+    // (The scan of every window costs a CTA more of these steps than it does the
+    // whole GPU, so each bound is four times as high.  256 documents of 512 KiB, with
+    // the bounds 1, 2, 4, 8 times as high and with none: 100 words 26, 19, 16, 16, 17
+    // ms, random bits 22, 13, 13, 13, 14, two-letter runs 31, 32, 33, 54, 67, ten words
+    // 45, 47, 56, 44, 45.)
+    const uint64_t wn = 4 * n, few = split ? work_few(wn) : work_most(wn, false);
+    uint64_t limit = work_most(wn, split != 0), newest = 0, before = 0;
     uint32_t step = kBySample;
     bool enter = true;
     for (bool again = false;; again = true) {
@@ -1028,7 +1033,7 @@ __device__ bool quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, co
       const uint64_t seen = *(volatile unsigned long long*)&K.qs->work;
       bool first = K.first;
       gsync(C.grp);
-      if (step == kBySample && !over && (!split || seen <= work_sample(n))) {
+      if (step == kBySample && !over && (!split || seen <= work_sample(wn))) {
         if (!split) break;
         step = kByRest;
         enter = false;
@@ -1048,7 +1053,7 @@ __device__ bool quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, co
         break;
       }
       before = seen;
-      limit = seen + (step == kByBoth ? few : work_most(n, false));
+      limit = seen + (step == kByBoth ? few : work_most(wn, false));
       if (threadIdx.x == 0) {
         C.chase.first = first;
         C.chase.probes = ~0ull;

@@ -1620,17 +1620,6 @@ unsigned sm_count() {
   return (unsigned)n;
 }
 
-// CTAs of a kernel that fit on one SM at once (at least 1).
-template <class F>
-unsigned resident_ctas(F* fn, int threads, size_t smem) {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    n = 1;
-  }
-  return (unsigned)n;
-}
-
 // Opt a kernel in to more than 48 KiB of dynamic shared memory, once per
 // device (the attribute is a property of the function on each device; the
 // template parameter gives every kernel its own flags).

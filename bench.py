@@ -433,7 +433,6 @@ def measure_batch(ndocs: int = 8192, min_len: int = 4 << 10, max_len: int = 16 <
 
     # Warm-up on the whole batch (the first call maps its memory).
     warm = bt.bt_build_batch(*args, o_kernel, nworkers=nworkers)
-    tuning = bt.bt_batch_report()
     for h in warm:
         bt.bt_free(h)
     kernel_s, kernel_blobs, rep, cyc = batch_arm(o_kernel)
@@ -461,8 +460,7 @@ def measure_batch(ndocs: int = 8192, min_len: int = 4 << 10, max_len: int = 16 <
             "speedup_vs_plain": plain_s / kernel_s, "speedup_vs_workers": workers_s / kernel_s,
             "workers_mb_per_s": total / workers_s / 1e6, "plain_mb_per_s": total / plain_s / 1e6,
             "identical_output_sample": {"docs": len(sample), "equal": bool(same)},
-            "kernel": rep, "autotune": {k: tuning[k] for k in ("threads", "ctas_per_sm", "chunk",
-                                                                "tuning_trials")},
+            "kernel": rep,
             "kernel_phase_share": dict(zip(phases, share)) if share else None,
             "nworkers": nworkers}
 
@@ -578,8 +576,9 @@ def scan_roofline(prof: dict, step_ms_total: float, traffic_ratio: float | None)
     achieved = scan["bytes"] / (scan["ms"] / 1e3) / 1e9 if scan["ms"] > 0 else None
     per_launch_bytes = scan["bytes"] / max(1, scan["launches"])
     return {
-        "kernel": "window search of a level (k_chase_scan and its bounds; k_scan_anchor, k_hits and "
-                  "k_candidates on levels of blocks under 27 bytes)",
+        "kernel": "a level's leftmost occurrences (bounds, comparisons and the search of the open keys; "
+                  "k_scan_anchor, k_hits and k_candidates on levels of blocks under 27 bytes): covered bytes "
+                  "per second, most of which are settled without being read",
         "bound": "hbm",
         "achieved": achieved,
         "peak": hbm if hbm else 6800.0,

@@ -82,8 +82,9 @@ typedef struct {
                                   other passes.                                */
 } bt_opts;
 
-/* flags: BT_FLAG_DENSE_SCAN probes the table at every window position instead
- * of the anchored scan (a diagnostic; both give the same tree).
+/* flags: BT_FLAG_DENSE_SCAN probes the table at every window position of every
+ * level (a diagnostic; the same tree.  Without it single levels go that way: those
+ * whose open keys share too few grams).
  * BT_FLAG_TINY_QUEUE caps the anchored scan's queue of proposed windows at 64
  * entries, so that nearly every anchored level takes the overflow path, a second scan
  * that tests the windows in place (a test hook; the same tree again). */
@@ -155,11 +156,13 @@ int bt_build_ex(const uint8_t* text, uint64_t n, uint32_t sigma, uint32_t tau,
  *
  * Documents of at most 2^30 bytes and 40 levels are built by one persistent
  * kernel launch per size class (the paper's section 3 levels and section 3.1
- * pass, per document): each CTA takes the next document from a device work
- * queue (longest first) and builds its whole tree -- alphabet, prefix
- * fingerprints, every level's scan, verification, marks, pointers and split,
- * pruning and counters -- level by level with barriers of the CTA, without
- * any host round trip.  The trees of one call share one device allocation,
+ * pass, per document): each CTA -- or, for few long documents, each cluster of
+ * CTAs; several narrow CTAs share an SM for short ones -- takes the next
+ * document from a device work queue (longest first) and builds its whole tree
+ * -- alphabet, prefix fingerprints, every level's pass by first occurrences or
+ * windows, verification, marks, pointers and split, pruning and counters --
+ * level by level with barriers of the CTA or cluster, without any host round
+ * trip.  The trees of one call share one device allocation,
  * released when the last of them is freed.  Larger documents, and every
  * document when opts->flags has BT_FLAG_BATCH_WORKERS, are built with
  * bt_build_ex on `nworkers` host threads (0: 8), one CUDA stream each.
@@ -296,8 +299,9 @@ const char* bt_strerror(int status);
  * window-scan, prefix-fingerprint, verification and counter kernels of every
  * build.  bt_profile_read aggregates, per kernel name: launches, total
  * milliseconds between the events, and the algorithmic bytes those launches
- * process (the covered bytes of the level for the window scan, n for the
- * prefix fingerprints, the compared bytes for verification).  It waits for
+ * process (the covered bytes of the level for the window scan, counted by its
+ * first scope -- the search of a level's open keys is a second one with none --,
+ * n for the prefix fingerprints, the compared bytes for verification).  It waits for
  * the recorded events.  Profiling state is process-wide; reads and resets
  * must not race with builds that record.
  */

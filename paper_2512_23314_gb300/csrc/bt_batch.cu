@@ -1663,7 +1663,9 @@ __device__ void build_doc(const M& m, const PrefixConst<M>& PC, const KrPow& pw,
 // 64 registers per thread: one CTA of 1024 threads per SM, or several narrower
 // ones (launch_shape).  A document belongs to a CTA, or to a cluster of them.
 // Compiled apart for the two: one kernel for both spilled 2000 bytes of stores and
-// 4160 of loads (-Xptxas -v), these 344 and 780 (one CTA), 972 and 2524 (cluster).
+// 4160 of loads (-Xptxas -v, modulus 2^61 - 1), these 344 and 780 (one CTA) and 972
+// and 2524 (cluster); with the bounded search of the open keys 712 and 1500, 932 and
+// 2244.
 template <class M, class GRP>
 __global__ void __launch_bounds__(kMaxBThreads, 1) k_batch(const __grid_constant__ BParams P, M m,
                                                            const __grid_constant__ PrefixConst<M> PC,
@@ -2029,9 +2031,9 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
       if (grid == 0) grid = 1;
     }
     // Fewer documents than SMs: a cluster of CTAs for each (not with a bound
-    // on the CTAs, which leaves SMs to other work).  One document of DNA copies
-    // by 1, 4, 8, 16 CTAs: 16 KiB 559, 664, 665, 675 us, 256 KiB 1319, 1100,
-    // 1065, 1059, 1 MiB 3280, 1769, 1522, 1418 -- from 128 KiB a document on.
+    // on the CTAs, which leaves SMs to other work).  One document of DNA copies,
+    // tau 2, leaf 32, by 1 and 16 CTAs: 130 KiB 1357 and 1355 us, 256 KiB 1539 and
+    // 1165, 1 MiB 4513 and 2163 -- from 128 KiB a document on.
     uint64_t bytes = 0;
     for (uint32_t q2 = r; q2 < e; q2++) bytes += order[q2]->n;
     uint32_t group = 1;
@@ -2144,7 +2146,7 @@ int run_batch(const M& m, const uint8_t* const* texts, const uint32_t* taus, con
 }
 
 // Texts up to this long are built by one CTA in one launch: at 4 KiB and four
-// levels it takes 240 us, some fifty launches and four round trips 350 us.  The
+// levels it takes 160 us, some fifty launches and four round trips 350 us.  The
 // line lies where one CTA is too slow for the counters of many symbols: random
 // bytes take about as long both ways at 16 KiB (DNA copies still half at 64 KiB).
 constexpr uint64_t kSoloText = 16u << 10;

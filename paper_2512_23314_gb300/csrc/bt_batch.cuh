@@ -2,7 +2,8 @@
 // the batched build (bt_batch.cu).
 //
 // A batch is built by one persistent kernel per size class of documents.
-// Every CTA (for few long documents: every cluster of CTAs) takes the next
+// Every CTA (one to an SM, narrower ones for short documents; for few long
+// documents: every cluster of CTAs) takes the next
 // document from a device work queue (an atomic
 // counter over the documents in decreasing length) and builds that
 // document's whole tree by itself, level by level (section 3's levels, the

@@ -2,8 +2,9 @@
 //
 // Device data layout (one tree, all in HBM):
 //   text        u8[n]          the input (the caller's device buffer, or a copy)
-//   H           u64[n + 1]     Karp-Rabin prefix fingerprints H(p) (section 2),
-//                              during construction only
+//   Hs          u64[n/32 + 1]  Karp-Rabin prefix fingerprints H(32 j) (section 2),
+//                              during construction only; at every position
+//                              where a level is scanned by windows
 //   per level l (blocks in text order):
 //     mw        u32[ceil(c/32)] mark bits, bit k%32 of word k/32
 //     mr        u32[words + 1] exclusive prefix popcounts of mw

@@ -1578,7 +1578,8 @@ __global__ void k_reset_jobs(unsigned int* mismatch, uint64_t c, LevelDev* ld) {
   }
 }
 
-// Gram length w: half the block, at most 16; anchor range W <= 64.
+// Gram length w: half the block (at most 13 bytes: longer blocks have no anchors);
+// anchor range W.
 // Each gram is selected with probability 2^-sbits, so a key has no selected
 // gram among its first npos positions with probability (1 - 2^-sbits)^npos;
 // sbits is the largest value in 0..3 that leaves well under one such key per

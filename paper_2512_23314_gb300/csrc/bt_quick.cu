@@ -22,7 +22,7 @@
 // instead of every place where any key's first gram occurs.  Windows tested
 // by the levels of a build: 256 MiB of versioned text 41.3 M before (14.5 M of
 // them matched a key), 7.3 M now; 2 GiB of DNA copies 469 M before, 37.5 M now.
-// The builds: 16.2 -> 11.5 ms and 172 -> 91 ms (export included).
+// The builds: 16.2 -> 6.7 ms and 178 -> 42 ms (export included).
 //
 // Selection.  A gram is selected when the least of the 13 hashes of its
 // 4-byte substrings is the first or the last of them (a closed syncmer,

@@ -1003,8 +1003,8 @@ __device__ bool quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, co
     // the bounds 1, 2, 4, 8 times as high and with none: 100 words 26, 19, 16, 16, 17
     // ms, random bits 22, 13, 13, 13, 14, two-letter runs 31, 32, 33, 54, 67, ten words
     // 45, 47, 56, 44, 45.)
-    const uint64_t wn = 4 * n, few = split ? work_few(wn) : work_most(wn, false);
-    uint64_t limit = work_most(wn, split != 0), newest = 0, before = 0;
+    const uint64_t wn = 4 * n, least = least_work_cta(n), few = split ? work_few(wn) : work_most(wn, false, least);
+    uint64_t limit = work_most(wn, split != 0, least), newest = 0, before = 0;
     uint32_t step = kBySample;
     bool enter = true;
     for (bool again = false;; again = true) {
@@ -1053,7 +1053,7 @@ __device__ bool quick_keys(const M& m, const PrefixConst<M>& PC, Cta<GRP>& C, co
         break;
       }
       before = seen;
-      limit = seen + (step == kByBoth ? few : work_most(wn, false));
+      limit = seen + (step == kByBoth ? few : work_most(wn, false, least));
       if (threadIdx.x == 0) {
         C.chase.first = first;
         C.chase.probes = ~0ull;

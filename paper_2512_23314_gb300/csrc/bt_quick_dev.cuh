@@ -321,7 +321,13 @@ struct __align__(16) CGram {  // F << 32 | offset; windows from `bound` on are o
 // 256 MiB).  With a list long enough for two parts the first sixteenth is a
 // sample: above n / 700 there (versions and copies stay below n / 800), or given up
 // at n / 64, first grams are tried on the same sixteenth, and the better way takes
-// the rest unless both are above n / 256.  No search goes on beyond n / 32.  The
+// the rest unless both are above n / 256.  No search goes on beyond n / 32.
+// Giving up has a price of its own, so no bound but the sample's comparisons is below
+// a fixed one.  On the grid 2^21 steps: with bounds of n / 32 + 4096 two-letter runs of
+// 256 KiB took 3.11 ms and random bits of 1 MiB 2.09, now 1.66 and 1.70 (1.65 and 1.68
+// without bounds); such runs of 512 KiB by 2^16, 2^18, 2^20: 3.24, 2.21, 2.08.  For one
+// CTA it is 2^17 on documents below 96 KiB and 2^12 on longer ones: 256 documents of
+// two-letter runs by 2^12 and 2^15, 32 KiB 5.6 and 4.7 ms, 128 KiB 9.8 and 14.7.  The
 // registration is given up too: keys that share a gram stand in one run of slots,
 // which each passes (80 ns a slot: 4 M keys of two-letter text took 30 ms).
 enum ChaseState : uint32_t {
@@ -333,7 +339,12 @@ enum ChaseState : uint32_t {
 constexpr uint32_t kWalkWork = 1, kTestWork = 6;
 __host__ __device__ inline uint64_t work_sample(uint64_t n) { return n / 700; }
 __host__ __device__ inline uint64_t work_few(uint64_t n) { return n / 256 + 4096; }
-__host__ __device__ inline uint64_t work_most(uint64_t n, bool sample) { return (sample ? n / 64 : n / 32) + 4096; }
+__host__ __device__ inline uint64_t work_most(uint64_t n, bool sample, uint64_t least) {
+  const uint64_t most = sample ? n / 64 : n / 32;
+  return most > least ? most : least;
+}
+constexpr uint64_t kLeastWork = 1u << 21;
+__host__ __device__ inline uint64_t least_work_cta(uint64_t n) { return n < (96u << 10) ? 1u << 17 : 1u << 12; }
 constexpr uint32_t kLongProbe = 64;  // slots; a walk counts from there on
 __host__ __device__ inline uint64_t probes_most(uint64_t nitems) { return 4 * nitems + (1u << 16); }
 

@@ -46,7 +46,7 @@ def test_against_the_oracle(n, tau, leaf):
 
 @pytest.mark.parametrize("n", [(9 << 20) + 77, 12 << 20])
 def test_lists_in_two_parts(n):
-    """More than 2^20 list entries: a sample of the list decides."""
+    """Around the length from which a sample of the list decides (2^21 entries)."""
     for i, text in enumerate(kinds(n, n % 1000)):
         d = torch.from_numpy(text).cuda()
         t = bt.Tree(d, 256, 4, 32)
@@ -71,6 +71,26 @@ def test_batches(docs, modulus):
         finally:
             for h in hs:
                 bt.bt_free(h)
+
+
+@pytest.mark.parametrize("n", [(2 << 20) + 5, (8 << 20) + 3, 40 << 20])
+def test_bounds_of_the_search(n):
+    """Around the least bound (2^21 steps) and above it, with lists of one part and (40 MiB) of two."""
+    for i, text in enumerate(kinds(n, n % 999)):
+        d = torch.from_numpy(text).cuda()
+        dense = bt.Tree(d, 256, 4, 32, bt.BuildOptions(dense_scan=True)).export()
+        assert bt.Tree(d, 256, 4, 32).export() == dense, i
+
+
+def test_windows_of_short_texts():
+    """A short text's search is not given up: its steps are cheaper than a second way (two-letter runs of 256 KiB
+    were given up and took twice as long).  Levels given up go by every window and test few (7 in all), this
+    search tests over a million on 7 levels."""
+    n = 256 << 10
+    r = np.random.default_rng(7)
+    text = np.repeat(r.integers(97, 99, n // 20, dtype=np.uint8), r.integers(1, 90, n // 20))[:n].copy()
+    t = bt.Tree(torch.from_numpy(text).cuda(), 256, 4, 32)
+    assert sum(s["candidates"] for s in t.stats()) > n
 
 
 def test_windows_per_position():
